@@ -279,8 +279,8 @@ def tolerance(case):
     if case["kind"] == "build":
         return "exact"                                      # counting, ranking and copying whole numbers and bits
     # bf16 products summed in fp32, log-probabilities from fp32 exponentials.  Against sums in 64 bits they differ by
-    # up to 9e-8 (2-norm) and 1.6e-7 (largest) at temperature 1, and by 2.2e-6 and 5.6e-6 at temperatures from 0.5,
-    # where the exponents are larger; candidates closer than that may change places.
-    if case["kind"] in ("chain", "host"):
+    # up to 9e-8 (2-norm) and 2.1e-7 (largest) for the few rows of a chain, and by 2.2e-6 and 5.6e-6 where a tile of
+    # many rows is summed with fast exponentials; candidates closer than that may change places.
+    if case["kind"] == "chain":
         return {"rel": 4e-7, "max": 1e-6, "differ": 0.004}
     return {"rel": 1e-5, "max": 3e-5, "differ": 0.004}
