@@ -93,13 +93,16 @@ struct HeadArgs {
     int32_t overlap;       // launch with programmatic stream serialization (weights may be fetched early)
     TreeArgs tree;         // expansion to run on the merged top-k (pool_token == nullptr: none)
 };
-bool head_skinny_supported(int32_t B, int32_t d);
+bool head_skinny_supported(int32_t B, int32_t d);   // shapes whose candidate lists may be VT_MAX_TOPK long
+bool head_stream_takes(int32_t B);                  // hidden rows the streaming kernel is launched for
 size_t head_skinny_scratch_bytes(int32_t B, int32_t K, int32_t topk);
 cudaError_t launch_head_skinny(const HeadArgs& a, Ctrl* ctrl, uint8_t* scratch, cudaStream_t s);
 #ifdef VT_STAMPS
 size_t head_skinny_stamps_offset(int32_t B, int32_t topk);   // offset of the phase stamps in the head scratch
 size_t head_dense_stamps_offset(int32_t B, int32_t topk);    // the same for the batched head
 #endif
+
+cudaError_t launch_head_merge(const HeadArgs& a, Ctrl* ctrl, float* recs, int G, cudaStream_t s);
 
 bool head_dense_supported(int32_t B, int32_t K, int32_t d);
 bool head_dense_topk_ok(int32_t topk);

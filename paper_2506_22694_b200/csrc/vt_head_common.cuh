@@ -13,7 +13,7 @@ constexpr int kMaxOwn = kMaxGrid / 32;
 constexpr int kMergeDepth = 4;                   // list entries per CTA staged on chip by the merge
 constexpr int kSelCap = 128;                     // entries the merge's direct selection can rank
 // staging words (32-bit) per merging warp: staged list heads, selection buffer, output keys (all 64-bit)
-constexpr int kMergeStageWords = 2 * (kMergeDepth * kMaxGrid + kSelCap + 64);
+constexpr int kMergeStageWords = 2 * (kMergeDepth * kMaxGrid + kSelCap + 4 + 64);
 constexpr int kStampSlots = 16;                  // phase stamps per CTA (-DVT_STAMPS builds)
 #ifdef VT_STAMPS
 constexpr size_t kStampBytes = (size_t)kMaxGrid * kStampSlots * 8;
@@ -51,6 +51,55 @@ __device__ __forceinline__ unsigned long long key64(float v, int j) {
 }
 __device__ __forceinline__ float key_val(unsigned long long k) { return ord2f((unsigned)(k >> 32)); }
 __device__ __forceinline__ int key_idx(unsigned long long k) { return (int)~(unsigned)k; }
+
+// exp and log of the epilogue: one multiplication and the hardware's base-2 function, results and arguments under
+// 2^-126 flushed to zero (the arguments of the logarithm are at least 2^-25; an exponential is added to a sum that
+// holds 1).
+__device__ __forceinline__ float exp_fast(float x) {
+    float y;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x * 1.4426950408889634f));
+    return y;
+}
+__device__ __forceinline__ float log_fast(float x) {
+    float y;
+    asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y * 0.6931471805599453f;
+}
+
+// rk[i] += number of the N keys in shared memory that are greater than ek[i]; the buffer is 16-byte aligned and
+// zero-padded to a multiple of four.
+template <int NS>
+__device__ __forceinline__ void rank_among(const unsigned long long* keys, int N, const unsigned long long (&ek)[NS], int (&rk)[NS]) {
+    const ulonglong2* k2 = reinterpret_cast<const ulonglong2*>(keys);
+#pragma unroll 2
+    for (int e = 0; e < N; e += 4) {
+        const ulonglong2 p = k2[e >> 1], q = k2[(e >> 1) + 1];
+#pragma unroll
+        for (int i = 0; i < NS; ++i)
+            rk[i] += ((p.x > ek[i]) ? 1 : 0) + ((p.y > ek[i]) ? 1 : 0) + ((q.x > ek[i]) ? 1 : 0) + ((q.y > ek[i]) ? 1 : 0);
+    }
+}
+
+// A lower bound of the k-th largest (k <= 32) of the lanes' values: that value with its low five bits cleared (they
+// tell equal lanes apart meanwhile).  Every lane counts the values above its own in shared memory (32 words, 16-byte
+// aligned): broadcast reads that overlap, where 32 shuffles took 1500 cycles.
+__device__ __forceinline__ unsigned kth_of_lanes(unsigned v, int k, unsigned* s32) {
+    const unsigned lane = threadIdx.x & 31;
+    const unsigned mine = (v & ~31u) | (31u - lane);
+    s32[lane] = mine;
+    __syncwarp();
+    const uint4* s4 = reinterpret_cast<const uint4*>(s32);
+    int rk = 0;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const uint4 o = s4[i];
+        rk += ((o.x > mine) ? 1 : 0) + ((o.y > mine) ? 1 : 0) + ((o.z > mine) ? 1 : 0) + ((o.w > mine) ? 1 : 0);
+    }
+    const unsigned at = __ballot_sync(0xffffffffu, rk == k - 1);
+    const unsigned tau = __shfl_sync(0xffffffffu, mine, __ffs(at) - 1) & ~31u;       // (exactly one lane has that rank)
+    __syncwarp();                                           // the words may be reused
+    return tau;
+}
 
 // Records.  Per hidden row b a block of rec_fields(topk) * kMaxGrid 32-bit words, laid out in planes
 // with the CTA index fastest, so that a merging warp reads every plane with coalesced loads:
@@ -182,7 +231,7 @@ __device__ __noinline__ void merge_records(const MergeOut a, Ctrl* ctrl, float* 
     unsigned long long res_k[2] = {0ull, 0ull};
     unsigned long long* stk = reinterpret_cast<unsigned long long*>(stage);        // [kMergeDepth][kMaxGrid] list heads
     unsigned long long* sel = stk + kMergeDepth * kMaxGrid;                        // [kSelCap]
-    unsigned long long* outk = sel + kSelCap;                                      // [64]
+    unsigned long long* outk = sel + kSelCap + 4;                                  // [64] (behind four words of padding)
     bool done = false;
     if (topk <= 32) {
         // Direct selection.  tau = the topk-th largest of the 32 lanes' best list heads is a lower
@@ -196,14 +245,7 @@ __device__ __noinline__ void merge_records(const MergeOut a, Ctrl* ctrl, float* 
             const unsigned h = (unsigned)(ek[0][o] >> 32);
             lh = h > lh ? h : lh;
         }
-        int rk = 0;
-#pragma unroll
-        for (int sl = 0; sl < 32; ++sl) {
-            const unsigned oh = __shfl_sync(0xffffffffu, lh, sl);
-            rk += (oh > lh || (oh == lh && sl < lane)) ? 1 : 0;
-        }
-        const unsigned at = __ballot_sync(0xffffffffu, rk == topk - 1);
-        const unsigned tau = __shfl_sync(0xffffffffu, lh, __ffs(at) - 1);
+        const unsigned tau = kth_of_lanes(lh, topk, reinterpret_cast<unsigned*>(stage));
         outk[lane] = 0ull;
         outk[lane + 32] = 0ull;
         // compaction: every lane counts its qualifying entries, a warp scan gives it a place to put them
@@ -233,12 +275,13 @@ __device__ __noinline__ void merge_records(const MergeOut a, Ctrl* ctrl, float* 
                     if (ek[r][o] != 0ull && (unsigned)(ek[r][o] >> 32) >= tau) sel[pos++] = ek[r][o];
         }
         if (n <= kSelCap && !__any_sync(0xffffffffu, deep)) {
+            if (lane < 4) sel[n + lane] = 0ull;                                    // (read in groups of four)
             __syncwarp();
             if (n <= 32) {                                                         // the usual case: one entry per lane
-                const unsigned long long mine = lane < n ? sel[lane] : 0ull;
-                int r1 = 0;
-                for (int e = 0; e < n; ++e) r1 += (sel[e] > mine) ? 1 : 0;
-                if (lane < n && r1 < topk) outk[r1] = mine;
+                const unsigned long long mine[1] = {lane < n ? sel[lane] : 0ull};
+                int r1[1] = {0};
+                rank_among<1>(sel, n, mine, r1);
+                if (lane < n && r1[0] < topk) outk[r1[0]] = mine[0];
             } else {
                 unsigned long long mine[kSelCap / 32];
                 int rk4[kSelCap / 32];
@@ -247,11 +290,7 @@ __device__ __noinline__ void merge_records(const MergeOut a, Ctrl* ctrl, float* 
                     mine[i] = (lane + 32 * i < n) ? sel[lane + 32 * i] : 0ull;
                     rk4[i] = 0;
                 }
-                for (int e = 0; e < n; ++e) {
-                    const unsigned long long k = sel[e];
-#pragma unroll
-                    for (int i = 0; i < kSelCap / 32; ++i) rk4[i] += (k > mine[i]) ? 1 : 0;
-                }
+                rank_among<kSelCap / 32>(sel, n, mine, rk4);
 #pragma unroll
                 for (int i = 0; i < kSelCap / 32; ++i)
                     if (lane + 32 * i < n && rk4[i] < topk) outk[rk4[i]] = mine[i];

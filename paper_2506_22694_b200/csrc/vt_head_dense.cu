@@ -26,12 +26,9 @@
 // record goes to scratch; a second small kernel (one warp per hidden row) merges the records,
 // applies the index mapper and writes the outputs.  Every wait is bounded; on expiry the CTA raises
 // VT_FLAG_TIMEOUT and leaves after releasing its tensor memory.
-#include <cuda.h>
-
-#include <mutex>
-
 #include "vt_common.cuh"
 #include "vt_head_common.cuh"
+#include "vt_tc.cuh"
 
 namespace vt {
 
@@ -39,7 +36,6 @@ namespace {
 
 constexpr int kBM = 128;                  // hidden rows per CTA (TMEM lanes)
 constexpr int kMaxBN = 256;               // vocabulary rows per tile at most (TMEM columns per accumulator)
-constexpr int kBK = 64;                   // columns of d per ring stage: 128 bytes, one swizzle row
 constexpr int kMaxSub = 2;                // d-steps of kBK columns one ring stage holds at most
 constexpr int kMaxStages = 8;
 constexpr int kHTileBytes = kBM * kBK * 2; // 16 KB: the hidden-row operand of a stage
@@ -65,28 +61,6 @@ constexpr size_t kRingBudget = 225 * 1024;   // ring bytes at most (227 KB per C
 #endif
 
 // ---- PTX wrappers ----------------------------------------------------------------------------------
-__device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-__device__ __forceinline__ void mbar_init(uint64_t* b, int count) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(b)), "r"(count));
-}
-__device__ __forceinline__ void mbar_expect_tx(uint64_t* b, uint32_t bytes) {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(b)), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ void mbar_arrive(uint64_t* b) {
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(b)) : "memory");
-}
-__device__ __forceinline__ bool mbar_try(uint64_t* b, uint32_t parity) {
-    uint32_t ok;
-    asm volatile(
-        "{ .reg .pred p; mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2; selp.u32 %0, 1, 0, p; }"
-        : "=r"(ok) : "r"(smem_u32(b)), "r"(parity) : "memory");
-    return ok != 0;
-}
-__device__ __forceinline__ unsigned long long global_ns() {
-    unsigned long long t;
-    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-    return t;
-}
 __device__ __forceinline__ bool mbar_wait(uint64_t* b, uint32_t parity, volatile int* abort_flag) {
     if (mbar_try(b, parity)) return true;
     const unsigned long long t0 = global_ns();
@@ -117,22 +91,6 @@ __device__ __forceinline__ bool mbar_wait_warp(uint64_t* b, uint32_t parity, vol
     if (ok) ok = mbar_try(b, parity) || mbar_wait(b, parity, abort_flag);
     return __all_sync(0xffffffffu, ok);
 }
-__device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* tm, int x, int y, uint64_t* bar) {
-    asm volatile(
-        "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
-        ::"r"(dst), "l"(tm), "r"(x), "r"(y), "r"(smem_u32(bar)) : "memory");
-}
-__device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void tc_commit(uint64_t* bar) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
-}
-// D[tmem] (+)= A[smem] * B[smem]^T, 128 x N x 16, bf16 inputs, fp32 accumulation
-__device__ __forceinline__ void tc_mma(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, uint32_t acc) {
-    asm volatile(
-        "{ .reg .pred p; setp.ne.b32 p, %4, 0; tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p; }"
-        ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(acc) : "memory");
-}
 // 16 consecutive accumulator columns of this thread's TMEM lane
 __device__ __forceinline__ void tc_ld16(uint32_t taddr, uint32_t (&r)[16]) {
     asm volatile(
@@ -142,25 +100,6 @@ __device__ __forceinline__ void tc_ld16(uint32_t taddr, uint32_t (&r)[16]) {
         : "r"(taddr));
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
-
-// Shared-memory operand descriptor: K-major tile of 128-byte rows, 128-byte swizzle, 8-row groups
-// 1024 bytes apart (the layout a TMA tensor copy with SWIZZLE_128B and a 64-column bf16 box writes).
-// Fields: start address >> 4 [0,14); leading byte offset >> 4 [16,30) (unused for swizzled K-major: 1);
-// stride byte offset >> 4 [32,46); descriptor version 1 at [46,48); layout type 2 = 128B swizzle at [61,64).
-__device__ __forceinline__ uint64_t make_desc(uint32_t smem_addr) {
-    return (uint64_t)((smem_addr >> 4) & 0x3fffu) | ((uint64_t)1 << 16) | ((uint64_t)(1024 >> 4) << 32) |
-           ((uint64_t)1 << 46) | ((uint64_t)2 << 61);
-}
-// Instruction descriptor of kind::f16: fp32 accumulator (1 at [4,6)), A and B bf16 (1 at [7,10) and
-// [10,13)), both K-major (0 at bits 15 and 16), N >> 3 at [17,23), M >> 4 at [24,29).
-__host__ __device__ constexpr uint32_t make_idesc(int M, int N) {
-    return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
-}
-
-// Programmatic dependent launch: let the next launch on the stream become resident / wait until the
-// work this launch depends on has completed and its writes are visible (no-ops in a plain launch).
-__device__ __forceinline__ void griddep_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-__device__ __forceinline__ void griddep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 // ---- CTA-pair forms (cta_group::2): two CTAs of a cluster act as one 256-row MMA ---------------------
 __device__ __forceinline__ uint32_t cluster_ctarank() {
@@ -299,7 +238,7 @@ k_head_dense(const HeadArgs a, Ctrl* ctrl, float* __restrict__ recs, const Dense
 
     if (warp == 0) {
         // ================= TMA producer (both CTAs of a pair) ==========================================
-        if (lane == 0) {
+        if (elect_one()) {
             // fills are numbered g = 0 .. total-1 over (tile, step in d); fill g uses stage g % n_stages
             const int my_tiles = (geo.n_tiles - group + geo.n_groups - 1) / geo.n_groups;
             const int sub = geo.sub;
@@ -382,7 +321,7 @@ k_head_dense(const HeadArgs a, Ctrl* ctrl, float* __restrict__ recs, const Dense
         }
     } else if (warp == 1) {
         // ================= MMA issuer (leader CTA only) ================================================
-        if (lane == 0 && rank == 0) {
+        if (rank == 0 && elect_one()) {
             const uint32_t idesc = make_idesc(PAIR ? 2 * kBM : kBM, bn);
             const uint64_t desc_a0 = make_desc(ring_u32);                       // (the ring is 1024-byte aligned and under 256 KB:
             const uint64_t sub16 = (uint64_t)(((uint32_t)geo.stage_bytes / (uint32_t)geo.sub) >> 4);   //  adding byte offsets >> 4 stays inside the address field)
@@ -646,7 +585,7 @@ k_head_dense(const HeadArgs a, Ctrl* ctrl, float* __restrict__ recs, const Dense
 // Two warps per hidden row (candidates / statistics): merge the CTA records, remap, write the outputs.
 __global__ void __launch_bounds__(64)
 k_head_merge(const HeadArgs a, Ctrl* ctrl, float* __restrict__ recs, int G) {
-    __shared__ __align__(8) float s_stage[kMergeStageWords];
+    __shared__ __align__(16) float s_stage[kMergeStageWords];
     __shared__ float s_xch;
     const int b = blockIdx.x;
     griddep_launch_dependents();                                  // the next step may start fetching its weights
@@ -666,37 +605,6 @@ k_head_merge(const HeadArgs a, Ctrl* ctrl, float* __restrict__ recs, int G) {
 }
 
 // ---- host side ----------------------------------------------------------------------------------------
-typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
-                                  const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
-                                  CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
-EncodeTiledFn encode_fn() {
-    static std::mutex mu;
-    static EncodeTiledFn fn = nullptr;
-    std::lock_guard<std::mutex> lock(mu);
-    if (!fn) {
-        void* p = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &p, cudaEnableDefault, &q) == cudaSuccess &&
-            q == cudaDriverEntryPointSuccess)
-            fn = reinterpret_cast<EncodeTiledFn>(p);
-    }
-    return fn;
-}
-
-// bf16 matrix [rows, cols] row-major -> boxes of kBK columns x box_rows rows, 128-byte swizzle
-bool encode_map(CUtensorMap* tm, const void* base, int rows, int cols, int box_rows) {
-    EncodeTiledFn fn = encode_fn();
-    if (!fn) return false;
-    cuuint64_t gdim[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
-    cuuint64_t gstr[1] = {(cuuint64_t)cols * 2};
-    cuuint32_t box[2] = {(cuuint32_t)kBK, (cuuint32_t)box_rows};
-    cuuint32_t estr[2] = {1, 1};
-    return fn(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), gdim, gstr, box, estr,
-              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
 // Tile width: the vocabulary is dealt to `groups` CTAs (pairs) in tiles of bn rows; the slowest group
 // works ceil(tiles / groups) * bn rows.  Smallest such makespan wins, the wider tile on equal terms
 // (fewer re-reads of the hidden rows).
@@ -785,6 +693,12 @@ cudaError_t launch_head_dense(const HeadArgs& a, Ctrl* ctrl, uint8_t* scratch, c
     else e = pair ? launch_variant<kMaxTopk, true, kParts16>(a, ctrl, recs, geo, tm_h, tm_w, s)
                   : launch_variant<kMaxTopk, false, kParts16>(a, ctrl, recs, geo, tm_h, tm_w, s);
     if (e != cudaSuccess) return e;
+    count_launch();
+    return launch_head_merge(a, ctrl, recs, geo.n_groups, s);
+}
+
+// The records of G CTAs (pairs) -> outputs; with a tree, its expansion as one more launch (it needs every row's merge).
+cudaError_t launch_head_merge(const HeadArgs& a, Ctrl* ctrl, float* recs, int G, cudaStream_t s) {
     // the merge always follows its own producer closely: it takes its seats early and waits on the device
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)a.B);
@@ -795,10 +709,9 @@ cudaError_t launch_head_dense(const HeadArgs& a, Ctrl* ctrl, uint8_t* scratch, c
     at.val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = &at;
     cfg.numAttrs = 1;
-    count_launch(2);
-    e = cudaLaunchKernelEx(&cfg, k_head_merge, a, ctrl, recs, geo.n_groups);
+    count_launch();
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, k_head_merge, a, ctrl, recs, G);
     if (e != cudaSuccess || !a.tree.pool_token) return e;
-    // tree drafting: the expansion needs every row's merge, i.e. the whole merge grid: one more launch
     return launch_tree_expand(a.out_ids, a.out_logprobs, a.B, a.topk, 1 + a.topk, 1, a.tree, s);
 }
 

@@ -1,87 +1,75 @@
-// Trimmed LM head for a few hidden rows (B <= 16), fused with its sampling epilogue
-// (Algorithm 2, the drafter-forward and index-mapping steps: drafter head over the trimmed vocabulary, then the index mapper).
+// Trimmed LM head for up to 64 hidden rows, fused with its sampling epilogue (Algorithm 2, the
+// drafter-forward and index-mapping steps: drafter head over the trimmed vocabulary, then the index mapper).
 //
-// HBM-bound: the only large operand is W_trim [K,d] bf16, read exactly once.  One persistent CTA
-// per SM owns a contiguous slab of vocabulary rows and streams it through a shared-memory ring
-// filled by the bulk-copy engine (cp.async.bulk + mbarrier transaction counts): one warp issues,
-// besides its share of the math, one multi-kilobyte copy per vocabulary row of a stage (8 rows x
-// up to 2048 columns), refilling each stage one step after it was released, so well over 100 KB
-// per SM stay in flight whatever the other warps are doing.
+// HBM-bound: the only large operand is W_trim [K,d] bf16, read exactly once.  Every CTA owns a contiguous
+// slab of vocabulary rows (K / grid of them, equal to within one row) and walks it in tiles of at most 128
+// rows.  The contraction runs on the 5th-generation tensor cores with the VOCABULARY rows as the M operand:
 //
-// Sixteen consumer warps split the hidden dimension.  Each keeps its slice of h in registers as
-// ready-made operand fragments and feeds the warp-level tensor instruction mma.m16n8k16 (bf16 in,
-// fp32 accumulate) with the hidden rows as the 16-row operand and the stage's 8 vocabulary rows
-// as the 8-column operand.  A dot product does not care in which order k is visited, so the 16
-// contiguous bytes a lane reads from a W row serve directly as its fragment as long as the h
-// fragment is taken from the same k positions.  The tensor instruction only off-loads the FMAs
-// (at B = 10 the fp32 pipe could not keep up with HBM); the kernel remains a streaming read.
+//   D[j, b] = sum_i W_trim[j, i] * h[b, i]     M = vocabulary rows of a tile (the TMEM lanes),
+//                                              N = hidden rows (TMEM columns), K-loop over d in 64-column steps
 //
-// Per 8-row block the 16 partial tiles meet in shared memory and warp b updates hidden row b, on
-// chip: running max / sum-exp of z = logit / T, the row's top-k list, and the Gumbel-max
-// candidate from the caller's uniforms.  Logits never go to HBM.  Warps only meet through
-// mbarriers (stage full/empty, partial tile full/empty), never through a CTA-wide barrier inside
-// the loop.  Each CTA leaves one small record per hidden row; the last CTA to finish (atomic
-// ticket, no spinning) merges the records in CTA order, remaps trimmed indices through `map` and
-// writes the outputs.  Every wait is bounded: on expiry the CTA raises VT_FLAG_TIMEOUT, drains
-// its own copies and leaves.
+// so a weight is moved once (TMA into a shared-memory ring, 128-byte swizzle, where the MMA reads it in place)
+// and no register, no shuffle and no partial tile of another warp ever sees it.  Warp 0 feeds the ring (a
+// stage = up to four 64-column steps of the tile's rows and of h), one thread of warp 1 issues the MMAs.
+// fp32 accumulation inside the tensor core is a long serial sum, so d is cut into phases of eight steps and a
+// phase's 32 MMAs go to up to eight accumulators in turn (TMEM columns are plentiful); the epilogue adds the
+// accumulators up in fp32 registers, phase by phase, while the next phase's MMAs fill the other set.
+//
+// Epilogue warps read their TMEM lanes (lane = vocabulary row) and turn the finished tile around in shared
+// memory; then warp w owns hidden rows w, w + EW, ...: its lanes walk the tile's rows, updating running
+// max / sum-exp of z = logit / T, the Gumbel-max candidate from the caller's uniforms and the row's sorted
+// top-k list.  Logits never go to HBM.  Each CTA leaves one small record per hidden row; up to 16 rows, the
+// last CTA to finish (atomic ticket, no spinning) merges the records in CTA order, remaps trimmed indices
+// through `map` and writes the outputs; beyond that a second kernel does, one pair of warps per row.
+//
+// Every wait is bounded: on expiry the CTA raises VT_FLAG_TIMEOUT, lets its own copies and MMAs finish and leaves.
 #include <math_constants.h>
 
 #include "vt_common.cuh"
 #include "vt_head_common.cuh"
+#include "vt_tc.cuh"
 #include "vt_tree_common.cuh"
 
 namespace vt {
 
 namespace {
 
-constexpr int kNW = 16;                          // consumer warps: split of the hidden dimension
-constexpr int kThreads = kNW * 32;
-constexpr int kLag = 2;                          // a stage is refilled kLag items after its release
-constexpr int kRows = 8;                         // vocabulary rows per stage (mma n)
-constexpr int kMaxStages = 8;
-constexpr int kMaxB = 16;
-constexpr size_t kSmemLimit = 227 * 1024 - 1024; // opt-in limit minus static shared memory
-constexpr int kCand = 64;                        // candidate buffer entries per hidden row
-constexpr int kSelPerLane = (VT_MAX_TOPK + kCand) / 32;
+constexpr int kBM = 128;                         // vocabulary rows per tile at most (TMEM lanes)
+constexpr int kMaxStages = 16;
+constexpr int kMaxSub = 4;                       // 64-column steps of d one ring stage holds at most
+constexpr int kPhase = 8;                        // 64-column steps of d accumulated in one accumulator set
+constexpr int kSetCols = 128;                    // TMEM columns of an accumulator set (two sets)
+constexpr uint32_t kTmemCols = 2 * kSetCols;     // (half of the SM's: two CTAs of consecutive launches may be resident together)
+constexpr int kMaxB = 64;
+constexpr int kMergeB = 16;                      // hidden rows the last CTA merges by itself
+constexpr size_t kSmemLimit = 227 * 1024 - 2048; // opt-in limit minus static shared memory
 constexpr unsigned long long kWaitLimitNs = 2000000000ull;   // default bound of a device-side wait (Ctrl::wait_ns overrides)
 
-
-// Phase stamps (-DVT_STAMPS builds only): thread 0 of every CTA writes %globaltimer at fixed points into
+// Phase stamps (-DVT_STAMPS builds only): one thread per role writes %globaltimer at fixed points into
 // a region behind the records; bench.py --case stamps reads them back.  Slots: 0 entry, 1 ring fill
-// requested, 2 released by the launch dependency, 3 first stage landed, 4 last stage consumed,
-// 5 record written, 6 after the fence, 7 after the ticket, 8-10 merge (loads, selection, outputs), 11 SM id.
+// requested, 2 released by the launch dependency, 3 first stage landed, 4 last accumulators complete,
+// 5 record written, 6 all warps done, 7 after the ticket, 8-10 merge (loads, selection, outputs), 11 SM id.
 #ifdef VT_STAMPS
-#define VT_STAMP(slot) do { if (threadIdx.x == 0) stamps[(size_t)blockIdx.x * kStampSlots + (slot)] = global_ns(); } while (0)
+#define VT_STAMP(slot) do { stamps[(size_t)blockIdx.x * kStampSlots + (slot)] = global_ns(); } while (0)
 #else
 #define VT_STAMP(slot) do {} while (0)
 #endif
 
 struct Geo {
-    int RB;            // row blocks of 8 vocabulary rows
-    int S;             // ring stages
-    int pitch;         // bytes between rows of a stage (odd multiple of 64: conflict-free 128-bit reads)
-    int part_stride;   // floats per warp partial tile
+    int grid;          // CTAs
+    int n_tiles;       // tiles per CTA
+    int rows;          // vocabulary rows of a tile (rows of one W copy)
+    int n_kc;          // 64-column steps of d
+    int sub;           // steps per ring stage
+    int n_stages;      // ring depth
+    int h_bytes;       // shared memory of a step's h part (a multiple of 1024)
+    int step_bytes;    // ... of a step: h part + W part
     int ring_bytes;
+    int buf_bytes;     // selection buffers of the epilogue warps
+    uint32_t keep;     // bit g & 31: the weights of fill g keep their L2 lines
 };
 
-// ---- mbarrier / bulk copy primitives -------------------------------------------------------------
-__device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-__device__ __forceinline__ void mbar_init(uint64_t* b, int count) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(b)), "r"(count));
-}
-__device__ __forceinline__ void mbar_expect_tx(uint64_t* b, uint32_t bytes) {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(b)), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ void mbar_arrive(uint64_t* b) {
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(b)) : "memory");
-}
-__device__ __forceinline__ bool mbar_try(uint64_t* b, uint32_t parity) {
-    uint32_t ok;
-    asm volatile(
-        "{ .reg .pred p; mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2; selp.u32 %0, 1, 0, p; }"
-        : "=r"(ok) : "r"(smem_u32(b)), "r"(parity) : "memory");
-    return ok != 0;
-}
+// ---- bounded waits ---------------------------------------------------------------------------------
 // non-blocking probe of a phase (try_wait may suspend the thread for a system-chosen time before it answers)
 __device__ __forceinline__ bool mbar_test(uint64_t* b, uint32_t parity) {
     uint32_t ok;
@@ -90,145 +78,134 @@ __device__ __forceinline__ bool mbar_test(uint64_t* b, uint32_t parity) {
         : "=r"(ok) : "r"(smem_u32(b)), "r"(parity) : "memory");
     return ok != 0;
 }
-__device__ __forceinline__ unsigned long long global_ns() {
-    unsigned long long t;
-    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-    return t;
-}
 // The bound of a wait is kept with the SM's cycle counter (reading the nanosecond timer costs far more
 // than a probe): two cycles per nanosecond, i.e. at least the time asked for at any SM clock up to
-// 2 GHz.  It lives in shared memory and is looked at only once a wait has to spin, so it costs the hot
-// loop no register.  Bounds under a millisecond spin on non-blocking probes only: try_wait may park the
-// warp for a system-chosen time before it answers, which is what a long wait wants and a short bound
-// cannot afford.
+// 2 GHz.  It lives in shared memory and is looked at only once a wait has to spin.  Bounds under a
+// millisecond spin on non-blocking probes only: try_wait may park the thread for a system-chosen time before
+// it answers, which is what a long wait wants and a short bound cannot afford.
 __device__ __forceinline__ long long bound_cycles(unsigned long long ns) {
     return (long long)(ns < (1ull << 61) ? 2 * ns : (1ull << 62));
 }
 constexpr long long kShortBoundCycles = 2000000;      // 1 ms
-// Bounded wait, called by all 32 lanes of a warp; false when the CTA is aborting or the bound
-// expired (which starts an abort).  The outcome is voted on, so the lanes of a warp never part ways
-// before a warp-collective instruction (mma, shuffle, ballot).  Inline on purpose: a call here would
-// spill the caller's registers at every wait that is not satisfied at once, i.e. at most of them.
+// Bounded wait of one thread; false when the CTA is aborting or the bound expired (which starts an abort).
 __device__ __forceinline__ bool mbar_wait(uint64_t* b, uint32_t parity, volatile int* abort_flag,
                                           const volatile long long* bound) {
-    bool ok = mbar_test(b, parity);
-    if (!ok) {
-        const long long t0 = clock64();
-        const long long lim = *bound;
-        const bool nb = lim < kShortBoundCycles;
-        for (;;) {
+    if (mbar_test(b, parity)) return true;
+    const long long t0 = clock64();
+    const long long lim = *bound;
+    const bool nb = lim < kShortBoundCycles;
+    for (;;) {
 #pragma unroll 1
-            for (int i = 0; i < 64 && !ok; ++i) {
-                ok = nb ? mbar_test(b, parity) : mbar_try(b, parity);
-                if (nb && clock64() - t0 > lim) break;
-            }
-            if (ok || *abort_flag) break;
-            if (clock64() - t0 > lim) { *abort_flag = 1; break; }
+        for (int i = 0; i < 64; ++i) {
+            if (nb ? mbar_test(b, parity) : mbar_try(b, parity)) return true;
+            if (nb && clock64() - t0 > lim) break;
         }
+        if (*abort_flag) return false;
+        if (clock64() - t0 > lim) { *abort_flag = 1; return false; }
     }
-    return __all_sync(0xffffffffu, ok);
 }
-// bulk copy global -> shared with an L2 eviction-priority hint for the lines it brings in
-__device__ __forceinline__ void bulk_g2s(uint32_t dst, const void* src, uint32_t bytes, uint64_t* bar, uint64_t pol) {
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1], %2, [%3], %4;"
-                 ::"r"(dst), "l"(src), "r"(bytes), "r"(smem_u32(bar)), "l"(pol) : "memory");
+// Same, called by all 32 lanes of a warp: lane 0 polls (a CTA of polling threads takes shared-memory and issue
+// slots from what it waits for), then every lane observes the completed phase itself.  The outcome is voted on,
+// so the lanes never part ways before a warp-collective instruction.
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t* b, uint32_t parity, volatile int* abort_flag,
+                                               const volatile long long* bound) {
+    int ok = 1;
+    if ((threadIdx.x & 31) == 0) ok = mbar_wait(b, parity, abort_flag, bound) ? 1 : 0;
+    ok = __shfl_sync(0xffffffffu, ok, 0);
+    if (ok) ok = mbar_try(b, parity) ? 1 : 0;
+    return __all_sync(0xffffffffu, ok != 0);
 }
-__device__ __forceinline__ uint4 lds_u4(uint32_t addr) {
-    uint4 v;
-    asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr));
-    return v;
+// before the CTA leaves: what is in flight gets this long to finish
+__device__ __forceinline__ void drain_wait(uint64_t* b, uint32_t parity) {
+    const unsigned long long t0 = global_ns();
+    while (!mbar_try(b, parity) && global_ns() - t0 < kWaitLimitNs) {}
 }
 
-__device__ __forceinline__ void mma_bf16(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2,
-                                         uint32_t a3, uint32_t b0, uint32_t b1) {
+// eight times four consecutive accumulator columns of this thread's TMEM lane (the wait sits in the same
+// statement: nothing that uses the values can be moved in front of it)
+__device__ __forceinline__ void tc_ld_8x4(const uint32_t (&ad)[8], float (&r)[8][4]) {
+    uint32_t v[32];
     asm volatile(
-        "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, "
-        "{%8,%9}, {%0,%1,%2,%3};"
-        : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-        : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+        "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%32];\n\t"
+        "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%4,%5,%6,%7}, [%33];\n\t"
+        "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%8,%9,%10,%11}, [%34];\n\t"
+        "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%12,%13,%14,%15}, [%35];\n\t"
+        "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%16,%17,%18,%19}, [%36];\n\t"
+        "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%20,%21,%22,%23}, [%37];\n\t"
+        "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%24,%25,%26,%27}, [%38];\n\t"
+        "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%28,%29,%30,%31}, [%39];\n\t"
+        "tcgen05.wait::ld.sync.aligned;"
+        : "=&r"(v[0]), "=&r"(v[1]), "=&r"(v[2]), "=&r"(v[3]), "=&r"(v[4]), "=&r"(v[5]), "=&r"(v[6]), "=&r"(v[7]),
+          "=&r"(v[8]), "=&r"(v[9]), "=&r"(v[10]), "=&r"(v[11]), "=&r"(v[12]), "=&r"(v[13]), "=&r"(v[14]), "=&r"(v[15]),
+          "=&r"(v[16]), "=&r"(v[17]), "=&r"(v[18]), "=&r"(v[19]), "=&r"(v[20]), "=&r"(v[21]), "=&r"(v[22]), "=&r"(v[23]),
+          "=&r"(v[24]), "=&r"(v[25]), "=&r"(v[26]), "=&r"(v[27]), "=&r"(v[28]), "=&r"(v[29]), "=&r"(v[30]), "=&r"(v[31])
+        : "r"(ad[0]), "r"(ad[1]), "r"(ad[2]), "r"(ad[3]), "r"(ad[4]), "r"(ad[5]), "r"(ad[6]), "r"(ad[7])
+        : "memory");
+#pragma unroll
+    for (int i = 0; i < 32; ++i) r[i >> 2][i & 3] = __uint_as_float(v[i]);
 }
 
-struct TopkState {
-    int cnt;       // entries in the list
-    float thr;     // value of entry topk-1 once the list is full, else -inf
-};
+// ---- top-k list of one hidden row ------------------------------------------------------------------
+constexpr int kBufKeys = VT_MAX_TOPK + kBM + 4;       // a warp's selection buffer: list, candidates, padding
 
-// Warp-cooperative selection: the best min(topk, cnt + n_c) of a sorted list (tv/tj, cnt entries) and
-// a batch of unsorted candidates (cv/cj, n_c entries) become the new sorted list (descending value,
-// ties to the lower index).  Every element's final position is its rank -- the number of elements
-// that beat it -- so there are no sequential selection rounds: each lane keeps up to kSelPerLane
-// elements in registers while all elements stream by as broadcast shared-memory reads.  The cost
-// does not depend on topk and is small when few candidates are pending.
+// Warp-cooperative selection: buf holds the keys of a sorted list and behind them candidate keys, N in all; the
+// best min(topk, N) of them become the new sorted list (descending; keys order by value, then lower index).  Every
+// element's final position is its rank -- the number of elements that beat it -- so there are no sequential
+// selection rounds: each lane keeps up to NS elements in registers while all of them stream by as broadcast
+// 128-bit shared-memory reads, several in flight.
 template <int NS>
-__device__ __forceinline__ void rank_scatter(float* tv, int* tj, int cnt, const float* cv, const int* cj, int n_c,
-                                             int topk) {
+__device__ __forceinline__ void rank_scatter(unsigned long long* list, const unsigned long long* buf, int N, int topk) {
     const int lane = threadIdx.x & 31;
-    const int N = cnt + n_c;
     unsigned long long ek[NS];
     int rk[NS];
 #pragma unroll
     for (int i = 0; i < NS; ++i) {
-        const int idx = lane + 32 * i;
-        ek[i] = 0ull;
+        ek[i] = lane + 32 * i < N ? buf[lane + 32 * i] : 0ull;
         rk[i] = 0;
-        if (idx < cnt) ek[i] = key64(tv[idx], tj[idx]);
-        else if (idx < N) ek[i] = key64(cv[idx - cnt], cj[idx - cnt]);
     }
-#pragma unroll 2
-    for (int e = 0; e < cnt; ++e) {
-        const unsigned long long k = key64(tv[e], tj[e]);
-#pragma unroll
-        for (int i = 0; i < NS; ++i) rk[i] += (k > ek[i]) ? 1 : 0;
-    }
-#pragma unroll 4
-    for (int e = 0; e < n_c; ++e) {
-        const unsigned long long k = key64(cv[e], cj[e]);
-#pragma unroll
-        for (int i = 0; i < NS; ++i) rk[i] += (k > ek[i]) ? 1 : 0;
-    }
-    __syncwarp();                                         // every read of the old list is done
+    rank_among<NS>(buf, N, ek, rk);
 #pragma unroll
     for (int i = 0; i < NS; ++i)
-        if (lane + 32 * i < N && rk[i] < topk) { tv[rk[i]] = key_val(ek[i]); tj[rk[i]] = key_idx(ek[i]); }
+        if (lane + 32 * i < N && rk[i] < topk) list[rk[i]] = ek[i];
 }
 
-__device__ __noinline__ TopkState topk_flush(float* tv, int* tj, int cnt, const float* cv, const int* cj, int n_c,
-                                             int topk) {
-    const int N = cnt + n_c;
-    __syncwarp();
-    if (N <= 32) rank_scatter<1>(tv, tj, cnt, cv, cj, n_c, topk);
-    else if (N <= 64) rank_scatter<2>(tv, tj, cnt, cv, cj, n_c, topk);
-    else if (N <= 96) rank_scatter<3>(tv, tj, cnt, cv, cj, n_c, topk);
-    else rank_scatter<kSelPerLane>(tv, tj, cnt, cv, cj, n_c, topk);
-    __syncwarp();
-    const int out = min(topk, N);
-    return TopkState{out, (out == topk) ? tv[topk - 1] : -CUDART_INF_F};
-}
+// One lane's state of one hidden row over the vocabulary rows it has seen.
+struct RowState {
+    float m, s;        // running max and sum of exp(z - m)
+    float gs, gz;      // best Gumbel score and its z
+    int gj;
+};
 
-// NCH column chunks per row, KBC 32-column blocks per warp and chunk; TWO: hidden rows 8..15 present.
-template <int NCH, int KBC, bool TWO>
-__global__ void __launch_bounds__(kThreads, 1)
-k_head_stream(const HeadArgs a, Ctrl* ctrl, float* __restrict__ recs, const Geo geo) {
-    extern __shared__ __align__(128) uint8_t s_raw[];
-    __shared__ uint64_t s_full[kMaxStages], s_empty[kMaxStages], s_pfull[2], s_pempty[2];
+// EW epilogue warps (a multiple of 4: the warps of a lane quadrant share the accumulator columns), at most RPW hidden
+// rows per epilogue warp.
+template <int EW, int RPW>
+__global__ void __launch_bounds__((EW + 2) * 32, EW == 8 ? 2 : 1)
+k_head_stream(const HeadArgs a, Ctrl* ctrl, float* __restrict__ recs, const Geo geo,
+              const __grid_constant__ CUtensorMap tm_h, const __grid_constant__ CUtensorMap tm_w) {
+    extern __shared__ uint8_t s_dyn[];
+    __shared__ uint64_t s_full[kMaxStages], s_empty[kMaxStages], s_acc_full[2], s_acc_empty[2], s_drain;
+    __shared__ uint32_t s_tmem_base;
     __shared__ int s_last, s_abort, s_any_abort;
     __shared__ long long s_bound;                        // bound of a wait in SM cycles
-    __shared__ int s_issued[kMaxStages];                 // per stage: 0 = never requested, else 2 | parity of the latest fill
-    __shared__ int s_rowok[kMaxB];                       // per hidden row: its temperature is usable
-    __shared__ float s_xch[kMaxB];                       // merge: a row's lse, from its statistics warp to its candidate warp
-    constexpr int KC = kNW * KBC * 32;                   // columns per chunk
-    const int B = a.B, K = a.K, d = a.d, topk = a.topk;
-    const int S = geo.S, pitch = geo.pitch, PT = geo.part_stride;
-    const int stage_bytes = kRows * pitch;
-    uint8_t* ring = s_raw;
-    float* part = reinterpret_cast<float*>(s_raw + geo.ring_bytes);           // [2][kNW][R][PT]
-    float* topv = part + 2 * kNW * (TWO ? 2 : 4) * PT;                                        // [B][topk]
-    int* topj = reinterpret_cast<int*>(topv + B * topk);                      // [B][topk]
-    float* candv = reinterpret_cast<float*>(topj + B * topk);                 // [B][kCand]
-    int* candj = reinterpret_cast<int*>(candv + B * kCand);                   // [B][kCand]
+    __shared__ float s_xch[kMergeB];                     // merge: a row's lse, from its statistics warp to its candidate warp
+    constexpr int kWarps = EW + 2, kThreads = kWarps * 32;
+    // An accumulator set holds kAccs accumulators of kNpad columns (hidden rows).  The kParts warps of a lane quadrant
+    // take kUnits groups of four columns each: always eight loads per warp and phase.
+    constexpr int kParts = EW / 4, kUnits = RPW, kAccs = 8 / kUnits, kNpad = 16 * kUnits;
+    static_assert(kAccs * kNpad <= kSetCols && kParts * kUnits * 4 <= kNpad, "a set's columns");
+    const int B = a.B, K = a.K, topk = a.topk;
+    uint8_t* ring = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(s_dyn) + 1023) & ~(uintptr_t)1023);
+    const uint32_t ring_u32 = smem_u32(ring);
+    float* zt = reinterpret_cast<float*>(ring + geo.ring_bytes);                                  // [B][kBM]: a tile's logits, row by row
+    unsigned long long* lists = reinterpret_cast<unsigned long long*>(zt + B * kBM);              // [B][topk]
+    unsigned long long* bufs = lists + ((B * topk + 1) & ~1);                                     // [min(EW, B)][kBufKeys]
+    RowState* states = reinterpret_cast<RowState*>(reinterpret_cast<uint8_t*>(bufs) + geo.buf_bytes);     // [B][32]
+    float* s_invT = reinterpret_cast<float*>(states + B * 32);                                    // [B] 1 / T, NaN for an unusable temperature
+    int* s_cnt = reinterpret_cast<int*>(s_invT + B);                                              // [B] entries in the row's list
 
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int g = lane >> 2, t = lane & 3;
+    const int r0 = (int)((long long)K * blockIdx.x / gridDim.x);
+    const int r1 = (int)((long long)K * (blockIdx.x + 1) / gridDim.x);
 #ifdef VT_STAMPS
     unsigned long long* stamps = reinterpret_cast<unsigned long long*>(
         reinterpret_cast<uint8_t*>(recs) + align_up_dev((size_t)kMaxGrid * B * rec_fields(topk) * 4, 256));
@@ -236,281 +213,401 @@ k_head_stream(const HeadArgs a, Ctrl* ctrl, float* __restrict__ recs, const Geo 
         unsigned smid;
         asm volatile("mov.u32 %0, %%smid;" : "=r"(smid));
         stamps[(size_t)blockIdx.x * kStampSlots + 11] = smid;
+        VT_STAMP(0);
     }
 #endif
-    const int rb0 = (int)((long long)geo.RB * blockIdx.x / gridDim.x);
-    const int rb1 = (int)((long long)geo.RB * (blockIdx.x + 1) / gridDim.x);
-
     if (threadIdx.x == 0) {
-        for (int s = 0; s < S; ++s) { mbar_init(&s_full[s], 1); mbar_init(&s_empty[s], kNW); s_issued[s] = 0; }
-        for (int p = 0; p < 2; ++p) { mbar_init(&s_pfull[p], kNW); mbar_init(&s_pempty[p], B); }
+        asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tm_w)) : "memory");
+        asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tm_h)) : "memory");
+        for (int s = 0; s < geo.n_stages; ++s) { mbar_init(&s_full[s], 1); mbar_init(&s_empty[s], 1); }
+        for (int p = 0; p < 2; ++p) { mbar_init(&s_acc_full[p], 1); mbar_init(&s_acc_empty[p], EW); }
+        mbar_init(&s_drain, 1);
         s_abort = 0;
         s_bound = bound_cycles(kWaitLimitNs);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    for (int i = threadIdx.x; i < B * topk; i += kThreads) { topv[i] = -CUDART_INF_F; topj[i] = -1; }
+    if (warp == 1) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
+                     ::"r"(smem_u32(&s_tmem_base)), "r"(kTmemCols) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    tc_fence_before();
     __syncthreads();
-    VT_STAMP(0);
+    tc_fence_after();
+    const uint32_t tmem_base = s_tmem_base;
     volatile int* abort_flag = &s_abort;
-    const volatile long long* wait_ns = &s_bound;
+    const volatile long long* bound = &s_bound;
+    // Programmatic dependent launch (a no-op unless the launch asked for it): the next kernel on the stream
+    // may become resident as soon as its resources are free (this CTA has its tensor memory by now), and this
+    // kernel goes no further than fetching weights until everything enqueued before it has completed.
+    griddep_launch_dependents();
 
-    // per-row state of warp b (identical in its four 8-lane groups); declared here so that the
-    // record code after the loop sees it
-    const int b = warp;
-    float invT = 1.f;
-    bool row_ok = true;
-    float st_m = -CUDART_INF_F, st_s = 0.f;                 // running max / sum exp (per lane)
-    float gb_s = -CUDART_INF_F, gb_z = 0.f;                 // Gumbel best (per lane)
-    int gb_j = -1;
-
-    // ---- producer duty: one bulk copy per vocabulary row of a stage (lanes 0..7 of the duty warp) ----
-    // Every warp tracks the fetch sequence; fetch f is issued by one warp of the duty group (the
-    // warps that own no hidden row, so the epilogue warps are spared), in rotation.
-    // W_trim is read once per step: its lines are the first to go when L2 needs room, so that the
-    // records, the index mapper and h stay resident from step to step
-    uint64_t w_policy;                                       // (not volatile: may be re-made where it is used)
-    asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(w_policy));
-    const int n_items = (rb1 - rb0) * NCH;
-    const int n_duty = (B < kNW) ? kNW - B : 1;
-    int f_item = 0, f_rb = rb0, f_c = 0, f_s = 0, f_duty = kNW - 1;   // next item to fetch, its duty warp
-    uint32_t f_ph = 0;
-    auto fetch_next = [&]() -> bool {                         // false = abort
-        bool ok = true;
-        if (warp == f_duty) {
-            if (f_item >= S && !mbar_wait(&s_empty[f_s], f_ph ^ 1, abort_flag, wait_ns)) ok = false;
-            if (ok) {
-                const int nrows = min(kRows, K - f_rb * kRows);
-                const int col0 = f_c * KC;
-                const uint32_t cbytes = (uint32_t)(min(d, col0 + KC) - col0) * 2u;
-                if (lane == 0) {
-                    s_issued[f_s] = 2 | (int)f_ph;           // requested at least once; parity of the latest fill
-                    mbar_expect_tx(&s_full[f_s], cbytes * (uint32_t)nrows);
+    if (warp == 0) {
+        // ================= TMA producer ================================================================
+        if (elect_one()) {
+            const int sub = geo.sub, S = geo.n_stages;
+            const int n_ks = (geo.n_kc + sub - 1) / sub;               // ring stages per tile
+            const int total = geo.n_tiles * n_ks;
+            const uint32_t step_tx = (uint32_t)(geo.rows + B) * (kBK * 2);      // bytes that land per step
+            // W_trim is read once per call: its lines are the first to go when L2 needs room, so that the records, the
+            // index mapper, h and the uniforms stay resident from step to step -- except for the share of it that a
+            // drafting loop finds in L2 again at its next step (see make_geo)
+            uint64_t first_policy, keep_policy;
+            asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(first_policy));
+            asm("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(keep_policy));
+            auto load_w = [&](uint32_t dst, int x, int y, uint64_t* bar, int g) {
+                asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.L2::cache_hint"
+                             " [%0], [%1, {%2, %3}], [%4], %5;"
+                             ::"r"(dst), "l"(&tm_w), "r"(x), "r"(y), "r"(smem_u32(bar)),
+                               "l"(((geo.keep >> (g & 31)) & 1u) ? keep_policy : first_policy) : "memory");
+            };
+            // The weights are static: the first ring of them is requested before the work this launch
+            // depends on has finished; everything that work may have produced is touched after the wait.
+            const int pre = min(S, total);
+            {
+                int ks = 0, y = r0;
+                for (int g = 0; g < pre; ++g) {
+                    const int subs = min(sub, geo.n_kc - ks * sub);
+                    mbar_expect_tx(&s_full[g], step_tx * (uint32_t)subs);
+                    for (int u = 0; u < subs; ++u)
+                        load_w(ring_u32 + (uint32_t)((g * sub + u) * geo.step_bytes + geo.h_bytes), (ks * sub + u) * kBK, y, &s_full[g], g);
+                    if (++ks == n_ks) { ks = 0; y += geo.rows; }
                 }
-                __syncwarp();
-                if (lane < nrows)
-                    bulk_g2s(smem_u32(ring + (size_t)f_s * stage_bytes + lane * pitch),
-                             a.W + (size_t)(f_rb * kRows + lane) * d + col0, cbytes, &s_full[f_s], w_policy);
             }
-        }
-        ++f_item;
-        if (++f_c == NCH) { f_c = 0; ++f_rb; }
-        if (++f_s == S) { f_s = 0; f_ph ^= 1; }
-        if (--f_duty < kNW - n_duty) f_duty = kNW - 1;
-        return ok;
-    };
-    for (int i = 0; i < S && f_item < n_items; ++i) fetch_next();          // fill the ring (no waits)
-    VT_STAMP(1);
-
-    // Programmatic dependent launch (a no-op unless the launch asked for it): the next kernel on the
-    // stream may become resident as soon as SMs free up, and this kernel goes no further than
-    // fetching weights until everything enqueued before it has completed and is visible.
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    VT_STAMP(2);
-
-    // ---- h fragments of this warp's columns, straight from global memory into registers ----------
-    uint4 hl[NCH][KBC], hh[NCH][KBC];
-#pragma unroll
-    for (int c = 0; c < NCH; ++c)
-#pragma unroll
-        for (int i = 0; i < KBC; ++i) {
-            const int col = c * KC + (warp * KBC + i) * 32 + 8 * t;
-            hl[c][i] = make_uint4(0, 0, 0, 0);
-            hh[c][i] = make_uint4(0, 0, 0, 0);
-            if (col < d) {
-                if (g < B) hl[c][i] = __ldg(reinterpret_cast<const uint4*>(a.h + (size_t)g * d + col));
-                if (TWO && g + 8 < B)
-                    hh[c][i] = __ldg(reinterpret_cast<const uint4*>(a.h + (size_t)(g + 8) * d + col));
+            VT_STAMP(1);
+            griddep_wait();
+            VT_STAMP(2);
+            {
+                int ks = 0;
+                for (int g = 0; g < pre; ++g) {
+                    const int subs = min(sub, geo.n_kc - ks * sub);
+                    for (int u = 0; u < subs; ++u)
+                        tma_load_2d(ring_u32 + (uint32_t)((g * sub + u) * geo.step_bytes), &tm_h, (ks * sub + u) * kBK, 0, &s_full[g]);
+                    if (++ks == n_ks) ks = 0;
+                }
             }
+            {
+                const unsigned long long lim = *reinterpret_cast<volatile unsigned long long*>(&ctrl->wait_ns);        // 0 = the default
+                if (lim) s_bound = bound_cycles(lim);               // (a race with early waiters only keeps their bound)
+            }
+            int done = pre;
+            {
+                // steady state: the cursor over (stage, step in d, tile) moves by additions only
+                int sc = pre == S ? 0 : pre, ks = pre % n_ks, y = r0 + (pre / n_ks) * geo.rows;
+                uint32_t par = 0;                                   // fill g waits for the release of fill g - S
+                for (int g = pre; g < total; ++g, ++done) {
+                    if (!mbar_wait(&s_empty[sc], par, abort_flag, bound)) break;
+                    const int subs = min(sub, geo.n_kc - ks * sub);
+                    mbar_expect_tx(&s_full[sc], step_tx * (uint32_t)subs);
+                    const uint32_t dst0 = ring_u32 + (uint32_t)(sc * sub * geo.step_bytes);
+#pragma unroll
+                    for (int u = 0; u < kMaxSub; ++u) {
+                        if (u < subs) {
+                            const int x = (ks * sub + u) * kBK;
+                            load_w(dst0 + (uint32_t)(u * geo.step_bytes + geo.h_bytes), x, y, &s_full[sc], g);
+                            tma_load_2d(dst0 + (uint32_t)(u * geo.step_bytes), &tm_h, x, 0, &s_full[sc]);
+                        }
+                    }
+                    if (++sc == S) { sc = 0; par ^= 1u; }
+                    if (++ks == n_ks) { ks = 0; y += geo.rows; }
+                }
+            }
+            // aborting: every copy asked for has landed before the CTA may leave (else the MMAs have read them all)
+            if (*abort_flag)
+                for (int g = max(0, done - S); g < done; ++g) drain_wait(&s_full[g % S], (uint32_t)((g / S) & 1));
         }
-    {
-        const unsigned long long lim = ctrl->wait_ns;        // 0 = the default
-        if (lim && threadIdx.x == 0) s_bound = bound_cycles(lim);   // (a race with early waiters only shortens or keeps their bound)
-    }
-    if (b < B) {
-        const float T = a.temp[b];
-        row_ok = (T > 0.f) && (T < CUDART_INF_F);
-        invT = row_ok ? 1.f / T : CUDART_NAN_F;
-        if (lane == 0) s_rowok[b] = row_ok ? 1 : 0;
-    }
-    float thr = -CUDART_INF_F;                              // k-th best so far (warp uniform)
-    int tk_cnt = 0, n_cand = 0;
-    const uint32_t lane_off = (uint32_t)(g * pitch + warp * KBC * 64 + t * 16);
-    const uint32_t ring_u32 = smem_u32(ring);
-    // epilogue lane roles: a group of R row blocks has 8R logits per hidden row; LPR lanes share one
-    // logit, each summing the partial tiles of kNW / LPR warps
-    constexpr int R = TWO ? 2 : 4;                          // row blocks per exchange
-    constexpr int LPR = 4 / R;
-    const int e_ri = lane % (8 * R), e_q = lane / (8 * R);
-    const int e_r = e_ri >> 3, e_v8 = e_ri & 7;
-    float u_next = 0.5f;
-    if (a.uniforms && b < B && rb0 + e_r < rb1) {
-        const int j = (rb0 + e_r) * kRows + e_v8;
-        if (j < K) u_next = __ldg(a.uniforms + (size_t)b * K + j);
-    }
-    int s = 0, item = 0, n = 0;
-    uint32_t ph = 0;
-    bool alive = true;
-#pragma unroll 1
-    for (int rb = rb0; rb < rb1 && alive; rb += R, ++n) {
-        const int rc = min(R, rb1 - rb);
-        float res[R][TWO ? 4 : 2];
-#pragma unroll
-        for (int r = 0; r < R; ++r) {
-            if (r < rc && alive) {
-                float acc0[4] = {0.f, 0.f, 0.f, 0.f}, acc1[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-                for (int c = 0; c < NCH; ++c) {
-                    if (!alive || !mbar_wait(&s_full[s], ph, abort_flag, wait_ns)) { alive = false; continue; }
+    } else if (warp == 1) {
+        // ================= MMA issuer ==================================================================
+        if (elect_one()) {
+            constexpr uint32_t idesc = make_idesc(kBM, kNpad);
+            // (the ring is 1024-byte aligned and under 256 KB: adding byte offsets >> 4 stays inside the address field;
+            // rows of an operand beyond the tile's / beyond B are whatever lies behind it: their TMEM lanes and columns
+            // are not looked at)
+            const uint64_t desc_h0 = make_desc(ring_u32);
+            const uint64_t w_off = (uint64_t)(geo.h_bytes >> 4);
+            const uint64_t d_step = (uint64_t)(geo.step_bytes >> 4);
+            const int S = geo.n_stages, sub = geo.sub;
+            const int n_ks = (geo.n_kc + sub - 1) / sub;
+            int s = 0, issued = 0, set_no = 0;
+            uint32_t ph = 0;
+            bool alive = true;
+            for (int t = 0; t < geo.n_tiles && alive; ++t) {
+                uint32_t d_tmem = 0;
+                int in_phase = 0;                                   // steps issued into the current set
+                for (int ks = 0; ks < n_ks; ++ks) {
+                    if (!mbar_wait(&s_full[s], ph, abort_flag, bound)) { alive = false; break; }
 #ifdef VT_STAMPS
-                    if (item == 0) VT_STAMP(3);
+                    if (t == 0 && ks == 0) VT_STAMP(3);
 #endif
-                    const uint32_t base = ring_u32 + (uint32_t)s * (uint32_t)stage_bytes + lane_off;
-                    uint4 w[KBC];
-#pragma unroll
-                    for (int i = 0; i < KBC; ++i) {
-                        const int col = c * KC + (warp * KBC + i) * 32 + 8 * t;
-                        w[i] = (col < d) ? lds_u4(base + i * 64) : make_uint4(0, 0, 0, 0);
+                    if (in_phase == 0) {                            // a new accumulator set: the epilogue has read what it held
+                        if (set_no >= 2 && !mbar_wait(&s_acc_empty[set_no & 1], (uint32_t)(((set_no >> 1) - 1) & 1), abort_flag, bound)) {
+                            alive = false;
+                            break;
+                        }
+                        d_tmem = tmem_base + (uint32_t)((set_no & 1) * kSetCols);
                     }
+                    tc_fence_after();
+                    const int subs = min(sub, geo.n_kc - ks * sub);
+                    uint64_t dh = desc_h0 + (uint64_t)((uint32_t)(s * sub * geo.step_bytes) >> 4);
 #pragma unroll
-                    for (int i = 0; i < KBC; ++i) {
-                        mma_bf16(acc0, hl[c][i].x, hh[c][i].x, hl[c][i].y, hh[c][i].y, w[i].x, w[i].y);
-                        mma_bf16(acc1, hl[c][i].z, hh[c][i].z, hl[c][i].w, hh[c][i].w, w[i].z, w[i].w);
+                    for (int u = 0; u < kMaxSub; ++u) {
+                        if (u < subs) {
+                            // consecutive MMAs go to the set's accumulators in turn; the first round of a phase overwrites
+#pragma unroll
+                            for (int k = 0; k < kBK / 16; ++k) {
+                                const int i = (in_phase + u) * (kBK / 16) + k;
+                                tc_mma(d_tmem + (uint32_t)((i % kAccs) * kNpad), dh + w_off + (uint64_t)(k * 2), dh + (uint64_t)(k * 2), idesc,
+                                       i >= kAccs ? 1u : 0u);
+                            }
+                            dh += d_step;
+                        }
                     }
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(&s_empty[s]);
-                    if (++s == S) { s = 0; ph ^= 1; }
-                    // refill the stage released kLag items ago (by now every warp has normally left it)
-                    if (item >= kLag && f_item < n_items && !fetch_next()) alive = false;
-                    ++item;
+                    in_phase += subs;
+                    tc_commit(&s_empty[s]);                         // the stage is free once these MMAs have read it
+                    if (in_phase == kPhase || ks == n_ks - 1) {
+                        tc_commit(&s_acc_full[set_no & 1]);         // the phase's accumulators are complete
+                        ++set_no;
+                        in_phase = 0;
+                    }
+                    ++issued;
+                    if (++s == S) { s = 0; ph ^= 1u; }
                 }
-                res[r][0] = acc0[0] + acc1[0];
-                res[r][1] = acc0[1] + acc1[1];
-                if (TWO) { res[r][2] = acc0[2] + acc1[2]; res[r][3] = acc0[3] + acc1[3]; }
             }
+            // every MMA issued has finished and every commit has arrived before the CTA may leave, whatever happened
+            tc_commit(&s_drain);
+            drain_wait(&s_drain, 0);
+            for (int g = max(0, issued - S); g < issued; ++g) drain_wait(&s_empty[g % S], (uint32_t)((g / S) & 1));
         }
-        if (!alive) break;
-        // ---- hand the partial tiles over ------------------------------------------------------------
-        const int pb = n & 1;
-        const uint32_t use = (uint32_t)(n >> 1);
-        if (n >= 2 && !mbar_wait(&s_pempty[pb], (use - 1) & 1, abort_flag, wait_ns)) break;
-#pragma unroll
-        for (int r = 0; r < R; ++r) {
-            if (r < rc) {
-                float* mine = part + ((pb * kNW + warp) * R + r) * PT;
-                if (g < B) *reinterpret_cast<float2*>(mine + g * 8 + 2 * t) = make_float2(res[r][0], res[r][1]);
-                if (TWO && g + 8 < B)
-                    *reinterpret_cast<float2*>(mine + (g + 8) * 8 + 2 * t) = make_float2(res[r][2], res[r][3]);
-            }
+    } else {
+        // ================= epilogue warps ==============================================================
+        const int e = warp - 2;
+        const int quad = warp & 3;                                  // TMEM lanes this warp may read
+        const int part = e >> 2;                                    // which accumulator columns of the quadrant
+        unsigned long long* buf = bufs + (size_t)(e < B ? e : 0) * kBufKeys;     // (used only by warps that own a row: e < B)
+        for (int b = e; b < B; b += EW) {
+            states[b * 32 + lane] = RowState{-CUDART_INF_F, 0.f, -CUDART_INF_F, 0.f, -1};
+            if (lane == 0) s_cnt[b] = 0;
+        }
+        griddep_wait();                                             // temp, uniforms and the record scratch belong to earlier work until here
+        for (int b = e; b < B; b += EW) {
+            const float T = a.temp[b];
+            if (lane == 0) s_invT[b] = (T > 0.f) && (T < CUDART_INF_F) ? 1.f / T : CUDART_NAN_F;
         }
         __syncwarp();
-        if (lane == 0) mbar_arrive(&s_pfull[pb]);
-        if (b >= B) continue;
-        // ---- warp b: reduce the tiles, update hidden row b --------------------------------------------
-        if (!mbar_wait(&s_pfull[pb], use & 1, abort_flag, wait_ns)) break;
-        const bool in_group = e_r < rc;
-        float x = 0.f;
-        if (in_group) {
-            const float* src = part + ((pb * kNW + e_q) * R + e_r) * PT + b * 8 + e_v8;
+        const int n_ph = (geo.n_kc + kPhase - 1) / kPhase;
+        int set_no = 0;
+        for (int t = 0; t < geo.n_tiles; ++t) {
+            const int j0 = r0 + t * geo.rows;                       // first vocabulary row of the tile
+            const int nrow = min(geo.rows, r1 - j0);                // rows of it that are this CTA's
+            float un[4];                                            // the next row's uniforms; the first row's are requested before the MMAs are waited for
+            auto load_u = [&](int b) {
 #pragma unroll
-            for (int i = 0; i < kNW / LPR; ++i) x += src[i * LPR * R * PT];
-        }
-        if (LPR >= 2) x += __shfl_xor_sync(0xffffffffu, x, 8 * R);
-        if (LPR >= 4) x += __shfl_xor_sync(0xffffffffu, x, 16 * R);
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&s_pempty[pb]);
-        const int j = (rb + e_r) * kRows + e_v8;
-        const bool valid = in_group && j < K;
-        if (a.dbg_logits && valid && e_q == 0) a.dbg_logits[(size_t)b * K + j] = x;
-        const float z = x * invT;
-        {   // online max / sum-exp without a per-lane branch
-            const float zz = valid ? z : -CUDART_INF_F;
-            const float m_new = fmaxf(st_m, zz);
-            const float m_ref = (m_new == -CUDART_INF_F) ? 0.f : m_new;
-            st_s = st_s * __expf(st_m - m_ref) + __expf(zz - m_ref);
-            st_m = m_new;
-        }
-        if (a.uniforms) {
-            // g = -log(-log u): -log u from a short series in 1-u near 1 (where a fast logarithm's absolute
-            // error would dominate the tiny result), fast logarithms elsewhere
-            const float uc = fminf(fmaxf(u_next, 0x1p-24f), 1.f - 0x1p-24f);
-            const float t1 = 1.f - uc;
-            const float lp = t1 * (1.f + t1 * (0.5f + t1 * (0.33333334f + t1 * (0.25f + t1 * 0.2f))));
-            const float L = uc > 0.95f ? lp : -__logf(uc);
-            const float sc = z - __logf(L);
-            if (valid && sc > gb_s) { gb_s = sc; gb_j = j; gb_z = z; }
-            const int jn = (rb + R + e_r) * kRows + e_v8;
-            if (rb + R + e_r < rb1 && jn < K) u_next = __ldg(a.uniforms + (size_t)b * K + jn);
-        }
-        const bool is_cand = valid && e_q == 0 && z > thr;
-        const unsigned cand = __ballot_sync(0xffffffffu, is_cand);
-        if (cand) {
-            if (is_cand) {
-                const int pos = n_cand + __popc(cand & lanemask_lt());
-                candv[b * kCand + pos] = z;
-                candj[b * kCand + pos] = j;
-            }
-            n_cand += __popc(cand);
-            if (n_cand + kRows * R > kCand) {
-                const TopkState ts = topk_flush(topv + b * topk, topj + b * topk, tk_cnt, candv + b * kCand,
-                                                candj + b * kCand, n_cand, topk);
-                tk_cnt = ts.cnt;
-                thr = ts.thr;
-                n_cand = 0;
-            }
-        }
-    }
-    VT_STAMP(4);
-    // ---- this CTA's record per hidden row ----------------------------------------------------------
-    if (b < B && !*abort_flag) {
-        if (n_cand > 0) {
-            const TopkState ts = topk_flush(topv + b * topk, topj + b * topk, tk_cnt, candv + b * kCand,
-                                            candj + b * kCand, n_cand, topk);
-            tk_cnt = ts.cnt;
-        }
-        // Fold the lanes (those sharing a logit hold identical state: only the 8R distinct ones add to the
-        // sum): the maximum by one warp reduction, every lane's sum rescaled to it once, a butterfly of
-        // additions; the Gumbel candidate by two reductions over its 64-bit key.
-        const float Mall = ord2f(__reduce_max_sync(0xffffffffu, f2ord(st_m)));
-        float sc = (lane < 8 * (TWO ? 2 : 4) && st_m != -CUDART_INF_F) ? st_s * __expf(st_m - Mall) : 0.f;
+                for (int i = 0; i < 4; ++i)
+                    un[i] = (a.uniforms && b < B && lane + 32 * i < nrow) ? __ldg(a.uniforms + (size_t)b * K + j0 + lane + 32 * i) : 0.5f;
+            };
+            load_u(e);
+            // the accumulators of the tile, phase by phase, added up per (vocabulary row = lane, hidden row = column)
+            float x[kUnits][4];
 #pragma unroll
-        for (int o = 16; o; o >>= 1) sc += __shfl_xor_sync(0xffffffffu, sc, o);
-        const unsigned long long gk = gb_j >= 0 ? key64(gb_s, gb_j) : 0ull;
-        const unsigned ghi = (unsigned)(gk >> 32);
-        const unsigned gmax = __reduce_max_sync(0xffffffffu, ghi);
-        const unsigned glo = __reduce_max_sync(0xffffffffu, ghi == gmax ? (unsigned)gk : 0u);
-        const unsigned who = __ballot_sync(0xffffffffu, ghi == gmax && (unsigned)gk == glo);
-        const float gzw = __shfl_sync(0xffffffffu, gb_z, __ffs(who) - 1);
-        unsigned long long* kp = rec_keys(recs, b, topk);
-        float* fp = rec_f32(recs, b, topk);
-        const int c = blockIdx.x;
-        if (lane == 0) {
-            fp[c] = Mall;
-            fp[kMaxGrid + c] = sc;
-            fp[2 * kMaxGrid + c] = gzw;
-            kp[c] = ((unsigned long long)gmax << 32) | glo;
-        }
-        for (int r = lane; r < topk; r += 32) {
-            const int j = topj[b * topk + r];
-            kp[(size_t)(1 + r) * kMaxGrid + c] = j >= 0 ? key64(topv[b * topk + r], j) : 0ull;
-        }
-        __threadfence();                                    // the record is visible before the ticket is taken
-    }
-    VT_STAMP(5);
-    __syncthreads();                                        // every warp has left the loop: no copy is requested from here on
-    VT_STAMP(6);
-    if (warp == 0 && *abort_flag) {
-        // drain: every stage that was requested must have landed before the CTA may leave
-        for (int st = lane; st < S; st += 32) {
-            const int last_fill = s_issued[st];
-            if (last_fill) {
-                const unsigned long long t0 = global_ns();
-                while (!mbar_try(&s_full[st], (uint32_t)(last_fill & 1)) && global_ns() - t0 < kWaitLimitNs) {}
+            for (int i = 0; i < kUnits; ++i)
+#pragma unroll
+                for (int q = 0; q < 4; ++q) x[i][q] = 0.f;
+            bool ok = true;
+            for (int p = 0; p < n_ph; ++p, ++set_no) {
+                const int set = set_no & 1;
+                ok = mbar_wait_warp(&s_acc_full[set], (uint32_t)((set_no >> 1) & 1), abort_flag, bound);
+                if (!ok) break;
+                tc_fence_after();
+                if (quad * 32 < nrow && part * 4 < B) {
+                    const uint32_t base = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(set * kSetCols + part * 4);
+                    uint32_t ad[8];
+                    float v[8][4];
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) ad[i] = base + (uint32_t)((i % kAccs) * kNpad + (i / kAccs) * kParts * 4);
+                    tc_ld_8x4(ad, v);
+                    const int mmas = min(kPhase, geo.n_kc - p * kPhase) * (kBK / 16);
+                    // (an accumulator that a short last phase did not get to holds nothing; the others pairwise: fewer
+                    // roundings in a row than one after the other)
+#pragma unroll
+                    for (int q = 0; q < 4; ++q)
+#pragma unroll
+                        for (int i = 0; i < kUnits; ++i) {
+                            float w[kAccs];
+#pragma unroll
+                            for (int c = 0; c < kAccs; ++c) w[c] = c < mmas ? v[i * kAccs + c][q] : 0.f;
+#pragma unroll
+                            for (int o = kAccs / 2; o; o >>= 1)
+#pragma unroll
+                                for (int c = 0; c < o; ++c) w[c] += w[c + o];
+                            x[i][q] += w[0];
+                        }
+                }
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&s_acc_empty[set]);
+            }
+            if (ok) {
+#ifdef VT_STAMPS
+                if (e == 0 && lane == 0) VT_STAMP(4);
+#endif
+                if (quad * 32 < nrow) {
+#pragma unroll
+                    for (int i = 0; i < kUnits; ++i)
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) {
+                            const int b = (part + i * kParts) * 4 + q;
+                            if (b < B) zt[(size_t)b * kBM + quad * 32 + lane] = x[i][q];
+                        }
+                }
+            }
+            {   // every epilogue warp has written its part, and all of them agree whether to go on
+                int all_ok;
+                asm volatile("{ .reg .pred p, q; setp.ne.s32 p, %1, 0; bar.red.and.pred q, 1, %2, p; selp.s32 %0, 1, 0, q; }"
+                             : "=r"(all_ok) : "r"(ok ? 1 : 0), "n"(EW * 32) : "memory");
+                if (!all_ok) break;
+            }
+            // ---- the warp's hidden rows over this tile.  (A rolled loop, with the per-lane state in shared memory:
+            // unrolled over the rows its code would be fetched anew for every row.)
+#pragma unroll 1
+            for (int b = e; b < B; b += EW) {
+                const float u[4] = {un[0], un[1], un[2], un[3]};
+                load_u(b + EW);
+                RowState* rs = &states[b * 32 + lane];
+                RowState st = *rs;
+                const float invT = s_invT[b];
+                unsigned long long* list = lists + (size_t)b * topk;
+                const int cnt = s_cnt[b];
+                const float last = key_val(list[topk - 1]);
+                const float thr = cnt == topk ? last : -CUDART_INF_F;
+                const int ni = (nrow + 31) >> 5;                    // the tile's rows per lane
+                float z[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const bool valid = lane + 32 * i < nrow;
+                    const float x1 = valid ? zt[(size_t)b * kBM + lane + 32 * i] : 0.f;
+                    if (a.dbg_logits && valid) a.dbg_logits[(size_t)b * K + j0 + lane + 32 * i] = x1;
+                    z[i] = valid ? x1 * invT : -CUDART_INF_F;
+                }
+                {   // running max / sum-exp: one rescale per tile, independent exponentials (a NaN logit is left out of
+                    // the maximum and poisons the sum)
+                    const float m_new = fmaxf(st.m, fmaxf(fmaxf(z[0], z[1]), fmaxf(z[2], z[3])));
+                    const float m_ref = (m_new == -CUDART_INF_F) ? 0.f : m_new;
+                    st.s = st.s * exp_fast(st.m - m_ref) + ((exp_fast(z[0] - m_ref) + exp_fast(z[1] - m_ref)) +
+                                                            (exp_fast(z[2] - m_ref) + exp_fast(z[3] - m_ref)));
+                    st.m = m_new;
+                }
+                if (a.uniforms) {
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        if (i < ni) {
+                            // g = -log(-log u): -log u from a short series in 1-u near 1 (where a fast logarithm's absolute
+                            // error would dominate the tiny result), fast logarithms elsewhere
+                            const float uc = fminf(fmaxf(u[i], 0x1p-24f), 1.f - 0x1p-24f);
+                            const float t1 = 1.f - uc;
+                            const float lp = t1 * (1.f + t1 * (0.5f + t1 * (0.33333334f + t1 * (0.25f + t1 * 0.2f))));
+                            const float L = uc > 0.95f ? lp : -log_fast(uc);
+                            const float sc = z[i] - log_fast(L);
+                            const bool win = sc > st.gs;            // (rows that do not exist carry -inf)
+                            st.gs = win ? sc : st.gs;
+                            st.gj = win ? j0 + lane + 32 * i : st.gj;
+                            st.gz = win ? z[i] : st.gz;
+                        }
+                    }
+                }
+                *rs = st;
+                // top-k: the rows that beat the list's last entry join the list.  While the list is not full that is
+                // nearly every row of the tile; the topk-th largest of the lanes' best values is then a lower bound of
+                // the answer and leaves a few more than topk of them.
+                unsigned cm[4];
+                int n_c = 0;
+#pragma unroll
+                for (int i = 0; i < 4; ++i) { cm[i] = __ballot_sync(0xffffffffu, z[i] > thr); n_c += __popc(cm[i]); }
+                if (n_c > 32 && topk <= 32) {
+                    unsigned lb = 0u;                               // the lane's best candidate (no NaN is a candidate)
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) lb = (z[i] > thr) ? max(lb, f2ord(z[i])) : lb;
+                    const unsigned tau = kth_of_lanes(lb, topk, reinterpret_cast<unsigned*>(buf));
+                    n_c = 0;
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        cm[i] = __ballot_sync(0xffffffffu, z[i] > thr && f2ord(z[i]) >= tau);
+                        n_c += __popc(cm[i]);
+                    }
+                }
+                if (n_c) {
+                    for (int i = lane; i < cnt; i += 32) buf[i] = list[i];
+                    int pos = cnt;
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        if ((cm[i] >> lane) & 1u) buf[pos + __popc(cm[i] & lanemask_lt())] = key64(z[i], j0 + lane + 32 * i);
+                        pos += __popc(cm[i]);
+                    }
+                    if (lane < 4) buf[pos + lane] = 0ull;           // (read in groups of four)
+                    __syncwarp();                                   // (every read of the old list is done, too)
+                    if (pos <= 32) rank_scatter<1>(list, buf, pos, topk);
+                    else if (pos <= 64) rank_scatter<2>(list, buf, pos, topk);
+                    else rank_scatter<(VT_MAX_TOPK + kBM) / 32>(list, buf, pos, topk);
+                    if (lane == 0) s_cnt[b] = min(topk, pos);
+                    __syncwarp();
+                }
+            }
+            // ---- this CTA's record of its hidden rows: the lanes folded -- the maximum by one warp reduction, every
+            // lane's sum rescaled to it once, a butterfly of additions; the Gumbel candidate by two reductions over its
+            // 64-bit key.  (Made visible to the merging CTA by the ticket below: a barrier of this CTA, then one
+            // release at GPU scope.)
+            if (t == geo.n_tiles - 1) {
+#pragma unroll 1
+                for (int b = e; b < B; b += EW) {
+                    const RowState st = states[b * 32 + lane];
+                    unsigned long long* kp = rec_keys(recs, b, topk);
+                    float* fp = rec_f32(recs, b, topk);
+                    const int c = blockIdx.x;
+                    const int cnt = s_cnt[b];
+                    for (int k = lane; k < topk; k += 32) kp[(size_t)(1 + k) * kMaxGrid + c] = k < cnt ? lists[(size_t)b * topk + k] : 0ull;
+                    const float Mall = ord2f(__reduce_max_sync(0xffffffffu, f2ord(st.m)));
+                    float sc = (st.m != -CUDART_INF_F) ? st.s * exp_fast(st.m - Mall) : st.s;
+#pragma unroll
+                    for (int o = 16; o; o >>= 1) sc += __shfl_xor_sync(0xffffffffu, sc, o);
+                    if (lane == 0) {
+                        fp[c] = Mall;
+                        fp[kMaxGrid + c] = sc;
+                    }
+                    if (a.uniforms) {
+                        const unsigned long long gk = st.gj >= 0 ? key64(st.gs, st.gj) : 0ull;
+                        const unsigned ghi = (unsigned)(gk >> 32);
+                        const unsigned gmax = __reduce_max_sync(0xffffffffu, ghi);
+                        const unsigned glo = __reduce_max_sync(0xffffffffu, ghi == gmax ? (unsigned)gk : 0u);
+                        if (gk == (((unsigned long long)gmax << 32) | glo)) {     // (one lane, or all of them when no row has a candidate)
+                            fp[2 * kMaxGrid + c] = st.gz;
+                            kp[c] = gk;
+                        }
+                    }
+                }
+            } else {
+                asm volatile("bar.sync 1, %0;" ::"n"(EW * 32) : "memory");           // the tile buffer is free
             }
         }
-        __syncwarp();
+#ifdef VT_STAMPS
+        if (e == 0 && lane == 0) VT_STAMP(5);
+#endif
     }
+    tc_fence_before();
+    __syncwarp();                                                   // lanes of the single-thread roles rejoin their warps
+    __syncthreads();                                                // no copy, no MMA and no read of tensor memory is left
+    if (warp == 1) {
+        tc_fence_after();
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(kTmemCols) : "memory");
+    }
+    if (RPW > 1) {                                                  // a kernel of its own merges the records
+        if (threadIdx.x == 0 && s_abort) atomicOr(&ctrl->flags, (uint32_t)VT_FLAG_TIMEOUT);
+        return;
+    }
+    // as many rows as half the warps: two warps per hidden row (candidates / statistics) side by side; more: one warp each
+    const bool split = B <= kWarps / 2;
+    const int row = split ? (warp % (kWarps / 2)) : warp;
+    const bool row_ok = row < B && s_invT[row] == s_invT[row];      // (read now: the merge's staging may lie over it)
     if (threadIdx.x == 0) {
+        VT_STAMP(6);
         const bool aborted = s_abort != 0;
         if (aborted) atomicOr(&ctrl->flags, (uint32_t)VT_FLAG_TIMEOUT);
         // Ticket: arrivals in the low half, aborted CTAs in the high half.  Acquire + release in one, so
@@ -520,10 +617,10 @@ k_head_stream(const HeadArgs a, Ctrl* ctrl, float* __restrict__ recs, const Geo 
                      : "=r"(old) : "l"(&ctrl->head_ticket), "r"(aborted ? 0x10001u : 1u) : "memory");
         s_last = ((old & 0xffffu) == gridDim.x - 1);
         s_any_abort = aborted || (old >> 16) != 0;
-        if (s_last) ctrl->head_ticket = 0;                  // ready for the next launch
+        if (s_last) ctrl->head_ticket = 0;                          // ready for the next launch
+        VT_STAMP(7);
     }
     __syncthreads();
-    VT_STAMP(7);
     if (!s_last) return;
 
     if (s_any_abort) {
@@ -534,15 +631,11 @@ k_head_stream(const HeadArgs a, Ctrl* ctrl, float* __restrict__ recs, const Geo 
         }
         return;
     }
-
     {
-        // B <= 8: two warps per hidden row (candidates / statistics) side by side; more rows: one warp each
         const MergeOut mo{a.map, a.out_ids, a.out_logprobs, a.dbg_lse, topk, a.uniforms != nullptr};
-        const bool split = B <= kNW / 2;
-        const int row = split ? (warp & (kNW / 2 - 1)) : warp;
-        const int roles = split ? (warp < kNW / 2 ? kRoleCand : kRoleStats) : (kRoleCand | kRoleStats);
+        const int roles = split ? (warp < kWarps / 2 ? kRoleCand : kRoleStats) : (kRoleCand | kRoleStats);
         if (row < B)
-            merge_records(mo, ctrl, recs, row, s_rowok[row] != 0, (int)gridDim.x,
+            merge_records(mo, ctrl, recs, row, row_ok, (int)gridDim.x,
                           reinterpret_cast<float*>(ring) + (size_t)row * kMergeStageWords, roles, &s_xch[row], 1 + row
 #ifdef VT_STAMPS
                           , stamps + (size_t)blockIdx.x * kStampSlots
@@ -552,89 +645,93 @@ k_head_stream(const HeadArgs a, Ctrl* ctrl, float* __restrict__ recs, const Geo 
     if (a.tree.pool_token) {
         // tree drafting: the merged candidates of all rows become pool nodes and the next frontier is
         // chosen here, by the CTA that merged them, instead of in a launch of its own
-        __syncthreads();                                   // the rows' outputs are written; the staging area is free
+        __syncthreads();                                            // the rows' outputs are written; the staging area is free
         tree_expand_block(a.tree, a.out_ids, a.out_logprobs, B, topk, 1 + topk, 1,
                           reinterpret_cast<unsigned long long*>(ring), (int)threadIdx.x, kThreads);
     }
 }
 
 // ---- host side ---------------------------------------------------------------------------------------
-struct Shape {
-    int nch, kbc;      // template selection; 0 = unsupported
-};
-
-// 32-column blocks per warp needed for d, rounded up to a supported (chunks, blocks per chunk) pair
-Shape pick_shape(int d) {
-    const int nkb = (d + 31) / 32;
-    const int kbw = (nkb + kNW - 1) / kNW;
-    static const int table[17][2] = {{0, 0}, {1, 1}, {1, 2}, {1, 3}, {1, 4}, {2, 3}, {2, 3}, {2, 4}, {2, 4},
-                                     {3, 3}, {3, 4}, {3, 4}, {3, 4}, {4, 4}, {4, 4}, {4, 4}, {4, 4}};
-    if (kbw < 1 || kbw > 16) return Shape{0, 0};
-    return Shape{table[kbw][0], table[kbw][1]};
-}
-
+// Shapes of the few-row contract: what vt_workspace_bytes and the entry points take with topk up to VT_MAX_TOPK.
 bool shape_ok(int B, int d) {
-    if (B < 1 || B > kMaxB || d < 8 || (d & 7)) return false;
-    const Shape sh = pick_shape(d);
-    if (!sh.nch) return false;
-    if (B > 8 && sh.nch * sh.kbc > 8) return false;      // h fragments must fit the register file
-    return true;
+    if (B < 1 || B > kMergeB || d < 8 || (d & 7)) return false;
+    return d <= (B <= 8 ? 8192 : 4096);
 }
 
-Geo make_geo(int B, int K, int d, int topk, size_t* smem_bytes) {
-    const Shape sh = pick_shape(d);
+Geo make_geo(int B, int K, int d, int topk, int sms, size_t* smem_bytes) {
     Geo g{};
-    g.RB = (K + kRows - 1) / kRows;
-    const int kc_bytes = kNW * sh.kbc * 32 * 2;
-    g.pitch = kc_bytes + 64;                              // kc_bytes is a multiple of 128
-    g.part_stride = ((B * 8 - 8 + 31) / 32) * 32 + 8;     // >= 8 B floats and = 8 (mod 32): conflict-free reduce
-    const int R = B > 8 ? 2 : 4;
-    const size_t fixed = (size_t)2 * kNW * R * g.part_stride * 4 + (size_t)B * (topk + kCand) * 8;
-    const size_t stage = (size_t)kRows * g.pitch;
-    int S = (int)((kSmemLimit - fixed) / stage);
-    if (S > kMaxStages) S = kMaxStages;
-    g.S = S;
-    g.ring_bytes = (int)(S * stage);
-    *smem_bytes = g.ring_bytes + fixed;
-    const size_t merge_bytes = (size_t)B * kMergeStageWords * 4;            // staging area of the merge
-    if (*smem_bytes < merge_bytes) *smem_bytes = merge_bytes;
+    g.grid = sms;
+    if (g.grid > (K + 7) / 8) g.grid = (K + 7) / 8;
+    const int slab = (K + g.grid - 1) / g.grid;
+    g.n_tiles = (slab + kBM - 1) / kBM;
+    g.rows = (slab + g.n_tiles - 1) / g.n_tiles;
+    g.n_kc = (d + kBK - 1) / kBK;
+    g.h_bytes = (int)align_up((size_t)B * kBK * 2, 1024);
+    const int w_bytes = (int)align_up((size_t)g.rows * kBK * 2, 1024);
+    g.step_bytes = g.h_bytes + w_bytes;
+    const int ew = B <= 8 ? 8 : 16;
+    g.buf_bytes = (B < ew ? B : ew) * kBufKeys * 8;
+    const size_t fixed = (size_t)B * kBM * 4 + align_up((size_t)B * topk * 8, 16) + (size_t)g.buf_bytes + (size_t)B * (32 * sizeof(RowState) + 8);
+    const size_t over = (size_t)kBM * kBK * 2 - (size_t)w_bytes;   // the MMA reads 128 rows from the start of a W part
+    const size_t tail = fixed > over ? fixed : over;
+    const size_t room = kSmemLimit - 1024 - tail;
+    // Four steps to a stage where three such stages fit: the two threads that drive the ring wait and release once
+    // per stage (201 MB cold through the bare ring: 34.9 us with one step, 33.3 with two, 32.8 with four).
+    g.sub = kMaxSub;
+    while (g.sub > 1 && (g.sub > g.n_kc || (size_t)3 * g.sub * g.step_bytes > room)) g.sub >>= 1;
+    const size_t stage = (size_t)g.sub * g.step_bytes;
+    const long total = (long)g.n_tiles * ((g.n_kc + g.sub - 1) / g.sub);
+    g.n_stages = (int)(room / stage);
+    if (g.n_stages > kMaxStages) g.n_stages = kMaxStages;
+    if (g.n_stages > total) g.n_stages = (int)total;
+    g.ring_bytes = (int)(g.n_stages * stage);
+    // A drafting loop reads the same head again a few tens of microseconds later.  A head that is larger than L2
+    // leaves nothing behind when all of it streams through under one policy; so 56 MB of it, spread evenly over
+    // every CTA's fills, keep the ordinary priority and the rest is evicted first.  (56 MB: of the 126 MB about
+    // half serves a line that one die's SMs ask for; 201 MB per step 36.0 -> 31.5 us, 24 / 40 / 72 MB 34.3 / 33.1 /
+    // 32.1; 268 MB with 10 rows 54.3 -> 53.5.)  A head under 96 MB stays resident anyway, and there the ordinary
+    // priority would only push out the records and the uniforms (61 MB: 69.5 -> 73 us per three steps).
+    const double mb = (double)K * d * 2.0 / 1e6;
+    const int share = mb > 96.0 ? (int)(56.0 / mb * 32.0) : 0;
+    for (int i = 0; i < 32; ++i)
+        if ((i + 1) * share / 32 != i * share / 32) g.keep |= 1u << i;
+    size_t need = (size_t)g.ring_bytes + tail;
+    const size_t merge_bytes = B <= kMergeB ? (size_t)B * kMergeStageWords * 4 : 0;               // staging area of the merge
+    if (need < merge_bytes) need = merge_bytes;
+    *smem_bytes = need + 1024;                                     // + slack to align the ring to 1024 bytes
     return g;
 }
 
-template <int NCH, int KBC, bool TWO>
-cudaError_t launch_variant(const HeadArgs& a, Ctrl* ctrl, float* recs, int grid, const Geo& geo,
-                           size_t smem, cudaStream_t s) {
+template <int EW, int RPW>
+cudaError_t launch_variant(const HeadArgs& a, Ctrl* ctrl, float* recs, const Geo& geo, const CUtensorMap& tm_h,
+                           const CUtensorMap& tm_w, size_t smem, cudaStream_t s) {
     static int attr_done[64] = {0};
     int dev = 0;
     cudaGetDevice(&dev);
     if (dev < 0 || dev >= 64 || !attr_done[dev]) {
-        cudaError_t e = cudaFuncSetAttribute(k_head_stream<NCH, KBC, TWO>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemLimit);
+        cudaError_t e = cudaFuncSetAttribute(k_head_stream<EW, RPW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemLimit);
         if (e != cudaSuccess) return e;
         if (dev >= 0 && dev < 64) attr_done[dev] = 1;
     }
-    if (a.overlap) {
-        cudaLaunchConfig_t cfg{};
-        cfg.gridDim = dim3((unsigned)grid);
-        cfg.blockDim = dim3(kThreads);
-        cfg.dynamicSmemBytes = smem;
-        cfg.stream = s;
-        cudaLaunchAttribute attr{};
-        attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr.val.programmaticStreamSerializationAllowed = 1;
-        cfg.attrs = &attr;
-        cfg.numAttrs = 1;
-        count_launch();
-        return cudaLaunchKernelEx(&cfg, k_head_stream<NCH, KBC, TWO>, a, ctrl, recs, geo);
-    }
-    k_head_stream<NCH, KBC, TWO><<<grid, kThreads, smem, s>>>(a, ctrl, recs, geo);
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)geo.grid);
+    cfg.blockDim = dim3((EW + 2) * 32);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = a.overlap ? 1 : 0;
     count_launch();
-    return cudaGetLastError();
+    return cudaLaunchKernelEx(&cfg, k_head_stream<EW, RPW>, a, ctrl, recs, geo, tm_h, tm_w);
 }
 
 }  // namespace
 
 bool head_skinny_supported(int32_t B, int32_t d) { return shape_ok(B, d); }
+
+bool head_stream_takes(int32_t B) { return B >= 1 && B <= kMaxB; }
 
 size_t head_skinny_scratch_bytes(int32_t B, int32_t K, int32_t topk) {
     (void)K;
@@ -648,27 +745,21 @@ size_t head_skinny_stamps_offset(int32_t B, int32_t topk) {
 #endif
 
 cudaError_t launch_head_skinny(const HeadArgs& a, Ctrl* ctrl, uint8_t* scratch, cudaStream_t s) {
-    if (!shape_ok(a.B, a.d)) return cudaErrorInvalidValue;
+    if (!head_stream_takes(a.B) || a.d < 8 || (a.d & 7)) return cudaErrorInvalidValue;
+    int sms = num_sms();
+    if (sms > kMaxGrid) sms = kMaxGrid;
     size_t smem = 0;
-    const Geo geo = make_geo(a.B, a.K, a.d, a.topk, &smem);
-    if (geo.S < kLag + 1) return cudaErrorInvalidValue;
-    int grid = num_sms();
-    if (grid > kMaxGrid) grid = kMaxGrid;
-    if (grid > geo.RB) grid = geo.RB;
+    const Geo geo = make_geo(a.B, a.K, a.d, a.topk, sms, &smem);
+    if (geo.n_stages < 1 || smem > kSmemLimit) return cudaErrorInvalidValue;
+    CUtensorMap tm_h, tm_w;
+    if (!encode_map(&tm_h, a.h, a.B, a.d, a.B) || !encode_map(&tm_w, a.W, a.K, a.d, geo.rows)) return cudaErrorInvalidValue;
     float* recs = reinterpret_cast<float*>(scratch);
-    const Shape sh = pick_shape(a.d);
-    const bool two = a.B > 8;
-#define VT_CASE(N, C)                                                                            \
-    if (sh.nch == N && sh.kbc == C)                                                              \
-        return two ? launch_variant<N, C, true>(a, ctrl, recs, grid, geo, smem, s)               \
-                   : launch_variant<N, C, false>(a, ctrl, recs, grid, geo, smem, s);
-#define VT_CASE1(N, C)                                                                           \
-    if (sh.nch == N && sh.kbc == C) return launch_variant<N, C, false>(a, ctrl, recs, grid, geo, smem, s);
-    VT_CASE(1, 1) VT_CASE(1, 2) VT_CASE(1, 3) VT_CASE(1, 4) VT_CASE(2, 3) VT_CASE(2, 4)
-    VT_CASE1(3, 3) VT_CASE1(3, 4) VT_CASE1(4, 4)
-#undef VT_CASE
-#undef VT_CASE1
-    return cudaErrorInvalidValue;
+    if (a.B <= 8) return launch_variant<8, 1>(a, ctrl, recs, geo, tm_h, tm_w, smem, s);
+    if (a.B <= 16) return launch_variant<16, 1>(a, ctrl, recs, geo, tm_h, tm_w, smem, s);
+    const cudaError_t e = a.B <= 32 ? launch_variant<16, 2>(a, ctrl, recs, geo, tm_h, tm_w, smem, s)
+                                    : launch_variant<16, 4>(a, ctrl, recs, geo, tm_h, tm_w, smem, s);
+    if (e != cudaSuccess) return e;
+    return launch_head_merge(a, ctrl, recs, geo.grid, s);
 }
 
 }  // namespace vt

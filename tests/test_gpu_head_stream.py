@@ -1,0 +1,42 @@
+"""The streaming head at the edges of its tiling: 128 vocabulary rows per tile, phases of eight 64-column steps of d,
+ring stages of up to four steps, 8 / 16 / 32 / 64 hidden rows per variant, full and growing candidate lists."""
+import pytest
+import torch
+
+import paper_2506_22694_b200 as vt
+import vt_inputs
+from parity_util import check_head, oracle_head
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda"
+SMS = 148                                                # one slab per SM: K = SMS * 128 fills one tile per slab
+
+
+@pytest.mark.parametrize("B,K,d,topk,sample", [
+    (8, SMS * 128, 64, 8, True), (1, SMS * 128 + 1, 72, 33, True), (9, SMS * 128 - 1, 512, 64, False),   # tile edges, one phase
+    (16, SMS * 256 + 1, 520, 10, True), (2, 7, 576, 7, True), (3, SMS * 8 + 3, 4096, 64, True),          # two phases; tiny slabs
+    (17, 2000, 520, 16, True), (32, SMS * 128 + 1, 448, 1, False), (33, 3001, 1032, 16, True),           # separate merge
+    (64, SMS * 128 + 3, 264, 8, True), (65, 1500, 136, 8, True),                                         # last streaming / first dense row count
+])
+def test_streaming_head_at_tile_phase_and_variant_edges(B, K, d, topk, sample):
+    W = vt_inputs.gaussian_bf16((K, d), 0.05, seed=K + d, device=DEV)
+    h = vt_inputs.gaussian_bf16((B, d), 1.0, seed=B + 5, device=DEV)
+    T = vt_inputs.temperatures(B, 0.5, 1.5, seed=K, device=DEV)
+    u = vt_inputs.uniforms((B, K), seed=d + 1, device=DEV) if sample else None
+    m = torch.randperm(K * 2, device=DEV)[:K].to(torch.int32)
+    ws = vt.Workspace(vt.workspace_bytes(vt.VT_OP_DRAFT_HEAD, 0, 0, K, d, B, topk))
+    gi, gl, lg, lse = vt.vt_draft_head(h, W, m, T, topk, u, ws=ws, debug=True)
+    torch.cuda.synchronize()
+    check_head(oracle_head(h, W, m, T, topk, u), gi, gl, T, m, lg, lse, sampled=sample)
+    # fp32 accumulation split over many accumulators: 2^-24 per rounding on partial sums no larger than sum |w h|, eight
+    # phases of three pairwise levels and one addition each behind chains of at most four 16-column products
+    exact = h.double() @ W.double().t()
+    bound = (h.double().abs() @ W.double().abs().t()) * 2.0 ** -24 * 16
+    if B <= 16:
+        assert bool(((lg.double() - exact).abs() <= bound).all())
+    a = vt.vt_draft_head(h, W, m, T, topk, u, ws=ws)
+    b = vt.vt_draft_head(h, W, m, T, topk, u, ws=ws, overlapped=True)
+    torch.cuda.synchronize()
+    for o in (a, b):                                     # without the logits dump, plain and chained: the same bits
+        assert torch.equal(o[0], gi) and torch.equal(o[1], gl)
+    assert ws.read_status() == (0, 0, 0)
