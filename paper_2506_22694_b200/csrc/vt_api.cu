@@ -39,6 +39,12 @@ constexpr int64_t kHostChunkIds = 1 << 24;     // ids per staged chunk of vt_bui
 
 bool hist_shape_ok(int32_t V) { return hist_supported(V); }
 
+// scratch that the histogram and the selection of a build share, one after the other
+size_t inner_bytes(int32_t V) {
+    const size_t h = hist_plan(V, 0, SIZE_MAX).bytes, c = select_cut_scratch_bytes(V);
+    return h > c ? h : c;
+}
+
 bool head_shape_ok(int32_t B, int32_t K, int32_t d, int32_t topk) {
     if (B < 1 || B > 256 || K < 1 || d < 8 || (d & 7) || topk < 1 || topk > VT_MAX_TOPK || topk > K)
         return false;
@@ -83,16 +89,14 @@ size_t vt_workspace_bytes(int op, int64_t n, int32_t V, int32_t K, int32_t d, in
     switch (op) {
         case VT_OP_HISTOGRAM:
             if (!hist_shape_ok(V) || n < 0) return 0;
-            return VT_CTRL_BYTES + hist_plan(V).bytes;
+            return VT_CTRL_BYTES + hist_plan(V, 0, SIZE_MAX).bytes;
         case VT_OP_SELECT_TOPK:
             if (V < 1 || K < 1 || K > V) return 0;
             return VT_CTRL_BYTES + select_cut_scratch_bytes(V);
         case VT_OP_BUILD_VOCAB:
         case VT_OP_BUILD_VOCAB_HOST: {
             if (!hist_shape_ok(V) || n < 0 || K < 1 || K > V) return 0;
-            size_t inner = hist_plan(V).bytes;
-            if (select_cut_scratch_bytes(V) > inner) inner = select_cut_scratch_bytes(V);
-            size_t total = VT_CTRL_BYTES + align_up((size_t)V * 4, 256) + inner;
+            size_t total = VT_CTRL_BYTES + align_up((size_t)V * 4, 256) + inner_bytes(V);
             if (op == VT_OP_BUILD_VOCAB_HOST) {
                 const int64_t chunk = n < kHostChunkIds ? (n > 0 ? n : 1) : kHostChunkIds;
                 total = align_up(total, 256) + 2 * align_up((size_t)chunk * 4, 256);
@@ -184,11 +188,12 @@ vt_status vt_histogram(const int32_t* ids, int64_t n, int32_t V, uint32_t* count
     if (n < 0 || n >= ((int64_t)1 << 32) || V < 1 || !counts || (n > 0 && !ids)) return VT_ERR_INVALID_ARG;
     if (!aligned(ids, 4) || !aligned(counts, 4)) return VT_ERR_INVALID_ARG;
     if (!hist_shape_ok(V)) return VT_ERR_UNSUPPORTED;
-    vt_status st = check_ws(ws, ws_bytes, vt_workspace_bytes(VT_OP_HISTOGRAM, n, V, 0, 0, 0, 0));
+    // (a workspace of the former, smaller size still serves: such a vocabulary is then counted the other way)
+    vt_status st = check_ws(ws, ws_bytes, VT_CTRL_BYTES + hist_min_bytes(V));
     if (st != VT_OK) return st;
     uint8_t* base = static_cast<uint8_t*>(ws);
     return from_cuda(launch_histogram(ids, n, V, counts, accumulate, reinterpret_cast<Ctrl*>(base),
-                                      base + VT_CTRL_BYTES, as_stream(stream)));
+                                      base + VT_CTRL_BYTES, ws_bytes - VT_CTRL_BYTES, as_stream(stream)));
 }
 
 vt_status vt_histogram_folded(const int32_t* ids, int64_t n, int32_t V, int32_t bins, uint32_t* counts, void* stream) {
@@ -293,7 +298,7 @@ vt_status vt_build_vocab(const int32_t* ids, int64_t n, int32_t V, int32_t K, in
     uint32_t* counts = reinterpret_cast<uint32_t*>(base + VT_CTRL_BYTES);
     uint8_t* inner = base + VT_CTRL_BYTES + align_up((size_t)V * 4, 256);
     cudaStream_t s = as_stream(stream);
-    cudaError_t e = launch_histogram(ids, n, V, counts, 0, reinterpret_cast<Ctrl*>(base), inner, s);
+    cudaError_t e = launch_histogram(ids, n, V, counts, 0, reinterpret_cast<Ctrl*>(base), inner, inner_bytes(V), s);
     if (e != cudaSuccess) return from_cuda(e);
     return from_cuda(launch_select_topk(counts, V, K, map, inv_map, inner, s));
 }
@@ -339,7 +344,7 @@ vt_status vt_build_vocab_host(const int32_t* ids_host, int64_t n, int32_t V, int
             e = cudaMemcpyAsync(stage[sl], ids_host + done, (size_t)m * 4, cudaMemcpyHostToDevice, copy_stream);
         if (e == cudaSuccess) e = cudaEventRecord(copied[sl], copy_stream);
         if (e == cudaSuccess) e = cudaStreamWaitEvent(s, copied[sl], 0);
-        if (e == cudaSuccess) e = launch_histogram(stage[sl], m, V, counts, 1, ctrl, inner, s);
+        if (e == cudaSuccess) e = launch_histogram(stage[sl], m, V, counts, 1, ctrl, inner, inner_bytes(V), s);
         if (e == cudaSuccess) e = cudaEventRecord(counted[sl], s);
         done += m;
     }

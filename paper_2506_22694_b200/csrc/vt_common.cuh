@@ -24,6 +24,24 @@ constexpr int kNumSMsFallback = 148;
 int num_sms();                    // SM count of the current device (cached per device)
 void count_launch(int n = 1);     // host-side launch counter behind vt_launch_count
 
+// A launch that may take its seats before the kernel in front of it on the stream has finished (programmatic stream
+// serialization): every kernel launched this way executes griddepcontrol.wait before it touches global memory.
+template <class Kernel, class... Args>
+inline cudaError_t launch_dependent(Kernel k, unsigned grid, unsigned block, size_t smem, cudaStream_t s, Args... args) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    count_launch();
+    return cudaLaunchKernelEx(&cfg, k, args...);
+}
+
 inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 #ifdef __CUDACC__
 __device__ __forceinline__ size_t align_up_dev(size_t x, size_t a) { return (x + a - 1) / a * a; }
@@ -32,6 +50,7 @@ __device__ __forceinline__ size_t align_up_dev(size_t x, size_t a) { return (x +
 // ---- launchers implemented in the .cu files (host functions) --------------------------------
 struct HistPlan {
     bool small;            // all bins fit in one CTA's shared memory
+    int parts;             // id ranges the packed kernel deals to different CTAs (0: not packed)
     size_t off_sample;     // uint32 [V]   sampled counts
     size_t off_packed;     // uint32 [V]   what the packed kernel counted (only when three bins per word fit)
     size_t off_gate;       // uint32 [4]   {recount, -, skipped ids (64 bits)} of the packed kernel
@@ -39,10 +58,13 @@ struct HistPlan {
     size_t off_table;      // uint2  [ceil(V/32)] hot-bin table {bitmap word, slot base}
     size_t bytes;          // scratch after the control block
 };
-HistPlan hist_plan(int32_t V);
+// scratch_bytes: what the caller has; a vocabulary that needs several id ranges is counted the packed way only
+// when the scratch holds the packed counts too (hist_min_bytes does not include them)
+HistPlan hist_plan(int32_t V, int64_t n, size_t scratch_bytes);
+size_t hist_min_bytes(int32_t V);
 bool hist_supported(int32_t V);   // V the counting kernels take (bins or lookup table fit shared memory)
 cudaError_t launch_histogram(const int32_t* ids, int64_t n, int32_t V, uint32_t* counts,
-                             int accumulate, Ctrl* ctrl, uint8_t* scratch, cudaStream_t s);
+                             int accumulate, Ctrl* ctrl, uint8_t* scratch, size_t scratch_bytes, cudaStream_t s);
 
 cudaError_t launch_hist_fold(const int32_t* ids, int64_t n, int32_t V, int32_t bins, uint32_t* counts, cudaStream_t s);
 
@@ -111,6 +133,10 @@ cudaError_t launch_head_dense(const HeadArgs& a, Ctrl* ctrl, uint8_t* scratch, c
 
 // ---- device helpers ----------------------------------------------------------------------------
 #ifdef __CUDACC__
+// Programmatic dependent launch: let the next launch on the stream become resident / wait until the
+// work this launch depends on has completed and its writes are visible (no-ops in a plain launch).
+__device__ __forceinline__ void griddep_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void griddep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 // Streaming 128-bit load: read-only path, do not keep the line in L1 (data is used once).
 __device__ __forceinline__ uint4 ld_stream_u4(const void* p) {
     uint4 v;

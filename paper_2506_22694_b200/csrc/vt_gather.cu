@@ -17,6 +17,8 @@ k_gather_rows(const uint16_t* __restrict__ W_full, const int32_t* __restrict__ m
     const int lane = threadIdx.x & 31;
     const int warps_total = gridDim.x * (kThreads / 32);
     const int gw = blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5);
+    griddep_launch_dependents();
+    griddep_wait();                                              // (the map comes from the kernel before)
     const int nvec = d >> 3;                                     // 16-byte vectors per row
     for (int j = gw; j < K; j += warps_total) {
         const int32_t src = map[j];
@@ -47,9 +49,7 @@ cudaError_t launch_gather_rows(const uint16_t* W_full, const int32_t* map, uint1
     int grid = (K + warps_per_cta - 1) / warps_per_cta;
     const int cap = num_sms() * kCtasPerSm;
     if (grid > cap) grid = cap;
-    k_gather_rows<<<grid, kThreads, 0, s>>>(W_full, map, W_trim, V, K, d, ctrl);
-    count_launch();
-    return cudaGetLastError();
+    return launch_dependent(k_gather_rows, (unsigned)grid, kThreads, 0, s, W_full, map, W_trim, V, K, d, ctrl);
 }
 
 }  // namespace vt

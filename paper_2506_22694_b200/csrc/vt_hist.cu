@@ -8,7 +8,9 @@
 //     three 10-bit fields to a word (k_hist_packed): one shared-memory add per token and nothing else.
 //     A field hands 512 counts on to global memory whenever it gets there; the add that would wrap a
 //     field notices, and the stream is then counted again by the kernels of the next case.
-//   * otherwise a short pre-pass samples the stream, picks the hottest bins that fit (about 49.8 K of
+//   * more bins than that, in two to four ranges that fit: the same kernel, every range dealt to its own share of
+//     the CTAs, each share reading the whole stream (the second and later readers find it in L2).
+//   * the recount: a short pre-pass samples the stream, picks the hottest bins that fit (about 49.8 K of
 //     them for 128256 bins), and the main pass keeps those in shared memory; the rare cold tokens go
 //     to L2 with one red.global each.  The hot set only steers traffic: counts are exact whichever
 //     bins were picked.
@@ -144,7 +146,17 @@ k_hist_small(const int32_t* __restrict__ ids, int64_t n, int32_t V, uint32_t* __
 #pragma unroll
         for (int r = 0; r < kRows; ++r) tally4(x[r]);
     }
-    for (int64_t v = v0 + trips * (kRows * kThreads) + threadIdx.x; v < v1; v += kThreads) tally4(ld_stream_u4(vec + v));
+    {   // the rest, at most kRows rows, all of it in flight
+        const int64_t left = v1 - (v0 + trips * (kRows * kThreads)) - threadIdx.x;
+        uint4 x[kRows];
+#pragma unroll
+        for (int r = 0; r < kRows; ++r)
+            if (r * kThreads < left) x[r] = ld_stream_u4(p + r * kThreads);
+#pragma unroll
+        for (int r = 0; r < kRows; ++r)
+            if (r * kThreads < left) tally4(x[r]);
+    }
+    griddep_launch_dependents();
     __syncthreads();
     for (int i = threadIdx.x; i < V; i += kThreads) {
         const int v = (i + blockIdx.x * (V / (int)gridDim.x)) % V;   // the CTAs' flushes spread over the whole array
@@ -213,7 +225,9 @@ __global__ void __launch_bounds__(kThreads, 1)
 k_hist_pick(const uint32_t* __restrict__ sample, int32_t V, int32_t H, uint2* __restrict__ table,
             const uint32_t* __restrict__ gate) {
     extern __shared__ __align__(16) uint8_t s_dyn[];
-    if (gate && *gate == 0) return;                        // the packed count stood: nothing to recount
+    griddep_launch_dependents();
+    griddep_wait();
+    if (gate && *reinterpret_cast<const volatile uint32_t*>(gate) == 0) return;   // the packed count stood: nothing to recount
     __shared__ uint32_t s_hist[kPickBins];
     __shared__ uint32_t s_warp[33];
     __shared__ uint32_t s_definite;
@@ -317,7 +331,9 @@ __global__ void __launch_bounds__(kThreads, 1)
 k_hist_hot(const int32_t* __restrict__ ids, int64_t n, int32_t V, uint32_t* __restrict__ counts,
            const uint2* __restrict__ table, int32_t H, Ctrl* ctrl, const uint32_t* __restrict__ gate) {
     extern __shared__ __align__(16) uint8_t s_raw[];
-    if (gate && *gate == 0) return;
+    griddep_launch_dependents();
+    griddep_wait();
+    if (gate && *reinterpret_cast<const volatile uint32_t*>(gate) == 0) return;
     const int T32 = (V + 31) >> 5;
     // The lookup is repacked for the main pass: one 4-byte word per 16 ids = {16 membership bits,
     // 16-bit slot of the first member} -- a 4-byte gather costs half the shared-memory wavefronts of
@@ -450,12 +466,21 @@ static uint32_t packed_words(int32_t V, uint32_t* magic) {
     return 0;
 }
 
+// SPLIT: the vocabulary is cut into `parts` ranges of Vp ids; CTA c counts range c % parts of share c / parts of the
+// stream, and a token outside the CTA's range costs the instructions but not the add.  (Neighbouring CTAs read the
+// same ids at about the same time: one of them from HBM, the others from L2.)
+template <bool SPLIT, bool SHORT>
 __global__ void __launch_bounds__(kThreads, 1)
-k_hist_packed(const int32_t* __restrict__ ids, int64_t n, int32_t V, uint32_t W, uint32_t M,
-              uint32_t* __restrict__ out, uint32_t* __restrict__ gate) {
+k_hist_packed(const int32_t* __restrict__ ids, int64_t n, int32_t V, int32_t Vp, int32_t parts, uint32_t W, uint32_t M,
+              uint32_t* __restrict__ all_out, uint32_t* __restrict__ gate) {
     extern __shared__ __align__(16) uint32_t s_fields[];
     __shared__ uint32_t s_hot;
     __shared__ uint32_t s_own[32];                           // the hot id's counts, one word per lane
+    const int part = SPLIT ? (int)blockIdx.x % parts : 0;
+    const int share = SPLIT ? (int)blockIdx.x / parts : (int)blockIdx.x, shares = SPLIT ? (int)gridDim.x / parts : (int)gridDim.x;
+    const uint32_t lo = SPLIT ? (uint32_t)part * (uint32_t)Vp : 0u;       // first id of the CTA's range
+    const uint32_t mine = SPLIT ? min((uint32_t)Vp, (uint32_t)V - lo) : (uint32_t)V;
+    uint32_t* __restrict__ out = all_out + lo;               // (ids are relative to lo from the range test on)
     for (uint32_t i = threadIdx.x; i < W; i += kThreads) s_fields[i] = 0;
     if (threadIdx.x == 0) s_hot = kNoId;
     if (threadIdx.x < 32) s_own[threadIdx.x] = 0;
@@ -487,6 +512,30 @@ k_hist_packed(const int32_t* __restrict__ ids, int64_t n, int32_t V, uint32_t W,
                 : "r"(id), "r"(M), "r"(neg_w), "r"(base), "r"(hot), "r"(own) : "memory");
         return old;
     };
+    // The same for an id that may lie outside the CTA's range: then nothing is added and the test does not fire.
+    auto add_if_mine = [&](uint32_t id, uint32_t& low) -> uint32_t {
+        uint32_t old;
+        asm volatile("{\n\t"
+            ".reg .pred ph, pm;\n\t"
+            ".reg .b32 f, w, sh, a, inc;\n\t"
+            "setp.lt.u32 pm, %2, %8;\n\t"
+            "mul.hi.u32 f, %2, %3;\n\t"
+            "mad.lo.u32 w, f, %4, %2;\n\t"
+            "mul.lo.u32 sh, f, 10;\n\t"
+            "shl.b32 inc, 1, sh;\n\t"
+            "shl.b32 %1, 511, sh;\n\t"
+            "mad.lo.u32 a, w, 4, %5;\n\t"
+            "setp.eq.u32 ph, %2, %6;\n\t"
+            "selp.u32 a, %7, a, ph;\n\t"
+            "selp.u32 inc, 1, inc, ph;\n\t"
+            "selp.u32 %1, 0x80000000, %1, ph;\n\t"
+            "selp.u32 %1, %1, 0x80000000, pm;\n\t"
+            "mov.u32 %0, 0;\n\t"
+            "@pm atom.shared.add.u32 %0, [a], inc;\n\t"
+            "}" : "=&r"(old), "=&r"(low)
+                : "r"(id), "r"(M), "r"(neg_w), "r"(base), "r"(hot), "r"(own), "r"(mine) : "memory");
+        return old;
+    };
     static_assert(kFieldBits == 10 && kSpill == 512, "written into the instructions above");
     // The add found the low nine bits of its field set: kSpill-1 (hand kSpill counts on) or kFieldMax (wrapped).
     auto settle_field = [&](uint32_t id, uint32_t old) {
@@ -499,29 +548,30 @@ k_hist_packed(const int32_t* __restrict__ ids, int64_t n, int32_t V, uint32_t W,
             if (*reinterpret_cast<volatile uint32_t*>(&s_hot) == kNoId) atomicCAS(&s_hot, kNoId, id);
         }
     };
+    auto add = [&](uint32_t id, uint32_t& low) -> uint32_t { return SPLIT ? add_if_mine(id, low) : add_one(id, low); };
     auto tally_in_range = [&](uint32_t id) {
         uint32_t low;
-        const uint32_t old = add_one(id, low);
-        if ((~old & low) == 0) settle_field(id, old);
+        const uint32_t old = add(id - lo, low);
+        if ((~old & low) == 0) settle_field(id - lo, old);
     };
     auto tally1 = [&](uint32_t id) {
-        if (id < (uint32_t)V) tally_in_range(id); else ++bad;
+        if (id < (uint32_t)V) tally_in_range(id); else bad += part == 0 ? 1 : 0;
     };
     // Four tokens of one 128-bit load: four adds in flight, their tests folded into one branch (taken once
     // in about kSpill / 4 loads).
     auto tally4 = [&](uint4 x) {
         if (max(max(x.x, x.y), max(x.z, x.w)) < (uint32_t)V) {       // one range test per 128-bit load
             uint32_t la, lb, lc, ld;
-            const uint32_t oa = add_one(x.x, la);
-            const uint32_t ob = add_one(x.y, lb);
-            const uint32_t oc = add_one(x.z, lc);
-            const uint32_t od = add_one(x.w, ld);
+            const uint32_t oa = add(x.x - lo, la);
+            const uint32_t ob = add(x.y - lo, lb);
+            const uint32_t oc = add(x.z - lo, lc);
+            const uint32_t od = add(x.w - lo, ld);
             const uint32_t za = ~oa & la, zb = ~ob & lb, zc = ~oc & lc, zd = ~od & ld;
             if (min(min(za, zb), min(zc, zd)) == 0) {
-                if (za == 0) settle_field(x.x, oa);
-                if (zb == 0) settle_field(x.y, ob);
-                if (zc == 0) settle_field(x.z, oc);
-                if (zd == 0) settle_field(x.w, od);
+                if (za == 0) settle_field(x.x - lo, oa);             // (at once: what is added meanwhile may wrap the field)
+                if (zb == 0) settle_field(x.y - lo, ob);
+                if (zc == 0) settle_field(x.z - lo, oc);
+                if (zd == 0) settle_field(x.w - lo, od);
             }
         } else {
             tally1(x.x); tally1(x.y); tally1(x.z); tally1(x.w);
@@ -536,38 +586,58 @@ k_hist_packed(const int32_t* __restrict__ ids, int64_t n, int32_t V, uint32_t W,
     if (head > n) head = n;
     const int64_t nvec = (n - head) >> 2;
     const int64_t tail0 = head + nvec * 4;
-    if (blockIdx.x == 0) {
+    if (share == 0) {
         if ((int64_t)threadIdx.x < head) tally1((uint32_t)ids[threadIdx.x]);
         const int64_t t = tail0 + threadIdx.x;
         if (t < n) tally1((uint32_t)ids[t]);
     }
     const uint4* vec = reinterpret_cast<const uint4*>(ids + head);
-    const int64_t v0 = nvec * blockIdx.x / gridDim.x;
-    const int64_t v1 = nvec * (blockIdx.x + 1) / gridDim.x;
+    const int64_t v0 = nvec * share / shares;
+    const int64_t v1 = nvec * (share + 1) / shares;
     const int64_t trips = (v1 - v0) / (kRows * kThreads);
     const uint4* p = vec + v0 + threadIdx.x;
-    for (int64_t t = 0; t < trips; ++t, p += kRows * kThreads) {
-        uint4 x[kRows];
+    if (SHORT) {
+        // The CTA's share is all careful trips (kShortIds): guarded rows, all of them requested before any is counted -- a
+        // small stream is nothing but this, and one load at a time it is nothing but their latencies (1e6 / 3e6 / 1e7 ids:
+        // 31 / 32 / 41 -> 25 / 29 / 37 us per call).  An instance of its own: the same code behind the long loop slowed
+        // that by 1 to 10 %.
+        for (int64_t v = v0 + threadIdx.x; v < v1; v += kRows * kThreads, p += kRows * kThreads) {
+            uint4 x[kRows];
 #pragma unroll
-        for (int r = 0; r < kRows; ++r) x[r] = ld_stream_u4(p + r * kThreads);
-        if (hot == kNoId) hot = *reinterpret_cast<volatile uint32_t*>(&s_hot);   // once set it stays
-        if (t < kCarefulTrips) {
+            for (int r = 0; r < kRows; ++r)
+                if (v + r * kThreads < v1) x[r] = ld_stream_u4(p + r * kThreads);
+            if (hot == kNoId) hot = *reinterpret_cast<volatile uint32_t*>(&s_hot);
 #pragma unroll
-            for (int r = 0; r < kRows; ++r) tally4_in_turn(x[r]);
-        } else {
-#pragma unroll
-            for (int r = 0; r < kRows; ++r) tally4(x[r]);
+            for (int r = 0; r < kRows; ++r)
+                if (v + r * kThreads < v1) tally4_in_turn(x[r]);
         }
+    } else {
+        for (int64_t t = 0; t < trips; ++t, p += kRows * kThreads) {
+            uint4 x[kRows];
+#pragma unroll
+            for (int r = 0; r < kRows; ++r) x[r] = ld_stream_u4(p + r * kThreads);
+            if (hot == kNoId) hot = *reinterpret_cast<volatile uint32_t*>(&s_hot);   // once set it stays
+            if (t < kCarefulTrips) {
+#pragma unroll
+                for (int r = 0; r < kRows; ++r) tally4_in_turn(x[r]);
+            } else {
+#pragma unroll
+                for (int r = 0; r < kRows; ++r) tally4(x[r]);
+            }
+        }
+        for (int64_t v = v0 + trips * (kRows * kThreads) + threadIdx.x; v < v1; v += kThreads) tally4_in_turn(ld_stream_u4(vec + v));
     }
-    for (int64_t v = v0 + trips * (kRows * kThreads) + threadIdx.x; v < v1; v += kThreads) tally4_in_turn(ld_stream_u4(vec + v));
+    griddep_launch_dependents();                             // (the settling kernel waits for this one's end)
     __syncthreads();
+    const uint32_t first = blockIdx.x * (W / gridDim.x);         // the CTAs' flushes spread over the whole array
     for (uint32_t i = threadIdx.x; i < W; i += kThreads) {
-        const uint32_t w = (i + blockIdx.x * (W / gridDim.x)) % W;   // the CTAs' flushes spread over the whole array
+        const uint32_t w = i + first < W ? i + first : i + first - W;
         const uint32_t x = s_fields[w];
+        if (x == 0) continue;
 #pragma unroll
         for (uint32_t f = 0; f < 3; ++f) {
             const uint32_t c = (x >> (f * kFieldBits)) & kFieldMax, id = f * W + w;
-            if (c && id < (uint32_t)V) atomicAdd(&out[id], c);
+            if (c && id < mine) atomicAdd(&out[id], c);
         }
     }
     if (threadIdx.x < 32) {                                  // (only lanes that had read s_hot added to s_own)
@@ -589,7 +659,9 @@ k_hist_settle(const int32_t* __restrict__ ids, int64_t n, int32_t V, const uint3
               const uint32_t* __restrict__ gate, Ctrl* ctrl) {
     __shared__ int s_tag[kSampleSlots];
     __shared__ uint32_t s_cnt[kSampleSlots];
-    const bool recount = gate[0] != 0;
+    griddep_launch_dependents();
+    griddep_wait();
+    const bool recount = *reinterpret_cast<const volatile uint32_t*>(gate) != 0;
     for (int v = blockIdx.x * kThreads + threadIdx.x; v < V; v += gridDim.x * kThreads) {
         const uint32_t c = recount ? 0u : packed[v];
         counts[v] = accumulate ? counts[v] + c : c;
@@ -666,28 +738,72 @@ bool hist_supported(int32_t V) {
     return ((size_t)V + 31) / 32 * 8 <= kMaxTableBytes;
 }
 
-static bool packed_fits(int32_t V) { return packed_words(V, nullptr) != 0; }
+constexpr int kMaxParts = 4;                   // (V <= 655360 by the lookup table: four ranges of at most 172 K ids)
+// Ranges the packed kernel needs for V bins, and the ids of one; 0: too many.
+static int packed_parts(int32_t V, int32_t* Vp) {
+    for (int p = 1; p <= kMaxParts; ++p) {
+        const int32_t each = (V + p - 1) / p;
+        if (packed_words(each, nullptr)) {
+            if (Vp) *Vp = each;
+            return p;
+        }
+    }
+    return 0;
+}
 
-HistPlan hist_plan(int32_t V) {
+static HistPlan plan_for(int32_t V, int parts) {
     HistPlan p{};
-    p.small = (size_t)V * 4 <= kDynSmem;
-    if (p.small) { p.off_sample = p.off_packed = p.off_gate = p.off_table = 0; p.bytes = 0; return p; }
+    p.parts = parts;
     const size_t T32 = ((size_t)V + 31) / 32;
     // sample, packed counts and gate lie together: one memset clears all three
     p.off_sample = 0;
     p.off_packed = (size_t)V * 4;
-    p.off_gate = packed_fits(V) ? 2 * (size_t)V * 4 : p.off_packed;
-    p.clear_bytes = packed_fits(V) ? p.off_gate + kGateWords * 4 : (size_t)V * 4;
+    p.off_gate = parts ? 2 * (size_t)V * 4 : p.off_packed;
+    // (the gate's 64-bit count of skipped ids wants an 8-byte boundary: V * 8 is one)
+    p.clear_bytes = parts ? p.off_gate + kGateWords * 4 : (size_t)V * 4;
     p.off_table = align_up(p.clear_bytes, 256);
     p.bytes = p.off_table + align_up(T32 * 8, 256);
     return p;
 }
 
+// Several ranges against the hot / cold kernels: P ranges cost 1.8 / 2.6 / 3.5 us per million ids (P = 2 / 3 / 4) and
+// 20-30 us per call, the hot / cold pair 1.3-1.4 us per million and 120-225 us per call for its pre-passes.  The lines
+// cross at 250 / 112 / 100 million ids; the ranges are taken up to 200 million / (P - 1).
+constexpr int64_t kSplitIds = 200000000;
+
+HistPlan hist_plan(int32_t V, int64_t n, size_t scratch_bytes) {
+    HistPlan p{};
+    p.small = (size_t)V * 4 <= kDynSmem;
+    if (p.small) return p;
+    const int parts = packed_parts(V, nullptr);
+    p = plan_for(V, parts);
+    if (parts > 1 && (n * (parts - 1) > kSplitIds || p.bytes > scratch_bytes)) p = plan_for(V, 0);
+    return p;
+}
+
+size_t hist_min_bytes(int32_t V) {
+    const HistPlan p = hist_plan(V, 0, SIZE_MAX);
+    return p.small ? 0 : p.parts > 1 ? plan_for(V, 0).bytes : p.bytes;
+}
+
+constexpr int64_t kShortIds = (int64_t)kCarefulTrips * kRows * kThreads * 4;       // ids of a CTA's careful trips
+
+template <bool SPLIT, bool SHORT>
+static cudaError_t launch_packed(int grid, const int32_t* ids, int64_t n, int32_t V, int32_t Vp, int parts, uint32_t W, uint32_t M,
+                                 uint32_t* packed, uint32_t* gate, cudaStream_t s) {
+    static int done[kMaxDevices] = {0};
+    const cudaError_t e = set_smem_once(reinterpret_cast<const void*>(k_hist_packed<SPLIT, SHORT>), kDynSmem, done);
+    if (e != cudaSuccess) return e;
+    k_hist_packed<SPLIT, SHORT><<<grid, kThreads, (size_t)W * 4, s>>>(ids, n, V, Vp, parts, W, M, packed, gate);
+    count_launch();
+    return cudaGetLastError();
+}
+
 cudaError_t launch_histogram(const int32_t* ids, int64_t n, int32_t V, uint32_t* counts,
-                             int accumulate, Ctrl* ctrl, uint8_t* scratch, cudaStream_t s) {
+                             int accumulate, Ctrl* ctrl, uint8_t* scratch, size_t scratch_bytes, cudaStream_t s) {
     cudaError_t e;
-    const HistPlan p = hist_plan(V);
-    const bool packed_path = !p.small && packed_fits(V) && n != 0;
+    const HistPlan p = hist_plan(V, n, scratch_bytes);
+    const bool packed_path = !p.small && p.parts != 0 && n != 0;
     if (!accumulate && !packed_path) {                     // (the packed path's second kernel writes every count)
         e = cudaMemsetAsync(counts, 0, (size_t)V * 4, s);
         if (e != cudaSuccess) return e;
@@ -714,7 +830,7 @@ cudaError_t launch_histogram(const int32_t* ids, int64_t n, int32_t V, uint32_t*
     uint2* table = reinterpret_cast<uint2*>(scratch + p.off_table);
     e = cudaMemsetAsync(scratch, 0, p.clear_bytes, s);
     if (e != cudaSuccess) return e;
-    static int done_pick[kMaxDevices] = {0}, done_hot[kMaxDevices] = {0}, done_packed[kMaxDevices] = {0};
+    static int done_pick[kMaxDevices] = {0}, done_hot[kMaxDevices] = {0};
     e = set_smem_once(reinterpret_cast<const void*>(k_hist_pick), kMaxTableBytes, done_pick);
     if (e != cudaSuccess) return e;
     e = set_smem_once(reinterpret_cast<const void*>(k_hist_hot), kDynSmem, done_hot);
@@ -722,29 +838,34 @@ cudaError_t launch_histogram(const int32_t* ids, int64_t n, int32_t V, uint32_t*
     // a refused launch must stop the chain: the main pass would count through an unwritten table
     const uint32_t* gate = nullptr;
     if (packed_path) {
-        // all bins in shared memory, packed; the three kernels after it return at once unless a field wrapped
-        e = set_smem_once(reinterpret_cast<const void*>(k_hist_packed), kDynSmem, done_packed);
-        if (e != cudaSuccess) return e;
+        // all bins in shared memory, packed; of the three kernels after it two return at once unless a field wrapped
         uint32_t M = 0;
-        const uint32_t W = packed_words(V, &M);
+        int32_t Vp = V;
+        const int parts = packed_parts(V, &Vp);
+        const uint32_t W = packed_words(Vp, &M);
         uint32_t* packed = reinterpret_cast<uint32_t*>(scratch + p.off_packed);
         uint32_t* g = reinterpret_cast<uint32_t*>(scratch + p.off_gate);
-        k_hist_packed<<<grid, kThreads, (size_t)W * 4, s>>>(ids, n, V, W, M, packed, g);
-        count_launch();
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        k_hist_settle<<<grid, kThreads, 0, s>>>(ids, n, V, packed, counts, accumulate, sample, g, ctrl);
+        int shares = parts > 1 ? sms / parts : sms;
+        if (shares < 1) shares = 1;
+        if (shares > grid) shares = grid;                  // (never more than one share per 4096 ids)
+        const bool brief = n <= (int64_t)shares * kShortIds;
+        if (parts == 1) e = brief ? launch_packed<false, true>(shares, ids, n, V, V, 1, W, M, packed, g, s)
+                                  : launch_packed<false, false>(shares, ids, n, V, V, 1, W, M, packed, g, s);
+        else e = brief ? launch_packed<true, true>(shares * parts, ids, n, V, Vp, parts, W, M, packed, g, s)
+                       : launch_packed<true, false>(shares * parts, ids, n, V, Vp, parts, W, M, packed, g, s);
+        if (e != cudaSuccess) return e;
+        e = launch_dependent(k_hist_settle, grid, kThreads, 0, s, ids, n, V, (const uint32_t*)packed, counts, accumulate, sample,
+                             (const uint32_t*)g, ctrl);
         gate = g;
     } else {
         k_hist_sample<<<grid, kThreads, 0, s>>>(ids, n, V, sample);
+        count_launch();
+        e = cudaGetLastError();
     }
-    count_launch();
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    k_hist_pick<<<1, kThreads, T32 * 8, s>>>(sample, V, H, table, gate);
-    count_launch();
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    k_hist_hot<<<grid, kThreads, kDynSmem, s>>>(ids, n, V, counts, table, H, ctrl, gate);
-    count_launch();
-    return cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    e = launch_dependent(k_hist_pick, 1, kThreads, T32 * 8, s, (const uint32_t*)sample, V, H, table, gate);
+    if (e != cudaSuccess) return e;
+    return launch_dependent(k_hist_hot, grid, kThreads, kDynSmem, s, ids, n, V, counts, (const uint2*)table, H, ctrl, gate);
 }
 
 }  // namespace vt

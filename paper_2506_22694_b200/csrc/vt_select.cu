@@ -365,6 +365,8 @@ k_select_sort(const uint32_t* counts, int32_t V, int32_t K, int32_t* map, int32_
     if (threadIdx.x < kDeals * kCluster) { (&s_load[0][0])[threadIdx.x] = 0; (&s_work[0][0])[threadIdx.x] = 0u; }
     if (threadIdx.x < kDeals) { s_lo[threadIdx.x] = 0x7fffffff; s_hi[threadIdx.x] = 0; s_cut_owner[threadIdx.x] = -1; }
     if (threadIdx.x == 0) { s_cut = -1; s_big = 0; s_K = 0; s_first = 0; s_T = 0; s_mass_before = 0; }
+    griddep_launch_dependents();
+    griddep_wait();                                     // (the counts come from the kernel before)
     __syncthreads();
     // phase 1: bucket counts (descending order: inverted bucket index), and per warp the ids of every exact count
     for (int i = w0 + lane; i < w1; i += 32 * kInFlight) {
@@ -737,11 +739,10 @@ cudaError_t launch_select_cut(const uint32_t* counts, int32_t V, int mode, doubl
     cudaError_t e = select_smem_attr();
     if (e != cudaSuccess) return e;
     if (mode == 0)
-        k_select_sort<1><<<kCluster, kThreads, kSelectSmem, s>>>(counts, V, 0, map, inv_map, keyA, valA, keyB, valB, pfrac, 0u, k_out);
-    else
-        k_select_sort<2><<<kCluster, kThreads, kSelectSmem, s>>>(counts, V, 0, map, inv_map, keyA, valA, keyB, valB, 1.0, min_count, k_out);
-    count_launch();
-    return cudaGetLastError();
+        return launch_dependent(k_select_sort<1>, kCluster, kThreads, kSelectSmem, s, counts, V, 0, map, inv_map, keyA, valA, keyB, valB,
+                                pfrac, 0u, k_out);
+    return launch_dependent(k_select_sort<2>, kCluster, kThreads, kSelectSmem, s, counts, V, 0, map, inv_map, keyA, valA, keyB, valB, 1.0,
+                            min_count, k_out);
 }
 
 size_t select_scratch_bytes(int32_t V) { return 4 * align_up((size_t)V * 4, 256); }
@@ -758,9 +759,8 @@ cudaError_t launch_select_topk(const uint32_t* counts, int32_t V, int32_t K, int
     if (e != cudaSuccess) return e;
     // (whatever K: even K = V is the selection's work when most ids were seen fewer than 1024 times -- 31 against
     // 56 us on the counts of 3 M tokens -- and costs it one bucket pass, 13 us, before the full ranking when not)
-    k_select_sort<0><<<kCluster, kThreads, kSelectSmem, s>>>(counts, V, K, map, inv_map, keyA, valA, keyB, valB, 1.0, 0u, nullptr);
-    count_launch();
-    return cudaGetLastError();
+    return launch_dependent(k_select_sort<0>, kCluster, kThreads, kSelectSmem, s, counts, V, K, map, inv_map, keyA, valA, keyB, valB, 1.0, 0u,
+                            (int32_t*)nullptr);
 }
 
 }  // namespace vt
