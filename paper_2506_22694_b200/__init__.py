@@ -102,12 +102,16 @@ def _check(call: str, status: int) -> None:
         raise VocabTrimError(call, status)
 
 
+# Marshalling.  A drafting step is a few tens of microseconds on the device, so what Python does per call shows: pointers
+# go to ctypes as plain integers (None = NULL), the raw stream handle comes from torch's C layer without a Stream
+# object, outputs are allocated through an input's new_empty, and the size of a caller's workspace is checked by the
+# library, which does it anyway.
 def _ptr(t):
-    return c_void_p(t.data_ptr()) if t is not None else c_void_p(0)
+    return t.data_ptr() if t is not None else None
 
 
-def _stream() -> c_void_p:
-    return c_void_p(torch.cuda.current_stream().cuda_stream)
+def _stream():
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
 
 
 def _dev(t: torch.Tensor, dtype, name: str) -> torch.Tensor:
@@ -145,12 +149,16 @@ class Workspace:
         return int(st), int(flags.value), int(bad.value)
 
 
-def _ws(ws: Workspace | None, need: int, like: torch.Tensor) -> Workspace:
+def _run(call: str, op: int, shape, ws: Workspace | None, like: torch.Tensor, *args, tail=()) -> None:
+    """One library call on the current stream: args, the workspace (the caller's, or one made for the call), the stream, tail."""
     if ws is None:
-        return Workspace(need, like.device)
-    if ws.nbytes < need:
-        raise VocabTrimError("workspace too small (%d < %d)" % (ws.nbytes, need), 3)
-    return ws
+        ws = Workspace(workspace_bytes(op, *shape), like.device)
+    status = getattr(lib(), call)(*args, ws.ptr, ws.nbytes, _stream(), *tail)
+    if status:
+        need = workspace_bytes(op, *shape) if status == 3 else 0
+        if ws.nbytes < need:
+            raise VocabTrimError("workspace too small (%d < %d)" % (ws.nbytes, need), 3)
+        raise VocabTrimError(call, status)
 
 
 def vt_histogram(ids: torch.Tensor, V: int, counts: torch.Tensor | None = None, accumulate: bool = False,
@@ -161,9 +169,8 @@ def vt_histogram(ids: torch.Tensor, V: int, counts: torch.Tensor | None = None, 
         counts = torch.empty(V, dtype=torch.int32, device=ids.device)
         accumulate = False
     _dev(counts, torch.int32, "counts")
-    ws = _ws(ws, workspace_bytes(VT_OP_HISTOGRAM, ids.numel(), V), ids)
-    _check("vt_histogram", lib().vt_histogram(_ptr(ids), ids.numel(), V, _ptr(counts), int(bool(accumulate)),
-                                              c_void_p(ws.ptr), ws.nbytes, _stream()))
+    n = ids.numel()
+    _run("vt_histogram", VT_OP_HISTOGRAM, (n, V), ws, ids, ids.data_ptr(), n, V, counts.data_ptr(), 1 if accumulate else 0)
     return counts
 
 
@@ -182,34 +189,27 @@ def vt_select_topk(counts: torch.Tensor, K: int, ws: Workspace | None = None):
     """Eq. 1 (token selection).  counts [V] -> (map int32 [K], inv_map int32 [V])."""
     _dev(counts, torch.int32, "counts")
     V = counts.numel()
-    map_ = torch.empty(K, dtype=torch.int32, device=counts.device)
-    inv = torch.empty(V, dtype=torch.int32, device=counts.device)
-    ws = _ws(ws, workspace_bytes(VT_OP_SELECT_TOPK, 0, V, K), counts)
-    _check("vt_select_topk", lib().vt_select_topk(_ptr(counts), V, K, _ptr(map_), _ptr(inv), c_void_p(ws.ptr),
-                                                  ws.nbytes, _stream()))
+    map_, inv = counts.new_empty(K), counts.new_empty(V)
+    _run("vt_select_topk", VT_OP_SELECT_TOPK, (0, V, K), ws, counts, counts.data_ptr(), V, K, map_.data_ptr(), inv.data_ptr())
     return map_, inv
 
 
 def _select_cut(counts: torch.Tensor, ws, call, *arg):
     _dev(counts, torch.int32, "counts")
     V = counts.numel()
-    map_ = torch.empty(V, dtype=torch.int32, device=counts.device)
-    inv = torch.empty(V, dtype=torch.int32, device=counts.device)
-    k_out = torch.empty(1, dtype=torch.int32, device=counts.device)
-    ws = _ws(ws, workspace_bytes(VT_OP_SELECT_TOPK, 0, V, V), counts)
-    fn = getattr(lib(), call)
-    _check(call, fn(_ptr(counts), V, *arg, _ptr(map_), _ptr(inv), _ptr(k_out), c_void_p(ws.ptr), ws.nbytes, _stream()))
+    map_, inv, k_out = counts.new_empty(V), counts.new_empty(V), counts.new_empty(1)
+    _run(call, VT_OP_SELECT_TOPK, (0, V, V), ws, counts, counts.data_ptr(), V, *arg, map_.data_ptr(), inv.data_ptr(), k_out.data_ptr())
     return k_out, map_, inv
 
 
 def vt_select_topp(counts: torch.Tensor, p: float, ws: Workspace | None = None):
     """Top-P selection (Method section): returns (K device int32 [1], map [V] whose first K entries are the trimmed vocabulary, inv_map [V])."""
-    return _select_cut(counts, ws, "vt_select_topp", c_double(float(p)))
+    return _select_cut(counts, ws, "vt_select_topp", float(p))
 
 
 def vt_select_minfreq(counts: torch.Tensor, min_count: int, ws: Workspace | None = None):
     """Minimum-frequency selection (Method section): returns (K device int32 [1], map [V] (first K entries), inv_map [V])."""
-    return _select_cut(counts, ws, "vt_select_minfreq", c_uint32(int(min_count)))
+    return _select_cut(counts, ws, "vt_select_minfreq", int(min_count) & 0xffffffff)
 
 
 def tree_pool(capacity: int, device="cuda"):
@@ -232,7 +232,7 @@ def vt_tree_expand(cand_ids: torch.Tensor, cand_logprobs: torch.Tensor, frontier
     _dev(tok, torch.int32, "pool token"), _dev(par, torch.int32, "pool parent"), _dev(sc, torch.float32, "pool score")
     if frontier_nodes is not None and _dev(frontier_nodes, torch.int32, "frontier_nodes").numel() != B:
         raise ValueError("frontier_nodes must have B entries")
-    nxt = torch.empty(n_front, dtype=torch.int32, device=cand_ids.device)
+    nxt = cand_ids.new_empty(n_front)
     _check("vt_tree_expand", lib().vt_tree_expand(
         _ptr(cand_ids), _ptr(cand_logprobs), B, ld - col0, ld, col0, _ptr(frontier_nodes), _ptr(tok), _ptr(par),
         _ptr(sc), pool_base, min(tok.numel(), par.numel(), sc.numel()), n_front, _ptr(nxt), _stream()))
@@ -263,12 +263,11 @@ def vt_draft_head_expand(h: torch.Tensor, W_trim: torch.Tensor, map_: torch.Tens
         out = (torch.empty((B, 1 + topk), dtype=torch.int32, device=h.device),
                torch.empty((B, 1 + topk), dtype=torch.float32, device=h.device))
     ids, lps = out
-    nxt = torch.empty(n_front, dtype=torch.int32, device=h.device)
-    ws = _ws(ws, workspace_bytes(VT_OP_DRAFT_HEAD, 0, 0, K, d, B, topk), h)
-    _check("vt_draft_head_expand", lib().vt_draft_head_expand(
-        _ptr(h), _ptr(W_trim), _ptr(map_), B, K, d, _ptr(temp), topk, _ptr(uniforms), _ptr(ids), _ptr(lps),
-        _ptr(frontier_nodes), _ptr(tok), _ptr(par), _ptr(sc), pool_base, min(tok.numel(), par.numel(), sc.numel()),
-        n_front, _ptr(nxt), c_void_p(ws.ptr), ws.nbytes, _stream()))
+    nxt = tok.new_empty(n_front)
+    _run("vt_draft_head_expand", VT_OP_DRAFT_HEAD, (0, 0, K, d, B, topk), ws, h,
+         h.data_ptr(), W_trim.data_ptr(), _ptr(map_), B, K, d, temp.data_ptr(), topk, _ptr(uniforms), ids.data_ptr(), lps.data_ptr(),
+         _ptr(frontier_nodes), tok.data_ptr(), par.data_ptr(), sc.data_ptr(), pool_base, min(tok.numel(), par.numel(), sc.numel()),
+         n_front, nxt.data_ptr())
     return ids, lps, nxt
 
 
@@ -278,7 +277,7 @@ def vt_tree_rerank(pool, n: int, budget: int):
     _dev(tok, torch.int32, "pool token"), _dev(par, torch.int32, "pool parent"), _dev(sc, torch.float32, "pool score")
     if n > min(tok.numel(), par.numel(), sc.numel()):
         raise ValueError("n exceeds the pool")
-    outs = [torch.empty(budget, dtype=torch.int32, device=tok.device) for _ in range(3)]
+    outs = [tok.new_empty(budget) for _ in range(3)]
     _check("vt_tree_rerank", lib().vt_tree_rerank(_ptr(tok), _ptr(par), _ptr(sc), n, budget, _ptr(outs[0]),
                                                   _ptr(outs[1]), _ptr(outs[2]), _stream()))
     return tuple(outs)
@@ -301,12 +300,9 @@ def vt_verify_greedy(token: torch.Tensor, parent: torch.Tensor | None, target: t
             raise ValueError("parent must be [S, N]")
     if tokens_total is not None:
         _dev(tokens_total, torch.int64, "tokens_total")
-    n_accept = torch.empty(S, dtype=torch.int32, device=token.device)
-    path = torch.empty(S, N, dtype=torch.int32, device=token.device)
-    emitted = torch.empty(S, N + 1, dtype=torch.int32, device=token.device)
+    n_accept, path, emitted = token.new_empty(S), token.new_empty((S, N)), token.new_empty((S, N + 1))
     _check("vt_verify_greedy", lib().vt_verify_greedy(
-        _ptr(token), _ptr(parent) if parent is not None else None, _ptr(target), S, N, _ptr(n_accept),
-        _ptr(path), _ptr(emitted), _ptr(tokens_total) if tokens_total is not None else None, _stream()))
+        _ptr(token), _ptr(parent), _ptr(target), S, N, _ptr(n_accept), _ptr(path), _ptr(emitted), _ptr(tokens_total), _stream()))
     return n_accept, path, emitted
 
 
@@ -335,11 +331,8 @@ def vt_build_vocab(ids: torch.Tensor, V: int, K: int, ws: Workspace | None = Non
     if not ids.is_cuda:
         return vt_build_vocab_host(ids, V, K, ws)
     _dev(ids, torch.int32, "ids")
-    map_ = torch.empty(K, dtype=torch.int32, device=ids.device)
-    inv = torch.empty(V, dtype=torch.int32, device=ids.device)
-    ws = _ws(ws, workspace_bytes(VT_OP_BUILD_VOCAB, ids.numel(), V, K), ids)
-    _check("vt_build_vocab", lib().vt_build_vocab(_ptr(ids), ids.numel(), V, K, _ptr(map_), _ptr(inv),
-                                                  c_void_p(ws.ptr), ws.nbytes, _stream()))
+    map_, inv, n = ids.new_empty(K), ids.new_empty(V), ids.numel()
+    _run("vt_build_vocab", VT_OP_BUILD_VOCAB, (n, V, K), ws, ids, ids.data_ptr(), n, V, K, map_.data_ptr(), inv.data_ptr())
     return map_, inv
 
 
@@ -350,10 +343,8 @@ def vt_build_vocab_host(ids_host: torch.Tensor, V: int, K: int, ws: Workspace | 
     if out is None:
         out = (torch.empty(K, dtype=torch.int32, device=device), torch.empty(V, dtype=torch.int32, device=device))
     map_, inv = out
-    ws = _ws(ws, workspace_bytes(VT_OP_BUILD_VOCAB_HOST, ids_host.numel(), V, K), map_)
-    _check("vt_build_vocab_host", lib().vt_build_vocab_host(
-        c_void_p(ids_host.data_ptr()), ids_host.numel(), V, K, _ptr(map_), _ptr(inv), c_void_p(ws.ptr),
-        ws.nbytes, _stream()))
+    n = ids_host.numel()
+    _run("vt_build_vocab_host", VT_OP_BUILD_VOCAB_HOST, (n, V, K), ws, map_, ids_host.data_ptr(), n, V, K, map_.data_ptr(), inv.data_ptr())
     return map_, inv
 
 
@@ -365,10 +356,10 @@ def vt_trim_head(W_full: torch.Tensor, map_: torch.Tensor, W_trim: torch.Tensor 
     V, d = W_full.shape
     K = map_.numel()
     if W_trim is None:
-        W_trim = torch.empty((K, d), dtype=torch.bfloat16, device=W_full.device)
+        W_trim = W_full.new_empty((K, d))
     _dev(W_trim, torch.bfloat16, "W_trim")
     _check("vt_trim_head", lib().vt_trim_head(_ptr(W_full), _ptr(map_), _ptr(W_trim), V, K, d,
-                                              c_void_p(ws.ptr if ws else 0), _stream()))
+                                              ws.ptr if ws else None, _stream()))
     return W_trim
 
 
@@ -393,18 +384,14 @@ def vt_draft_head(h: torch.Tensor, W_trim: torch.Tensor, map_: torch.Tensor | No
         out = (torch.empty((B, 1 + topk), dtype=torch.int32, device=h.device),
                torch.empty((B, 1 + topk), dtype=torch.float32, device=h.device))
     ids, lps = out
-    ws = _ws(ws, workspace_bytes(VT_OP_DRAFT_HEAD, 0, 0, K, d, B, topk), h)
-    args = [_ptr(h), _ptr(W_trim), _ptr(map_), B, K, d, _ptr(temp), topk, _ptr(uniforms), _ptr(ids), _ptr(lps),
-            c_void_p(ws.ptr), ws.nbytes, _stream()]
+    args = (h.data_ptr(), W_trim.data_ptr(), _ptr(map_), B, K, d, temp.data_ptr(), topk, _ptr(uniforms), ids.data_ptr(), lps.data_ptr())
+    shape = (0, 0, K, d, B, topk)
     if debug:
         logits = torch.empty((B, K), dtype=torch.float32, device=h.device)
         lse = torch.empty(B, dtype=torch.float32, device=h.device)
-        _check("vt_draft_head_debug", lib().vt_draft_head_debug(*args, _ptr(logits), _ptr(lse)))
+        _run("vt_draft_head_debug", VT_OP_DRAFT_HEAD, shape, ws, h, *args, tail=(logits.data_ptr(), lse.data_ptr()))
         return ids, lps, logits, lse
-    if overlapped:
-        _check("vt_draft_head_overlapped", lib().vt_draft_head_overlapped(*args))
-    else:
-        _check("vt_draft_head", lib().vt_draft_head(*args))
+    _run("vt_draft_head_overlapped" if overlapped else "vt_draft_head", VT_OP_DRAFT_HEAD, shape, ws, h, *args)
     return ids, lps
 
 
@@ -418,7 +405,6 @@ def vt_draft_head_host(h_host: torch.Tensor, W_trim: torch.Tensor, map_: torch.T
     K = W_trim.shape[0]
     ids, lps = out_host
     _check("vt_draft_head_host", lib().vt_draft_head_host(
-        c_void_p(h_host.data_ptr()), _ptr(W_trim), _ptr(map_), B, K, d, c_void_p(temp_host.data_ptr()), topk,
-        c_void_p(uniforms_host.data_ptr() if uniforms_host is not None else 0), c_void_p(ids.data_ptr()),
-        c_void_p(lps.data_ptr()), c_void_p(ws.ptr), ws.nbytes, _stream()))
+        h_host.data_ptr(), _ptr(W_trim), _ptr(map_), B, K, d, temp_host.data_ptr(), topk, _ptr(uniforms_host),
+        ids.data_ptr(), lps.data_ptr(), ws.ptr, ws.nbytes, _stream()))
     return ids, lps
