@@ -174,20 +174,23 @@ __device__ __noinline__ void merge_records(const MergeOut a, Ctrl* ctrl, float* 
             hz[o] = (on && a.sampled) ? ld_cg_f32(fp + 2 * kMaxGrid + c) : 0.f;
             hk[o] = (on && a.sampled) ? ld_cg_u64(kp + c) : 0ull;
         }
-        // this lane's CTAs in CTA order, then across lanes: the row's maximum by one warp reduction,
-        // every lane's sum rescaled to it once, a butterfly of additions (a fixed order: the result does
-        // not depend on which CTA finished when)
-        float M = -CUDART_INF_F, S = 0.f, gz = 0.f;
+        // the row's maximum over this lane's CTAs and by one warp reduction, every CTA's sum rescaled to it once, added in
+        // CTA order, a butterfly of additions (a fixed order: the result does not depend on which CTA finished when)
+        float M = hm[0], gz = 0.f;
         unsigned long long gk = 0ull;
 #pragma unroll
+        for (int o = 1; o < kMaxOwn; ++o) M = fmaxf(M, hm[o]);
+#pragma unroll
         for (int o = 0; o < kMaxOwn; ++o) {
-            lse_merge(M, S, hm[o], hs[o]);
             const bool w = hk[o] > gk;
             gk = w ? hk[o] : gk;
             gz = w ? hz[o] : gz;
         }
         const float Mall = ord2f(__reduce_max_sync(0xffffffffu, f2ord(M)));
-        float sc = (M == -CUDART_INF_F) ? 0.f : S * __expf(M - Mall);
+        const float Mref = Mall == -CUDART_INF_F ? 0.f : Mall;
+        float sc = 0.f;
+#pragma unroll
+        for (int o = 0; o < kMaxOwn; ++o) sc += hs[o] * exp_fast(hm[o] - Mref);   // (hm = -inf: nothing but a NaN sum counts)
 #pragma unroll
         for (int o = 16; o; o >>= 1) sc += __shfl_xor_sync(0xffffffffu, sc, o);
         lse = Mall + logf(sc);

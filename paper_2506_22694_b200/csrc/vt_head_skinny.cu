@@ -187,6 +187,7 @@ k_head_stream(const HeadArgs a, Ctrl* ctrl, float* __restrict__ recs, const Geo 
     __shared__ uint32_t s_tmem_base;
     __shared__ int s_last, s_abort, s_any_abort;
     __shared__ long long s_bound;                        // bound of a wait in SM cycles
+    __shared__ int s_rowok[kMergeB];                     // merge: the row's temperature is usable
     __shared__ float s_xch[kMergeB];                     // merge: a row's lse, from its statistics warp to its candidate warp
     constexpr int kWarps = EW + 2, kThreads = kWarps * 32;
     // An accumulator set holds kAccs accumulators of kNpad columns (hidden rows).  The kParts warps of a lane quadrant
@@ -391,7 +392,9 @@ k_head_stream(const HeadArgs a, Ctrl* ctrl, float* __restrict__ recs, const Geo 
         griddep_wait();                                             // temp, uniforms and the record scratch belong to earlier work until here
         for (int b = e; b < B; b += EW) {
             const float T = a.temp[b];
-            if (lane == 0) s_invT[b] = (T > 0.f) && (T < CUDART_INF_F) ? 1.f / T : CUDART_NAN_F;
+            const bool good = (T > 0.f) && (T < CUDART_INF_F);
+            if (lane == 0) s_invT[b] = good ? 1.f / T : CUDART_NAN_F;
+            if (RPW == 1 && lane == 0) s_rowok[b] = good ? 1 : 0;
         }
         __syncwarp();
         const int n_ph = (geo.n_kc + kPhase - 1) / kPhase;
@@ -514,7 +517,6 @@ k_head_stream(const HeadArgs a, Ctrl* ctrl, float* __restrict__ recs, const Geo 
                         }
                     }
                 }
-                *rs = st;
                 // top-k: the rows that beat the list's last entry join the list.  While the list is not full that is
                 // nearly every row of the tile; the topk-th largest of the lanes' best values is then a lower bound of
                 // the answer and leaves a few more than topk of them.
@@ -534,6 +536,7 @@ k_head_stream(const HeadArgs a, Ctrl* ctrl, float* __restrict__ recs, const Geo 
                         n_c += __popc(cm[i]);
                     }
                 }
+                int now = cnt;                                      // entries of the list from here on
                 if (n_c) {
                     for (int i = lane; i < cnt; i += 32) buf[i] = list[i];
                     int pos = cnt;
@@ -547,43 +550,42 @@ k_head_stream(const HeadArgs a, Ctrl* ctrl, float* __restrict__ recs, const Geo 
                     if (pos <= 32) rank_scatter<1>(list, buf, pos, topk);
                     else if (pos <= 64) rank_scatter<2>(list, buf, pos, topk);
                     else rank_scatter<(VT_MAX_TOPK + kBM) / 32>(list, buf, pos, topk);
-                    if (lane == 0) s_cnt[b] = min(topk, pos);
+                    now = min(topk, pos);
                     __syncwarp();
                 }
-            }
-            // ---- this CTA's record of its hidden rows: the lanes folded -- the maximum by one warp reduction, every
-            // lane's sum rescaled to it once, a butterfly of additions; the Gumbel candidate by two reductions over its
-            // 64-bit key.  (Made visible to the merging CTA by the ticket below: a barrier of this CTA, then one
-            // release at GPU scope.)
-            if (t == geo.n_tiles - 1) {
-#pragma unroll 1
-                for (int b = e; b < B; b += EW) {
-                    const RowState st = states[b * 32 + lane];
-                    unsigned long long* kp = rec_keys(recs, b, topk);
-                    float* fp = rec_f32(recs, b, topk);
-                    const int c = blockIdx.x;
-                    const int cnt = s_cnt[b];
-                    for (int k = lane; k < topk; k += 32) kp[(size_t)(1 + k) * kMaxGrid + c] = k < cnt ? lists[(size_t)b * topk + k] : 0ull;
-                    const float Mall = ord2f(__reduce_max_sync(0xffffffffu, f2ord(st.m)));
-                    float sc = (st.m != -CUDART_INF_F) ? st.s * exp_fast(st.m - Mall) : st.s;
+                if (t + 1 < geo.n_tiles) {
+                    *rs = st;
+                    if (lane == 0) s_cnt[b] = now;
+                    continue;
+                }
+                // ---- last tile: this CTA's record of the hidden row, the lanes folded -- the maximum by one warp reduction,
+                // every lane's sum rescaled to it once, a butterfly of additions; the Gumbel candidate by two reductions
+                // over its 64-bit key.  (Made visible to the merging CTA by the ticket below: a barrier of this CTA, then
+                // one release at GPU scope.)
+                unsigned long long* kp = rec_keys(recs, b, topk);
+                float* fp = rec_f32(recs, b, topk);
+                const int c = blockIdx.x;
+                for (int k = lane; k < topk; k += 32) kp[(size_t)(1 + k) * kMaxGrid + c] = k < now ? list[k] : 0ull;
+                const float Mall = ord2f(__reduce_max_sync(0xffffffffu, f2ord(st.m)));
+                float sc = (st.m != -CUDART_INF_F) ? st.s * exp_fast(st.m - Mall) : st.s;
 #pragma unroll
-                    for (int o = 16; o; o >>= 1) sc += __shfl_xor_sync(0xffffffffu, sc, o);
-                    if (lane == 0) {
-                        fp[c] = Mall;
-                        fp[kMaxGrid + c] = sc;
-                    }
-                    if (a.uniforms) {
-                        const unsigned long long gk = st.gj >= 0 ? key64(st.gs, st.gj) : 0ull;
-                        const unsigned ghi = (unsigned)(gk >> 32);
-                        const unsigned gmax = __reduce_max_sync(0xffffffffu, ghi);
-                        const unsigned glo = __reduce_max_sync(0xffffffffu, ghi == gmax ? (unsigned)gk : 0u);
-                        if (gk == (((unsigned long long)gmax << 32) | glo)) {     // (one lane, or all of them when no row has a candidate)
-                            fp[2 * kMaxGrid + c] = st.gz;
-                            kp[c] = gk;
-                        }
+                for (int o = 16; o; o >>= 1) sc += __shfl_xor_sync(0xffffffffu, sc, o);
+                if (lane == 0) {
+                    fp[c] = Mall;
+                    fp[kMaxGrid + c] = sc;
+                }
+                if (a.uniforms) {
+                    const unsigned long long gk = st.gj >= 0 ? key64(st.gs, st.gj) : 0ull;
+                    const unsigned ghi = (unsigned)(gk >> 32);
+                    const unsigned gmax = __reduce_max_sync(0xffffffffu, ghi);
+                    const unsigned glo = __reduce_max_sync(0xffffffffu, ghi == gmax ? (unsigned)gk : 0u);
+                    if (gk == (((unsigned long long)gmax << 32) | glo)) {     // (one lane, or all of them when no row has a candidate)
+                        fp[2 * kMaxGrid + c] = st.gz;
+                        kp[c] = gk;
                     }
                 }
-            } else {
+            }
+            if (t + 1 < geo.n_tiles) {
                 asm volatile("bar.sync 1, %0;" ::"n"(EW * 32) : "memory");           // the tile buffer is free
             }
         }
@@ -602,10 +604,6 @@ k_head_stream(const HeadArgs a, Ctrl* ctrl, float* __restrict__ recs, const Geo 
         if (threadIdx.x == 0 && s_abort) atomicOr(&ctrl->flags, (uint32_t)VT_FLAG_TIMEOUT);
         return;
     }
-    // as many rows as half the warps: two warps per hidden row (candidates / statistics) side by side; more: one warp each
-    const bool split = B <= kWarps / 2;
-    const int row = split ? (warp % (kWarps / 2)) : warp;
-    const bool row_ok = row < B && s_invT[row] == s_invT[row];      // (read now: the merge's staging may lie over it)
     if (threadIdx.x == 0) {
         VT_STAMP(6);
         const bool aborted = s_abort != 0;
@@ -632,11 +630,19 @@ k_head_stream(const HeadArgs a, Ctrl* ctrl, float* __restrict__ recs, const Geo 
         return;
     }
     {
+        // Who merges what: a row's candidates and its statistics side by side on two warps while the warps beyond the rows
+        // can take the statistics in at most two turns each (then they are done before the candidates are); else one
+        // warp each does both.
+        const int n_stat = kWarps - B;
+        const bool split = 2 * n_stat >= B;
+        const bool is_stat = split && warp >= B;
+        const int row = is_stat ? warp - B : warp;
         const MergeOut mo{a.map, a.out_ids, a.out_logprobs, a.dbg_lse, topk, a.uniforms != nullptr};
-        const int roles = split ? (warp < kWarps / 2 ? kRoleCand : kRoleStats) : (kRoleCand | kRoleStats);
-        if (row < B)
-            merge_records(mo, ctrl, recs, row, row_ok, (int)gridDim.x,
-                          reinterpret_cast<float*>(ring) + (size_t)row * kMergeStageWords, roles, &s_xch[row], 1 + row
+        const int roles = is_stat ? kRoleStats : split ? kRoleCand : (kRoleCand | kRoleStats);
+#pragma unroll 1
+        for (int r = row; r < B; r += is_stat ? n_stat : B)
+            merge_records(mo, ctrl, recs, r, s_rowok[r] != 0, (int)gridDim.x,
+                          reinterpret_cast<float*>(ring) + (size_t)r * kMergeStageWords, roles, &s_xch[r], 1 + r
 #ifdef VT_STAMPS
                           , stamps + (size_t)blockIdx.x * kStampSlots
 #endif

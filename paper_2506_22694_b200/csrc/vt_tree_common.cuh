@@ -17,15 +17,26 @@ __device__ __forceinline__ unsigned long long node_key(float s, int i) {
     return ((unsigned long long)score_ord(s) << 32) | (uint32_t)~(uint32_t)i;     // greater key = preferred
 }
 
-// rank of keys[i] among keys[0..n): number of strictly greater keys (keys are distinct)
+// rank among keys[0..n): number of strictly greater keys (keys are distinct).  All lanes read the same words, two keys
+// to a 128-bit broadcast and eight loads in flight: keys is 16-byte aligned and padded with zeros to a multiple of
+// kKeyGroup (a key of a node is never 0).
+constexpr int kKeyGroup = 16;
+__device__ __forceinline__ int padded_keys(int n) { return (n + kKeyGroup - 1) / kKeyGroup * kKeyGroup; }
 __device__ __forceinline__ int rank_of(const unsigned long long* keys, int n, unsigned long long mine) {
+    const ulonglong2* k2 = reinterpret_cast<const ulonglong2*>(keys);
     int r = 0;
-    for (int j = 0; j < n; ++j) r += keys[j] > mine;  // all lanes read the same word: a broadcast
+    for (int j = 0; j < n; j += kKeyGroup) {
+#pragma unroll
+        for (int q = 0; q < kKeyGroup / 2; ++q) {
+            const ulonglong2 k = k2[j / 2 + q];
+            r += (k.x > mine ? 1 : 0) + (k.y > mine ? 1 : 0);
+        }
+    }
     return r;
 }
 
 // One depth of the expansion by the `nthreads` threads `tid` of a CTA that all call it; s_key holds
-// B * topk keys.  Contains two CTA barriers.
+// B * topk keys, padded to a multiple of kKeyGroup.  Contains a CTA barrier.
 __device__ __forceinline__ void tree_expand_block(const TreeArgs& t, const int32_t* __restrict__ cand_ids,
                                                   const float* __restrict__ cand_lp, int32_t B, int32_t topk,
                                                   int32_t ld, int32_t col0, unsigned long long* s_key, int tid,
@@ -45,6 +56,7 @@ __device__ __forceinline__ void tree_expand_block(const TreeArgs& t, const int32
         t.pool_score[node] = s;
         s_key[i] = node_key(s, i);
     }
+    if (n_new + tid < padded_keys(n_new)) s_key[n_new + tid] = 0ull;
     __syncthreads();
     for (int i = tid; i < n_new; i += nthreads) {
         const int r = rank_of(s_key, n_new, s_key[i]);

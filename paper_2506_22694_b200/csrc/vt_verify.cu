@@ -16,6 +16,8 @@ k_verify_greedy(const int32_t* __restrict__ token, const int32_t* __restrict__ p
                 int32_t* __restrict__ path, int32_t* __restrict__ emitted, unsigned long long* tokens_total) {
     const int lane = threadIdx.x & 31;
     const int64_t s = (int64_t)blockIdx.x * kWarpsPerCta + (threadIdx.x >> 5);
+    griddep_launch_dependents();
+    griddep_wait();                                                // (the draft comes from the kernel before)
     if (s >= S) return;                                            // whole warps leave together
     const int32_t* tok = token + s * N;
     const int32_t* par = parent ? parent + s * N : nullptr;
@@ -61,10 +63,7 @@ cudaError_t launch_verify_greedy(const int32_t* token, const int32_t* parent, co
                                  unsigned long long* tokens_total, cudaStream_t st) {
     if (S == 0) return cudaSuccess;
     const unsigned grid = (unsigned)((S + kWarpsPerCta - 1) / kWarpsPerCta);
-    k_verify_greedy<<<grid, kWarpsPerCta * 32, 0, st>>>(token, parent, target, S, N, n_accept, path, emitted,
-                                                        tokens_total);
-    count_launch();
-    return cudaGetLastError();
+    return launch_dependent(k_verify_greedy, grid, kWarpsPerCta * 32, 0, st, token, parent, target, S, N, n_accept, path, emitted, tokens_total);
 }
 
 }  // namespace vt
