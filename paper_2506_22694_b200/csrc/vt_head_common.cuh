@@ -55,16 +55,19 @@ __device__ __forceinline__ int key_idx(unsigned long long k) { return (int)~(uns
 // exp and log of the epilogue: one multiplication and the hardware's base-2 function, results and arguments under
 // 2^-126 flushed to zero (the arguments of the logarithm are at least 2^-25; an exponential is added to a sum that
 // holds 1).
-__device__ __forceinline__ float exp_fast(float x) {
+constexpr float kLog2e = 1.4426950408889634f, kLn2 = 0.6931471805599453f;
+__device__ __forceinline__ float exp2_fast(float x) {
     float y;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x * 1.4426950408889634f));
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
 }
-__device__ __forceinline__ float log_fast(float x) {
+__device__ __forceinline__ float log2_fast(float x) {
     float y;
     asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y * 0.6931471805599453f;
+    return y;
 }
+__device__ __forceinline__ float exp_fast(float x) { return exp2_fast(x * kLog2e); }
+__device__ __forceinline__ float log_fast(float x) { return log2_fast(x) * kLn2; }
 
 // rk[i] += number of the N keys in shared memory that are greater than ek[i]; the buffer is 16-byte aligned and
 // zero-padded to a multiple of four.

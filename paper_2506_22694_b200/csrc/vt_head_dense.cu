@@ -433,51 +433,56 @@ k_head_dense(const HeadArgs a, Ctrl* ctrl, float* __restrict__ recs, const Dense
                 // Warp-uniform from here on (j0 and K are): rows that do not exist simply carry nv = 0,
                 // i.e. columns of -inf, so the warp votes below always see all 32 lanes.
                 if (j0 < K) {
-                    const int nv = row_live ? min(kCh, K - j0) : 0;
+                    // (a hidden row that does not exist has zeros for logits: its lane goes along and is never looked at)
+                    const int nv = min(kCh, K - j0);
                     float z[kCh];
-                    float cmax = -CUDART_INF_F;
+                    if (nv == kCh) {
 #pragma unroll
-                    for (int i = 0; i < kCh; ++i) {
-                        z[i] = (i < nv) ? __uint_as_float(r[i]) * invT : -CUDART_INF_F;
-                        cmax = fmaxf(cmax, z[i]);
+                        for (int i = 0; i < kCh; ++i) z[i] = __uint_as_float(r[i]) * invT;
+                    } else {
+#pragma unroll
+                        for (int i = 0; i < kCh; ++i) z[i] = (i < nv) ? __uint_as_float(r[i]) * invT : -CUDART_INF_F;
                     }
+                    float cmax = z[0];
+#pragma unroll
+                    for (int i = 1; i < kCh; ++i) cmax = fmaxf(cmax, z[i]);
                     if (a.dbg_logits && row_live) {
 #pragma unroll
                         for (int i = 0; i < kCh; ++i)
                             if (i < nv) a.dbg_logits[(size_t)b * K + j0 + i] = __uint_as_float(r[i]);
                     }
-                    // running max / sum-exp: one rescale per chunk, independent exponentials
+                    // running max / sum-exp: one rescale per chunk, independent exponentials, two sums
                     const float m_new = fmaxf(st.m, cmax);
                     const float m_ref = (m_new == -CUDART_INF_F) ? 0.f : m_new;
-                    float acc = 0.f;
+                    const float m2 = m_ref * -kLog2e;
+                    float acc0 = 0.f, acc1 = 0.f;
 #pragma unroll
-                    for (int i = 0; i < kCh; ++i) acc += __expf(z[i] - m_ref);
-                    st.s = st.s * __expf(st.m - m_ref) + acc;
+                    for (int i = 0; i < kCh; i += 2) {
+                        acc0 += exp2_fast(fmaf(z[i], kLog2e, m2));
+                        acc1 += exp2_fast(fmaf(z[i + 1], kLog2e, m2));
+                    }
+                    st.s = st.s * exp_fast(st.m - m_ref) + (acc0 + acc1);
                     st.m = m_new;
                     if (a.uniforms) {
 #pragma unroll
                         for (int i = 0; i < kCh; ++i) {
                             // g = -log(-log u): -log u from a short series in 1-u near 1 (where the fast
-                            // logarithm's absolute error would dominate), fast logarithms elsewhere
-                            const float uc = fminf(fmaxf(u[i], 0x1p-24f), 1.f - 0x1p-24f);
-                            const float t = 1.f - uc;
+                            // logarithm's absolute error would dominate), fast logarithms elsewhere; u is clamped to
+                            // [2^-24, 1 - 2^-24] where each of the two looks at it
+                            const float t = fmaxf(1.f - u[i], 0x1p-24f);
                             const float lp = t * (1.f + t * (0.5f + t * (0.33333334f + t * (0.25f + t * 0.2f))));
-                            const float L = uc > 0.95f ? lp : -__logf(uc);
-                            const float sc = z[i] - __logf(L);
-                            const bool win = sc > st.gb_s;            // invalid columns carry z = -inf
+                            const float L = u[i] > 0.95f ? lp : log2_fast(fmaxf(u[i], 0x1p-24f)) * -kLn2;
+                            const float sc = fmaf(log2_fast(L), -kLn2, z[i]);
+                            const bool win = sc > st.gb_s;            // columns that do not exist carry z = -inf
                             st.gb_s = win ? sc : st.gb_s;
                             st.gb_j = win ? j0 + i : st.gb_j;
                             st.gb_z = win ? z[i] : st.gb_z;
                         }
                     }
-                    // top-k: pull the chunk's maxima out in descending order while they beat the list's
-                    // last entry.  The loop is warp-uniform (it runs while any row of the warp still has
-                    // a candidate) and everything inside is select-based: one row's insertions never
-                    // make the other 31 rows branch.
-                    // a NaN logit poisons the row's lse (reported through VT_FLAG_NAN_ROW) but must not hide the
-                    // chunk's other candidates: it competes as -inf
-#pragma unroll
-                    for (int i = 0; i < kCh; ++i) z[i] = (z[i] == z[i]) ? z[i] : -CUDART_INF_F;
+                    // top-k: pull the chunk's candidates into the list while they beat its last entry.  The loop is
+                    // warp-uniform (it runs while any row of the warp still has a candidate) and everything inside is
+                    // select-based: one row's insertions never make the other 31 rows branch.  A NaN logit poisons the
+                    // row's lse (reported through VT_FLAG_NAN_ROW) and is no candidate (it beats nothing).
                     // candidates: the columns that beat the list's last entry as it stands; they go in by
                     // ascending column (equal values keep the lower column ahead), one per trip of a warp-
                     // uniform loop that runs while any row still has one.  A candidate that has fallen under
