@@ -1,8 +1,8 @@
 // Top-K vocabulary selection (Eq. 1, first line: V_trim = V[Top-K(c,k)]) in rank order, and the Method
 // section's two other rules (Top-P, minimum frequency) over the same ranking.
 //
-// V is about 1e5: the job is latency-bound, not bandwidth-bound.  It runs as ONE thread-block cluster of
-// 8 CTAs (one launch, no grid-wide spin) that talk through distributed shared memory between hardware
+// V is about 1e5: the job is latency-bound, not bandwidth-bound.  It runs as ONE thread-block cluster of 8 or 16
+// CTAs (one launch, no grid-wide spin) that talk through distributed shared memory between hardware
 // cluster barriers.  Two algorithms live here:
 //
 //  * the selection (k_select_sort, further down): one pass of bucket counts finds where the K-th key lies;
@@ -26,7 +26,7 @@ namespace vt {
 
 namespace {
 
-constexpr int kCluster = 8;
+constexpr int kWide = 16, kPortable = 8;         // CTAs per cluster: sixteen where the device can place such a cluster
 constexpr int kThreads = 1024;
 constexpr int kWarps = kThreads / 32;
 constexpr int kDigits = 256;
@@ -40,10 +40,30 @@ constexpr uint32_t kWorkCap = 6u << 10;          // key comparisons one CTA spen
 constexpr size_t kSelectSmem = sizeof(uint32_t) * 4 * kFine + sizeof(uint32_t) * 2 * kSortCap + sizeof(uint16_t) * (1024 / 32) * kExact;
 constexpr int kMassAt = 32 << 10;                // where in the key buffer the buckets' token mass lives while that buffer is idle
 static_assert(kMassAt + sizeof(unsigned long long) * kFine <= sizeof(uint32_t) * 2 * kSortCap, "the token mass fits the idle key buffer");
-static_assert(sizeof(uint32_t) * (kFine / 8) * (1 + 8) + sizeof(unsigned long long) * (kFine / 8) <= kMassAt, "... behind the exchange's sums");
+static_assert(sizeof(uint32_t) * (kFine / 8) * (1 + 8) + sizeof(unsigned long long) * (kFine / 8) <= kMassAt &&
+              sizeof(uint32_t) * (kFine / 16) * (1 + 16) + sizeof(unsigned long long) * (kFine / 16) <= kMassAt, "... behind the exchange's sums");
 constexpr int kDeals = 2;                        // ways of dealing the buckets to the CTAs that are tried
 constexpr uint32_t kKeyCost0 = 64, kKeyCost1 = 1024;   // comparisons a key is counted as, besides those with its bucket's keys, in each
 static_assert(sizeof(uint32_t) * 4 * kFine >= sizeof(uint32_t) * kWarps * kDigits, "the full ranking reuses the bucket arrays");
+
+// Sum of the warp totals in front of this warp, and of all: every warp for itself, one read per lane and one or two warp
+// reductions (a loop over the totals is a chain of up to 32 shared-memory reads: 1000 cycles for the last warp).
+__device__ __forceinline__ uint32_t warps_before(const uint32_t* totals, int warp, uint32_t* all = nullptr) {
+    const uint32_t t = totals[threadIdx.x & 31];
+    if (all) *all = __reduce_add_sync(0xffffffffu, t);
+    return __reduce_add_sync(0xffffffffu, (int)(threadIdx.x & 31) < warp ? t : 0u);
+}
+__device__ __forceinline__ unsigned long long warps_before(const unsigned long long* totals, int warp, unsigned long long* all) {
+    const unsigned long long t = totals[threadIdx.x & 31];
+    unsigned long long b = (int)(threadIdx.x & 31) < warp ? t : 0ull, a = t;
+#pragma unroll
+    for (int o = 16; o; o >>= 1) {
+        a += __shfl_xor_sync(0xffffffffu, a, o);
+        b += __shfl_xor_sync(0xffffffffu, b, o);
+    }
+    *all = a;
+    return b;
+}
 
 // What the full ranking needs to find K itself (Top-P / minimum frequency): the cut bucket's ranks
 // [first, end) from the bucket pass and what lies before them.
@@ -60,6 +80,7 @@ struct CutSpec {
 // ---- full ranking: least-significant-digit radix sort over the whole cluster -------------------------
 // s_wcnt: [kWarps][kDigits] words of shared memory.  With `spec`, K is read off the sorted counts before the
 // ranking is emitted (every CTA works it out for itself: the same reads, the same answer).
+template <int kCluster>
 __device__ void lsd_rank_all(cg::cluster_group& cluster, const uint32_t* counts, int32_t V, int32_t K, int32_t* map,
                              int32_t* inv_map, uint32_t* keyA, uint32_t* valA, uint32_t* keyB, uint32_t* valB,
                              uint32_t (*s_wcnt)[kDigits], const CutSpec* spec = nullptr) {
@@ -317,7 +338,7 @@ __device__ __forceinline__ uint32_t fine_bucket(uint32_t c) {
 // emitted.  map[0, K) and inv_map are written; k_out receives K.  When the run does not fit (see above) or
 // the histogram is degenerate (no tokens, nothing down to the cut), the full ranking takes over here too and
 // reads K off the sorted counts of the cut bucket's ranks.
-template <int MODE>
+template <int MODE, int kCluster>
 __global__ void __cluster_dims__(kCluster, 1, 1) __launch_bounds__(kThreads, 1)
 k_select_sort(const uint32_t* counts, int32_t V, int32_t K, int32_t* map, int32_t* inv_map, uint32_t* keyA, uint32_t* valA, uint32_t* keyB,
               uint32_t* valB, double pfrac, uint32_t min_count, int32_t* k_out) {
@@ -340,10 +361,10 @@ k_select_sort(const uint32_t* counts, int32_t V, int32_t K, int32_t* map, int32_
     __shared__ unsigned long long s_wmass[kWarps + 1];
     __shared__ unsigned long long s_mass_before;    // token mass of the buckets above the cut
     __shared__ int s_cut_owner[kDeals], s_K, s_first;
-    __shared__ uint32_t s_load[kDeals][kCluster];  // keys each CTA would have to rank, per way of dealing the buckets
+    __shared__ uint32_t s_run0[kDeals][kCluster];  // first rank of the keys each CTA would have to rank, per way of dealing the buckets
     __shared__ uint32_t s_work[kDeals][kCluster];  // key comparisons that would take: sum of squared bucket sizes, in units of 1024
     __shared__ uint32_t s_T;
-    __shared__ int s_cut, s_lo[kDeals], s_hi[kDeals], s_big;
+    __shared__ int s_cut, s_big;
 
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     // ids of this CTA: a contiguous slice; every warp walks a contiguous piece of it in id order (128 bytes per
@@ -362,8 +383,8 @@ k_select_sort(const uint32_t* counts, int32_t V, int32_t K, int32_t* map, int32_
         if (MODE == 1) s_mass[i] = 0ull;
     }
     for (int i = threadIdx.x; i < kWarps * kExact / 8; i += kThreads) reinterpret_cast<uint4*>(s_ws2)[i] = make_uint4(0, 0, 0, 0);
-    if (threadIdx.x < kDeals * kCluster) { (&s_load[0][0])[threadIdx.x] = 0; (&s_work[0][0])[threadIdx.x] = 0u; }
-    if (threadIdx.x < kDeals) { s_lo[threadIdx.x] = 0x7fffffff; s_hi[threadIdx.x] = 0; s_cut_owner[threadIdx.x] = -1; }
+    if (threadIdx.x < kDeals * kCluster) { (&s_run0[0][0])[threadIdx.x] = 0xffffffffu; (&s_work[0][0])[threadIdx.x] = 0u; }
+    if (threadIdx.x < kDeals) s_cut_owner[threadIdx.x] = -1;
     if (threadIdx.x == 0) { s_cut = -1; s_big = 0; s_K = 0; s_first = 0; s_T = 0; s_mass_before = 0; }
     griddep_launch_dependents();
     griddep_wait();                                     // (the counts come from the kernel before)
@@ -409,8 +430,8 @@ k_select_sort(const uint32_t* counts, int32_t V, int32_t K, int32_t* map, int32_
     // buckets), the bucket of the K-th key, who ranks what
     constexpr int BPT = kFine / kThreads;
     static_assert(BPT == 4, "one 128-bit load per peer and thread");
-    // The eight CTAs' counts meet in two steps, so that 48 KB instead of 128 KB cross between the SMs per CTA: CTA r
-    // adds up the buckets [r * kSlice, (r + 1) * kSlice) of all eight (and, per peer, what the peers before it hold),
+    // The CTAs' counts meet in two steps, so that (with eight of them) 48 KB instead of 128 KB cross between the SMs per CTA: CTA r
+    // adds up the buckets [r * kSlice, (r + 1) * kSlice) of all (and, per peer, what the peers before it hold),
     // leaves the sums in its own shared memory (the key buffer is idle until the ranking), and after one more cluster
     // barrier every CTA reads the totals and its own row of the prefix table from the bucket's summing CTA.
     constexpr int kSlice = kFine / kCluster;                         // buckets summed by one CTA
@@ -419,15 +440,18 @@ k_select_sort(const uint32_t* counts, int32_t V, int32_t K, int32_t* map, int32_
     unsigned long long* s_mtot = reinterpret_cast<unsigned long long*>(s_pre + kCluster * kSlice);   // [kSlice] token mass (MODE 1)
     if (threadIdx.x < kSlice / BPT) {
         const int i4 = (int)rank * (kSlice / BPT) + (int)threadIdx.x;   // which 128-bit group of the bucket arrays
-        uint4 pv[kCluster];
-#pragma unroll
-        for (unsigned c = 0; c < kCluster; ++c)                     // all eight remote loads in flight
-            pv[c] = reinterpret_cast<const uint4*>(cluster.map_shared_rank(s_hist, c))[i4];
         uint4 run = make_uint4(0, 0, 0, 0);
 #pragma unroll
-        for (unsigned c = 0; c < kCluster; ++c) {
-            reinterpret_cast<uint4*>(s_pre + c * kSlice)[threadIdx.x] = run;
-            run.x += pv[c].x; run.y += pv[c].y; run.z += pv[c].z; run.w += pv[c].w;
+        for (unsigned c0 = 0; c0 < kCluster; c0 += 8) {
+            uint4 pv[8];
+#pragma unroll
+            for (unsigned c = 0; c < 8; ++c)                        // eight remote loads in flight
+                pv[c] = reinterpret_cast<const uint4*>(cluster.map_shared_rank(s_hist, c0 + c))[i4];
+#pragma unroll
+            for (unsigned c = 0; c < 8; ++c) {
+                reinterpret_cast<uint4*>(s_pre + (c0 + c) * kSlice)[threadIdx.x] = run;
+                run.x += pv[c].x; run.y += pv[c].y; run.z += pv[c].z; run.w += pv[c].w;
+            }
         }
         reinterpret_cast<uint4*>(s_tot)[threadIdx.x] = run;
         if (MODE == 1) {
@@ -490,8 +514,7 @@ k_select_sort(const uint32_t* counts, int32_t V, int32_t K, int32_t* map, int32_
     }
     if (lane == 31) s_warp[warp] = incl;
     __syncthreads();
-    uint32_t start = incl - sum;
-    for (int w = 0; w < warp; ++w) start += s_warp[w];
+    uint32_t start = incl - sum + warps_before(s_warp, warp);
     unsigned long long mstart = mincl - msum, mtotal = 0;
     // Top-P: target = ceil(p * total) is the one fp64 product; what is compared with it are integers, and while the
     // total is under 2^53 (every prefix then converts exactly) they are compared as integers -- fp64 conversions of
@@ -500,8 +523,7 @@ k_select_sort(const uint32_t* counts, int32_t V, int32_t K, int32_t* map, int32_
     unsigned long long itarget = 0;
     bool as_int = true;
     if (MODE == 1) {
-        for (int w = 0; w < warp; ++w) mstart += s_wmass[w];
-        for (int w = 0; w < kWarps; ++w) mtotal += s_wmass[w];
+        mstart += warps_before(s_wmass, warp, &mtotal);
         if (lane == 0) target = ceil(pfrac * (double)mtotal);
         target = __shfl_sync(0xffffffffu, target, 0);
         as_int = mtotal < (1ull << 53);
@@ -540,7 +562,7 @@ k_select_sort(const uint32_t* counts, int32_t V, int32_t K, int32_t* map, int32_
     CutSpec spec{MODE, cut >= 0 && T > 0, (uint32_t)s_first, T, s_mass_before, target, min_count, k_out};
     if (MODE != 0 && !spec.valid) {                     // no tokens at all / nothing as frequent as asked: K = 1 of the full ranking
         cluster.sync();                                 // peers are done reading this CTA's counts
-        lsd_rank_all(cluster, counts, V, V, map, inv_map, keyA, valA, keyB, valB,
+        lsd_rank_all<kCluster>(cluster, counts, V, V, map, inv_map, keyA, valA, keyB, valB,
                      reinterpret_cast<uint32_t (*)[kDigits]>(s_dyn), &spec);
         return;
     }
@@ -551,7 +573,7 @@ k_select_sort(const uint32_t* counts, int32_t V, int32_t K, int32_t* map, int32_
     // Two deals are tried and the first that fits is taken: the second, with a higher key cost and so closer to
     // equal key counts, is for rankings of 50 K keys and more, where the first one's leading CTA would get more
     // tiny buckets than its shared memory holds.
-    int deal = -1;
+    int deal = -1, r0 = 0, n = 0;                       // this CTA's run: first rank, keys
     for (int d = 0; d < kDeals && deal < 0; ++d) {      // (the same trips in every thread of every CTA: same inputs)
         const uint32_t kc = d == 0 ? kKeyCost0 : kKeyCost1;
         uint32_t cost[BPT], csum = 0;
@@ -569,43 +591,58 @@ k_select_sort(const uint32_t* counts, int32_t V, int32_t K, int32_t* map, int32_
         }
         if (lane == 31) s_warp[warp] = cincl;            // (a barrier lies between this and the last reads of the array)
         __syncthreads();
-        uint32_t cstart = cincl - csum, ctotal = 0;
-        for (int w = 0; w < kWarps; ++w) {
-            if (w < warp) cstart += s_warp[w];
-            ctotal += s_warp[w];
-        }
+        uint32_t ctotal;
+        uint32_t cstart = cincl - csum + warps_before(s_warp, warp, &ctotal);
+        // owner of a bucket = floor(cost before it * CTAs / total cost), by comparisons (a 64-bit division per bucket and
+        // atomics from every bucket into a few words were 3 us here).  Ranks grow with the buckets, so all that is
+        // needed of a CTA's run is its first rank: it ends where the next one begins.
+        uint32_t st = s_gstart[threadIdx.x * BPT];
 #pragma unroll
         for (int q = 0; q < BPT; ++q) {
             const int b = threadIdx.x * BPT + q;
-            if (b <= cut && b < first_exact && tot[q] > 0) {
-                const uint32_t st = s_gstart[b];
+            const bool on = cost[q] > 0;                              // (down to the cut, inexact, not empty)
+            const unsigned act = __ballot_sync(0xffffffffu, on);
+            if (on) {
                 const int lb = low_bits_of_bucket(kFine - 1 - b);
                 if (tot[q] > (uint32_t)kCountCap || (lb + id_bits(V) > 32 && tot[q] > kWideCap)) s_big = 1;
-                const unsigned owner = min((unsigned)kCluster - 1u, (unsigned)(((unsigned long long)cstart * kCluster) / max(ctotal, 1u)));
-                atomicAdd(&s_load[d][owner], tot[q]);
-                if (tot[q] <= (uint32_t)kCountCap) atomicAdd(&s_work[d][owner], (tot[q] * tot[q] + 1023u) >> 10);
-                if (owner == rank) {
-                    atomicMin(&s_lo[d], (int)st);
-                    atomicMax(&s_hi[d], (int)(st + tot[q]));
+                const unsigned long long c8 = (unsigned long long)cstart * kCluster;
+                unsigned owner = 0;
+#pragma unroll
+                for (int k = 1; k < kCluster; ++k) owner += c8 >= (unsigned long long)ctotal * (unsigned)k ? 1u : 0u;
+                const unsigned peers = __match_any_sync(act, owner);
+                const uint32_t w = __reduce_add_sync(peers, tot[q] <= (uint32_t)kCountCap ? (tot[q] * tot[q] + 1023u) >> 10 : 0u);
+                if (lane == __ffs(peers) - 1) {                       // (the lowest lane has the lowest rank)
+                    atomicMin(&s_run0[d][owner], st);
+                    if (w) atomicAdd(&s_work[d][owner], w);
                 }
                 if (b == cut) s_cut_owner[d] = (int)owner;
             }
+            __syncwarp();
             cstart += cost[q];
+            st += tot[q];
         }
         __syncthreads();
         bool ok = s_big == 0;
-        for (int c = 0; c < kCluster; ++c) ok = ok && s_load[d][c] <= (uint32_t)kSortCap && s_work[d][c] <= kWorkCap;
+        uint32_t end = cut >= first_exact ? s_gstart[first_exact] : T;          // (exact buckets come after all others)
+#pragma unroll
+        for (int c = kCluster - 1; c >= 0; --c) {
+            const uint32_t first = s_run0[d][c];
+            const uint32_t load = first == 0xffffffffu ? 0u : end - first;
+            ok = ok && load <= (uint32_t)kSortCap && s_work[d][c] <= kWorkCap;
+            if (c == (int)rank) { r0 = load ? (int)first : 0; n = (int)load; }
+            if (load) end = first;
+        }
         if (ok) deal = d;
     }
     const bool fits = deal >= 0;
     if (!fits) {                                        // the same decision in every CTA (same inputs)
         cluster.sync();                                 // peers are done reading this CTA's counts
         if (MODE != 0) {
-            lsd_rank_all(cluster, counts, V, V, map, inv_map, keyA, valA, keyB, valB,
+            lsd_rank_all<kCluster>(cluster, counts, V, V, map, inv_map, keyA, valA, keyB, valB,
                          reinterpret_cast<uint32_t (*)[kDigits]>(s_dyn), &spec);
             return;
         }
-        lsd_rank_all(cluster, counts, V, K, map, inv_map, keyA, valA, keyB, valB,
+        lsd_rank_all<kCluster>(cluster, counts, V, K, map, inv_map, keyA, valA, keyB, valB,
                      reinterpret_cast<uint32_t (*)[kDigits]>(s_dyn));
         return;
     }
@@ -651,7 +688,6 @@ k_select_sort(const uint32_t* counts, int32_t V, int32_t K, int32_t* map, int32_
     // counts differ in their low bits only, so what is compared is a 32-bit word (those low bits, then ~id) held in
     // shared memory for the CTA's whole run of buckets, four to a load (neighbouring lanes mostly share a bucket:
     // the reads are broadcasts).  The 64-bit keys stay where phase 3 put them and are read from there.
-    const int r0 = s_lo[deal], n = s_hi[deal] > s_lo[deal] ? s_hi[deal] - s_lo[deal] : 0;
     const unsigned long long* run = pairs + r0;
     uint32_t* s_c = reinterpret_cast<uint32_t*>(s_run);                 // [kSortCap]
     uint32_t* s_place = s_c + kSortCap;                                 // [kSortCap] MODE 1 / 2: the keys' ranks
@@ -715,34 +751,76 @@ k_select_sort(const uint32_t* counts, int32_t V, int32_t K, int32_t* map, int32_
 
 }  // namespace
 
-static cudaError_t select_smem_attr() {
-    static int attr_done[64] = {0};
+// Attributes of one instance on the current device, and whether it can run there at all.
+template <int MODE, int CL>
+static cudaError_t select_prepare(bool* fits) {
+    cudaError_t e = cudaFuncSetAttribute(k_select_sort<MODE, CL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSelectSmem);
+    if (e == cudaSuccess && CL > kPortable) e = cudaFuncSetAttribute(k_select_sort<MODE, CL>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e != cudaSuccess || !fits) return e;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(CL);
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = kSelectSmem;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = CL;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, k_select_sort<MODE, CL>, &cfg) != cudaSuccess) { cudaGetLastError(); n = 0; }
+    *fits = n > 0;
+    return cudaSuccess;
+}
+
+// CTAs per cluster on the current device (found out once per device): sixteen need a GPC with as many SMs to itself,
+// which a device that lends out part of its SMs may not have.
+static cudaError_t select_width(int* width) {
+    static int known[64] = {0};
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
-    if (dev >= 0 && dev < 64 && attr_done[dev]) return cudaSuccess;
-    e = cudaFuncSetAttribute(k_select_sort<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSelectSmem);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_select_sort<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSelectSmem);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_select_sort<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSelectSmem);
-    if (e == cudaSuccess && dev >= 0 && dev < 64) attr_done[dev] = 1;
-    return e;
+    if (dev >= 0 && dev < 64 && known[dev]) { *width = known[dev]; return cudaSuccess; }
+    bool wide = false;
+    e = select_prepare<0, kWide>(&wide);
+    if (e == cudaSuccess) e = select_prepare<1, kWide>(nullptr);
+    if (e == cudaSuccess) e = select_prepare<2, kWide>(nullptr);
+    if (e == cudaSuccess) e = select_prepare<0, kPortable>(nullptr);
+    if (e == cudaSuccess) e = select_prepare<1, kPortable>(nullptr);
+    if (e == cudaSuccess) e = select_prepare<2, kPortable>(nullptr);
+    if (e != cudaSuccess) return e;
+    *width = wide ? kWide : kPortable;
+    if (dev >= 0 && dev < 64) known[dev] = *width;
+    return cudaSuccess;
 }
 
-// Top-P (mode 0) / minimum frequency (mode 1): the selection kernel in the mode that finds K on its way.
-cudaError_t launch_select_cut(const uint32_t* counts, int32_t V, int mode, double pfrac, uint32_t min_count,
-                              int32_t* map, int32_t* inv_map, int32_t* k_out, uint8_t* scratch, cudaStream_t s) {
+// Sixteen CTAs halve what is done per id and cost every cluster barrier and exchange a little more (us, eight / sixteen,
+// counts of 3e6 tokens: V = 4096 12.5 / 14.8, 24000 15.2 / 15.8, 48000 16.6 / 17.2, 80000 18.9 / 18.3, 128256 23.0 /
+// 20.2, 256000 34.4 / 24.9; Top-P 0.9 crosses at the same place).
+constexpr int32_t kNarrowIds = 65536;
+
+template <int MODE>
+static cudaError_t launch_select(const uint32_t* counts, int32_t V, int32_t K, int32_t* map, int32_t* inv_map, uint8_t* scratch, double pfrac,
+                                 uint32_t min_count, int32_t* k_out, cudaStream_t s) {
     const size_t seg = align_up((size_t)V * 4, 256);
     uint32_t* keyA = reinterpret_cast<uint32_t*>(scratch);
     uint32_t* valA = reinterpret_cast<uint32_t*>(scratch + seg);
     uint32_t* keyB = reinterpret_cast<uint32_t*>(scratch + 2 * seg);
     uint32_t* valB = reinterpret_cast<uint32_t*>(scratch + 3 * seg);
-    cudaError_t e = select_smem_attr();
+    int width = 0;
+    const cudaError_t e = select_width(&width);
     if (e != cudaSuccess) return e;
-    if (mode == 0)
-        return launch_dependent(k_select_sort<1>, kCluster, kThreads, kSelectSmem, s, counts, V, 0, map, inv_map, keyA, valA, keyB, valB,
-                                pfrac, 0u, k_out);
-    return launch_dependent(k_select_sort<2>, kCluster, kThreads, kSelectSmem, s, counts, V, 0, map, inv_map, keyA, valA, keyB, valB, 1.0,
-                            min_count, k_out);
+    return width == kWide && V > kNarrowIds ? launch_dependent(k_select_sort<MODE, kWide>, kWide, kThreads, kSelectSmem, s, counts, V, K, map, inv_map, keyA, valA,
+                                             keyB, valB, pfrac, min_count, k_out)
+                          : launch_dependent(k_select_sort<MODE, kPortable>, kPortable, kThreads, kSelectSmem, s, counts, V, K, map, inv_map, keyA,
+                                             valA, keyB, valB, pfrac, min_count, k_out);
+}
+
+// Top-P (mode 0) / minimum frequency (mode 1): the selection kernel in the mode that finds K on its way.
+cudaError_t launch_select_cut(const uint32_t* counts, int32_t V, int mode, double pfrac, uint32_t min_count,
+                              int32_t* map, int32_t* inv_map, int32_t* k_out, uint8_t* scratch, cudaStream_t s) {
+    return mode == 0 ? launch_select<1>(counts, V, 0, map, inv_map, scratch, pfrac, 0u, k_out, s)
+                     : launch_select<2>(counts, V, 0, map, inv_map, scratch, 1.0, min_count, k_out, s);
 }
 
 size_t select_scratch_bytes(int32_t V) { return 4 * align_up((size_t)V * 4, 256); }
@@ -750,17 +828,9 @@ size_t select_cut_scratch_bytes(int32_t V) { return select_scratch_bytes(V); }
 
 cudaError_t launch_select_topk(const uint32_t* counts, int32_t V, int32_t K, int32_t* map,
                                int32_t* inv_map, uint8_t* scratch, cudaStream_t s) {
-    const size_t seg = align_up((size_t)V * 4, 256);
-    uint32_t* keyA = reinterpret_cast<uint32_t*>(scratch);
-    uint32_t* valA = reinterpret_cast<uint32_t*>(scratch + seg);
-    uint32_t* keyB = reinterpret_cast<uint32_t*>(scratch + 2 * seg);
-    uint32_t* valB = reinterpret_cast<uint32_t*>(scratch + 3 * seg);
-    cudaError_t e = select_smem_attr();
-    if (e != cudaSuccess) return e;
     // (whatever K: even K = V is the selection's work when most ids were seen fewer than 1024 times -- 31 against
     // 56 us on the counts of 3 M tokens -- and costs it one bucket pass, 13 us, before the full ranking when not)
-    return launch_dependent(k_select_sort<0>, kCluster, kThreads, kSelectSmem, s, counts, V, K, map, inv_map, keyA, valA, keyB, valB, 1.0, 0u,
-                            (int32_t*)nullptr);
+    return launch_select<0>(counts, V, K, map, inv_map, scratch, 1.0, 0u, nullptr, s);
 }
 
 }  // namespace vt
