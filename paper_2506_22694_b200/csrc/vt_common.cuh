@@ -12,10 +12,11 @@ namespace vt {
 // leaves `ticket` words at zero when it finishes.
 struct Ctrl {
     uint32_t flags;               // sticky VT_FLAG_* bits
-    uint32_t head_ticket;         // "last CTA merges" ticket of the head kernels (wraps to 0)
+    uint32_t head_ticket;         // "last block" ticket of the head's merge kernel (wraps to 0)
     unsigned long long n_bad;     // ids skipped by the histogram
     unsigned long long wait_ns;   // bound of a device-side wait in nanoseconds (0 = the built-in default)
-    uint32_t pad[58];
+    uint32_t head_aborted;        // a CTA of the head kernel gave up on a wait: its call's merge reports and clears it
+    uint32_t pad[57];
 };
 static_assert(sizeof(Ctrl) == VT_CTRL_BYTES, "control block size");
 

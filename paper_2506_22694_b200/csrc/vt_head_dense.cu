@@ -29,6 +29,7 @@
 #include "vt_common.cuh"
 #include "vt_head_common.cuh"
 #include "vt_tc.cuh"
+#include "vt_tree_common.cuh"
 
 namespace vt {
 
@@ -581,17 +582,27 @@ k_head_dense(const HeadArgs a, Ctrl* ctrl, float* __restrict__ recs, const Dense
         if (PAIR) asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"((uint32_t)kTmemCols) : "memory");
         else asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"((uint32_t)kTmemCols) : "memory");
     }
-    if (threadIdx.x == 0 && s_abort) atomicOr(&ctrl->flags, (uint32_t)VT_FLAG_TIMEOUT);
+    if (threadIdx.x == 0 && s_abort) {
+        atomicOr(&ctrl->flags, (uint32_t)VT_FLAG_TIMEOUT);
+        atomicOr(&ctrl->head_aborted, 1u);                        // the merge reports every row as missing
+    }
 #ifdef VT_STAMPS
     if (threadIdx.x == 0) VT_DSTAMP(11);
 #endif
 }
 
-// Two warps per hidden row (candidates / statistics): merge the CTA records, remap, write the outputs.
+// Two warps per hidden row (candidates / statistics): merge the CTA records, remap, write the outputs.  After a
+// wait that expired somewhere the records are incomplete: every row is reported as missing.  FUSE: tree drafting --
+// the block that finishes last turns the merged candidates into pool nodes and chooses the next frontier, so that
+// a tree depth needs no launch for it.  (Dynamic shared memory, sized by the need: the block has to fit beside the
+// head kernel's CTA to take its seat early.)
+constexpr size_t kFuseBytes = 128u << 20;                          // heads up to this size (see launch_head_merge)
+constexpr int kFuseNodes = 512;                                   // new nodes the 64 threads of a block rank (else a kernel of 1024 threads)
 __global__ void __launch_bounds__(64)
-k_head_merge(const HeadArgs a, Ctrl* ctrl, float* __restrict__ recs, int G) {
-    __shared__ __align__(16) float s_stage[kMergeStageWords];
+k_head_merge(const HeadArgs a, Ctrl* ctrl, float* __restrict__ recs, int G, int fuse) {
+    extern __shared__ __align__(16) float s_stage[];              // [kMergeStageWords], and over it the keys of the expansion
     __shared__ float s_xch;
+    __shared__ int s_last;
     const int b = blockIdx.x;
     griddep_launch_dependents();                                  // the next step may start fetching its weights
     griddep_wait();                                               // the records are complete
@@ -600,13 +611,36 @@ k_head_merge(const HeadArgs a, Ctrl* ctrl, float* __restrict__ recs, int G) {
         reinterpret_cast<uint8_t*>(recs) + align_up_dev((size_t)kMaxGrid * a.B * rec_fields(a.topk) * 4, 256));
     if (b == 0 && threadIdx.x == 0) stamps[12] = global_ns();
 #endif
-    const float T = a.temp[b];
-    const bool row_ok = (T > 0.f) && (T < CUDART_INF_F);
-    const MergeOut mo{a.map, a.out_ids, a.out_logprobs, a.dbg_lse, a.topk, a.uniforms != nullptr};
-    merge_records(mo, ctrl, recs, b, row_ok, G, s_stage, threadIdx.x < 32 ? kRoleCand : kRoleStats, &s_xch, 1);
+    const bool aborted = *reinterpret_cast<volatile uint32_t*>(&ctrl->head_aborted) != 0u;
+    if (aborted) {
+        for (int i = threadIdx.x; i < 1 + a.topk; i += 64) {
+            a.out_ids[(size_t)b * (1 + a.topk) + i] = -1;
+            a.out_logprobs[(size_t)b * (1 + a.topk) + i] = CUDART_NAN_F;
+        }
+    } else {
+        const float T = a.temp[b];
+        const bool row_ok = (T > 0.f) && (T < CUDART_INF_F);
+        const MergeOut mo{a.map, a.out_ids, a.out_logprobs, a.dbg_lse, a.topk, a.uniforms != nullptr};
+        merge_records(mo, ctrl, recs, b, row_ok, G, s_stage, threadIdx.x < 32 ? kRoleCand : kRoleStats, &s_xch, 1);
+    }
 #ifdef VT_STAMPS
     if (b == 0 && threadIdx.x == 0) stamps[13] = global_ns();
 #endif
+    if (!fuse && !aborted) return;
+    __syncthreads();                                              // the row's outputs are written
+    if (threadIdx.x == 0) {
+        unsigned old;
+        asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], %2;" : "=r"(old) : "l"(&ctrl->head_ticket), "r"(1u) : "memory");
+        s_last = old == gridDim.x - 1;
+        if (s_last) {                                             // every block has looked: ready for the next launch
+            ctrl->head_ticket = 0;
+            ctrl->head_aborted = 0;
+        }
+    }
+    __syncthreads();
+    if (!s_last || !fuse) return;
+    tree_expand_block(a.tree, a.out_ids, a.out_logprobs, a.B, a.topk, 1 + a.topk, 1, reinterpret_cast<unsigned long long*>(s_stage),
+                      (int)threadIdx.x, 64);
 }
 
 // ---- host side ----------------------------------------------------------------------------------------
@@ -705,18 +739,15 @@ cudaError_t launch_head_dense(const HeadArgs& a, Ctrl* ctrl, uint8_t* scratch, c
 // The records of G CTAs (pairs) -> outputs; with a tree, its expansion as one more launch (it needs every row's merge).
 cudaError_t launch_head_merge(const HeadArgs& a, Ctrl* ctrl, float* recs, int G, cudaStream_t s) {
     // the merge always follows its own producer closely: it takes its seats early and waits on the device
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3((unsigned)a.B);
-    cfg.blockDim = dim3(64);
-    cfg.stream = s;
-    cudaLaunchAttribute at{};
-    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at.val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = &at;
-    cfg.numAttrs = 1;
-    count_launch();
-    const cudaError_t e = cudaLaunchKernelEx(&cfg, k_head_merge, a, ctrl, recs, G);
-    if (e != cudaSuccess || !a.tree.pool_token) return e;
+    const int n_new = a.B * a.topk;
+    // The expansion inside the merge saves a launch, as a kernel of its own (sixteen times the threads, launched ahead as a
+    // dependent) it is 1-2 us shorter: a depth over a small head is bound by its launches (depth-3 tree over 61 MB: 77
+    // with the kernel, 70 fused), over a large one by the device (six depths over 268 MB: 306 / 317).
+    const bool fuse = a.tree.pool_token && n_new <= kFuseNodes && (size_t)a.K * a.d * 2 <= kFuseBytes;
+    size_t smem = (size_t)kMergeStageWords * 4;
+    if (fuse && (size_t)padded_keys(n_new) * 8 > smem) smem = (size_t)padded_keys(n_new) * 8;
+    const cudaError_t e = launch_dependent(k_head_merge, (unsigned)a.B, 64, smem, s, a, ctrl, recs, G, fuse ? 1 : 0);
+    if (e != cudaSuccess || !a.tree.pool_token || fuse) return e;
     return launch_tree_expand(a.out_ids, a.out_logprobs, a.B, a.topk, 1 + a.topk, 1, a.tree, s);
 }
 

@@ -18,9 +18,16 @@
 // Epilogue warps read their TMEM lanes (lane = vocabulary row) and turn the finished tile around in shared
 // memory; then warp w owns hidden rows w, w + EW, ...: its lanes walk the tile's rows, updating running
 // max / sum-exp of z = logit / T, the Gumbel-max candidate from the caller's uniforms and the row's sorted
-// top-k list.  Logits never go to HBM.  Each CTA leaves one small record per hidden row; up to 16 rows, the
-// last CTA to finish (atomic ticket, no spinning) merges the records in CTA order, remaps trimmed indices
-// through `map` and writes the outputs; beyond that a second kernel does, one pair of warps per row.
+// top-k list.  Logits never go to HBM.  Each CTA leaves one small record per hidden row; a second kernel, one
+// pair of warps per row, merges them in CTA order, remaps trimmed indices through `map` and writes the outputs
+// (vt_head_dense.cu).  It takes its seats while this one runs, and a CTA here is gone as soon as its record is
+// written, which lets the next step's weights in; the merge by the last CTA to finish (atomic ticket) kept them
+// out for its 4-6 us (us per chained step, one CTA / second kernel: 1 row of 5000 x 2048 14.8 / 11.7, 10 rows of
+// 32768 x 4096 46.1 / 43.5; one launch more on the host).
+//
+// What bounds it: the HBM read of W_trim (201 MB, cold: 35.7 us per chained step = 0.86 of the measured copy rate;
+// the warp-level MMA kernel before it 38.8) and, for small heads, a fixed chain of about 9 us: h by TMA 0.5, MMAs
+// 25-45 cycles each, epilogue 2, merge and two launch dependencies 5.
 //
 // Every wait is bounded: on expiry the CTA raises VT_FLAG_TIMEOUT, lets its own copies and MMAs finish and leaves.
 #include <math_constants.h>
@@ -28,7 +35,6 @@
 #include "vt_common.cuh"
 #include "vt_head_common.cuh"
 #include "vt_tc.cuh"
-#include "vt_tree_common.cuh"
 
 namespace vt {
 
@@ -41,14 +47,14 @@ constexpr int kPhase = 8;                        // 64-column steps of d accumul
 constexpr int kSetCols = 128;                    // TMEM columns of an accumulator set (two sets)
 constexpr uint32_t kTmemCols = 2 * kSetCols;     // (half of the SM's: two CTAs of consecutive launches may be resident together)
 constexpr int kMaxB = 64;
-constexpr int kMergeB = 16;                      // hidden rows the last CTA merges by itself
 constexpr size_t kSmemLimit = 227 * 1024 - 2048; // opt-in limit minus static shared memory
 constexpr unsigned long long kWaitLimitNs = 2000000000ull;   // default bound of a device-side wait (Ctrl::wait_ns overrides)
 
 // Phase stamps (-DVT_STAMPS builds only): one thread per role writes %globaltimer at fixed points into
 // a region behind the records; bench.py --case stamps reads them back.  Slots: 0 entry, 1 ring fill
 // requested, 2 released by the launch dependency, 3 first stage landed, 4 last accumulators complete,
-// 5 record written, 6 all warps done, 7 after the ticket, 8-10 merge (loads, selection, outputs), 11 SM id.
+// 5 record written, 6 all warps done, 11 SM id; CTA 0 also carries the merge
+// kernel's 12 start and 13 end for hidden row 0.
 #ifdef VT_STAMPS
 #define VT_STAMP(slot) do { stamps[(size_t)blockIdx.x * kStampSlots + (slot)] = global_ns(); } while (0)
 #else
@@ -59,6 +65,7 @@ struct Geo {
     int grid;          // CTAs
     int n_tiles;       // tiles per CTA
     int rows;          // vocabulary rows of a tile (rows of one W copy)
+    int mma_rows;      // M of the MMA: 64 where a tile has no more rows, else 128
     int n_kc;          // 64-column steps of d
     int sub;           // steps per ring stage
     int n_stages;      // ring depth
@@ -185,11 +192,8 @@ k_head_stream(const HeadArgs a, Ctrl* ctrl, float* __restrict__ recs, const Geo 
     extern __shared__ uint8_t s_dyn[];
     __shared__ uint64_t s_full[kMaxStages], s_empty[kMaxStages], s_acc_full[2], s_acc_empty[2], s_drain;
     __shared__ uint32_t s_tmem_base;
-    __shared__ int s_last, s_abort, s_any_abort;
+    __shared__ int s_abort;
     __shared__ long long s_bound;                        // bound of a wait in SM cycles
-    __shared__ int s_rowok[kMergeB];                     // merge: the row's temperature is usable
-    __shared__ float s_xch[kMergeB];                     // merge: a row's lse, from its statistics warp to its candidate warp
-    constexpr int kWarps = EW + 2, kThreads = kWarps * 32;
     // An accumulator set holds kAccs accumulators of kNpad columns (hidden rows).  The kParts warps of a lane quadrant
     // take kUnits groups of four columns each: always eight loads per warp and phase.
     constexpr int kParts = EW / 4, kUnits = RPW, kAccs = 8 / kUnits, kNpad = 16 * kUnits;
@@ -320,7 +324,7 @@ k_head_stream(const HeadArgs a, Ctrl* ctrl, float* __restrict__ recs, const Geo 
     } else if (warp == 1) {
         // ================= MMA issuer ==================================================================
         if (elect_one()) {
-            constexpr uint32_t idesc = make_idesc(kBM, kNpad);
+            const uint32_t idesc = make_idesc(geo.mma_rows, kNpad);
             // (the ring is 1024-byte aligned and under 256 KB: adding byte offsets >> 4 stays inside the address field;
             // rows of an operand beyond the tile's / beyond B are whatever lies behind it: their TMEM lanes and columns
             // are not looked at)
@@ -383,6 +387,7 @@ k_head_stream(const HeadArgs a, Ctrl* ctrl, float* __restrict__ recs, const Geo 
         // ================= epilogue warps ==============================================================
         const int e = warp - 2;
         const int quad = warp & 3;                                  // TMEM lanes this warp may read
+        const int qrows = geo.mma_rows / 4;                         // vocabulary rows in them (M = 64 fills the first 16 of 32)
         const int part = e >> 2;                                    // which accumulator columns of the quadrant
         unsigned long long* buf = bufs + (size_t)(e < B ? e : 0) * kBufKeys;     // (used only by warps that own a row: e < B)
         for (int b = e; b < B; b += EW) {
@@ -392,9 +397,7 @@ k_head_stream(const HeadArgs a, Ctrl* ctrl, float* __restrict__ recs, const Geo 
         griddep_wait();                                             // temp, uniforms and the record scratch belong to earlier work until here
         for (int b = e; b < B; b += EW) {
             const float T = a.temp[b];
-            const bool good = (T > 0.f) && (T < CUDART_INF_F);
-            if (lane == 0) s_invT[b] = good ? 1.f / T : CUDART_NAN_F;
-            if (RPW == 1 && lane == 0) s_rowok[b] = good ? 1 : 0;
+            if (lane == 0) s_invT[b] = (T > 0.f) && (T < CUDART_INF_F) ? 1.f / T : CUDART_NAN_F;
         }
         __syncwarp();
         const int n_ph = (geo.n_kc + kPhase - 1) / kPhase;
@@ -421,7 +424,7 @@ k_head_stream(const HeadArgs a, Ctrl* ctrl, float* __restrict__ recs, const Geo 
                 ok = mbar_wait_warp(&s_acc_full[set], (uint32_t)((set_no >> 1) & 1), abort_flag, bound);
                 if (!ok) break;
                 tc_fence_after();
-                if (quad * 32 < nrow && part * 4 < B) {
+                if (quad * qrows < nrow && part * 4 < B) {
                     const uint32_t base = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(set * kSetCols + part * 4);
                     uint32_t ad[8];
                     float v[8][4];
@@ -453,13 +456,13 @@ k_head_stream(const HeadArgs a, Ctrl* ctrl, float* __restrict__ recs, const Geo 
 #ifdef VT_STAMPS
                 if (e == 0 && lane == 0) VT_STAMP(4);
 #endif
-                if (quad * 32 < nrow) {
+                if (quad * qrows < nrow && lane < qrows) {
 #pragma unroll
                     for (int i = 0; i < kUnits; ++i)
 #pragma unroll
                         for (int q = 0; q < 4; ++q) {
                             const int b = (part + i * kParts) * 4 + q;
-                            if (b < B) zt[(size_t)b * kBM + quad * 32 + lane] = x[i][q];
+                            if (b < B) zt[(size_t)b * kBM + quad * qrows + lane] = x[i][q];
                         }
                 }
             }
@@ -560,8 +563,7 @@ k_head_stream(const HeadArgs a, Ctrl* ctrl, float* __restrict__ recs, const Geo 
                 }
                 // ---- last tile: this CTA's record of the hidden row, the lanes folded -- the maximum by one warp reduction,
                 // every lane's sum rescaled to it once, a butterfly of additions; the Gumbel candidate by two reductions
-                // over its 64-bit key.  (Made visible to the merging CTA by the ticket below: a barrier of this CTA, then
-                // one release at GPU scope.)
+                // over its 64-bit key.  (The merge kernel starts when this grid has ended.)
                 unsigned long long* kp = rec_keys(recs, b, topk);
                 float* fp = rec_f32(recs, b, topk);
                 const int c = blockIdx.x;
@@ -600,67 +602,19 @@ k_head_stream(const HeadArgs a, Ctrl* ctrl, float* __restrict__ recs, const Geo 
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(kTmemCols) : "memory");
     }
-    if (RPW > 1) {                                                  // a kernel of its own merges the records
-        if (threadIdx.x == 0 && s_abort) atomicOr(&ctrl->flags, (uint32_t)VT_FLAG_TIMEOUT);
-        return;
-    }
     if (threadIdx.x == 0) {
-        VT_STAMP(6);
-        const bool aborted = s_abort != 0;
-        if (aborted) atomicOr(&ctrl->flags, (uint32_t)VT_FLAG_TIMEOUT);
-        // Ticket: arrivals in the low half, aborted CTAs in the high half.  Acquire + release in one, so
-        // that the last CTA's loads below see every other CTA's record.
-        unsigned old;
-        asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], %2;"
-                     : "=r"(old) : "l"(&ctrl->head_ticket), "r"(aborted ? 0x10001u : 1u) : "memory");
-        s_last = ((old & 0xffffu) == gridDim.x - 1);
-        s_any_abort = aborted || (old >> 16) != 0;
-        if (s_last) ctrl->head_ticket = 0;                          // ready for the next launch
-        VT_STAMP(7);
-    }
-    __syncthreads();
-    if (!s_last) return;
-
-    if (s_any_abort) {
-        // a bounded wait expired somewhere: the records are incomplete; report every row as missing
-        for (int i = threadIdx.x; i < B * (1 + topk); i += kThreads) {
-            a.out_ids[i] = -1;
-            a.out_logprobs[i] = CUDART_NAN_F;
+        if (s_abort) {
+            atomicOr(&ctrl->flags, (uint32_t)VT_FLAG_TIMEOUT);
+            atomicOr(&ctrl->head_aborted, 1u);                      // the merge reports every row as missing
         }
-        return;
-    }
-    {
-        // Who merges what: a row's candidates and its statistics side by side on two warps while the warps beyond the rows
-        // can take the statistics in at most two turns each (then they are done before the candidates are); else one
-        // warp each does both.
-        const int n_stat = kWarps - B;
-        const bool split = 2 * n_stat >= B;
-        const bool is_stat = split && warp >= B;
-        const int row = is_stat ? warp - B : warp;
-        const MergeOut mo{a.map, a.out_ids, a.out_logprobs, a.dbg_lse, topk, a.uniforms != nullptr};
-        const int roles = is_stat ? kRoleStats : split ? kRoleCand : (kRoleCand | kRoleStats);
-#pragma unroll 1
-        for (int r = row; r < B; r += is_stat ? n_stat : B)
-            merge_records(mo, ctrl, recs, r, s_rowok[r] != 0, (int)gridDim.x,
-                          reinterpret_cast<float*>(ring) + (size_t)r * kMergeStageWords, roles, &s_xch[r], 1 + r
-#ifdef VT_STAMPS
-                          , stamps + (size_t)blockIdx.x * kStampSlots
-#endif
-                          );
-    }
-    if (a.tree.pool_token) {
-        // tree drafting: the merged candidates of all rows become pool nodes and the next frontier is
-        // chosen here, by the CTA that merged them, instead of in a launch of its own
-        __syncthreads();                                            // the rows' outputs are written; the staging area is free
-        tree_expand_block(a.tree, a.out_ids, a.out_logprobs, B, topk, 1 + topk, 1,
-                          reinterpret_cast<unsigned long long*>(ring), (int)threadIdx.x, kThreads);
+        VT_STAMP(6);
     }
 }
 
 // ---- host side ---------------------------------------------------------------------------------------
 // Shapes of the few-row contract: what vt_workspace_bytes and the entry points take with topk up to VT_MAX_TOPK.
 bool shape_ok(int B, int d) {
-    if (B < 1 || B > kMergeB || d < 8 || (d & 7)) return false;
+    if (B < 1 || B > 16 || d < 8 || (d & 7)) return false;
     return d <= (B <= 8 ? 8192 : 4096);
 }
 
@@ -671,6 +625,8 @@ Geo make_geo(int B, int K, int d, int topk, int sms, size_t* smem_bytes) {
     const int slab = (K + g.grid - 1) / g.grid;
     g.n_tiles = (slab + kBM - 1) / kBM;
     g.rows = (slab + g.n_tiles - 1) / g.n_tiles;
+    // (M = 64 and N = 16: 25 cycles per MMA instead of 40 -- a part of what a step of a small head waits for)
+    g.mma_rows = g.rows <= 64 ? 64 : kBM;
     g.n_kc = (d + kBK - 1) / kBK;
     g.h_bytes = (int)align_up((size_t)B * kBK * 2, 1024);
     const int w_bytes = (int)align_up((size_t)g.rows * kBK * 2, 1024);
@@ -678,7 +634,7 @@ Geo make_geo(int B, int K, int d, int topk, int sms, size_t* smem_bytes) {
     const int ew = B <= 8 ? 8 : 16;
     g.buf_bytes = (B < ew ? B : ew) * kBufKeys * 8;
     const size_t fixed = (size_t)B * kBM * 4 + align_up((size_t)B * topk * 8, 16) + (size_t)g.buf_bytes + (size_t)B * (32 * sizeof(RowState) + 8);
-    const size_t over = (size_t)kBM * kBK * 2 - (size_t)w_bytes;   // the MMA reads 128 rows from the start of a W part
+    const size_t over = (size_t)g.mma_rows * kBK * 2 - (size_t)w_bytes;   // the MMA reads that many rows from the start of a W part
     const size_t tail = fixed > over ? fixed : over;
     const size_t room = kSmemLimit - 1024 - tail;
     // Four steps to a stage where three such stages fit: the two threads that drive the ring wait and release once
@@ -701,10 +657,7 @@ Geo make_geo(int B, int K, int d, int topk, int sms, size_t* smem_bytes) {
     const int share = mb > 96.0 ? (int)(56.0 / mb * 32.0) : 0;
     for (int i = 0; i < 32; ++i)
         if ((i + 1) * share / 32 != i * share / 32) g.keep |= 1u << i;
-    size_t need = (size_t)g.ring_bytes + tail;
-    const size_t merge_bytes = B <= kMergeB ? (size_t)B * kMergeStageWords * 4 : 0;               // staging area of the merge
-    if (need < merge_bytes) need = merge_bytes;
-    *smem_bytes = need + 1024;                                     // + slack to align the ring to 1024 bytes
+    *smem_bytes = (size_t)g.ring_bytes + tail + 1024;              // + slack to align the ring to 1024 bytes
     return g;
 }
 
@@ -760,9 +713,9 @@ cudaError_t launch_head_skinny(const HeadArgs& a, Ctrl* ctrl, uint8_t* scratch, 
     CUtensorMap tm_h, tm_w;
     if (!encode_map(&tm_h, a.h, a.B, a.d, a.B) || !encode_map(&tm_w, a.W, a.K, a.d, geo.rows)) return cudaErrorInvalidValue;
     float* recs = reinterpret_cast<float*>(scratch);
-    if (a.B <= 8) return launch_variant<8, 1>(a, ctrl, recs, geo, tm_h, tm_w, smem, s);
-    if (a.B <= 16) return launch_variant<16, 1>(a, ctrl, recs, geo, tm_h, tm_w, smem, s);
-    const cudaError_t e = a.B <= 32 ? launch_variant<16, 2>(a, ctrl, recs, geo, tm_h, tm_w, smem, s)
+    const cudaError_t e = a.B <= 8 ? launch_variant<8, 1>(a, ctrl, recs, geo, tm_h, tm_w, smem, s)
+                        : a.B <= 16 ? launch_variant<16, 1>(a, ctrl, recs, geo, tm_h, tm_w, smem, s)
+                        : a.B <= 32 ? launch_variant<16, 2>(a, ctrl, recs, geo, tm_h, tm_w, smem, s)
                                     : launch_variant<16, 4>(a, ctrl, recs, geo, tm_h, tm_w, smem, s);
     if (e != cudaSuccess) return e;
     return launch_head_merge(a, ctrl, recs, geo.grid, s);

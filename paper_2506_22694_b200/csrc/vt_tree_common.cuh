@@ -21,7 +21,7 @@ __device__ __forceinline__ unsigned long long node_key(float s, int i) {
 // to a 128-bit broadcast and eight loads in flight: keys is 16-byte aligned and padded with zeros to a multiple of
 // kKeyGroup (a key of a node is never 0).
 constexpr int kKeyGroup = 16;
-__device__ __forceinline__ int padded_keys(int n) { return (n + kKeyGroup - 1) / kKeyGroup * kKeyGroup; }
+__host__ __device__ inline int padded_keys(int n) { return (n + kKeyGroup - 1) / kKeyGroup * kKeyGroup; }
 __device__ __forceinline__ int rank_of(const unsigned long long* keys, int n, unsigned long long mine) {
     const ulonglong2* k2 = reinterpret_cast<const ulonglong2*>(keys);
     int r = 0;
@@ -37,8 +37,8 @@ __device__ __forceinline__ int rank_of(const unsigned long long* keys, int n, un
 
 // One depth of the expansion by the `nthreads` threads `tid` of a CTA that all call it; s_key holds
 // B * topk keys, padded to a multiple of kKeyGroup.  Contains a CTA barrier.
-__device__ __forceinline__ void tree_expand_block(const TreeArgs& t, const int32_t* __restrict__ cand_ids,
-                                                  const float* __restrict__ cand_lp, int32_t B, int32_t topk,
+__device__ __forceinline__ void tree_expand_block(const TreeArgs& t, const int32_t* cand_ids,
+                                                  const float* cand_lp, int32_t B, int32_t topk,
                                                   int32_t ld, int32_t col0, unsigned long long* s_key, int tid,
                                                   int nthreads) {
     const int n_new = B * topk;
@@ -47,11 +47,11 @@ __device__ __forceinline__ void tree_expand_block(const TreeArgs& t, const int32
         int32_t par = t.frontier ? t.frontier[b] : -1;
         if (par < -1 || par >= t.pool_base) par = -1;                   // memory safety; callers pass earlier nodes
         const float base = par < 0 ? 0.0f : t.pool_score[par];         // earlier depth: not written by this launch
-        const float lp = cand_lp[(int64_t)b * ld + col0 + j];
+        const float lp = ld_cg_f32(cand_lp + (int64_t)b * ld + col0 + j);    // (written by other blocks of this launch)
         const float step = (lp != lp) ? lp : fminf(lp, 0.0f);          // a log-probability is never positive
         const float s = base + step;
         const int node = t.pool_base + i;
-        t.pool_token[node] = cand_ids[(int64_t)b * ld + col0 + j];
+        t.pool_token[node] = ld_cg_s32(cand_ids + (int64_t)b * ld + col0 + j);
         t.pool_parent[node] = par;
         t.pool_score[node] = s;
         s_key[i] = node_key(s, i);
