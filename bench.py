@@ -44,8 +44,8 @@ L2_BYTES = 126 * 1024 * 1024
 FALLBACK_HBM_GBS = 6650.0
 
 PROFILE_KERNEL_SOURCES = {           # kernel -> the sources whose change invalidates its captured counters
-    "k_head_stream": ("vt_head_skinny.cu", "vt_head_common.cuh"),
-    "k_head_dense": ("vt_head_dense.cu", "vt_head_common.cuh"),
+    "k_head_stream": ("vt_head_skinny.cu", "vt_head_common.cuh", "vt_tc.cuh"),
+    "k_head_dense": ("vt_head_dense.cu", "vt_head_common.cuh", "vt_tc.cuh"),
     "k_hist_packed": ("vt_hist.cu",),
 }
 
@@ -611,14 +611,12 @@ def stamps_case(vt, vt_build, dev, args):
                 x = view.cpu().numpy().reshape(ctas.value, slots.value)
                 x = x[x[:, 0] > 0]
                 t_rel = x[:, 2].min()
-                last = int(np.argmax(x[:, 8]))
                 row = {"ctas": int(x.shape[0]), "entry_first": (x[:, 0].min() - t_rel) / 1e3}
-                for k in range(2, 8):
+                for k in range(2, 7):
                     row[STAMP_NAMES[k] + "_last"] = (x[:, k].max() - t_rel) / 1e3
                 row["last_stage_consumed_median"] = float(np.median(x[:, 4] - t_rel)) / 1e3
                 row["last_stage_consumed_first"] = (x[:, 4].min() - t_rel) / 1e3
-                for k in range(8, 11):
-                    row[STAMP_NAMES[k]] = (x[last, k] - t_rel) / 1e3
+                row["merge_started"], row["merge_row0_written"] = (x[0, 12] - t_rel) / 1e3, (x[0, 13] - t_rel) / 1e3
                 rows.append(row)
             rec[mode] = {k: round(float(np.median([r[k] for r in rows])), 2) for k in rows[0]}
             e0, e1 = _events()

@@ -266,9 +266,9 @@ vt_status vt_trim_head(const uint16_t *W_full, const int32_t *map, uint16_t *W_t
  *                                   columns 1.. = candidates in descending z, ties to lower index
  *   out_logprobs [B, 1+topk] fp32 : log softmax(logits/T_b) of the id in the same column
  * Uniforms are clamped to [2^-24, 1-2^-24].  Limits: d % 8 == 0, 1 <= topk <= min(K, 64),
- * 1 <= B <= 256.  B <= 16 with d <= 8192 (B <= 8) or d <= 4096 runs the streaming kernel; every
- * other shape runs the dense tensor-core kernel, which keeps its top-k lists in registers and
- * takes topk <= 16 (VT_ERR_UNSUPPORTED beyond).
+ * 1 <= B <= 256.  B <= 16 with d <= 8192 (B <= 8) or d <= 4096 takes topk up to VT_MAX_TOPK, every
+ * other shape topk <= 16 (VT_ERR_UNSUPPORTED beyond).  Up to 32 rows (64 over a large head) run the
+ * streaming kernel, more rows the batched one.
  */
 vt_status vt_draft_head(const uint16_t *h, const uint16_t *W_trim, const int32_t *map, int32_t B,
                         int32_t K, int32_t d, const float *temp, int32_t topk,
@@ -293,9 +293,9 @@ vt_status vt_draft_head_overlapped(const uint16_t *h, const uint16_t *W_trim, co
 /*
  * One tree depth in one call: vt_draft_head_overlapped followed by vt_tree_expand on its candidates
  * (out_ids / out_logprobs columns 1..topk), with the same arguments, results and limits as those two
- * (Algorithm 2, the drafter-forward and index-mapping steps with the draft tree of Section 4.1).  For the streaming kernel's shapes
- * (B <= 16) the expansion runs inside the head kernel, in the CTA that merges the rows, so a tree
- * depth costs one launch; other shapes chain the expansion kernel behind the merge.  The caller's
+ * (Algorithm 2, the drafter-forward and index-mapping steps with the draft tree of Section 4.1).  Over a
+ * head of up to 128 MB the expansion runs inside the merge kernel, in the block that finishes last;
+ * otherwise it is a kernel behind the merge.  The caller's
  * promise about W_trim is that of vt_draft_head_overlapped.
  */
 vt_status vt_draft_head_expand(const uint16_t *h, const uint16_t *W_trim, const int32_t *map, int32_t B,

@@ -170,8 +170,7 @@ const char* vt_status_str(vt_status s) {
 #ifdef VT_STAMPS
 int32_t vt_stamps_region(int32_t B, int32_t d, int32_t topk, size_t* offset, int32_t* slots, int32_t* max_ctas) {
     if (!offset || !slots || !max_ctas) return 0;
-    if (head_stream_takes(B)) *offset = VT_CTRL_BYTES + head_skinny_stamps_offset(B, topk);
-    else if (head_dense_supported(B, 1, d)) *offset = VT_CTRL_BYTES + head_dense_stamps_offset(B, topk);
+    if (head_dense_supported(B, 1, d)) *offset = VT_CTRL_BYTES + head_dense_stamps_offset(B, topk);
     else return 0;
     *slots = 16;
     *max_ctas = 160;
@@ -381,7 +380,7 @@ static vt_status draft_head_impl(const uint16_t* h, const uint16_t* W_trim, cons
     if (st != VT_OK) return st;
     uint8_t* base = static_cast<uint8_t*>(ws);
     HeadArgs a{h, W_trim, map, B, K, d, temp, topk, uniforms, out_ids, out_logprobs, out_logits, out_lse, overlap, tree};
-    if (head_stream_takes(B))
+    if (head_stream_takes(B, K, d))
         return from_cuda(launch_head_skinny(a, reinterpret_cast<Ctrl*>(base), base + VT_CTRL_BYTES,
                                             as_stream(stream)));
     return from_cuda(launch_head_dense(a, reinterpret_cast<Ctrl*>(base), base + VT_CTRL_BYTES,

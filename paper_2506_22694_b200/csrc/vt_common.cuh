@@ -117,7 +117,7 @@ struct HeadArgs {
     TreeArgs tree;         // expansion to run on the merged top-k (pool_token == nullptr: none)
 };
 bool head_skinny_supported(int32_t B, int32_t d);   // shapes whose candidate lists may be VT_MAX_TOPK long
-bool head_stream_takes(int32_t B);                  // hidden rows the streaming kernel is launched for
+bool head_stream_takes(int32_t B, int32_t K, int32_t d);      // calls the streaming kernel is launched for
 size_t head_skinny_scratch_bytes(int32_t B, int32_t K, int32_t topk);
 cudaError_t launch_head_skinny(const HeadArgs& a, Ctrl* ctrl, uint8_t* scratch, cudaStream_t s);
 #ifdef VT_STAMPS

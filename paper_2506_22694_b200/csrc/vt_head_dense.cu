@@ -1,4 +1,4 @@
-// Batched-serving head (17 <= B <= 256 hidden rows): the projection is a real dense contraction
+// Batched-serving head (33 to 256 hidden rows; which of 33 to 64 see head_stream_takes): the projection is a real dense contraction
 // and runs on the 5th-generation tensor cores (Algorithm 2, the drafter-forward and index-mapping steps, with many sequences and
 // tree nodes drafted at once).
 //
@@ -151,6 +151,7 @@ struct DenseGeo {
     int n_stages;     // ring depth
     int stage_bytes;  // bytes one CTA stages per step: hidden rows + its share of the vocabulary rows
     int n_groups;     // CTAs (or CTA pairs) walking the tiles round-robin
+    int h_rows;       // hidden rows a copy brings (the rest of the MMA's 128 is whatever lies there: lanes nobody looks at)
     int sub;          // d-steps per ring stage (1 or 2): one wait and one release per stage, so two steps per stage halve
                       // what the two single threads that drive the ring spend per MMA; taken when three such stages fit
 };
@@ -266,7 +267,9 @@ k_head_dense(const HeadArgs a, Ctrl* ctrl, float* __restrict__ recs, const Dense
                     else tma_load_2d(dst, &tm_h, kc * kBK, 0, &s_full[s]);
                 }
             };
-            auto bytes_of = [&](int g) { return (uint32_t)(PAIR ? 2 : 1) * sub_bytes * (uint32_t)subs_of(g); };
+            // what lands per step: the hidden rows of the copy and this CTA's share of the vocabulary rows
+            const uint32_t step_tx = (uint32_t)(geo.h_rows + w_rows) * (kBK * 2);
+            auto bytes_of = [&](int g) { return (uint32_t)(PAIR ? 2 : 1) * step_tx * (uint32_t)subs_of(g); };
             // The weights are static: the first ring of them is requested before the work this launch
             // depends on has finished; everything that work may have produced is touched after the wait.
             const int pre = min(n_stages, total);
@@ -287,7 +290,7 @@ k_head_dense(const HeadArgs a, Ctrl* ctrl, float* __restrict__ recs, const Dense
                 for (int g = pre; g < total; ++g, ++done) {
                     if (!mbar_wait(&s_empty[sc], par, abort_flag)) break;
                     const int subs = min(sub, geo.n_kc - ks * sub);
-                    if (rank == 0) mbar_expect_tx(&s_full[sc], pair_mul * sub_bytes * (uint32_t)subs);
+                    if (rank == 0) mbar_expect_tx(&s_full[sc], pair_mul * step_tx * (uint32_t)subs);
                     const uint32_t dst0 = ring_u32 + (uint32_t)sc * (uint32_t)geo.stage_bytes;
                     const uint32_t bar = full0 + (uint32_t)(sc * sizeof(uint64_t));
                     const int row_w = (group + tl * geo.n_groups) * bn + (PAIR ? (int)rank * w_rows : 0);
@@ -434,7 +437,7 @@ k_head_dense(const HeadArgs a, Ctrl* ctrl, float* __restrict__ recs, const Dense
                 // Warp-uniform from here on (j0 and K are): rows that do not exist simply carry nv = 0,
                 // i.e. columns of -inf, so the warp votes below always see all 32 lanes.
                 if (j0 < K) {
-                    // (a hidden row that does not exist has zeros for logits: its lane goes along and is never looked at)
+                    // (the lane of a hidden row that does not exist goes along with whatever it has and is never looked at)
                     const int nv = min(kCh, K - j0);
                     float z[kCh];
                     if (nv == kCh) {
@@ -721,9 +724,10 @@ cudaError_t launch_head_dense(const HeadArgs& a, Ctrl* ctrl, uint8_t* scratch, c
     int max_groups = pair ? num_sms() / 2 : num_sms();
     if (max_groups > kMaxGrid) max_groups = kMaxGrid;
     if (max_groups < 1) return cudaErrorInvalidValue;
-    const DenseGeo geo = make_geo(a.K, a.d, pair, max_groups);
+    DenseGeo geo = make_geo(a.K, a.d, pair, max_groups);
+    geo.h_rows = pair ? kBM : a.B;
     CUtensorMap tm_h, tm_w;
-    if (!encode_map(&tm_h, a.h, a.B, a.d, kBM) || !encode_map(&tm_w, a.W, a.K, a.d, pair ? geo.bn / 2 : geo.bn))
+    if (!encode_map(&tm_h, a.h, a.B, a.d, geo.h_rows) || !encode_map(&tm_w, a.W, a.K, a.d, pair ? geo.bn / 2 : geo.bn))
         return cudaErrorInvalidValue;
     float* recs = reinterpret_cast<float*>(scratch);
     cudaError_t e;

@@ -690,7 +690,13 @@ cudaError_t launch_variant(const HeadArgs& a, Ctrl* ctrl, float* recs, const Geo
 
 bool head_skinny_supported(int32_t B, int32_t d) { return shape_ok(B, d); }
 
-bool head_stream_takes(int32_t B) { return B >= 1 && B <= kMaxB; }
+// Up to 32 rows this kernel is the faster one at every size (us per call, this / batched kernel: 24 rows of 5000 x 2048
+// 15.8 / 18.5, of 20001 x 3072 30.7 / 39.2, of 80000 x 3072 83 / 146).  From 33 to 64 its second pass over h for slabs of
+// more than 128 rows and four hidden rows per epilogue warp cost as much as the batched kernel's idle lanes: 40 rows of
+// 123 MB 40.4 / 39.6, of 268 MB 58.5 / 64.0, of 491 MB 99.5 / 146.5; the line is drawn between the first two.
+bool head_stream_takes(int32_t B, int32_t K, int32_t d) {
+    return B >= 1 && (B <= 32 || (B <= kMaxB && (size_t)K * d * 2 >= ((size_t)192 << 20)));
+}
 
 size_t head_skinny_scratch_bytes(int32_t B, int32_t K, int32_t topk) {
     (void)K;
@@ -704,7 +710,7 @@ size_t head_skinny_stamps_offset(int32_t B, int32_t topk) {
 #endif
 
 cudaError_t launch_head_skinny(const HeadArgs& a, Ctrl* ctrl, uint8_t* scratch, cudaStream_t s) {
-    if (!head_stream_takes(a.B) || a.d < 8 || (a.d & 7)) return cudaErrorInvalidValue;
+    if (!head_stream_takes(a.B, a.K, a.d) || a.d < 8 || (a.d & 7)) return cudaErrorInvalidValue;
     int sms = num_sms();
     if (sms > kMaxGrid) sms = kMaxGrid;
     size_t smem = 0;
