@@ -317,9 +317,10 @@ k_head_stream(const HeadArgs a, Ctrl* ctrl, float* __restrict__ recs, const Geo 
                     if (++ks == n_ks) { ks = 0; y += geo.rows; }
                 }
             }
-            // aborting: every copy asked for has landed before the CTA may leave (else the MMAs have read them all)
-            if (*abort_flag)
-                for (int g = max(0, done - S); g < done; ++g) drain_wait(&s_full[g % S], (uint32_t)((g / S) & 1));
+            // Every copy asked for has landed before the CTA may leave, whatever the other roles do from here on: a wait of
+            // theirs may expire after this thread's last request, and then nobody else looks at these stages again.  (The last
+            // fill of a stage is its barrier's last phase; in an undisturbed run the MMAs finish later than this.)
+            for (int g = max(0, done - S); g < done; ++g) drain_wait(&s_full[g % S], (uint32_t)((g / S) & 1));
         }
     } else if (warp == 1) {
         // ================= MMA issuer ==================================================================

@@ -40,3 +40,28 @@ def test_streaming_head_at_tile_phase_and_variant_edges(B, K, d, topk, sample):
     for o in (a, b):                                     # without the logits dump, plain and chained: the same bits
         assert torch.equal(o[0], gi) and torch.equal(o[1], gl)
     assert ws.read_status() == (0, 0, 0)
+
+
+@pytest.mark.parametrize("B,K,d,topk", [(1, 5000, 2048, 8), (8, 3000, 512, 10), (20, 4000, 1024, 8)])
+def test_an_expired_wait_with_every_copy_already_asked_for(B, K, d, topk):
+    """A CTA's whole share fits its ring: the producer has made its last request by the time a wait of another role expires
+    (bound of 1 ns, set by the host), and still nothing may be in flight when the CTA leaves.  The calls right behind it
+    use the same shared memory and must return what an undisturbed call does."""
+    W = vt_inputs.gaussian_bf16((K, d), 0.02, seed=31, device=DEV)
+    h = vt_inputs.gaussian_bf16((B, d), 1.0, seed=32, device=DEV)
+    T = vt_inputs.temperatures(B, 1.0, 1.0, 0, device=DEV)
+    ws = vt.Workspace(vt.workspace_bytes(vt.VT_OP_DRAFT_HEAD, 0, 0, K, d, B, topk))
+    good = tuple(t.clone() for t in vt.vt_draft_head(h, W, None, T, topk, ws=ws))
+    for overlapped in (False, True):
+        ws.set_wait_limit(1)
+        gi, gl = vt.vt_draft_head(h, W, None, T, topk, ws=ws, overlapped=overlapped)
+        ws.set_wait_limit(0)
+        after = [vt.vt_draft_head(h, W, None, T, topk, ws=ws, overlapped=overlapped) for _ in range(3)]
+        st, flags, _ = ws.read_status()
+        if st == 5:
+            assert flags & vt.VT_FLAG_TIMEOUT and bool((gi == -1).all()) and bool(torch.isnan(gl).all())
+        else:                                            # no wait had to spin after the bound was read
+            assert st == 0 and torch.equal(gi, good[0]) and torch.equal(gl, good[1])
+        for ids, lps in after:
+            assert torch.equal(ids, good[0]) and torch.equal(lps, good[1])
+    assert ws.read_status() == (0, 0, 0)
