@@ -455,15 +455,16 @@ k_head_dense(const HeadArgs a, Ctrl* ctrl, float* __restrict__ recs, const Dense
                         for (int i = 0; i < kCh; ++i)
                             if (i < nv) a.dbg_logits[(size_t)b * K + j0 + i] = __uint_as_float(r[i]);
                     }
-                    // running max / sum-exp: one rescale per chunk, independent exponentials, two sums
+                    // running max / sum-exp: one rescale per chunk, independent exponentials, two sums.  The maximum is
+                    // subtracted before the scaling to base 2: z - m is exact or nearly so whatever the size of the logits,
+                    // while z * log2e - round(m * log2e) carries half a unit of m * log2e into every exponent of the chunk
                     const float m_new = fmaxf(st.m, cmax);
                     const float m_ref = (m_new == -CUDART_INF_F) ? 0.f : m_new;
-                    const float m2 = m_ref * -kLog2e;
                     float acc0 = 0.f, acc1 = 0.f;
 #pragma unroll
                     for (int i = 0; i < kCh; i += 2) {
-                        acc0 += exp2_fast(fmaf(z[i], kLog2e, m2));
-                        acc1 += exp2_fast(fmaf(z[i + 1], kLog2e, m2));
+                        acc0 += exp_fast(z[i] - m_ref);
+                        acc1 += exp_fast(z[i + 1] - m_ref);
                     }
                     st.s = st.s * exp_fast(st.m - m_ref) + (acc0 + acc1);
                     st.m = m_new;
