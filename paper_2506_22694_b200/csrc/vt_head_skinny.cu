@@ -95,8 +95,7 @@ __device__ __forceinline__ long long bound_cycles(unsigned long long ns) {
 }
 constexpr long long kShortBoundCycles = 2000000;      // 1 ms
 // Bounded wait of one thread; false when the CTA is aborting or the bound expired (which starts an abort).
-__device__ __forceinline__ bool mbar_wait(uint64_t* b, uint32_t parity, volatile int* abort_flag,
-                                          const volatile long long* bound) {
+__device__ __forceinline__ bool mbar_wait(uint64_t* b, uint32_t parity, volatile int* abort_flag, const long long* bound) {
     if (mbar_test(b, parity)) return true;
     const long long t0 = clock64();
     const long long lim = *bound;
@@ -114,8 +113,7 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* b, uint32_t parity, volatile
 // Same, called by all 32 lanes of a warp: lane 0 polls (a CTA of polling threads takes shared-memory and issue
 // slots from what it waits for), then every lane observes the completed phase itself.  The outcome is voted on,
 // so the lanes never part ways before a warp-collective instruction.
-__device__ __forceinline__ bool mbar_wait_warp(uint64_t* b, uint32_t parity, volatile int* abort_flag,
-                                               const volatile long long* bound) {
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t* b, uint32_t parity, volatile int* abort_flag, const long long* bound) {
     int ok = 1;
     if ((threadIdx.x & 31) == 0) ok = mbar_wait(b, parity, abort_flag, bound) ? 1 : 0;
     ok = __shfl_sync(0xffffffffu, ok, 0);
@@ -228,8 +226,12 @@ k_head_stream(const HeadArgs a, Ctrl* ctrl, float* __restrict__ recs, const Geo 
         for (int p = 0; p < 2; ++p) { mbar_init(&s_acc_full[p], 1); mbar_init(&s_acc_empty[p], EW); }
         mbar_init(&s_drain, 1);
         s_abort = 0;
-        s_bound = bound_cycles(kWaitLimitNs);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (threadIdx.x == 64) {                             // (beside the barriers' and the tensor memory's set-up, which take as long)
+        // the caller's bound, 0 = the default: written with the host waiting for it, so it is final before any later launch
+        const unsigned long long ns = *reinterpret_cast<volatile unsigned long long*>(&ctrl->wait_ns);
+        s_bound = bound_cycles(ns ? ns : kWaitLimitNs);
     }
     if (warp == 1) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
@@ -241,7 +243,6 @@ k_head_stream(const HeadArgs a, Ctrl* ctrl, float* __restrict__ recs, const Geo 
     tc_fence_after();
     const uint32_t tmem_base = s_tmem_base;
     volatile int* abort_flag = &s_abort;
-    const volatile long long* bound = &s_bound;
     // Programmatic dependent launch (a no-op unless the launch asked for it): the next kernel on the stream
     // may become resident as soon as its resources are free (this CTA has its tensor memory by now), and this
     // kernel goes no further than fetching weights until everything enqueued before it has completed.
@@ -291,17 +292,13 @@ k_head_stream(const HeadArgs a, Ctrl* ctrl, float* __restrict__ recs, const Geo 
                     if (++ks == n_ks) ks = 0;
                 }
             }
-            {
-                const unsigned long long lim = *reinterpret_cast<volatile unsigned long long*>(&ctrl->wait_ns);        // 0 = the default
-                if (lim) s_bound = bound_cycles(lim);               // (a race with early waiters only keeps their bound)
-            }
             int done = pre;
             {
                 // steady state: the cursor over (stage, step in d, tile) moves by additions only
                 int sc = pre == S ? 0 : pre, ks = pre % n_ks, y = r0 + (pre / n_ks) * geo.rows;
                 uint32_t par = 0;                                   // fill g waits for the release of fill g - S
                 for (int g = pre; g < total; ++g, ++done) {
-                    if (!mbar_wait(&s_empty[sc], par, abort_flag, bound)) break;
+                    if (!mbar_wait(&s_empty[sc], par, abort_flag, &s_bound)) break;
                     const int subs = min(sub, geo.n_kc - ks * sub);
                     mbar_expect_tx(&s_full[sc], step_tx * (uint32_t)subs);
                     const uint32_t dst0 = ring_u32 + (uint32_t)(sc * sub * geo.step_bytes);
@@ -334,6 +331,8 @@ k_head_stream(const HeadArgs a, Ctrl* ctrl, float* __restrict__ recs, const Geo 
             const uint64_t d_step = (uint64_t)(geo.step_bytes >> 4);
             const int S = geo.n_stages, sub = geo.sub;
             const int n_ks = (geo.n_kc + sub - 1) / sub;
+            // (h is asked for after the dependency, so no stage is complete before it; its bound must not count earlier work)
+            griddep_wait();
             int s = 0, issued = 0, set_no = 0;
             uint32_t ph = 0;
             bool alive = true;
@@ -341,12 +340,12 @@ k_head_stream(const HeadArgs a, Ctrl* ctrl, float* __restrict__ recs, const Geo 
                 uint32_t d_tmem = 0;
                 int in_phase = 0;                                   // steps issued into the current set
                 for (int ks = 0; ks < n_ks; ++ks) {
-                    if (!mbar_wait(&s_full[s], ph, abort_flag, bound)) { alive = false; break; }
+                    if (!mbar_wait(&s_full[s], ph, abort_flag, &s_bound)) { alive = false; break; }
 #ifdef VT_STAMPS
                     if (t == 0 && ks == 0) VT_STAMP(3);
 #endif
                     if (in_phase == 0) {                            // a new accumulator set: the epilogue has read what it held
-                        if (set_no >= 2 && !mbar_wait(&s_acc_empty[set_no & 1], (uint32_t)(((set_no >> 1) - 1) & 1), abort_flag, bound)) {
+                        if (set_no >= 2 && !mbar_wait(&s_acc_empty[set_no & 1], (uint32_t)(((set_no >> 1) - 1) & 1), abort_flag, &s_bound)) {
                             alive = false;
                             break;
                         }
@@ -422,7 +421,7 @@ k_head_stream(const HeadArgs a, Ctrl* ctrl, float* __restrict__ recs, const Geo 
             bool ok = true;
             for (int p = 0; p < n_ph; ++p, ++set_no) {
                 const int set = set_no & 1;
-                ok = mbar_wait_warp(&s_acc_full[set], (uint32_t)((set_no >> 1) & 1), abort_flag, bound);
+                ok = mbar_wait_warp(&s_acc_full[set], (uint32_t)((set_no >> 1) & 1), abort_flag, &s_bound);
                 if (!ok) break;
                 tc_fence_after();
                 if (quad * qrows < nrow && part * 4 < B) {
