@@ -32,6 +32,8 @@
 // Every wait is bounded: on expiry the CTA raises VT_FLAG_TIMEOUT, lets its own copies and MMAs finish and leaves.
 #include <math_constants.h>
 
+#include <type_traits>
+
 #include "vt_common.cuh"
 #include "vt_head_common.cuh"
 #include "vt_tc.cuh"
@@ -68,6 +70,7 @@ struct Geo {
     int mma_rows;      // M of the MMA: 64 where a tile has no more rows, else 128
     int n_kc;          // 64-column steps of d
     int sub;           // steps per ring stage
+    int issuers;       // warps that issue MMAs, stages dealt to them in turn (see make_geo)
     int n_stages;      // ring depth
     int h_bytes;       // shared memory of a step's h part (a multiple of 1024)
     int step_bytes;    // ... of a step: h part + W part
@@ -94,19 +97,24 @@ __device__ __forceinline__ long long bound_cycles(unsigned long long ns) {
     return (long long)(ns < (1ull << 61) ? 2 * ns : (1ull << 62));
 }
 constexpr long long kShortBoundCycles = 2000000;      // 1 ms
-// Bounded wait of one thread; false when the CTA is aborting or the bound expired (which starts an abort).
-__device__ __forceinline__ bool mbar_wait(uint64_t* b, uint32_t parity, volatile int* abort_flag, const long long* bound) {
+// Bounded wait of one thread; false when the CTA is aborting or the bound expired (which starts an abort).  A role that
+// waits before the launch dependency is released passes `released`: earlier work on the stream does not count, the clock
+// starts when that flag is up (until then the bound is a thousand times the default).
+__device__ __forceinline__ bool mbar_wait(uint64_t* b, uint32_t parity, volatile int* abort_flag, const long long* bound,
+                                          volatile int* released = nullptr) {
     if (mbar_test(b, parity)) return true;
-    const long long t0 = clock64();
-    const long long lim = *bound;
-    const bool nb = lim < kShortBoundCycles;
+    bool counts = !released || *released;
+    long long t0 = clock64();
     for (;;) {
+        const long long lim = counts ? *bound : 1000 * bound_cycles(kWaitLimitNs);
+        const bool nb = lim < kShortBoundCycles;
 #pragma unroll 1
         for (int i = 0; i < 64; ++i) {
             if (nb ? mbar_test(b, parity) : mbar_try(b, parity)) return true;
             if (nb && clock64() - t0 > lim) break;
         }
         if (*abort_flag) return false;
+        if (!counts && *released) { counts = true; t0 = clock64(); continue; }
         if (clock64() - t0 > lim) { *abort_flag = 1; return false; }
     }
 }
@@ -122,6 +130,7 @@ __device__ __forceinline__ bool mbar_wait_warp(uint64_t* b, uint32_t parity, vol
 }
 // before the CTA leaves: what is in flight gets this long to finish
 __device__ __forceinline__ void drain_wait(uint64_t* b, uint32_t parity) {
+    if (mbar_try(b, parity)) return;                     // (the usual case; reading the timer costs 0.1 us)
     const unsigned long long t0 = global_ns();
     while (!mbar_try(b, parity) && global_ns() - t0 < kWaitLimitNs) {}
 }
@@ -181,20 +190,26 @@ struct RowState {
     int gj;
 };
 
+// The variant of up to eight hidden rows may have a second warp for the MMAs (the last one; see make_geo).  With sixteen
+// epilogue warps one more slows them down by more than it gives (9 rows of 12000 x 2048 13.3 us without, 15.8 with it).
+__host__ __device__ constexpr int max_issuers(int ew) { return ew == 8 ? 2 : 1; }
+
 // EW epilogue warps (a multiple of 4: the warps of a lane quadrant share the accumulator columns), at most RPW hidden
 // rows per epilogue warp.
 template <int EW, int RPW>
-__global__ void __launch_bounds__((EW + 2) * 32, EW == 8 ? 2 : 1)
+__global__ void __launch_bounds__((EW + 1 + max_issuers(EW)) * 32, EW == 8 ? 2 : 1)
 k_head_stream(const HeadArgs a, Ctrl* ctrl, float* __restrict__ recs, const Geo geo,
               const __grid_constant__ CUtensorMap tm_h, const __grid_constant__ CUtensorMap tm_w) {
     extern __shared__ uint8_t s_dyn[];
     __shared__ uint64_t s_full[kMaxStages], s_empty[kMaxStages], s_acc_full[2], s_acc_empty[2], s_drain;
     __shared__ uint32_t s_tmem_base;
     __shared__ int s_abort;
+    __shared__ int s_issued[2];                          // ring stages each issuer has released
+    __shared__ int s_released;                           // the launch dependency is
     __shared__ long long s_bound;                        // bound of a wait in SM cycles
     // An accumulator set holds kAccs accumulators of kNpad columns (hidden rows).  The kParts warps of a lane quadrant
     // take kUnits groups of four columns each: always eight loads per warp and phase.
-    constexpr int kParts = EW / 4, kUnits = RPW, kAccs = 8 / kUnits, kNpad = 16 * kUnits;
+    constexpr int kParts = EW / 4, kUnits = RPW, kAccs = 8 / kUnits, kNpad = 16 * kUnits, kIssuers = max_issuers(EW);
     static_assert(kAccs * kNpad <= kSetCols && kParts * kUnits * 4 <= kNpad, "a set's columns");
     const int B = a.B, K = a.K, topk = a.topk;
     uint8_t* ring = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(s_dyn) + 1023) & ~(uintptr_t)1023);
@@ -223,9 +238,11 @@ k_head_stream(const HeadArgs a, Ctrl* ctrl, float* __restrict__ recs, const Geo 
         asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tm_w)) : "memory");
         asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tm_h)) : "memory");
         for (int s = 0; s < geo.n_stages; ++s) { mbar_init(&s_full[s], 1); mbar_init(&s_empty[s], 1); }
-        for (int p = 0; p < 2; ++p) { mbar_init(&s_acc_full[p], 1); mbar_init(&s_acc_empty[p], EW); }
-        mbar_init(&s_drain, 1);
+        for (int p = 0; p < 2; ++p) { mbar_init(&s_acc_full[p], geo.issuers); mbar_init(&s_acc_empty[p], EW); }
+        mbar_init(&s_drain, geo.issuers);
         s_abort = 0;
+        s_issued[0] = s_issued[1] = 0;
+        s_released = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (threadIdx.x == 64) {                             // (beside the barriers' and the tensor memory's set-up, which take as long)
@@ -282,6 +299,7 @@ k_head_stream(const HeadArgs a, Ctrl* ctrl, float* __restrict__ recs, const Geo 
             }
             VT_STAMP(1);
             griddep_wait();
+            *const_cast<volatile int*>(&s_released) = 1;
             VT_STAMP(2);
             {
                 int ks = 0;
@@ -319,69 +337,84 @@ k_head_stream(const HeadArgs a, Ctrl* ctrl, float* __restrict__ recs, const Geo 
             // fill of a stage is its barrier's last phase; in an undisturbed run the MMAs finish later than this.)
             for (int g = max(0, done - S); g < done; ++g) drain_wait(&s_full[g % S], (uint32_t)((g / S) & 1));
         }
-    } else if (warp == 1) {
-        // ================= MMA issuer ==================================================================
-        if (elect_one()) {
+    } else if (warp == 1 || (kIssuers == 2 && warp == EW + 2)) {
+        // ================= MMA issuers =================================================================
+        const int me = warp == 1 ? 0 : 1, ni = geo.issuers;
+        if (me < ni && elect_one()) {
             const uint32_t idesc = make_idesc(geo.mma_rows, kNpad);
             // (the ring is 1024-byte aligned and under 256 KB: adding byte offsets >> 4 stays inside the address field;
             // rows of an operand beyond the tile's / beyond B are whatever lies behind it: their TMEM lanes and columns
             // are not looked at)
             const uint64_t desc_h0 = make_desc(ring_u32);
-            const uint64_t w_off = (uint64_t)(geo.h_bytes >> 4);
-            const uint64_t d_step = (uint64_t)(geo.step_bytes >> 4);
+            const uint32_t desc_lo = (uint32_t)desc_h0, desc_hi = (uint32_t)(desc_h0 >> 32);
+            const uint32_t w_off = (uint32_t)(geo.h_bytes >> 4), d_step = (uint32_t)(geo.step_bytes >> 4);
             const int S = geo.n_stages, sub = geo.sub;
-            const int n_ks = (geo.n_kc + sub - 1) / sub;
-            // (h is asked for after the dependency, so no stage is complete before it; its bound must not count earlier work)
-            griddep_wait();
-            int s = 0, issued = 0, set_no = 0;
+            const int n_ks = (geo.n_kc + sub - 1) / sub, spp = kPhase / sub;       // ring stages per tile / per phase
+            const int total = geo.n_tiles * n_ks;
+            // Every MMA of a stage: consecutive ones go to this issuer's N accumulators (from column d on) in turn, the first
+            // round of a phase overwrites.  in_phase: this issuer's steps in the phase so far.  Accumulators and flags are
+            // constants of the unrolled code (an odd step swaps the halves of eight accumulators).
+            auto issue = [&](auto accs, uint32_t d, uint32_t lo, int subs, int in_phase) {
+                constexpr int N = decltype(accs)::value;
+                const uint32_t odd = N > 4 ? (uint32_t)(in_phase & 1) * (4 * kNpad) : 0u;
+                const uint32_t d_even = d + odd, d_odd = N > 4 ? d + 4 * kNpad - odd : d;
+                auto steps = [&](auto later) {
+#pragma unroll
+                    for (int u = 0; u < kMaxSub; ++u)
+                        if (u < subs) {
+#pragma unroll
+                            for (int k = 0; k < kBK / 16; ++k)
+                                tc_mma_lo(((u & 1) ? d_odd : d_even) + (uint32_t)((k % N) * kNpad), lo + (uint32_t)u * d_step + w_off + (uint32_t)(2 * k),
+                                          lo + (uint32_t)u * d_step + (uint32_t)(2 * k), desc_hi, idesc,
+                                          (decltype(later)::value || u * (kBK / 16) + k >= N) ? 1u : 0u);
+                        }
+                };
+                if (in_phase * (kBK / 16) >= N) steps(std::true_type{}); else steps(std::false_type{});
+            };
+            // (no griddep_wait here: h is asked for after it, so no stage is complete before; waking up from it costs 0.3 us
+            // that a probe on the stage does not)
+            int s = me, own = me, first = 0, set_no = 0;            // own: this issuer's next stage, first: the phase's first
             uint32_t ph = 0;
             bool alive = true;
             for (int t = 0; t < geo.n_tiles && alive; ++t) {
-                uint32_t d_tmem = 0;
-                int in_phase = 0;                                   // steps issued into the current set
-                for (int ks = 0; ks < n_ks; ++ks) {
-                    if (!mbar_wait(&s_full[s], ph, abort_flag, &s_bound)) { alive = false; break; }
+                for (int ks0 = 0; ks0 < n_ks && alive; ks0 += spp) {
+                    // a new accumulator set: the epilogue has read what it held
+                    if (set_no >= 2 && !mbar_wait(&s_acc_empty[set_no & 1], (uint32_t)(((set_no >> 1) - 1) & 1), abort_flag, &s_bound)) {
+                        alive = false;
+                        break;
+                    }
+                    const uint32_t d_tmem = tmem_base + (uint32_t)((set_no & 1) * kSetCols);
+                    const int end = first + min(spp, n_ks - ks0);
+                    int in_phase = 0;
+                    for (; own < end; own += ni) {
+                        if (!mbar_wait(&s_full[s], ph, abort_flag, &s_bound, &s_released)) { alive = false; break; }
 #ifdef VT_STAMPS
-                    if (t == 0 && ks == 0) VT_STAMP(3);
+                        if (own == 0) VT_STAMP(3);
 #endif
-                    if (in_phase == 0) {                            // a new accumulator set: the epilogue has read what it held
-                        if (set_no >= 2 && !mbar_wait(&s_acc_empty[set_no & 1], (uint32_t)(((set_no >> 1) - 1) & 1), abort_flag, &s_bound)) {
-                            alive = false;
-                            break;
-                        }
-                        d_tmem = tmem_base + (uint32_t)((set_no & 1) * kSetCols);
+                        tc_fence_after();
+                        const int subs = min(sub, geo.n_kc - (ks0 + own - first) * sub);
+                        const uint32_t lo = desc_lo + ((uint32_t)(s * sub * geo.step_bytes) >> 4);
+                        if (kIssuers == 2 && ni == 2)
+                            issue(std::integral_constant<int, kAccs / 2>{}, d_tmem + (uint32_t)(me * (kAccs / 2) * kNpad), lo, subs, in_phase);
+                        else
+                            issue(std::integral_constant<int, kAccs>{}, d_tmem, lo, subs, in_phase);
+                        in_phase += subs;
+                        tc_commit(&s_empty[s]);                     // the stage is free once these MMAs have read it
+                        s += ni;
+                        if (s >= S) { s -= S; ph ^= 1u; }
                     }
-                    tc_fence_after();
-                    const int subs = min(sub, geo.n_kc - ks * sub);
-                    uint64_t dh = desc_h0 + (uint64_t)((uint32_t)(s * sub * geo.step_bytes) >> 4);
-#pragma unroll
-                    for (int u = 0; u < kMaxSub; ++u) {
-                        if (u < subs) {
-                            // consecutive MMAs go to the set's accumulators in turn; the first round of a phase overwrites
-#pragma unroll
-                            for (int k = 0; k < kBK / 16; ++k) {
-                                const int i = (in_phase + u) * (kBK / 16) + k;
-                                tc_mma(d_tmem + (uint32_t)((i % kAccs) * kNpad), dh + w_off + (uint64_t)(k * 2), dh + (uint64_t)(k * 2), idesc,
-                                       i >= kAccs ? 1u : 0u);
-                            }
-                            dh += d_step;
-                        }
-                    }
-                    in_phase += subs;
-                    tc_commit(&s_empty[s]);                         // the stage is free once these MMAs have read it
-                    if (in_phase == kPhase || ks == n_ks - 1) {
-                        tc_commit(&s_acc_full[set_no & 1]);         // the phase's accumulators are complete
-                        ++set_no;
-                        in_phase = 0;
-                    }
-                    ++issued;
-                    if (++s == S) { s = 0; ph ^= 1u; }
+                    if (alive) tc_commit(&s_acc_full[set_no & 1]);  // this issuer's part of the phase's accumulators is complete
+                    first = end;
+                    ++set_no;
                 }
             }
-            // every MMA issued has finished and every commit has arrived before the CTA may leave, whatever happened
+            s_issued[me] = (own - me) / ni;
+            // every MMA issued has finished and every commit has arrived before the CTA may leave (a stage's last release: its
+            // barrier moves no further)
             tc_commit(&s_drain);
             drain_wait(&s_drain, 0);
-            for (int g = max(0, issued - S); g < issued; ++g) drain_wait(&s_empty[g % S], (uint32_t)((g / S) & 1));
+            if (alive)
+                for (int g = own - ni; g >= max(0, total - S); g -= ni) drain_wait(&s_empty[g % S], (uint32_t)((g / S) & 1));
         }
     } else {
         // ================= epilogue warps ==============================================================
@@ -401,6 +434,7 @@ k_head_stream(const HeadArgs a, Ctrl* ctrl, float* __restrict__ recs, const Geo 
         }
         __syncwarp();
         const int n_ph = (geo.n_kc + kPhase - 1) / kPhase;
+        const int n_ks = (geo.n_kc + geo.sub - 1) / geo.sub, spp = kPhase / geo.sub;     // ring stages per tile / per phase
         int set_no = 0;
         for (int t = 0; t < geo.n_tiles; ++t) {
             const int j0 = r0 + t * geo.rows;                       // first vocabulary row of the tile
@@ -431,16 +465,22 @@ k_head_stream(const HeadArgs a, Ctrl* ctrl, float* __restrict__ recs, const Geo 
 #pragma unroll
                     for (int i = 0; i < 8; ++i) ad[i] = base + (uint32_t)((i % kAccs) * kNpad + (i / kAccs) * kParts * 4);
                     tc_ld_8x4(ad, v);
-                    const int mmas = min(kPhase, geo.n_kc - p * kPhase) * (kBK / 16);
-                    // (an accumulator that a short last phase did not get to holds nothing; the others pairwise: fewer
-                    // roundings in a row than one after the other)
+                    // (an accumulator that a short last phase did not get to holds nothing: those beyond its MMAs or, where
+                    // it is one stage, the half of the issuer that had no stage; the others pairwise: fewer roundings in a
+                    // row than one after the other)
+                    int c0 = 0, c1 = min(kPhase, geo.n_kc - p * kPhase) * (kBK / 16);
+                    if (kIssuers == 2 && geo.issuers == 2) {
+                        const bool one = n_ks - p * spp == 1;
+                        c0 = one && ((t * n_ks + p * spp) & 1) ? kAccs / 2 : 0;
+                        c1 = one ? c0 + kAccs / 2 : kAccs;
+                    }
 #pragma unroll
                     for (int q = 0; q < 4; ++q)
 #pragma unroll
                         for (int i = 0; i < kUnits; ++i) {
                             float w[kAccs];
 #pragma unroll
-                            for (int c = 0; c < kAccs; ++c) w[c] = c < mmas ? v[i * kAccs + c][q] : 0.f;
+                            for (int c = 0; c < kAccs; ++c) w[c] = c >= c0 && c < c1 ? v[i * kAccs + c][q] : 0.f;
 #pragma unroll
                             for (int o = kAccs / 2; o; o >>= 1)
 #pragma unroll
@@ -599,6 +639,18 @@ k_head_stream(const HeadArgs a, Ctrl* ctrl, float* __restrict__ recs, const Geo 
     __syncwarp();                                                   // lanes of the single-thread roles rejoin their warps
     __syncthreads();                                                // no copy, no MMA and no read of tensor memory is left
     if (warp == 1) {
+        if (s_abort && lane == 0) {
+            // a wait expired somewhere: the last release of every stage that was released has arrived, whoever issued it
+            const int S = geo.n_stages, ni = geo.issuers;
+            int top = -1;
+            for (int i = 0; i < ni; ++i) top = max(top, i + ni * (s_issued[i] - 1));
+            for (int g = top; g > top - S && g >= 0; --g) {
+                int r = g;
+                while (r >= 0 && r / ni >= s_issued[r % ni]) r -= S;
+                if (r >= 0) drain_wait(&s_empty[r % S], (uint32_t)((r / S) & 1));
+            }
+        }
+        __syncwarp();
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(kTmemCols) : "memory");
     }
@@ -646,6 +698,14 @@ Geo make_geo(int B, int K, int d, int topk, int sms, size_t* smem_bytes) {
     g.n_stages = (int)(room / stage);
     if (g.n_stages > kMaxStages) g.n_stages = kMaxStages;
     if (g.n_stages > total) g.n_stages = (int)total;
+    // A single thread needs 250-300 cycles per 64-column step for its waits, releases and four MMAs, which a small head waits
+    // for from the moment h has landed; two threads take every other stage each (one row, L2, one / two issuers: 3000 x
+    // 1024 8.8 / 7.9 us, 5000 x 3072 15.0 / 12.9, 8000 x 4096 16.4 / 13.1, 20001 x 3072 22.4 / 20.3).  An issuer that is ahead must not take
+    // a stage's former fill, which the other one has yet to wait for, for the one it expects: it is at most two phases less
+    // a stage ahead (an accumulator set is read before its next use), so the ring has to be longer than that, or never
+    // reused, or even (a stage then always has the same issuer).  A large head's ring of three stages is none of these; there
+    // the copies are what is waited for (three stages of four steps, one issuer / six of two, two issuers: 788 MB 114.4 / 116.5).
+    g.issuers = max_issuers(ew) == 2 && (g.n_stages >= total || (g.n_stages & 1) == 0 || g.n_stages >= 2 * kPhase / g.sub) ? 2 : 1;
     g.ring_bytes = (int)(g.n_stages * stage);
     // A drafting loop reads the same head again a few tens of microseconds later.  A head that is larger than L2
     // leaves nothing behind when all of it streams through under one policy; so 56 MB of it, spread evenly over
@@ -674,7 +734,7 @@ cudaError_t launch_variant(const HeadArgs& a, Ctrl* ctrl, float* recs, const Geo
     }
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)geo.grid);
-    cfg.blockDim = dim3((EW + 2) * 32);
+    cfg.blockDim = dim3((unsigned)(EW + 1 + geo.issuers) * 32);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
     cudaLaunchAttribute attr{};
