@@ -151,7 +151,25 @@ __device__ __forceinline__ void st_stream_u4(void* p, uint4 v) {
                  "r"(v.z), "r"(v.w)
                  : "memory");
 }
-// Load that bypasses L1 (partials written by other CTAs of the same grid).
+// Loads through L2: what other CTAs of the same grid have written, and in a dependent launch the results of the kernels in
+// front of it.  Such a launch may be resident while they still write, so their results are neither constant during the
+// kernel (which the non-coherent path of __ldg and of const __restrict__ pointers takes for granted) nor to be read
+// before griddep_wait (volatile, as that is: the two keep their order).
+__device__ __forceinline__ uint32_t ld_cg_u32(const uint32_t* p) {
+    uint32_t v;
+    asm volatile("ld.global.cg.u32 %0, [%1];" : "=r"(v) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ uint2 ld_cg_u2(const uint2* p) {
+    uint2 v;
+    asm volatile("ld.global.cg.v2.u32 {%0,%1}, [%2];" : "=r"(v.x), "=r"(v.y) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ float4 ld_cg_f4(const float4* p) {
+    float4 v;
+    asm volatile("ld.global.cg.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
+    return v;
+}
 __device__ __forceinline__ float ld_cg_f32(const float* p) {
     float v;
     asm volatile("ld.global.cg.f32 %0, [%1];" : "=f"(v) : "l"(p));

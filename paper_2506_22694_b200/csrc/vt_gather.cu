@@ -12,7 +12,7 @@ constexpr int kThreads = 256;
 constexpr int kCtasPerSm = 8;
 
 __global__ void __launch_bounds__(kThreads)
-k_gather_rows(const uint16_t* __restrict__ W_full, const int32_t* __restrict__ map,
+k_gather_rows(const uint16_t* __restrict__ W_full, const int32_t* map,
               uint16_t* __restrict__ W_trim, int32_t V, int32_t K, int32_t d, Ctrl* ctrl) {
     const int lane = threadIdx.x & 31;
     const int warps_total = gridDim.x * (kThreads / 32);
@@ -21,7 +21,7 @@ k_gather_rows(const uint16_t* __restrict__ W_full, const int32_t* __restrict__ m
     griddep_wait();                                              // (the map comes from the kernel before)
     const int nvec = d >> 3;                                     // 16-byte vectors per row
     for (int j = gw; j < K; j += warps_total) {
-        const int32_t src = map[j];
+        const int32_t src = ld_cg_s32(map + j);
         uint4* dst = reinterpret_cast<uint4*>(W_trim + (size_t)j * d);
         if ((uint32_t)src >= (uint32_t)V) {                      // bad entry: flag, zero the row
             if (lane == 0 && ctrl) atomicOr(&ctrl->flags, (uint32_t)VT_FLAG_BAD_MAP);

@@ -216,7 +216,7 @@ __device__ __noinline__ void merge_records(const MergeOut a, Ctrl* ctrl, float* 
             if (a.sampled) {
                 const bool ok = row_ok && gwin != 0ull;
                 const int gj = key_idx(gwin);
-                oid[0] = ok ? (a.map ? __ldg(a.map + gj) : gj) : -1;
+                oid[0] = ok ? (a.map ? ld_cg_s32(a.map + gj) : gj) : -1;
                 olp[0] = ok ? gzw - lse : CUDART_NAN_F;
                 bad = bad || !ok;
             }
@@ -362,7 +362,7 @@ __device__ __noinline__ void merge_records(const MergeOut a, Ctrl* ctrl, float* 
         const int r = lane + 32 * sl;
         okv[sl] = r < topk && row_ok && res_k[sl] != 0ull;
         const int j = key_idx(res_k[sl]);
-        ids[sl] = okv[sl] ? (a.map ? __ldg(a.map + j) : j) : -1;
+        ids[sl] = okv[sl] ? (a.map ? ld_cg_s32(a.map + j) : j) : -1;
         zv[sl] = key_val(res_k[sl]);
     }
     if (roles == kRoleCand) {

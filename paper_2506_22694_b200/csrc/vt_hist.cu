@@ -222,12 +222,11 @@ __device__ uint32_t block_excl_scan(uint32_t x, uint32_t* s_warp /*[33]*/, uint3
 // ---- pre-pass 2: choose at most H hot bins from the sampled counts, build the lookup table ------
 // hot = sampled count >= tau, plus (in id order) as many bins with count == tau-1 as still fit.
 __global__ void __launch_bounds__(kThreads, 1)
-k_hist_pick(const uint32_t* __restrict__ sample, int32_t V, int32_t H, uint2* __restrict__ table,
-            const uint32_t* __restrict__ gate) {
+k_hist_pick(const uint32_t* sample, int32_t V, int32_t H, uint2* __restrict__ table, const uint32_t* gate) {
     extern __shared__ __align__(16) uint8_t s_dyn[];
     griddep_launch_dependents();
     griddep_wait();
-    if (gate && *reinterpret_cast<const volatile uint32_t*>(gate) == 0) return;   // the packed count stood: nothing to recount
+    if (gate && ld_cg_u32(gate) == 0) return;               // the packed count stood: nothing to recount
     __shared__ uint32_t s_hist[kPickBins];
     __shared__ uint32_t s_warp[33];
     __shared__ uint32_t s_definite;
@@ -244,7 +243,7 @@ k_hist_pick(const uint32_t* __restrict__ sample, int32_t V, int32_t H, uint2* __
 #pragma unroll
             for (int q = 0; q < kPickLoads; ++q) {
                 const int v = v0 + q * kThreads;
-                cs[q] = v < V ? __ldg(sample + v) : 0xffffffffu;
+                cs[q] = v < V ? ld_cg_u32(sample + v) : 0xffffffffu;
             }
 #pragma unroll
             for (int q = 0; q < kPickLoads; ++q) {
@@ -282,7 +281,7 @@ k_hist_pick(const uint32_t* __restrict__ sample, int32_t V, int32_t H, uint2* __
 #pragma unroll
         for (int q = 0; q < kPickLoads; ++q) {
             const int v = (w0 + q * (kThreads / 32)) * 32 + lane;
-            cs[q] = v < V ? min(__ldg(sample + v), (uint32_t)(kPickBins - 1)) : 0xffffffffu;
+            cs[q] = v < V ? min(ld_cg_u32(sample + v), (uint32_t)(kPickBins - 1)) : 0xffffffffu;
         }
 #pragma unroll
         for (int q = 0; q < kPickLoads; ++q) {
@@ -329,11 +328,11 @@ k_hist_pick(const uint32_t* __restrict__ sample, int32_t V, int32_t H, uint2* __
 // ---- main pass: hot bins in shared memory, cold bins through L2 ----------------------------------
 __global__ void __launch_bounds__(kThreads, 1)
 k_hist_hot(const int32_t* __restrict__ ids, int64_t n, int32_t V, uint32_t* __restrict__ counts,
-           const uint2* __restrict__ table, int32_t H, Ctrl* ctrl, const uint32_t* __restrict__ gate) {
+           const uint2* table, int32_t H, Ctrl* ctrl, const uint32_t* gate) {
     extern __shared__ __align__(16) uint8_t s_raw[];
     griddep_launch_dependents();
     griddep_wait();
-    if (gate && *reinterpret_cast<const volatile uint32_t*>(gate) == 0) return;
+    if (gate && ld_cg_u32(gate) == 0) return;
     const int T32 = (V + 31) >> 5;
     // The lookup is repacked for the main pass: one 4-byte word per 16 ids = {16 membership bits,
     // 16-bit slot of the first member} -- a 4-byte gather costs half the shared-memory wavefronts of
@@ -341,7 +340,7 @@ k_hist_hot(const int32_t* __restrict__ ids, int64_t n, int32_t V, uint32_t* __re
     uint32_t* s_t16 = reinterpret_cast<uint32_t*>(s_raw);                       // [2 * T32]
     uint32_t* s_cnt = reinterpret_cast<uint32_t*>(s_raw + (size_t)T32 * 8);
     for (int i = threadIdx.x; i < T32; i += kThreads) {
-        const uint2 e = table[i];
+        const uint2 e = ld_cg_u2(table + i);
         s_t16[2 * i] = (e.x & 0xffffu) | (e.y << 16);
         s_t16[2 * i + 1] = (e.x >> 16) | ((e.y + __popc(e.x & 0xffffu)) << 16);
     }
@@ -654,21 +653,22 @@ k_hist_packed(const int32_t* __restrict__ ids, int64_t n, int32_t V, int32_t Vp,
 // wrapped, counts is left as the recount needs it (zero unless accumulating) and the recount's sampling
 // pre-pass runs here.
 __global__ void __launch_bounds__(kThreads, 1)
-k_hist_settle(const int32_t* __restrict__ ids, int64_t n, int32_t V, const uint32_t* __restrict__ packed,
+k_hist_settle(const int32_t* __restrict__ ids, int64_t n, int32_t V, const uint32_t* packed,
               uint32_t* __restrict__ counts, int accumulate, uint32_t* __restrict__ sample,
-              const uint32_t* __restrict__ gate, Ctrl* ctrl) {
+              const uint32_t* gate, Ctrl* ctrl) {
     __shared__ int s_tag[kSampleSlots];
     __shared__ uint32_t s_cnt[kSampleSlots];
     griddep_launch_dependents();
     griddep_wait();
-    const bool recount = *reinterpret_cast<const volatile uint32_t*>(gate) != 0;
+    const bool recount = ld_cg_u32(gate) != 0;
     for (int v = blockIdx.x * kThreads + threadIdx.x; v < V; v += gridDim.x * kThreads) {
-        const uint32_t c = recount ? 0u : packed[v];
+        const uint32_t c = recount ? 0u : ld_cg_u32(packed + v);
         counts[v] = accumulate ? counts[v] + c : c;
     }
     if (!recount) {
         if (blockIdx.x == 0 && threadIdx.x == 0) {
-            const unsigned long long bad = *reinterpret_cast<const unsigned long long*>(gate + 2);
+            const uint2 skipped = ld_cg_u2(reinterpret_cast<const uint2*>(gate + 2));
+            const unsigned long long bad = (unsigned long long)skipped.y << 32 | skipped.x;
             if (bad) {
                 atomicAdd(&ctrl->n_bad, bad);
                 atomicOr(&ctrl->flags, (uint32_t)VT_FLAG_BAD_ID);

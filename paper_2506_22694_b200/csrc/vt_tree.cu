@@ -12,7 +12,7 @@ constexpr int kTreeThreads = 1024;
 constexpr int kTreeMax = 4096;                       // nodes one call ranks (VT_TREE_MAX_NODES)
 
 __global__ void __launch_bounds__(kTreeThreads, 1)
-k_tree_expand(const int32_t* __restrict__ cand_ids, const float* __restrict__ cand_lp, int32_t B, int32_t topk,
+k_tree_expand(const int32_t* cand_ids, const float* cand_lp, int32_t B, int32_t topk,
               int32_t ld, int32_t col0, const TreeArgs t) {
     __shared__ __align__(16) unsigned long long s_key[kTreeMax];
     griddep_launch_dependents();
@@ -21,9 +21,8 @@ k_tree_expand(const int32_t* __restrict__ cand_ids, const float* __restrict__ ca
 }
 
 __global__ void __launch_bounds__(kTreeThreads, 1)
-k_tree_rerank(const int32_t* __restrict__ pool_token, const int32_t* __restrict__ pool_parent,
-              const float* __restrict__ pool_score, int32_t n, int32_t budget, int32_t* __restrict__ out_nodes,
-              int32_t* __restrict__ out_token, int32_t* __restrict__ out_parent) {
+k_tree_rerank(const int32_t* pool_token, const int32_t* pool_parent, const float* pool_score, int32_t n,
+              int32_t budget, int32_t* __restrict__ out_nodes, int32_t* __restrict__ out_token, int32_t* __restrict__ out_parent) {
     __shared__ __align__(16) unsigned long long s_key[kTreeMax];
     __shared__ uint32_t s_sel[kTreeMax / 32];        // bit i: node i is kept
     __shared__ int s_before[kTreeMax / 32];          // kept nodes in earlier words
@@ -31,7 +30,7 @@ k_tree_rerank(const int32_t* __restrict__ pool_token, const int32_t* __restrict_
     griddep_launch_dependents();
     griddep_wait();                                  // (the pool comes from the kernels before)
     const int words = (n + 31) / 32;
-    for (int i = threadIdx.x; i < n; i += (int)blockDim.x) s_key[i] = node_key(pool_score[i], i);
+    for (int i = threadIdx.x; i < n; i += (int)blockDim.x) s_key[i] = node_key(ld_cg_f32(pool_score + i), i);
     if (n + (int)threadIdx.x < padded_keys(n)) s_key[n + threadIdx.x] = 0ull;
     for (int w = threadIdx.x; w < words; w += (int)blockDim.x) s_sel[w] = 0;
     __syncthreads();
@@ -59,14 +58,14 @@ k_tree_rerank(const int32_t* __restrict__ pool_token, const int32_t* __restrict_
         const uint32_t bit = 1u << (i & 31);
         if (!(s_sel[i >> 5] & bit)) continue;
         const int pos = s_before[i >> 5] + __popc(s_sel[i >> 5] & (bit - 1));
-        const int32_t par = pool_parent[i];
+        const int32_t par = ld_cg_s32(pool_parent + i);
         int32_t ppos = -1;
         if (par >= 0) {
             const bool ok = par < n && (s_sel[par >> 5] >> (par & 31) & 1u);
             ppos = ok ? s_before[par >> 5] + __popc(s_sel[par >> 5] & ((1u << (par & 31)) - 1)) : -2;
         }
         out_nodes[pos] = i;
-        out_token[pos] = pool_token[i];
+        out_token[pos] = ld_cg_s32(pool_token + i);
         out_parent[pos] = ppos;
     }
     for (int k = m + threadIdx.x; k < budget; k += (int)blockDim.x) {

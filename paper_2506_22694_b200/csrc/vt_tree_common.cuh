@@ -44,9 +44,9 @@ __device__ __forceinline__ void tree_expand_block(const TreeArgs& t, const int32
     const int n_new = B * topk;
     for (int i = tid; i < n_new; i += nthreads) {
         const int b = i / topk, j = i - b * topk;
-        int32_t par = t.frontier ? t.frontier[b] : -1;
+        int32_t par = t.frontier ? ld_cg_s32(t.frontier + b) : -1;
         if (par < -1 || par >= t.pool_base) par = -1;                   // memory safety; callers pass earlier nodes
-        const float base = par < 0 ? 0.0f : t.pool_score[par];         // earlier depth: not written by this launch
+        const float base = par < 0 ? 0.0f : ld_cg_f32(t.pool_score + par);         // earlier depth: not written by this launch
         const float lp = ld_cg_f32(cand_lp + (int64_t)b * ld + col0 + j);    // (written by other blocks of this launch)
         const float step = (lp != lp) ? lp : fminf(lp, 0.0f);          // a log-probability is never positive
         const float s = base + step;

@@ -11,8 +11,7 @@ namespace {
 constexpr int kWarpsPerCta = 8;
 
 __global__ void __launch_bounds__(kWarpsPerCta * 32)
-k_verify_greedy(const int32_t* __restrict__ token, const int32_t* __restrict__ parent,
-                const int32_t* __restrict__ target, int32_t S, int32_t N, int32_t* __restrict__ n_accept,
+k_verify_greedy(const int32_t* token, const int32_t* parent, const int32_t* __restrict__ target, int32_t S, int32_t N, int32_t* __restrict__ n_accept,
                 int32_t* __restrict__ path, int32_t* __restrict__ emitted, unsigned long long* tokens_total) {
     const int lane = threadIdx.x & 31;
     const int64_t s = (int64_t)blockIdx.x * kWarpsPerCta + (threadIdx.x >> 5);
@@ -35,8 +34,8 @@ k_verify_greedy(const int32_t* __restrict__ token, const int32_t* __restrict__ p
             const int i = base + lane;
             bool hit = false;
             if (i < N) {
-                const int32_t p = par ? par[i] : i - 1;
-                hit = (p == cur) & (tok[i] == want);
+                const int32_t p = par ? ld_cg_s32(par + i) : i - 1;
+                hit = (p == cur) & (ld_cg_s32(tok + i) == want);
             }
             const unsigned m = __ballot_sync(0xffffffffu, hit);
             if (m) { next = base + __ffs(m) - 1; break; }          // lowest index among equal siblings
@@ -44,7 +43,7 @@ k_verify_greedy(const int32_t* __restrict__ token, const int32_t* __restrict__ p
         if (next == INT_MAX) break;
         if (lane == 0) {
             if (my_path) my_path[n] = next;
-            if (my_emit) my_emit[n] = tok[next];
+            if (my_emit) my_emit[n] = ld_cg_s32(tok + next);
         }
         ++n;
         cur = next;
