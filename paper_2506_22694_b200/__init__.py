@@ -242,8 +242,9 @@ def vt_tree_expand(cand_ids: torch.Tensor, cand_logprobs: torch.Tensor, frontier
 def vt_draft_head_expand(h: torch.Tensor, W_trim: torch.Tensor, map_: torch.Tensor | None, temp: torch.Tensor,
                          topk: int, uniforms: torch.Tensor | None, frontier_nodes: torch.Tensor | None, pool,
                          pool_base: int, n_front: int, ws: Workspace | None = None, out=None):
-    """One tree depth in one call: the head (as vt_draft_head(..., overlapped=True)) and the expansion of
-    its candidates into the node pool.  Returns (out_ids, out_logprobs, next_frontier [n_front])."""
+    """One tree depth in one call: the head (as vt_draft_head(..., overlapped=True), with the same promise: W_trim is not
+    written by work still pending on the stream) and the expansion of its candidates into the node pool.  Returns
+    (out_ids, out_logprobs, next_frontier [n_front])."""
     _dev(h, torch.bfloat16, "h")
     _dev(W_trim, torch.bfloat16, "W_trim")
     _dev(temp, torch.float32, "temp")
@@ -368,7 +369,9 @@ def vt_draft_head(h: torch.Tensor, W_trim: torch.Tensor, map_: torch.Tensor | No
                   out=None, debug: bool = False, overlapped: bool = False):
     """Algorithm 2 (the drafter's head over the trimmed vocabulary and the index mapping; head part).  Returns (out_ids int32 [B,1+topk], out_logprobs fp32
     [B,1+topk]); with debug=True also (logits fp32 [B,K], lse fp32 [B]).  overlapped=True uses
-    vt_draft_head_overlapped (drafting loops with static weights; see the header)."""
+    vt_draft_head_overlapped, for drafting loops with static weights: W_trim is fetched before the work in front of the
+    call has finished, so it must not be written by work still pending on the stream.  After vt_trim_head (or any other
+    write to it) synchronise, or make one plain call first."""
     _dev(h, torch.bfloat16, "h")
     _dev(W_trim, torch.bfloat16, "W_trim")
     _dev(temp, torch.float32, "temp")

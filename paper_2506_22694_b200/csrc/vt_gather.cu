@@ -17,7 +17,7 @@ k_gather_rows(const uint16_t* __restrict__ W_full, const int32_t* map,
     const int lane = threadIdx.x & 31;
     const int warps_total = gridDim.x * (kThreads / 32);
     const int gw = blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5);
-    griddep_launch_dependents();
+    // (no griddep_launch_dependents: a head call behind this one would ask for W_trim before it is written)
     griddep_wait();                                              // (the map comes from the kernel before)
     const int nvec = d >> 3;                                     // 16-byte vectors per row
     for (int j = gw; j < K; j += warps_total) {
