@@ -774,21 +774,24 @@ static cudaError_t select_prepare(bool* fits) {
 }
 
 // CTAs per cluster on the current device (found out once per device): sixteen need a GPC with as many SMs to itself,
-// which a device that lends out part of its SMs may not have.
+// which a device that lends out part of its SMs may not have.  Whatever is refused to the instances of sixteen leaves the
+// selection with eight; so does a launch of sixteen that is refused where the stream's context owns fewer SMs (below).
 static cudaError_t select_width(int* width) {
     static int known[64] = {0};
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if (dev >= 0 && dev < 64 && known[dev]) { *width = known[dev]; return cudaSuccess; }
-    bool wide = false;
-    e = select_prepare<0, kWide>(&wide);
-    if (e == cudaSuccess) e = select_prepare<1, kWide>(nullptr);
-    if (e == cudaSuccess) e = select_prepare<2, kWide>(nullptr);
-    if (e == cudaSuccess) e = select_prepare<0, kPortable>(nullptr);
+    e = select_prepare<0, kPortable>(nullptr);
     if (e == cudaSuccess) e = select_prepare<1, kPortable>(nullptr);
     if (e == cudaSuccess) e = select_prepare<2, kPortable>(nullptr);
     if (e != cudaSuccess) return e;
+    bool wide = false;
+    if (select_prepare<0, kWide>(&wide) != cudaSuccess || select_prepare<1, kWide>(nullptr) != cudaSuccess ||
+        select_prepare<2, kWide>(nullptr) != cudaSuccess) {
+        cudaGetLastError();
+        wide = false;
+    }
     *width = wide ? kWide : kPortable;
     if (dev >= 0 && dev < 64) known[dev] = *width;
     return cudaSuccess;
@@ -810,10 +813,14 @@ static cudaError_t launch_select(const uint32_t* counts, int32_t V, int32_t K, i
     int width = 0;
     const cudaError_t e = select_width(&width);
     if (e != cudaSuccess) return e;
-    return width == kWide && V > kNarrowIds ? launch_dependent(k_select_sort<MODE, kWide>, kWide, kThreads, kSelectSmem, s, counts, V, K, map, inv_map, keyA, valA,
-                                             keyB, valB, pfrac, min_count, k_out)
-                          : launch_dependent(k_select_sort<MODE, kPortable>, kPortable, kThreads, kSelectSmem, s, counts, V, K, map, inv_map, keyA,
-                                             valA, keyB, valB, pfrac, min_count, k_out);
+    if (width == kWide && V > kNarrowIds) {
+        if (launch_dependent(k_select_sort<MODE, kWide>, kWide, kThreads, kSelectSmem, s, counts, V, K, map, inv_map, keyA, valA, keyB, valB, pfrac,
+                             min_count, k_out) == cudaSuccess)
+            return cudaSuccess;
+        cudaGetLastError();
+    }
+    return launch_dependent(k_select_sort<MODE, kPortable>, kPortable, kThreads, kSelectSmem, s, counts, V, K, map, inv_map, keyA, valA, keyB, valB,
+                            pfrac, min_count, k_out);
 }
 
 // Top-P (mode 0) / minimum frequency (mode 1): the selection kernel in the mode that finds K on its way.
