@@ -68,7 +68,7 @@ k_tree_rerank(const int32_t* pool_token, const int32_t* pool_parent, const float
         out_token[pos] = ld_cg_s32(pool_token + i);
         out_parent[pos] = ppos;
     }
-    for (int k = m + threadIdx.x; k < budget; k += (int)blockDim.x) {
+    for (int64_t k = m + threadIdx.x; k < budget; k += blockDim.x) {
         out_nodes[k] = -1;
         out_token[k] = -1;
         out_parent[k] = -1;
@@ -89,8 +89,8 @@ cudaError_t launch_tree_rerank(const int32_t* pool_token, const int32_t* pool_pa
                                int32_t* out_parent, cudaStream_t st) {
     // as many threads as there are nodes to place (a quarter of the CTA for a tree of depth 3): the rest would only meet
     // at the barriers
-    int threads = (n > budget ? n : budget) + 31 & ~31;
-    if (threads > kTreeThreads) threads = kTreeThreads;
+    const int most = n > budget ? n : budget;
+    const int threads = most < kTreeThreads ? (most + 31) & ~31 : kTreeThreads;
     return launch_dependent(k_tree_rerank, 1, (unsigned)threads, 0, st, pool_token, pool_parent, pool_score, n, budget, out_nodes, out_token,
                             out_parent);
 }
