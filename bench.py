@@ -567,8 +567,8 @@ def dense_case(vt, dev, steps=200, warmup=20):
             "frac_of_lower_bound": max(t_tensor, t_hbm) / (ms * 1e3)}
 
 
-STAMP_NAMES = ("entry", "ring_requested", "released", "first_stage_landed", "last_stage_consumed", "record_written",
-               "after_fence_barrier", "after_ticket", "merge_loads_done", "merge_selection_done", "merge_outputs_written")
+STAMP_NAMES = ("entry", "ring_requested", "released", "first_stage_landed", "last_accumulators_complete", "record_written",
+               "leaving")
 
 
 DENSE_STAMP_NAMES = ("entry", "set_up", "released", "first_stage_landed", "mmas_issued_first_tile", "mmas_issued_last_tile",
@@ -614,8 +614,8 @@ def stamps_case(vt, vt_build, dev, args):
                 row = {"ctas": int(x.shape[0]), "entry_first": (x[:, 0].min() - t_rel) / 1e3}
                 for k in range(2, 7):
                     row[STAMP_NAMES[k] + "_last"] = (x[:, k].max() - t_rel) / 1e3
-                row["last_stage_consumed_median"] = float(np.median(x[:, 4] - t_rel)) / 1e3
-                row["last_stage_consumed_first"] = (x[:, 4].min() - t_rel) / 1e3
+                row["last_accumulators_median"] = float(np.median(x[:, 4] - t_rel)) / 1e3
+                row["last_accumulators_first"] = (x[:, 4].min() - t_rel) / 1e3
                 row["merge_started"], row["merge_row0_written"] = (x[0, 12] - t_rel) / 1e3, (x[0, 13] - t_rel) / 1e3
                 rows.append(row)
             rec[mode] = {k: round(float(np.median([r[k] for r in rows])), 2) for k in rows[0]}

@@ -121,8 +121,7 @@ bool head_stream_takes(int32_t B, int32_t K, int32_t d);      // calls the strea
 size_t head_skinny_scratch_bytes(int32_t B, int32_t K, int32_t topk);
 cudaError_t launch_head_skinny(const HeadArgs& a, Ctrl* ctrl, uint8_t* scratch, cudaStream_t s);
 #ifdef VT_STAMPS
-size_t head_skinny_stamps_offset(int32_t B, int32_t topk);   // offset of the phase stamps in the head scratch
-size_t head_dense_stamps_offset(int32_t B, int32_t topk);    // the same for the batched head
+size_t head_stamps_offset(int32_t B, int32_t topk);   // offset of the phase stamps in the scratch of either head
 #endif
 
 cudaError_t launch_head_merge(const HeadArgs& a, Ctrl* ctrl, float* recs, int G, cudaStream_t s);

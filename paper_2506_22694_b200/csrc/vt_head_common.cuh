@@ -135,14 +135,12 @@ struct MergeOut {
 // roles that two warps can run side by side when the CTA has warps to spare:
 //   kRoleStats: log-sum-exp over all CTAs, the Gumbel-max winner (column 0 when sampling);
 //   kRoleCand : the topk best list entries over all CTAs (columns 1..topk; column 0 when not sampling).
-// The candidate log-probabilities need the row's lse: a warp with both roles computes it first; two
-// warps sharing a row pass it through `xch` (shared memory) and meet at the named barrier `bar_id`
-// (64 threads).  All record loads of a role are issued before their first use.
+// The candidate log-probabilities need the row's lse: the two warps pass it through `xch` (shared memory) and
+// meet at the named barrier `bar_id` (64 threads).  All record loads of a role are issued before their first use.
 constexpr int kRoleCand = 1, kRoleStats = 2;
 
 __device__ __noinline__ void merge_records(const MergeOut a, Ctrl* ctrl, float* recs, int b, bool row_ok, int G,
-                                           float* stage, int roles, volatile float* xch, int bar_id,
-                                           unsigned long long* stamp = nullptr) {
+                                           float* stage, int role, volatile float* xch, int bar_id) {
     const int lane = threadIdx.x & 31;
     const int topk = a.topk;
     const unsigned long long* kp = rec_keys(recs, b, topk);
@@ -150,12 +148,10 @@ __device__ __noinline__ void merge_records(const MergeOut a, Ctrl* ctrl, float* 
     const int row_w = 1 + topk;
     int* oid = a.out_ids + (size_t)b * row_w;
     float* olp = a.out_logprobs + (size_t)b * row_w;
-    float lse = 0.f;
 
-    // the candidate role's loads go out first in any case
     const int depth = min(topk, kMergeDepth);
     unsigned long long ek[kMergeDepth][kMaxOwn];
-    if (roles & kRoleCand) {
+    if (role == kRoleCand) {
 #pragma unroll
         for (int r = 0; r < kMergeDepth; ++r)
 #pragma unroll
@@ -165,7 +161,7 @@ __device__ __noinline__ void merge_records(const MergeOut a, Ctrl* ctrl, float* 
             }
     }
 
-    if (roles & kRoleStats) {
+    if (role == kRoleStats) {
         float hm[kMaxOwn], hs[kMaxOwn], hz[kMaxOwn];
         unsigned long long hk[kMaxOwn];
 #pragma unroll
@@ -196,11 +192,9 @@ __device__ __noinline__ void merge_records(const MergeOut a, Ctrl* ctrl, float* 
         for (int o = 0; o < kMaxOwn; ++o) sc += hs[o] * exp_fast(hm[o] - Mref);   // (hm = -inf: nothing but a NaN sum counts)
 #pragma unroll
         for (int o = 16; o; o >>= 1) sc += __shfl_xor_sync(0xffffffffu, sc, o);
-        lse = Mall + logf(sc);
-        if (roles == kRoleStats) {                          // the candidate warp of this row is waiting for it
-            if (lane == 0) *xch = lse;
-            asm volatile("bar.sync %0, 64;" ::"r"(bar_id) : "memory");
-        }
+        const float lse = Mall + logf(sc);
+        if (lane == 0) *xch = lse;                          // the candidate warp of this row is waiting for it
+        asm volatile("bar.sync %0, 64;" ::"r"(bar_id) : "memory");
         unsigned long long gwin = 0ull;
         float gzw = 0.f;
         if (a.sampled) {
@@ -224,15 +218,8 @@ __device__ __noinline__ void merge_records(const MergeOut a, Ctrl* ctrl, float* 
             if (!row_ok) atomicOr(&ctrl->flags, (uint32_t)VT_FLAG_BAD_TEMP);
             else if (bad) atomicOr(&ctrl->flags, (uint32_t)VT_FLAG_NAN_ROW);
         }
+        return;
     }
-    if (!(roles & kRoleCand)) return;
-#ifdef VT_STAMPS
-    if (stamp && lane == 0 && b == 0) {
-        unsigned long long t;
-        asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t) : "l"(ek[0][0] + ek[kMergeDepth - 1][kMaxOwn - 1]));   // after the loads
-        stamp[8] = t;
-    }
-#endif
 
     unsigned long long res_k[2] = {0ull, 0ull};
     unsigned long long* stk = reinterpret_cast<unsigned long long*>(stage);        // [kMergeDepth][kMaxGrid] list heads
@@ -346,13 +333,6 @@ __device__ __noinline__ void merge_records(const MergeOut a, Ctrl* ctrl, float* 
             if (lane == (r & 31)) res_k[r >> 5] = win;
         }
     }
-#ifdef VT_STAMPS
-    if (stamp && lane == 0 && b == 0) {
-        unsigned long long t;
-        asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t) : "l"(res_k[0]));
-        stamp[9] = t;
-    }
-#endif
     // the gathers through the index mapper go out before the wait for the row's lse
     int ids[2];
     float zv[2];
@@ -365,10 +345,8 @@ __device__ __noinline__ void merge_records(const MergeOut a, Ctrl* ctrl, float* 
         ids[sl] = okv[sl] ? (a.map ? ld_cg_s32(a.map + j) : j) : -1;
         zv[sl] = key_val(res_k[sl]);
     }
-    if (roles == kRoleCand) {
-        asm volatile("bar.sync %0, 64;" ::"r"(bar_id) : "memory");
-        lse = *xch;
-    }
+    asm volatile("bar.sync %0, 64;" ::"r"(bar_id) : "memory");
+    const float lse = *xch;
     bool miss = false;
 #pragma unroll
     for (int sl = 0; sl < 2; ++sl) {
@@ -383,13 +361,6 @@ __device__ __noinline__ void merge_records(const MergeOut a, Ctrl* ctrl, float* 
     }
     const bool any_missing = __any_sync(0xffffffffu, miss);
     if (lane == 0 && row_ok && any_missing) atomicOr(&ctrl->flags, (uint32_t)VT_FLAG_NAN_ROW);
-#ifdef VT_STAMPS
-    if (stamp && lane == 0 && b == 0) {
-        unsigned long long t;
-        asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t) :: "memory");   // the stores above needed the gathered ids
-        stamp[10] = t;
-    }
-#endif
 }
 
 }  // namespace

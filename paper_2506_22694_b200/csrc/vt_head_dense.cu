@@ -23,7 +23,7 @@
 // columns each -- 16 columns at a time: running max / sum-exp of z = logit / T_b, Gumbel-max candidate
 // from the caller's uniforms, and a sorted top-k list kept in registers.  Logits never go to HBM.  The
 // two column halves of a row are merged through shared memory; per CTA (pair) and hidden row one
-// record goes to scratch; a second small kernel (one warp per hidden row) merges the records,
+// record goes to scratch; a second small kernel (two warps per hidden row) merges the records,
 // applies the index mapper and writes the outputs.  Every wait is bounded; on expiry the CTA raises
 // VT_FLAG_TIMEOUT and leaves after releasing its tensor memory.
 #include "vt_common.cuh"
@@ -40,9 +40,9 @@ constexpr int kMaxBN = 256;               // vocabulary rows per tile at most (T
 constexpr int kMaxSub = 2;                // d-steps of kBK columns one ring stage holds at most
 constexpr int kMaxStages = 8;
 constexpr int kHTileBytes = kBM * kBK * 2; // 16 KB: the hidden-row operand of a stage
-constexpr int kParts8 = 2, kParts16 = 2;  // epilogue warps per TMEM lane quadrant for lists of 8 / 16 (3 and 4 were no
+constexpr int kParts = 2;                  // epilogue warps per TMEM lane quadrant (3 and 4 were no
                                           // faster: the epilogue is bound by the instructions it issues, not by latency)
-constexpr int epi_threads(int parts) { return (2 + 4 * parts) * 32; }   // TMA producer, MMA issuer, epilogue warps
+constexpr int kThreads = (2 + 4 * kParts) * 32;   // TMA producer, MMA issuer, epilogue warps
 constexpr int kCh = 16;                   // accumulator columns per epilogue step (keeps the row state in registers)
 constexpr int kTmemCols = 512;            // 2 accumulator stages x kMaxBN columns
 constexpr int kMaxTopk = 16;              // top-k list lives in registers
@@ -182,11 +182,11 @@ __device__ __forceinline__ void list_insert(float (&tv)[KT], int (&tj)[KT], floa
 }
 
 // KT: capacity of the register top-k list (8 or kMaxTopk).  PAIR: two CTAs of a cluster form one MMA.
-// PARTS: epilogue warps per TMEM lane quadrant; each takes a contiguous share of a tile's 16-column chunks.
+// Each of the epilogue warps of a TMEM lane quadrant takes a contiguous share of a tile's 16-column chunks.
 // The epilogue is a long chain of dependent arithmetic per column: it runs at the rate the schedulers can
 // interleave warps, so more warps per scheduler shorten it almost in proportion.
-template <int KT, bool PAIR, int PARTS>
-__global__ void __launch_bounds__(epi_threads(PARTS), 1)
+template <int KT, bool PAIR>
+__global__ void __launch_bounds__(kThreads, 1)
 k_head_dense(const HeadArgs a, Ctrl* ctrl, float* __restrict__ recs, const DenseGeo geo,
              const __grid_constant__ CUtensorMap tm_h, const __grid_constant__ CUtensorMap tm_w) {
     extern __shared__ uint8_t s_dyn[];
@@ -213,7 +213,7 @@ k_head_dense(const HeadArgs a, Ctrl* ctrl, float* __restrict__ recs, const Dense
         asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tm_h)) : "memory");
         asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tm_w)) : "memory");
         for (int s = 0; s < kMaxStages; ++s) { mbar_init(&s_full[s], 1); mbar_init(&s_empty[s], 1); }
-        for (int p = 0; p < 2; ++p) { mbar_init(&s_acc_full[p], 1); mbar_init(&s_acc_empty[p], (PAIR ? 2 : 1) * 4 * PARTS); }
+        for (int p = 0; p < 2; ++p) { mbar_init(&s_acc_full[p], 1); mbar_init(&s_acc_empty[p], (PAIR ? 2 : 1) * 4 * kParts); }
         s_abort = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -382,7 +382,7 @@ k_head_dense(const HeadArgs a, Ctrl* ctrl, float* __restrict__ recs, const Dense
         const int quad = warp & 3;                            // TMEM lanes this warp may read
         const int part = ew >> 2;                             // which share of the tile's chunks
         const int n_ch_tile = bn / kCh;
-        const int ch_lo = part * n_ch_tile / PARTS, ch_hi = (part + 1) * n_ch_tile / PARTS;
+        const int ch_lo = part * n_ch_tile / kParts, ch_hi = (part + 1) * n_ch_tile / kParts;
         const int b = (int)rank * kBM + quad * 32 + lane;
         const bool row_live = b < B;
         griddep_wait();                                       // temp, uniforms and the record scratch belong to earlier work until here
@@ -534,10 +534,10 @@ k_head_dense(const HeadArgs a, Ctrl* ctrl, float* __restrict__ recs, const Dense
 #pragma unroll
             for (int p = 0; p < KT; ++p) { x[(5 + p) * kBM] = st.tv[p]; x[(5 + KT + p) * kBM] = __int_as_float(st.tj[p]); }
         }
-        asm volatile("bar.sync 1, %0;" ::"n"(4 * PARTS * 32) : "memory");
+        asm volatile("bar.sync 1, %0;" ::"n"(4 * kParts * 32) : "memory");
         if (part == 0 && ok && row_live) {
 #pragma unroll 1
-            for (int o = 0; o < PARTS - 1; ++o) {
+            for (int o = 0; o < kParts - 1; ++o) {
                 const float* x = xch + (size_t)o * kXchFields * kBM + slot;
                 lse_merge(st.m, st.s, x[0 * kBM], x[1 * kBM]);
                 const float os = x[2 * kBM];
@@ -670,7 +670,7 @@ DenseGeo make_geo(int32_t K, int32_t d, bool pair, int max_groups) {
     return g;
 }
 
-template <int KT, bool PAIR, int PARTS>
+template <int KT, bool PAIR>
 cudaError_t launch_variant(const HeadArgs& a, Ctrl* ctrl, float* recs, const DenseGeo& geo, const CUtensorMap& tm_h,
                            const CUtensorMap& tm_w, cudaStream_t s) {
     static int attr_done[64] = {0};
@@ -678,14 +678,14 @@ cudaError_t launch_variant(const HeadArgs& a, Ctrl* ctrl, float* recs, const Den
     int dev = 0;
     cudaGetDevice(&dev);
     if (dev < 0 || dev >= 64 || !attr_done[dev]) {
-        cudaError_t e = cudaFuncSetAttribute(k_head_dense<KT, PAIR, PARTS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        cudaError_t e = cudaFuncSetAttribute(k_head_dense<KT, PAIR>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              (int)(kRingBudget + 1024));
         if (e != cudaSuccess) return e;
         if (dev >= 0 && dev < 64) attr_done[dev] = 1;
     }
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)(PAIR ? 2 * geo.n_groups : geo.n_groups));
-    cfg.blockDim = dim3(epi_threads(PARTS));
+    cfg.blockDim = dim3(kThreads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
     cudaLaunchAttribute at[2];
@@ -697,7 +697,7 @@ cudaError_t launch_variant(const HeadArgs& a, Ctrl* ctrl, float* recs, const Den
     at[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
     cfg.numAttrs = a.overlap ? 2 : 1;
-    return cudaLaunchKernelEx(&cfg, k_head_dense<KT, PAIR, PARTS>, a, ctrl, recs, geo, tm_h, tm_w);
+    return cudaLaunchKernelEx(&cfg, k_head_dense<KT, PAIR>, a, ctrl, recs, geo, tm_h, tm_w);
 }
 
 }  // namespace
@@ -714,7 +714,7 @@ size_t head_dense_scratch_bytes(int32_t B, int32_t K, int32_t topk) {
 }
 
 #ifdef VT_STAMPS
-size_t head_dense_stamps_offset(int32_t B, int32_t topk) {
+size_t head_stamps_offset(int32_t B, int32_t topk) {
     return align_up((size_t)kMaxGrid * B * rec_fields(topk) * 4, 256);
 }
 #endif
@@ -732,10 +732,10 @@ cudaError_t launch_head_dense(const HeadArgs& a, Ctrl* ctrl, uint8_t* scratch, c
         return cudaErrorInvalidValue;
     float* recs = reinterpret_cast<float*>(scratch);
     cudaError_t e;
-    if (a.topk <= 8) e = pair ? launch_variant<8, true, kParts8>(a, ctrl, recs, geo, tm_h, tm_w, s)
-                              : launch_variant<8, false, kParts8>(a, ctrl, recs, geo, tm_h, tm_w, s);
-    else e = pair ? launch_variant<kMaxTopk, true, kParts16>(a, ctrl, recs, geo, tm_h, tm_w, s)
-                  : launch_variant<kMaxTopk, false, kParts16>(a, ctrl, recs, geo, tm_h, tm_w, s);
+    if (a.topk <= 8) e = pair ? launch_variant<8, true>(a, ctrl, recs, geo, tm_h, tm_w, s)
+                              : launch_variant<8, false>(a, ctrl, recs, geo, tm_h, tm_w, s);
+    else e = pair ? launch_variant<kMaxTopk, true>(a, ctrl, recs, geo, tm_h, tm_w, s)
+                  : launch_variant<kMaxTopk, false>(a, ctrl, recs, geo, tm_h, tm_w, s);
     if (e != cudaSuccess) return e;
     count_launch();
     return launch_head_merge(a, ctrl, recs, geo.n_groups, s);

@@ -763,12 +763,6 @@ size_t head_skinny_scratch_bytes(int32_t B, int32_t K, int32_t topk) {
     return align_up((size_t)kMaxGrid * B * rec_fields(topk) * 4, 256) + kStampBytes;
 }
 
-#ifdef VT_STAMPS
-size_t head_skinny_stamps_offset(int32_t B, int32_t topk) {
-    return align_up((size_t)kMaxGrid * B * rec_fields(topk) * 4, 256);
-}
-#endif
-
 cudaError_t launch_head_skinny(const HeadArgs& a, Ctrl* ctrl, uint8_t* scratch, cudaStream_t s) {
     if (!head_stream_takes(a.B, a.K, a.d) || a.d < 8 || (a.d & 7)) return cudaErrorInvalidValue;
     int sms = num_sms();

@@ -581,7 +581,9 @@ k_select_sort(const uint32_t* counts, int32_t V, int32_t K, int32_t* map, int32_
         for (int q = 0; q < BPT; ++q) {
             const int b = threadIdx.x * BPT + q;
             const uint32_t sz = (b <= cut && b < first_exact) ? tot[q] : 0u;    // (ids of exact buckets are placed directly)
-            cost[q] = sz * (min(sz, (uint32_t)kCountCap) + kc);                 // (<= 128 K keys in all: the sum fits 32 bits)
+            cost[q] = sz * (min(sz, (uint32_t)kCountCap) + kc);                 // (at most 3072 a key: fits 32 bits while the keys fit the
+                                                                                // CTAs; with more it may wrap, and whatever deal comes of it fails
+                                                                                // the load test below, whose loads add up to all keys)
             csum += cost[q];
         }
         uint32_t cincl = csum;

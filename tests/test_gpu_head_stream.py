@@ -1,5 +1,6 @@
 """The streaming head at the edges of its tiling: 128 vocabulary rows per tile, phases of eight 64-column steps of d,
-ring stages of up to four steps, 8 / 16 / 32 / 64 hidden rows per variant, full and growing candidate lists."""
+ring stages of up to four steps, 8 / 16 / 32 hidden rows per variant (64: over large heads only, tested with those),
+full and growing candidate lists."""
 import pytest
 import torch
 
@@ -15,8 +16,8 @@ SMS = 148                                                # one slab per SM: K = 
 @pytest.mark.parametrize("B,K,d,topk,sample", [
     (8, SMS * 128, 64, 8, True), (1, SMS * 128 + 1, 72, 33, True), (9, SMS * 128 - 1, 512, 64, False),   # tile edges, one phase
     (16, SMS * 256 + 1, 520, 10, True), (2, 7, 576, 7, True), (3, SMS * 8 + 3, 4096, 64, True),          # two phases; tiny slabs
-    (17, 2000, 520, 16, True), (32, SMS * 128 + 1, 448, 1, False), (33, 3001, 1032, 16, True),           # separate merge
-    (64, SMS * 128 + 3, 264, 8, True), (65, 1500, 136, 8, True),                                         # last streaming / first dense row count
+    (17, 2000, 520, 16, True), (32, SMS * 128 + 1, 448, 1, False), (33, 3001, 1032, 16, True),           # last streaming row counts
+    (64, SMS * 128 + 3, 264, 8, True), (65, 1500, 136, 8, True),                                         # and batched ones
 ])
 def test_streaming_head_at_tile_phase_and_variant_edges(B, K, d, topk, sample):
     W = vt_inputs.gaussian_bf16((K, d), 0.05, seed=K + d, device=DEV)
