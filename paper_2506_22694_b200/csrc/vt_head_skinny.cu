@@ -10,7 +10,8 @@
 //
 // so a weight is moved once (TMA into a shared-memory ring, 128-byte swizzle, where the MMA reads it in place)
 // and no register, no shuffle and no partial tile of another warp ever sees it.  Warp 0 feeds the ring (a
-// stage = up to four 64-column steps of the tile's rows and of h), one thread of warp 1 issues the MMAs.
+// stage = up to four 64-column steps of the tile's rows and of h), one thread of warp 1 issues the MMAs (up to eight
+// hidden rows: it and one of the last warp, every other stage each).
 // fp32 accumulation inside the tensor core is a long serial sum, so d is cut into phases of eight steps and a
 // phase's 32 MMAs go to up to eight accumulators in turn (TMEM columns are plentiful); the epilogue adds the
 // accumulators up in fp32 registers, phase by phase, while the next phase's MMAs fill the other set.
@@ -25,9 +26,9 @@
 // out for its 4-6 us (us per chained step, one CTA / second kernel: 1 row of 5000 x 2048 14.8 / 11.7, 10 rows of
 // 32768 x 4096 46.1 / 43.5; one launch more on the host).
 //
-// What bounds it: the HBM read of W_trim (201 MB, cold: 35.7 us per chained step = 0.86 of the measured copy rate;
-// the warp-level MMA kernel before it 38.8) and, for small heads, a fixed chain of about 9 us: h by TMA 0.5, MMAs
-// 25-45 cycles each, epilogue 2, merge and two launch dependencies 5.
+// What bounds it: the HBM read of W_trim (201 MB, cold: 35.0-36.7 us per chained step by box = 0.84-0.88 of the measured
+// copy rate; the warp-level MMA kernel before it 38.3-39.8) and, for small heads, a fixed chain of about 8 us: h by TMA
+// 0.5, two threads' issue of the MMAs (about 45 cycles each), epilogue 2, merge and two launch dependencies 5.
 //
 // Every wait is bounded: on expiry the CTA raises VT_FLAG_TIMEOUT, lets its own copies and MMAs finish and leaves.
 #include <math_constants.h>
