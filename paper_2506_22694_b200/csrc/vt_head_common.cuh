@@ -341,10 +341,16 @@ __device__ __noinline__ void merge_records(const MergeOut a, Ctrl* ctrl, float* 
     for (int sl = 0; sl < 2; ++sl) {
         const int r = lane + 32 * sl;
         okv[sl] = r < topk && row_ok && res_k[sl] != 0ull;
-        const int j = key_idx(res_k[sl]);
-        ids[sl] = okv[sl] ? (a.map ? ld_cg_s32(a.map + j) : j) : -1;
+        ids[sl] = okv[sl] ? key_idx(res_k[sl]) : 0;
         zv[sl] = key_val(res_k[sl]);
     }
+    if (a.map) {                                            // (both loads unconditional: no branch around either)
+        const int i0 = ld_cg_s32(a.map + ids[0]), i1 = ld_cg_s32(a.map + ids[1]);
+        ids[0] = i0;
+        ids[1] = i1;
+    }
+    ids[0] = okv[0] ? ids[0] : -1;
+    ids[1] = okv[1] ? ids[1] : -1;
     asm volatile("bar.sync %0, 64;" ::"r"(bar_id) : "memory");
     const float lse = *xch;
     bool miss = false;

@@ -421,12 +421,12 @@ k_head_dense(const HeadArgs a, Ctrl* ctrl, float* __restrict__ recs, const Dense
                     if (vec_u && j0 + kCh <= K) {
 #pragma unroll
                         for (int i = 0; i < kCh / 4; ++i) {
-                            const float4 q = ld_cg_f4(reinterpret_cast<const float4*>(up) + i);
+                            const float4 q = reinterpret_cast<const float4*>(up)[i];
                             u[4 * i] = q.x; u[4 * i + 1] = q.y; u[4 * i + 2] = q.z; u[4 * i + 3] = q.w;
                         }
                     } else {
 #pragma unroll
-                        for (int i = 0; i < kCh; ++i) u[i] = (j0 + i < K) ? ld_cg_f32(up + i) : 0.5f;
+                        for (int i = 0; i < kCh; ++i) u[i] = (j0 + i < K) ? up[i] : 0.5f;
                     }
                 }
                 const int jn = (ch + 2 < ch_hi) ? j0 + 2 * kCh : jt + geo.n_groups * bn + ch_lo * kCh;

@@ -444,7 +444,7 @@ k_head_stream(const HeadArgs a, Ctrl* ctrl, float* __restrict__ recs, const Geo 
             auto load_u = [&](int b) {
 #pragma unroll
                 for (int i = 0; i < 4; ++i)
-                    un[i] = (a.uniforms && b < B && lane + 32 * i < nrow) ? ld_cg_f32(a.uniforms + (size_t)b * K + j0 + lane + 32 * i) : 0.5f;
+                    un[i] = (a.uniforms && b < B && lane + 32 * i < nrow) ? a.uniforms[(size_t)b * K + j0 + lane + 32 * i] : 0.5f;
             };
             load_u(e);
             // the accumulators of the tile, phase by phase, added up per (vocabulary row = lane, hidden row = column)

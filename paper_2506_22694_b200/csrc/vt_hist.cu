@@ -243,7 +243,8 @@ k_hist_pick(const uint32_t* sample, int32_t V, int32_t H, uint2* __restrict__ ta
 #pragma unroll
             for (int q = 0; q < kPickLoads; ++q) {
                 const int v = v0 + q * kThreads;
-                cs[q] = v < V ? ld_cg_u32(sample + v) : 0xffffffffu;
+                const uint32_t c = ld_cg_u32(sample + min(v, V - 1));       // (no branch around a load)
+                cs[q] = v < V ? c : 0xffffffffu;
             }
 #pragma unroll
             for (int q = 0; q < kPickLoads; ++q) {
@@ -281,7 +282,8 @@ k_hist_pick(const uint32_t* sample, int32_t V, int32_t H, uint2* __restrict__ ta
 #pragma unroll
         for (int q = 0; q < kPickLoads; ++q) {
             const int v = (w0 + q * (kThreads / 32)) * 32 + lane;
-            cs[q] = v < V ? min(ld_cg_u32(sample + v), (uint32_t)(kPickBins - 1)) : 0xffffffffu;
+            const uint32_t c = ld_cg_u32(sample + min(v, V - 1));
+            cs[q] = v < V ? min(c, (uint32_t)(kPickBins - 1)) : 0xffffffffu;
         }
 #pragma unroll
         for (int q = 0; q < kPickLoads; ++q) {

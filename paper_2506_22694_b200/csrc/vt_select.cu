@@ -393,7 +393,7 @@ k_select_sort(const uint32_t* counts, int32_t V, int32_t K, int32_t* map, int32_
     for (int i = w0 + lane; i < w1; i += 32 * kInFlight) {
         uint32_t c[kInFlight];
 #pragma unroll
-        for (int q = 0; q < kInFlight; ++q) c[q] = i + q * 32 < w1 ? ld_cg_u32(counts + i + q * 32) : 0u;
+        for (int q = 0; q < kInFlight; ++q) c[q] = ld_cg_u32(counts + min(i + q * 32, w1 - 1));      // (no branch around a load)
 #pragma unroll
         for (int q = 0; q < kInFlight; ++q)
             if (i + q * 32 < w1) {
@@ -655,7 +655,7 @@ k_select_sort(const uint32_t* counts, int32_t V, int32_t K, int32_t* map, int32_
     for (int i = w0 + lane; i < w1 + lane; i += 32 * kInFlight) {      // (every lane of the warp makes every trip)
         uint32_t c[kInFlight];
 #pragma unroll
-        for (int q = 0; q < kInFlight; ++q) c[q] = i + q * 32 < w1 ? ld_cg_u32(counts + i + q * 32) : 0u;
+        for (int q = 0; q < kInFlight; ++q) c[q] = ld_cg_u32(counts + min(i + q * 32, w1 - 1));      // (no branch around a load)
 #pragma unroll
         for (int q = 0; q < kInFlight; ++q) {
             const int id = i + q * 32;
