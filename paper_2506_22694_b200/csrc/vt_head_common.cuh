@@ -12,8 +12,10 @@ constexpr int kMaxGrid = 160;                    // merge: each lane owns at mos
 constexpr int kMaxOwn = kMaxGrid / 32;
 constexpr int kMergeDepth = 4;                   // list entries per CTA staged on chip by the merge
 constexpr int kSelCap = 128;                     // entries the merge's direct selection can rank
-// staging words (32-bit) per merging warp: staged list heads, selection buffer, output keys (all 64-bit)
-constexpr int kMergeStageWords = 2 * (kMergeDepth * kMaxGrid + kSelCap + 4 + 64);
+// staging words (32-bit) per merging warp: the staged list heads, or before it comes to that the selection buffer and the
+// output keys (all 64-bit)
+constexpr int kMergeStageWords = 2 * kMergeDepth * kMaxGrid;
+static_assert(2 * (kSelCap + 4 + 64) <= kMergeStageWords, "both uses fit");
 constexpr int kStampSlots = 16;                  // phase stamps per CTA (-DVT_STAMPS builds)
 #ifdef VT_STAMPS
 constexpr size_t kStampBytes = (size_t)kMaxGrid * kStampSlots * 8;
@@ -223,7 +225,7 @@ __device__ __noinline__ void merge_records(const MergeOut a, Ctrl* ctrl, float* 
 
     unsigned long long res_k[2] = {0ull, 0ull};
     unsigned long long* stk = reinterpret_cast<unsigned long long*>(stage);        // [kMergeDepth][kMaxGrid] list heads
-    unsigned long long* sel = stk + kMergeDepth * kMaxGrid;                        // [kSelCap]
+    unsigned long long* sel = stk;                                                 // [kSelCap] (in the same place: one or the other)
     unsigned long long* outk = sel + kSelCap + 4;                                  // [64] (behind four words of padding)
     bool done = false;
     if (topk <= 32) {
@@ -294,6 +296,7 @@ __device__ __noinline__ void merge_records(const MergeOut a, Ctrl* ctrl, float* 
         }
     }
     if (!done) {
+        __syncwarp();                                                              // (the selection buffer has been given up)
         // heads of the lists: entry r of CTA c at stk[r * kMaxGrid + c]
 #pragma unroll
         for (int o = 0; o < kMaxOwn; ++o)

@@ -50,7 +50,11 @@ constexpr int kPhase = 8;                        // 64-column steps of d accumul
 constexpr int kSetCols = 128;                    // TMEM columns of an accumulator set (two sets)
 constexpr uint32_t kTmemCols = 2 * kSetCols;     // (half of the SM's: two CTAs of consecutive launches may be resident together)
 constexpr int kMaxB = 64;
-constexpr size_t kSmemLimit = 227 * 1024 - 2048; // opt-in limit minus static shared memory
+// Dynamic shared memory at most: what an SM has less 1 KB per block, the static part and a block of the merge kernel, which
+// has its seat while the next step's CTAs come in.  Where it did not fit beside them, the CTAs of the SMs it sits on
+// started 2-3 us after all others (one row, L2: 5000 x 3072 12.9 -> 11.7 us, 5000
+// x 4096 14.6 -> 13.2).
+constexpr size_t kSmemLimit = 228 * 1024 - (1024 + 512) - (kMergeStageWords * 4 + 1024 + 128);
 constexpr unsigned long long kWaitLimitNs = 2000000000ull;   // default bound of a device-side wait (Ctrl::wait_ns overrides)
 
 // Phase stamps (-DVT_STAMPS builds only): one thread per role writes %globaltimer at fixed points into
@@ -69,12 +73,16 @@ struct Geo {
     int n_tiles;       // tiles per CTA
     int rows;          // vocabulary rows of a tile (rows of one W copy)
     int mma_rows;      // M of the MMA: 64 where a tile has no more rows, else 128
-    int n_kc;          // 64-column steps of d
+    int n_kc;          // 64-column steps of d, rounded up to a multiple of comb
+    int comb;          // steps an MMA takes side by side (see make_geo)
+    int pitch;         // vocabulary rows from one step's W part to the next one's
+    int h_steps;       // steps of h one copy brings: a whole stage's, or one
     int sub;           // steps per ring stage
+    int spp;           // ring stages accumulated in one accumulator set: a phase
     int issuers;       // warps that issue MMAs, stages dealt to them in turn (see make_geo)
     int n_stages;      // ring depth
     int h_bytes;       // shared memory of a step's h part (a multiple of 1024)
-    int step_bytes;    // ... of a step: h part + W part
+    int step_bytes;    // ... of a step: W part + h part; a stage holds its W parts and behind them its h parts
     int ring_bytes;
     int buf_bytes;     // selection buffers of the epilogue warps
     uint32_t keep;     // bit g & 31: the weights of fill g keep their L2 lines
@@ -196,8 +204,8 @@ struct RowState {
 __host__ __device__ constexpr int max_issuers(int ew) { return ew == 8 ? 2 : 1; }
 
 // EW epilogue warps (a multiple of 4: the warps of a lane quadrant share the accumulator columns), at most RPW hidden
-// rows per epilogue warp.
-template <int EW, int RPW>
+// rows per epilogue warp.  COMB: an MMA takes several steps of d side by side (see make_geo).
+template <int EW, int RPW, bool COMB>
 __global__ void __launch_bounds__((EW + 1 + max_issuers(EW)) * 32, EW == 8 ? 2 : 1)
 k_head_stream(const HeadArgs a, Ctrl* ctrl, float* __restrict__ recs, const Geo geo,
               const __grid_constant__ CUtensorMap tm_h, const __grid_constant__ CUtensorMap tm_w) {
@@ -212,6 +220,9 @@ k_head_stream(const HeadArgs a, Ctrl* ctrl, float* __restrict__ recs, const Geo 
     // take kUnits groups of four columns each: always eight loads per warp and phase.
     constexpr int kParts = EW / 4, kUnits = RPW, kAccs = 8 / kUnits, kNpad = 16 * kUnits, kIssuers = max_issuers(EW);
     static_assert(kAccs * kNpad <= kSetCols && kParts * kUnits * 4 <= kNpad, "a set's columns");
+    // Steps side by side: a set holds c_accs accumulators of c_cols columns, kNrow of them per step.
+    constexpr int kNrow = EW;                            // (8 or 16 hidden rows at most)
+    const int c_cols = (geo.comb == 2 ? 2 : 4) * kNrow, c_accs = min(4, kSetCols / c_cols);
     const int B = a.B, K = a.K, topk = a.topk;
     uint8_t* ring = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(s_dyn) + 1023) & ~(uintptr_t)1023);
     const uint32_t ring_u32 = smem_u32(ring);
@@ -272,7 +283,12 @@ k_head_stream(const HeadArgs a, Ctrl* ctrl, float* __restrict__ recs, const Geo 
             const int sub = geo.sub, S = geo.n_stages;
             const int n_ks = (geo.n_kc + sub - 1) / sub;               // ring stages per tile
             const int total = geo.n_tiles * n_ks;
-            const uint32_t step_tx = (uint32_t)(geo.rows + B) * (kBK * 2);      // bytes that land per step
+            // bytes that land: per step, and per stage (h in one copy: all its rows and steps, zeros where there are none)
+            const bool h_whole = RPW == 1 && geo.h_steps > 1;
+            const uint32_t step_tx = (uint32_t)(geo.rows + (h_whole ? 0 : B)) * (kBK * 2);
+            const uint32_t stage_tx = h_whole ? (uint32_t)(geo.h_steps * geo.h_bytes) : 0u;
+            const uint32_t w_step = (uint32_t)geo.pitch * (kBK * 2), h_step = (uint32_t)geo.h_bytes;
+            const uint32_t stage_bytes = (uint32_t)(sub * geo.step_bytes), h_off = (uint32_t)sub * w_step;
             // W_trim is read once per call: its lines are the first to go when L2 needs room, so that the records, the
             // index mapper, h and the uniforms stay resident from step to step -- except for the share of it that a
             // drafting loop finds in L2 again at its next step (see make_geo)
@@ -292,9 +308,9 @@ k_head_stream(const HeadArgs a, Ctrl* ctrl, float* __restrict__ recs, const Geo 
                 int ks = 0, y = r0;
                 for (int g = 0; g < pre; ++g) {
                     const int subs = min(sub, geo.n_kc - ks * sub);
-                    mbar_expect_tx(&s_full[g], step_tx * (uint32_t)subs);
+                    mbar_expect_tx(&s_full[g], stage_tx + step_tx * (uint32_t)subs);
                     for (int u = 0; u < subs; ++u)
-                        load_w(ring_u32 + (uint32_t)((g * sub + u) * geo.step_bytes + geo.h_bytes), (ks * sub + u) * kBK, y, &s_full[g], g);
+                        load_w(ring_u32 + (uint32_t)g * stage_bytes + (uint32_t)u * w_step, (ks * sub + u) * kBK, y, &s_full[g], g);
                     if (++ks == n_ks) { ks = 0; y += geo.rows; }
                 }
             }
@@ -305,9 +321,14 @@ k_head_stream(const HeadArgs a, Ctrl* ctrl, float* __restrict__ recs, const Geo 
             {
                 int ks = 0;
                 for (int g = 0; g < pre; ++g) {
+                    if (h_whole) {
+                        tma_load_3d(ring_u32 + (uint32_t)g * stage_bytes + h_off, &tm_h, 0, 0, ks * sub, &s_full[g]);
+                        if (++ks == n_ks) ks = 0;
+                        continue;
+                    }
                     const int subs = min(sub, geo.n_kc - ks * sub);
                     for (int u = 0; u < subs; ++u)
-                        tma_load_2d(ring_u32 + (uint32_t)((g * sub + u) * geo.step_bytes), &tm_h, (ks * sub + u) * kBK, 0, &s_full[g]);
+                        tma_load_2d(ring_u32 + (uint32_t)g * stage_bytes + h_off + (uint32_t)u * h_step, &tm_h, (ks * sub + u) * kBK, 0, &s_full[g]);
                     if (++ks == n_ks) ks = 0;
                 }
             }
@@ -319,14 +340,15 @@ k_head_stream(const HeadArgs a, Ctrl* ctrl, float* __restrict__ recs, const Geo 
                 for (int g = pre; g < total; ++g, ++done) {
                     if (!mbar_wait(&s_empty[sc], par, abort_flag, &s_bound)) break;
                     const int subs = min(sub, geo.n_kc - ks * sub);
-                    mbar_expect_tx(&s_full[sc], step_tx * (uint32_t)subs);
-                    const uint32_t dst0 = ring_u32 + (uint32_t)(sc * sub * geo.step_bytes);
+                    mbar_expect_tx(&s_full[sc], stage_tx + step_tx * (uint32_t)subs);
+                    const uint32_t dst0 = ring_u32 + (uint32_t)sc * stage_bytes;
+                    if (h_whole) tma_load_3d(dst0 + h_off, &tm_h, 0, 0, ks * sub, &s_full[sc]);
 #pragma unroll
                     for (int u = 0; u < kMaxSub; ++u) {
                         if (u < subs) {
                             const int x = (ks * sub + u) * kBK;
-                            load_w(dst0 + (uint32_t)(u * geo.step_bytes + geo.h_bytes), x, y, &s_full[sc], g);
-                            tma_load_2d(dst0 + (uint32_t)(u * geo.step_bytes), &tm_h, x, 0, &s_full[sc]);
+                            load_w(dst0 + (uint32_t)u * w_step, x, y, &s_full[sc], g);
+                            if (!h_whole) tma_load_2d(dst0 + h_off + (uint32_t)u * h_step, &tm_h, x, 0, &s_full[sc]);
                         }
                     }
                     if (++sc == S) { sc = 0; par ^= 1u; }
@@ -342,20 +364,21 @@ k_head_stream(const HeadArgs a, Ctrl* ctrl, float* __restrict__ recs, const Geo 
         // ================= MMA issuers =================================================================
         const int me = warp == 1 ? 0 : 1, ni = geo.issuers;
         if (me < ni && elect_one()) {
-            const uint32_t idesc = make_idesc(geo.mma_rows, kNpad);
+            const int comb = geo.comb;
+            const uint32_t idesc = make_idesc(geo.mma_rows, COMB ? c_cols : kNpad);
             // (the ring is 1024-byte aligned and under 256 KB: adding byte offsets >> 4 stays inside the address field;
             // rows of an operand beyond the tile's / beyond B are whatever lies behind it: their TMEM lanes and columns
             // are not looked at)
             const uint64_t desc_h0 = make_desc(ring_u32);
             const uint32_t desc_lo = (uint32_t)desc_h0, desc_hi = (uint32_t)(desc_h0 >> 32);
-            const uint32_t w_off = (uint32_t)(geo.h_bytes >> 4), d_step = (uint32_t)(geo.step_bytes >> 4);
+            const uint32_t w16 = (uint32_t)geo.pitch * (kBK * 2 / 16), h16 = (uint32_t)(geo.h_bytes >> 4);      // operand steps >> 4
             const int S = geo.n_stages, sub = geo.sub;
-            const int n_ks = (geo.n_kc + sub - 1) / sub, spp = kPhase / sub;       // ring stages per tile / per phase
+            const int n_ks = (geo.n_kc + sub - 1) / sub, spp = geo.spp;            // ring stages per tile / per phase
             const int total = geo.n_tiles * n_ks;
             // Every MMA of a stage: consecutive ones go to this issuer's N accumulators (from column d on) in turn, the first
             // round of a phase overwrites.  in_phase: this issuer's steps in the phase so far.  Accumulators and flags are
             // constants of the unrolled code (an odd step swaps the halves of eight accumulators).
-            auto issue = [&](auto accs, uint32_t d, uint32_t lo, int subs, int in_phase) {
+            auto issue = [&](auto accs, uint32_t d, uint32_t w_lo, uint32_t h_lo, int subs, int in_phase) {
                 constexpr int N = decltype(accs)::value;
                 const uint32_t odd = N > 4 ? (uint32_t)(in_phase & 1) * (4 * kNpad) : 0u;
                 const uint32_t d_even = d + odd, d_odd = N > 4 ? d + 4 * kNpad - odd : d;
@@ -365,12 +388,29 @@ k_head_stream(const HeadArgs a, Ctrl* ctrl, float* __restrict__ recs, const Geo 
                         if (u < subs) {
 #pragma unroll
                             for (int k = 0; k < kBK / 16; ++k)
-                                tc_mma_lo(((u & 1) ? d_odd : d_even) + (uint32_t)((k % N) * kNpad), lo + (uint32_t)u * d_step + w_off + (uint32_t)(2 * k),
-                                          lo + (uint32_t)u * d_step + (uint32_t)(2 * k), desc_hi, idesc,
+                                tc_mma_lo(((u & 1) ? d_odd : d_even) + (uint32_t)((k % N) * kNpad), w_lo + (uint32_t)u * w16 + (uint32_t)(2 * k),
+                                          h_lo + (uint32_t)u * h16 + (uint32_t)(2 * k), desc_hi, idesc,
                                           (decltype(later)::value || u * (kBK / 16) + k >= N) ? 1u : 0u);
                         }
                 };
                 if (in_phase * (kBK / 16) >= N) steps(std::true_type{}); else steps(std::false_type{});
+            };
+            // The same with `comb` steps side by side: an MMA's vocabulary rows are those of `comb` W parts, its columns those
+            // of as many h parts, and of the product only the blocks on the diagonal are looked at.
+            const int my_accs = c_accs / ni;
+            auto issue_comb = [&](uint32_t d, uint32_t w_lo, uint32_t h_lo, int subs, int in_phase) {
+                d += (uint32_t)(me * my_accs * c_cols);
+#pragma unroll
+                for (int g = 0; g < kMaxSub / 2; ++g) {
+                    if (g * comb < subs) {
+#pragma unroll
+                        for (int k = 0; k < kBK / 16; ++k)
+                            tc_mma_lo(d + (uint32_t)((k & (my_accs - 1)) * c_cols), w_lo + (uint32_t)(2 * k), h_lo + (uint32_t)(2 * k), desc_hi, idesc,
+                                      in_phase + g > 0 || k >= my_accs ? 1u : 0u);
+                        w_lo += (uint32_t)comb * w16;
+                        h_lo += (uint32_t)comb * h16;
+                    }
+                }
             };
             // (no griddep_wait here: h is asked for after it, so no stage is complete before; waking up from it costs 0.3 us
             // that a probe on the stage does not)
@@ -394,11 +434,13 @@ k_head_stream(const HeadArgs a, Ctrl* ctrl, float* __restrict__ recs, const Geo 
 #endif
                         tc_fence_after();
                         const int subs = min(sub, geo.n_kc - (ks0 + own - first) * sub);
-                        const uint32_t lo = desc_lo + ((uint32_t)(s * sub * geo.step_bytes) >> 4);
-                        if (kIssuers == 2 && ni == 2)
-                            issue(std::integral_constant<int, kAccs / 2>{}, d_tmem + (uint32_t)(me * (kAccs / 2) * kNpad), lo, subs, in_phase);
+                        const uint32_t w_lo = desc_lo + ((uint32_t)(s * sub * geo.step_bytes) >> 4), h_lo = w_lo + (uint32_t)sub * w16;
+                        if (COMB)
+                            issue_comb(d_tmem, w_lo, h_lo, subs, in_phase);
+                        else if (kIssuers == 2 && ni == 2)
+                            issue(std::integral_constant<int, kAccs / 2>{}, d_tmem + (uint32_t)(me * (kAccs / 2) * kNpad), w_lo, h_lo, subs, in_phase);
                         else
-                            issue(std::integral_constant<int, kAccs>{}, d_tmem, lo, subs, in_phase);
+                            issue(std::integral_constant<int, kAccs>{}, d_tmem, w_lo, h_lo, subs, in_phase);
                         in_phase += subs;
                         tc_commit(&s_empty[s]);                     // the stage is free once these MMAs have read it
                         s += ni;
@@ -434,8 +476,12 @@ k_head_stream(const HeadArgs a, Ctrl* ctrl, float* __restrict__ recs, const Geo 
             if (lane == 0) s_invT[b] = (T > 0.f) && (T < CUDART_INF_F) ? 1.f / T : CUDART_NAN_F;
         }
         __syncwarp();
-        const int n_ph = (geo.n_kc + kPhase - 1) / kPhase;
-        const int n_ks = (geo.n_kc + geo.sub - 1) / geo.sub, spp = kPhase / geo.sub;     // ring stages per tile / per phase
+        const int n_ks = (geo.n_kc + geo.sub - 1) / geo.sub, spp = geo.spp;     // ring stages per tile / per phase
+        const int n_ph = (n_ks + spp - 1) / spp;
+        // steps side by side: this warp's TMEM lanes belong to one step's rows or to two's
+        const int comb = COMB ? geo.comb : 1;
+        const int step_a = COMB ? quad * 32 / geo.pitch : 0, step_b = COMB ? min((quad * 32 + 31) / geo.pitch, comb - 1) : 0;
+        const bool in_b = quad * 32 + lane >= step_b * geo.pitch;
         int set_no = 0;
         for (int t = 0; t < geo.n_tiles; ++t) {
             const int j0 = r0 + t * geo.rows;                       // first vocabulary row of the tile
@@ -459,7 +505,26 @@ k_head_stream(const HeadArgs a, Ctrl* ctrl, float* __restrict__ recs, const Geo 
                 ok = mbar_wait_warp(&s_acc_full[set], (uint32_t)((set_no >> 1) & 1), abort_flag, &s_bound);
                 if (!ok) break;
                 tc_fence_after();
-                if (quad * qrows < nrow && part * 4 < B) {
+                if (COMB) {
+                    if (quad * 32 < comb * geo.pitch && part * 4 < B) {
+                        const uint32_t base = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(set * kSetCols + part * 4);
+                        uint32_t ad[8];
+                        float v[8][4];
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) ad[i] = base + (uint32_t)((i & (c_accs - 1)) * c_cols + (i < 4 ? step_a : step_b) * kNrow);
+                        tc_ld_8x4(ad, v);
+                        // (a short last phase of one stage: the other issuer's accumulators hold nothing)
+                        const bool one = kIssuers == 2 && geo.issuers == 2 && n_ks - p * spp == 1;
+                        const int c0 = one && ((p * spp) & 1) ? c_accs / 2 : 0, c1 = one ? c0 + c_accs / 2 : c_accs;
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) {
+                            float w[4];
+#pragma unroll
+                            for (int c = 0; c < 4; ++c) w[c] = c >= c0 && c < c1 ? (in_b ? v[4 + c][q] : v[c][q]) : 0.f;
+                            x[0][q] += (w[0] + w[2]) + (w[1] + w[3]);
+                        }
+                    }
+                } else if (quad * qrows < nrow && part * 4 < B) {
                     const uint32_t base = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(set * kSetCols + part * 4);
                     uint32_t ad[8];
                     float v[8][4];
@@ -497,7 +562,7 @@ k_head_stream(const HeadArgs a, Ctrl* ctrl, float* __restrict__ recs, const Geo 
 #ifdef VT_STAMPS
                 if (e == 0 && lane == 0) VT_STAMP(4);
 #endif
-                if (quad * qrows < nrow && lane < qrows) {
+                if (COMB ? quad * 32 < comb * geo.pitch : quad * qrows < nrow && lane < qrows) {
 #pragma unroll
                     for (int i = 0; i < kUnits; ++i)
 #pragma unroll
@@ -531,7 +596,14 @@ k_head_stream(const HeadArgs a, Ctrl* ctrl, float* __restrict__ recs, const Geo 
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
                     const bool valid = lane + 32 * i < nrow;
-                    const float x1 = valid ? zt[(size_t)b * kBM + lane + 32 * i] : 0.f;
+                    float x1 = valid ? zt[(size_t)b * kBM + lane + 32 * i] : 0.f;
+                    if (COMB && i < 2) {                            // the logit's parts of the steps that lay side by side (tiles of up to 64 rows)
+                        const float* zc = zt + (size_t)b * kBM + lane + 32 * i;
+                        const float p1 = valid ? zc[geo.pitch] : 0.f;
+                        const float p2 = valid && comb > 2 ? zc[2 * geo.pitch] : 0.f;
+                        const float p3 = valid && comb > 3 ? zc[3 * geo.pitch] : 0.f;
+                        x1 = (x1 + p1) + (p2 + p3);
+                    }
                     if (a.dbg_logits && valid) a.dbg_logits[(size_t)b * K + j0 + lane + 32 * i] = x1;
                     z[i] = valid ? x1 * invT : -CUDART_INF_F;
                 }
@@ -678,27 +750,48 @@ Geo make_geo(int B, int K, int d, int topk, int sms, size_t* smem_bytes) {
     const int slab = (K + g.grid - 1) / g.grid;
     g.n_tiles = (slab + kBM - 1) / kBM;
     g.rows = (slab + g.n_tiles - 1) / g.n_tiles;
-    // (M = 64 and N = 16: 25 cycles per MMA instead of 40 -- a part of what a step of a small head waits for)
-    g.mma_rows = g.rows <= 64 ? 64 : kBM;
     g.n_kc = (d + kBK - 1) / kBK;
     g.h_bytes = (int)align_up((size_t)B * kBK * 2, 1024);
-    const int w_bytes = (int)align_up((size_t)g.rows * kBK * 2, 1024);
-    g.step_bytes = g.h_bytes + w_bytes;
     const int ew = B <= 8 ? 8 : 16;
+    // Tiles of up to 64 rows and up to 16 hidden rows: an MMA takes about 40 cycles whatever its size, so two to four steps
+    // of d go into one, side by side: vocabulary rows [c * pitch, (c + 1) * pitch) are those of step c, columns [c * 8 or 16,
+    // ...) its hidden rows, and the blocks of the product where both are of the same step are its result.  The rest is
+    // computed for nothing; steps beyond d are copies of zeros.  (One row, L2, two issuers
+    // without / with: 3000 x 2048 9.8 / 8.3 us, 3000 x 4096 12.6 / 9.9, 5000 x 3072 11.7 / 10.2, 8000 x 4096 13.5 / 12.6; 9 rows of
+    // 5000 x 3072 17.1 / 15.2, 16 rows 15.9 / 15.8; the warp-level kernel before took 8.4, 11.0, 12.6, 15.4; 16.8, 21.1.)
+    g.comb = 1;
+    g.pitch = (int)align_up((size_t)g.rows, 8);
+    if (B <= 16 && g.rows <= 64 && g.n_kc > 1) {
+        if (g.pitch < 16) g.pitch = 16;                                    // (a TMEM quadrant then holds rows of two steps at most)
+        g.comb = kBM / g.pitch < 4 ? kBM / g.pitch : 4;
+        if (g.comb > g.n_kc) g.comb = g.n_kc;
+        g.n_kc = (g.n_kc + g.comb - 1) / g.comb * g.comb;
+    }
+    g.mma_rows = g.comb == 1 && g.rows <= 64 ? 64 : kBM;
+    const int w_bytes = g.pitch * kBK * 2;
+    g.step_bytes = g.h_bytes + w_bytes;
     g.buf_bytes = (B < ew ? B : ew) * kBufKeys * 8;
     const size_t fixed = (size_t)B * kBM * 4 + align_up((size_t)B * topk * 8, 16) + (size_t)g.buf_bytes + (size_t)B * (32 * sizeof(RowState) + 8);
-    const size_t over = (size_t)g.mma_rows * kBK * 2 - (size_t)w_bytes;   // the MMA reads that many rows from the start of a W part
-    const size_t tail = fixed > over ? fixed : over;
+    // the MMA reads mma_rows rows from the start of a W part: what may lie beyond the ring's end
+    const long over = (long)g.mma_rows * kBK * 2 - (long)g.comb * g.step_bytes;
+    const size_t tail = (long)fixed > over ? fixed : (size_t)over;
     const size_t room = kSmemLimit - 1024 - tail;
     // Four steps to a stage where three such stages fit: the two threads that drive the ring wait and release once
     // per stage (201 MB cold through the bare ring: 34.9 us with one step, 33.3 with two, 32.8 with four).
-    g.sub = kMaxSub;
-    while (g.sub > 1 && (g.sub > g.n_kc || (size_t)3 * g.sub * g.step_bytes > room)) g.sub >>= 1;
+    g.sub = kMaxSub / g.comb * g.comb;
+    while (g.sub > g.comb && (g.sub > g.n_kc || (size_t)3 * g.sub * g.step_bytes > room)) g.sub >>= 1;
+    // h of a stage in one copy where its rows end on a step: the producer spends 50 ns on every copy it asks for
+    g.h_steps = B <= 16 && d % kBK == 0 ? g.sub : 1;
     const size_t stage = (size_t)g.sub * g.step_bytes;
     const long total = (long)g.n_tiles * ((g.n_kc + g.sub - 1) / g.sub);
     g.n_stages = (int)(room / stage);
     if (g.n_stages > kMaxStages) g.n_stages = kMaxStages;
     if (g.n_stages > total) g.n_stages = (int)total;
+    // A phase: eight steps, up to four MMAs in a row per accumulator.  Steps side by side need half the accumulations where
+    // there are three or four of them and two issuers; there a phase may be twice as long, and it pays: reading a set takes the
+    // epilogue as long as the MMAs of four stages.
+    g.spp = kPhase / g.sub;
+    if (g.comb >= 3 && ew == 8 && (g.n_stages >= total || g.n_stages >= 4 * g.spp)) g.spp *= 2;
     // A single thread needs 250-300 cycles per 64-column step for its waits, releases and four MMAs, which a small head waits
     // for from the moment h has landed; two threads take every other stage each (one row, L2, one / two issuers: 3000 x
     // 1024 8.8 / 7.9 us, 5000 x 3072 15.0 / 12.9, 8000 x 4096 16.4 / 13.1, 20001 x 3072 22.4 / 20.3).  An issuer that is ahead must not take
@@ -706,7 +799,7 @@ Geo make_geo(int B, int K, int d, int topk, int sms, size_t* smem_bytes) {
     // a stage ahead (an accumulator set is read before its next use), so the ring has to be longer than that, or never
     // reused, or even (a stage then always has the same issuer).  A large head's ring of three stages is none of these; there
     // the copies are what is waited for (three stages of four steps, one issuer / six of two, two issuers: 788 MB 114.4 / 116.5).
-    g.issuers = max_issuers(ew) == 2 && (g.n_stages >= total || (g.n_stages & 1) == 0 || g.n_stages >= 2 * kPhase / g.sub) ? 2 : 1;
+    g.issuers = max_issuers(ew) == 2 && (g.n_stages >= total || (g.n_stages & 1) == 0 || g.n_stages >= 2 * g.spp) ? 2 : 1;
     g.ring_bytes = (int)(g.n_stages * stage);
     // A drafting loop reads the same head again a few tens of microseconds later.  A head that is larger than L2
     // leaves nothing behind when all of it streams through under one policy; so 56 MB of it, spread evenly over
@@ -722,14 +815,14 @@ Geo make_geo(int B, int K, int d, int topk, int sms, size_t* smem_bytes) {
     return g;
 }
 
-template <int EW, int RPW>
+template <int EW, int RPW, bool COMB>
 cudaError_t launch_variant(const HeadArgs& a, Ctrl* ctrl, float* recs, const Geo& geo, const CUtensorMap& tm_h,
                            const CUtensorMap& tm_w, size_t smem, cudaStream_t s) {
     static int attr_done[64] = {0};
     int dev = 0;
     cudaGetDevice(&dev);
     if (dev < 0 || dev >= 64 || !attr_done[dev]) {
-        cudaError_t e = cudaFuncSetAttribute(k_head_stream<EW, RPW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemLimit);
+        cudaError_t e = cudaFuncSetAttribute(k_head_stream<EW, RPW, COMB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemLimit);
         if (e != cudaSuccess) return e;
         if (dev >= 0 && dev < 64) attr_done[dev] = 1;
     }
@@ -744,7 +837,7 @@ cudaError_t launch_variant(const HeadArgs& a, Ctrl* ctrl, float* recs, const Geo
     cfg.attrs = &attr;
     cfg.numAttrs = a.overlap ? 1 : 0;
     count_launch();
-    return cudaLaunchKernelEx(&cfg, k_head_stream<EW, RPW>, a, ctrl, recs, geo, tm_h, tm_w);
+    return cudaLaunchKernelEx(&cfg, k_head_stream<EW, RPW, COMB>, a, ctrl, recs, geo, tm_h, tm_w);
 }
 
 }  // namespace
@@ -772,12 +865,16 @@ cudaError_t launch_head_skinny(const HeadArgs& a, Ctrl* ctrl, uint8_t* scratch, 
     const Geo geo = make_geo(a.B, a.K, a.d, a.topk, sms, &smem);
     if (geo.n_stages < 1 || smem > kSmemLimit) return cudaErrorInvalidValue;
     CUtensorMap tm_h, tm_w;
-    if (!encode_map(&tm_h, a.h, a.B, a.d, a.B) || !encode_map(&tm_w, a.W, a.K, a.d, geo.rows)) return cudaErrorInvalidValue;
+    const int box_h = geo.h_steps > 1 ? geo.h_bytes / (kBK * 2) : a.B;
+    if (!encode_map(&tm_h, a.h, a.B, a.d, box_h, geo.h_steps > 1 ? geo.h_steps : 0) || !encode_map(&tm_w, a.W, a.K, a.d, geo.rows)) return cudaErrorInvalidValue;
     float* recs = reinterpret_cast<float*>(scratch);
-    const cudaError_t e = a.B <= 8 ? launch_variant<8, 1>(a, ctrl, recs, geo, tm_h, tm_w, smem, s)
-                        : a.B <= 16 ? launch_variant<16, 1>(a, ctrl, recs, geo, tm_h, tm_w, smem, s)
-                        : a.B <= 32 ? launch_variant<16, 2>(a, ctrl, recs, geo, tm_h, tm_w, smem, s)
-                                    : launch_variant<16, 4>(a, ctrl, recs, geo, tm_h, tm_w, smem, s);
+    const bool comb = geo.comb > 1;
+    const cudaError_t e = a.B <= 8 ? (comb ? launch_variant<8, 1, true>(a, ctrl, recs, geo, tm_h, tm_w, smem, s)
+                                           : launch_variant<8, 1, false>(a, ctrl, recs, geo, tm_h, tm_w, smem, s))
+                        : a.B <= 16 ? (comb ? launch_variant<16, 1, true>(a, ctrl, recs, geo, tm_h, tm_w, smem, s)
+                                            : launch_variant<16, 1, false>(a, ctrl, recs, geo, tm_h, tm_w, smem, s))
+                        : a.B <= 32 ? launch_variant<16, 2, false>(a, ctrl, recs, geo, tm_h, tm_w, smem, s)
+                                    : launch_variant<16, 4, false>(a, ctrl, recs, geo, tm_h, tm_w, smem, s);
     if (e != cudaSuccess) return e;
     return launch_head_merge(a, ctrl, recs, geo.grid, s);
 }

@@ -48,6 +48,11 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* tm,
         "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
         ::"r"(dst), "l"(tm), "r"(x), "r"(y), "r"(smem_u32(bar)) : "memory");
 }
+__device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* tm, int x, int y, int z, uint64_t* bar) {
+    asm volatile(
+        "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];"
+        ::"r"(dst), "l"(tm), "r"(x), "r"(y), "r"(z), "r"(smem_u32(bar)) : "memory");
+}
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_commit(uint64_t* bar) {
@@ -112,12 +117,13 @@ const MapFns& map_fns() {
     return fns;
 }
 
-// bf16 matrix [rows, cols] row-major -> boxes of kBK columns x box_rows rows, 128-byte swizzle.  Encoding a map
+// bf16 matrix [rows, cols] row-major -> boxes of kBK columns x box_rows rows, 128-byte swizzle; with steps > 0 boxes of
+// `steps` of those behind one another, as a third dimension (cols a multiple of kBK).  Encoding a map
 // takes the host about 2.5 us, two of them 5 of a call's 12; the last few shapes of a thread are kept encoded (a
 // shape, not a matrix: the address is put in on every call, which costs a tenth of that).
-bool encode_map(CUtensorMap* tm, const void* base, int rows, int cols, int box_rows) {
+bool encode_map(CUtensorMap* tm, const void* base, int rows, int cols, int box_rows, int steps = 0) {
     struct Shape {
-        int rows, cols, box_rows;
+        int rows, cols, box_rows, steps;
         CUtensorMap map;
     };
     constexpr int kShapes = 8;
@@ -126,19 +132,19 @@ bool encode_map(CUtensorMap* tm, const void* base, int rows, int cols, int box_r
     const MapFns& fn = map_fns();
     if (!fn.encode) return false;
     for (int i = 0; i < kShapes; ++i)
-        if (kept[i].rows == rows && kept[i].cols == cols && kept[i].box_rows == box_rows) {
+        if (kept[i].rows == rows && kept[i].cols == cols && kept[i].box_rows == box_rows && kept[i].steps == steps) {
             *tm = kept[i].map;
             return fn.replace(tm, const_cast<void*>(base)) == CUDA_SUCCESS;
         }
-    cuuint64_t gdim[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
-    cuuint64_t gstr[1] = {(cuuint64_t)cols * 2};
-    cuuint32_t box[2] = {(cuuint32_t)kBK, (cuuint32_t)box_rows};
-    cuuint32_t estr[2] = {1, 1};
-    if (fn.encode(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), gdim, gstr, box, estr,
+    cuuint64_t gdim[3] = {(cuuint64_t)(steps ? kBK : cols), (cuuint64_t)rows, (cuuint64_t)(cols / kBK)};
+    cuuint64_t gstr[2] = {(cuuint64_t)cols * 2, (cuuint64_t)kBK * 2};
+    cuuint32_t box[3] = {(cuuint32_t)kBK, (cuuint32_t)box_rows, (cuuint32_t)steps};
+    cuuint32_t estr[3] = {1, 1, 1};
+    if (fn.encode(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, steps ? 3 : 2, const_cast<void*>(base), gdim, gstr, box, estr,
                   CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
         return false;
-    kept[next] = Shape{rows, cols, box_rows, *tm};
+    kept[next] = Shape{rows, cols, box_rows, steps, *tm};
     next = (next + 1) % kShapes;
     return true;
 }
