@@ -293,9 +293,9 @@ vt_status vt_draft_head_overlapped(const uint16_t *h, const uint16_t *W_trim, co
 /*
  * One tree depth in one call: vt_draft_head_overlapped followed by vt_tree_expand on its candidates
  * (out_ids / out_logprobs columns 1..topk), with the same arguments, results and limits as those two
- * (Algorithm 2, the drafter-forward and index-mapping steps with the draft tree of Section 4.1).  Over a
- * head of up to 128 MB the expansion runs inside the merge kernel, in the block that finishes last;
- * otherwise it is a kernel behind the merge.  The caller's
+ * (Algorithm 2, the drafter-forward and index-mapping steps with the draft tree of Section 4.1).  Up to
+ * 64 new nodes (B * topk) are expanded inside the merge kernel, in the block that finishes last;
+ * for more there is a kernel behind the merge.  The caller's
  * promise about W_trim is that of vt_draft_head_overlapped.
  */
 vt_status vt_draft_head_expand(const uint16_t *h, const uint16_t *W_trim, const int32_t *map, int32_t B,

@@ -600,8 +600,7 @@ k_head_dense(const HeadArgs a, Ctrl* ctrl, float* __restrict__ recs, const Dense
 // the block that finishes last turns the merged candidates into pool nodes and chooses the next frontier, so that
 // a tree depth needs no launch for it.  (Dynamic shared memory, sized by the need: the block has to fit beside the
 // head kernel's CTA to take its seat early.)
-constexpr size_t kFuseBytes = 128u << 20;                          // heads up to this size (see launch_head_merge)
-constexpr int kFuseNodes = 512;                                   // new nodes the 64 threads of a block rank (else a kernel of 1024 threads)
+constexpr int kFuseNodes = 64;                                    // new nodes that a block of 64 threads expands (see launch_head_merge)
 __global__ void __launch_bounds__(64)
 k_head_merge(const HeadArgs a, Ctrl* ctrl, float* __restrict__ recs, int G, int fuse) {
     extern __shared__ __align__(16) float s_stage[];              // [kMergeStageWords], and over it the keys of the expansion
@@ -745,10 +744,10 @@ cudaError_t launch_head_dense(const HeadArgs& a, Ctrl* ctrl, uint8_t* scratch, c
 cudaError_t launch_head_merge(const HeadArgs& a, Ctrl* ctrl, float* recs, int G, cudaStream_t s) {
     // the merge always follows its own producer closely: it takes its seats early and waits on the device
     const int n_new = a.B * a.topk;
-    // The expansion inside the merge saves a launch, as a kernel of its own (sixteen times the threads, launched ahead as a
-    // dependent) it is 1-2 us shorter: a depth over a small head is bound by its launches (depth-3 tree over 61 MB: 77
-    // with the kernel, 70 fused), over a large one by the device (six depths over 268 MB: 306 / 317).
-    const bool fuse = a.tree.pool_token && n_new <= kFuseNodes && (size_t)a.K * a.d * 2 <= kFuseBytes;
+    // The expansion inside the merge saves a launch; as a kernel of its own it has sixteen times the threads.  What decides is
+    // one node per thread (us per depth, fused / kernel, heads of 60, 128, 268 MB: 8 nodes 15.1 / 16.1, 23.3 / 24.0, 41.9 / 42.3; 64
+    // nodes 15.5 / 17.2, 23.8 / 24.8, 42.6 / 43.0; 100 nodes 20.7 / 20.7, 27.8 / 26.3, 46.0 / 44.7; 512 nodes 43.5 / 28.3, 49.3 / 34.8, 70.4 / 55.7).
+    const bool fuse = a.tree.pool_token && n_new <= kFuseNodes;
     size_t smem = (size_t)kMergeStageWords * 4;
     if (fuse && (size_t)padded_keys(n_new) * 8 > smem) smem = (size_t)padded_keys(n_new) * 8;
     const cudaError_t e = launch_dependent(k_head_merge, (unsigned)a.B, 64, smem, s, a, ctrl, recs, G, fuse ? 1 : 0);

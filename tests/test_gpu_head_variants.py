@@ -54,8 +54,8 @@ def test_many_rows_over_large_heads(B, d, mb, extra, topk, sample):
 
 
 @pytest.mark.parametrize("B,K,d,topk,depths", [
-    (8, 33_001, 2048, 8, 4),                             # over 128 MB: a kernel behind the merge, the next depth's head behind that
-    (64, 3000, 256, 8, 2), (57, 3000, 256, 9, 2), (64, 2000, 264, 16, 2),     # 512, 513 and 1024 new nodes
+    (8, 33_001, 2048, 8, 4), (13, 33_001, 2048, 5, 4),   # 64 new nodes: in the merge; 65: a kernel behind it, the next depth's head behind that
+    (64, 3000, 256, 8, 2), (57, 3000, 256, 9, 2), (64, 2000, 264, 16, 2),     # 512, 513 and 1024 of them
 ])
 def test_expansion_behind_the_merge_equals_head_then_expansion(B, K, d, topk, depths):
     """Depths back to back, nothing in between: ids, log-probabilities, pool and frontier are those of the two calls."""

@@ -143,7 +143,7 @@ def test_head_to_tree_to_verification_on_the_trimmed_vocabulary():
 @pytest.mark.parametrize("K,d,topk,n_front,depth,sample", [(4096, 512, 8, 8, 3, False), (3000, 1024, 10, 10, 4, True),
                                                             (700, 72, 4, 6, 3, True), (2048, 256, 16, 16, 2, False)])
 def test_head_with_fused_expansion_equals_head_then_expansion(K, d, topk, n_front, depth, sample):
-    """vt_draft_head_expand (the expansion in the merge's last block) against vt_draft_head
+    """vt_draft_head_expand (one call per depth) against vt_draft_head
     followed by vt_tree_expand: same ids, log-probs, pool and frontier, bit for bit; the pool is also what
     the oracle's expansion makes of those candidates."""
     W = vt_inputs.gaussian_bf16((K, d), 0.05, seed=K + 1, device=DEV)
@@ -176,7 +176,7 @@ def test_head_with_fused_expansion_equals_head_then_expansion(K, d, topk, n_fron
 
 
 def test_fused_expansion_on_the_dense_path_and_argument_checks():
-    K, d, topk, B = 1500, 128, 8, 40                         # more rows than a tree's depth has: batched kernel, fused expansion
+    K, d, topk, B = 1500, 128, 8, 40                         # more rows than a tree's depth has: batched kernel, expansion behind the merge
     W = vt_inputs.gaussian_bf16((K, d), 0.05, seed=3, device=DEV)
     h = vt_inputs.gaussian_bf16((B, d), 1.0, seed=4, device=DEV)
     T = torch.ones(B, device=DEV)
