@@ -26,6 +26,8 @@
 // record goes to scratch; a second small kernel (two warps per hidden row) merges the records,
 // applies the index mapper and writes the outputs.  Every wait is bounded; on expiry the CTA raises
 // VT_FLAG_TIMEOUT and leaves after releasing its tensor memory.
+#include <cfloat>
+
 #include "vt_common.cuh"
 #include "vt_head_common.cuh"
 #include "vt_tc.cuh"
@@ -39,15 +41,11 @@ constexpr int kBM = 128;                  // hidden rows per CTA (TMEM lanes)
 constexpr int kMaxBN = 256;               // vocabulary rows per tile at most (TMEM columns per accumulator)
 constexpr int kMaxSub = 2;                // d-steps of kBK columns one ring stage holds at most
 constexpr int kMaxStages = 8;
-constexpr int kHTileBytes = kBM * kBK * 2; // 16 KB: the hidden-row operand of a stage
-constexpr int kParts = 2;                  // epilogue warps per TMEM lane quadrant (3 and 4 were no
-                                          // faster: the epilogue is bound by the instructions it issues, not by latency)
-constexpr int kThreads = (2 + 4 * kParts) * 32;   // TMA producer, MMA issuer, epilogue warps
 constexpr int kCh = 16;                   // accumulator columns per epilogue step (keeps the row state in registers)
 constexpr int kTmemCols = 512;            // 2 accumulator stages x kMaxBN columns
-constexpr int kMaxTopk = 16;              // top-k list lives in registers
+constexpr int kMaxTopk = 16;              // the list's values live in registers
 constexpr unsigned long long kWaitLimitNs = 2000000000ull;
-constexpr size_t kRingBudget = 225 * 1024;   // ring bytes at most (227 KB per CTA less alignment slack and statics)
+constexpr size_t kSmemBudget = 225 * 1024;   // ring and candidate entries at most (227 KB per CTA less alignment slack and statics)
 
 // Phase stamps (-DVT_STAMPS builds only): one thread per role writes %globaltimer into a region behind the
 // records; bench.py --case stamps reads them back.  Slots per CTA: 0 entry, 1 set up (barriers, tensor
@@ -92,14 +90,23 @@ __device__ __forceinline__ bool mbar_wait_warp(uint64_t* b, uint32_t parity, vol
     if (ok) ok = mbar_try(b, parity) || mbar_wait(b, parity, abort_flag);
     return __all_sync(0xffffffffu, ok);
 }
-// 16 consecutive accumulator columns of this thread's TMEM lane
-__device__ __forceinline__ void tc_ld16(uint32_t taddr, uint32_t (&r)[16]) {
+// 16 consecutive columns of this thread's TMEM lane.  (The wait sits in the same statement: nothing that uses the values can be
+// moved in front of it.)
+__device__ __forceinline__ void tc_ld16(uint32_t taddr, float (&r)[16]) {
     asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
-          "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-        : "r"(taddr));
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];\n\t"
+        "tcgen05.wait::ld.sync.aligned;"
+        : "=&f"(r[0]), "=&f"(r[1]), "=&f"(r[2]), "=&f"(r[3]), "=&f"(r[4]), "=&f"(r[5]), "=&f"(r[6]), "=&f"(r[7]), "=&f"(r[8]),
+          "=&f"(r[9]), "=&f"(r[10]), "=&f"(r[11]), "=&f"(r[12]), "=&f"(r[13]), "=&f"(r[14]), "=&f"(r[15])
+        : "r"(taddr) : "memory");
+}
+// 16 consecutive columns written; complete when it returns
+__device__ __forceinline__ void tc_st16(uint32_t taddr, const float (&r)[16]) {
+    asm volatile(
+        "tcgen05.st.sync.aligned.32x32b.x16.b32 [%16], {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15};\n\t"
+        "tcgen05.wait::st.sync.aligned;"
+        ::"f"(r[0]), "f"(r[1]), "f"(r[2]), "f"(r[3]), "f"(r[4]), "f"(r[5]), "f"(r[6]), "f"(r[7]), "f"(r[8]), "f"(r[9]), "f"(r[10]),
+          "f"(r[11]), "f"(r[12]), "f"(r[13]), "f"(r[14]), "f"(r[15]), "r"(taddr) : "memory");
 }
 
 // ---- CTA-pair forms (cta_group::2): two CTAs of a cluster act as one 256-row MMA ---------------------
@@ -147,11 +154,13 @@ __device__ __forceinline__ void tc_mma_pair(uint32_t d_tmem, uint64_t a_desc, ui
 struct DenseGeo {
     int n_tiles;      // vocabulary tiles of bn rows
     int n_kc;         // ring steps per tile: ceil(d / kBK)
-    int bn;           // vocabulary rows per tile (per CTA pair when paired); a multiple of 32, <= kMaxBN
+    int bn;           // vocabulary rows per tile (per CTA pair when paired); a multiple of 16, <= kMaxBN
     int n_stages;     // ring depth
     int stage_bytes;  // bytes one CTA stages per step: hidden rows + its share of the vocabulary rows
     int n_groups;     // CTAs (or CTA pairs) walking the tiles round-robin
     int h_rows;       // hidden rows a copy brings (the rest of the MMA's 128 is whatever lies there: lanes nobody looks at)
+    int h_bytes;      // shared memory of a step's hidden rows (a multiple of 1024); its vocabulary rows lie behind them
+    int ring_bytes;
     int sub;          // d-steps per ring stage (1 or 2): one wait and one release per stage, so two steps per stage halve
                       // what the two single threads that drive the ring spend per MMA; taken when three such stages fit
 };
@@ -163,30 +172,75 @@ struct RowState {
     float gb_s, gb_z;         // best Gumbel score and its z
     int gb_j;
     float tv[KT];             // top-k list at the END of the arrays (slots KT-topk .. KT-1, descending)
-    int tj[KT];               // behind +inf sentinels: the insertion threshold is always slot KT-1
+    int tj[KT];               // behind +inf sentinels: the insertion threshold is always slot KT-1; -1: no entry
 };
 
 // Insert (cv, cj) into the sorted list with selects only; equal values keep the entry already there.
 template <int KT>
 __device__ __forceinline__ void list_insert(float (&tv)[KT], int (&tj)[KT], float cv, int cj) {
+    bool gt[KT];
 #pragma unroll
-    for (int p = 0; p < KT; ++p) {
-        const bool sw = cv > tv[p];
-        const float ov = tv[p];
-        const int oj = tj[p];
-        tv[p] = sw ? cv : ov;
-        tj[p] = sw ? cj : oj;
-        cv = sw ? ov : cv;
-        cj = sw ? oj : cj;
+    for (int p = 0; p < KT; ++p) gt[p] = cv > tv[p];
+#pragma unroll
+    for (int p = KT - 1; p >= 1; --p) {
+        tv[p] = gt[p] ? (gt[p - 1] ? tv[p - 1] : cv) : tv[p];
+        tj[p] = gt[p] ? (gt[p - 1] ? tj[p - 1] : cj) : tj[p];
     }
+    tv[0] = gt[0] ? cv : tv[0];
+    tj[0] = gt[0] ? cj : tj[0];
 }
 
-// KT: capacity of the register top-k list (8 or kMaxTopk).  PAIR: two CTAs of a cluster form one MMA.
-// Each of the epilogue warps of a TMEM lane quadrant takes a contiguous share of a tile's 16-column chunks.
-// The epilogue is a long chain of dependent arithmetic per column: it runs at the rate the schedulers can
-// interleave warps, so more warps per scheduler shorten it almost in proportion.
-template <int KT, bool PAIR>
-__global__ void __launch_bounds__(kThreads, 1)
+// ---- sorting networks (descending, everything in registers) ------------------------------------------
+__device__ __forceinline__ void order2(float& a, float& b) {
+    const float hi = fmaxf(a, b), lo = fminf(a, b);
+    a = hi;
+    b = lo;
+}
+__device__ __forceinline__ void order2(unsigned long long& a, unsigned long long& b) {
+    const bool sw = b > a;
+    const unsigned long long hi = sw ? b : a, lo = sw ? a : b;
+    a = hi;
+    b = lo;
+}
+__device__ __forceinline__ float larger(float a, float b) { return fmaxf(a, b); }
+__device__ __forceinline__ unsigned long long larger(unsigned long long a, unsigned long long b) { return b > a ? b : a; }
+// Batcher's odd-even merge sort of v[O .. O + N), N a power of two (the indices are template arguments: they have to be constants)
+template <int O, int N, int R, class T, int A>
+__device__ __forceinline__ void odd_even_merge(T (&v)[A]) {
+    if constexpr (2 * R < N) {
+        odd_even_merge<O, N, 2 * R>(v);
+        odd_even_merge<O + R, N, 2 * R>(v);
+#pragma unroll
+        for (int i = O + R; i + R < O + N; i += 2 * R) order2(v[i], v[i + R]);
+    } else {
+        order2(v[O], v[O + R]);
+    }
+}
+template <int O, int N, class T, int A>
+__device__ __forceinline__ void sort_desc(T (&v)[A]) {
+    if constexpr (N > 1) {
+        sort_desc<O, N / 2>(v);
+        sort_desc<O + N / 2, N / 2>(v);
+        odd_even_merge<O, N, 1>(v);
+    }
+}
+// list <- the N largest of list and v[O .. O + N), both descending: the larger ones of opposite ends are those, in bitonic
+// order, which half-cleaners sort
+template <int O, int N, class T, int A>
+__device__ __forceinline__ void merge_desc(T (&list)[N], const T (&v)[A]) {
+#pragma unroll
+    for (int i = 0; i < N; ++i) list[i] = larger(list[i], v[O + N - 1 - i]);
+#pragma unroll
+    for (int k = N / 2; k >= 1; k >>= 1)
+#pragma unroll
+        for (int i = 0; i < N; ++i)
+            if ((i & k) == 0) order2(list[i], list[i + k]);
+}
+
+// KT: capacity of the list (8 or kMaxTopk).  PAIR: two CTAs of a cluster form one MMA.  PARTS: epilogue warps per TMEM lane
+// quadrant, each with a contiguous share of a tile's 16-column chunks.  Warps whose lanes hold no hidden row leave at once.
+template <int KT, bool PAIR, int PARTS>
+__global__ void __launch_bounds__((2 + 4 * PARTS) * 32, 1)
 k_head_dense(const HeadArgs a, Ctrl* ctrl, float* __restrict__ recs, const DenseGeo geo,
              const __grid_constant__ CUtensorMap tm_h, const __grid_constant__ CUtensorMap tm_w) {
     extern __shared__ uint8_t s_dyn[];
@@ -207,13 +261,15 @@ k_head_dense(const HeadArgs a, Ctrl* ctrl, float* __restrict__ recs, const Dense
     const int group = PAIR ? (int)(blockIdx.x >> 1) : (int)blockIdx.x;
     const int bn = geo.bn, n_stages = geo.n_stages;
     const int w_rows = PAIR ? bn / 2 : bn;                         // vocabulary rows this CTA stages per step
+    // epilogue warps of a CTA with this many of the hidden rows that have any of them to look after
+    auto live_warps = [&](int rows) { return (min(max(rows, 0), kBM) + 31) / 32 * PARTS; };
 
     if (threadIdx.x == 0) {
         // the two tensor maps are fetched now, not by the first copy that needs them
         asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tm_h)) : "memory");
         asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tm_w)) : "memory");
         for (int s = 0; s < kMaxStages; ++s) { mbar_init(&s_full[s], 1); mbar_init(&s_empty[s], 1); }
-        for (int p = 0; p < 2; ++p) { mbar_init(&s_acc_full[p], 1); mbar_init(&s_acc_empty[p], (PAIR ? 2 : 1) * 4 * kParts); }
+        for (int p = 0; p < 2; ++p) { mbar_init(&s_acc_full[p], 1); mbar_init(&s_acc_empty[p], live_warps(B) + (PAIR ? live_warps(B - kBM) : 0)); }
         s_abort = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -246,14 +302,14 @@ k_head_dense(const HeadArgs a, Ctrl* ctrl, float* __restrict__ recs, const Dense
             const int sub = geo.sub;
             const int n_ks = (geo.n_kc + sub - 1) / sub;               // ring stages per tile
             const int total = my_tiles * n_ks;
-            const uint32_t sub_bytes = (uint32_t)geo.stage_bytes / (uint32_t)sub;
+            const uint32_t sub_bytes = (uint32_t)geo.stage_bytes / (uint32_t)sub, h_bytes = (uint32_t)geo.h_bytes;
             const uint32_t full0 = PAIR ? mapa_u32(smem_u32(&s_full[0]), 0) : 0u;      // the leader's full barriers
             auto subs_of = [&](int g) { return min(sub, geo.n_kc - (g % n_ks) * sub); };
             auto load_w = [&](int g) {
                 const int s = g % n_stages, tile = group + (g / n_ks) * geo.n_groups;
                 for (int u = 0; u < subs_of(g); ++u) {
                     const int kc = (g % n_ks) * sub + u;
-                    const uint32_t dst = ring_u32 + (uint32_t)s * (uint32_t)geo.stage_bytes + (uint32_t)u * sub_bytes + kHTileBytes;
+                    const uint32_t dst = ring_u32 + (uint32_t)s * (uint32_t)geo.stage_bytes + (uint32_t)u * sub_bytes + h_bytes;
                     if (PAIR) tma_load_2d_pair(dst, &tm_w, kc * kBK, tile * bn + (int)rank * w_rows, full0 + (uint32_t)(s * sizeof(uint64_t)));
                     else tma_load_2d(dst, &tm_w, kc * kBK, tile * bn, &s_full[s]);
                 }
@@ -300,10 +356,10 @@ k_head_dense(const HeadArgs a, Ctrl* ctrl, float* __restrict__ recs, const Dense
                             const int x = (ks * sub + u) * kBK;
                             if (PAIR) {
                                 tma_load_2d_pair(dst0 + (uint32_t)u * sub_bytes, &tm_h, x, (int)rank * kBM, bar);
-                                tma_load_2d_pair(dst0 + (uint32_t)u * sub_bytes + kHTileBytes, &tm_w, x, row_w, bar);
+                                tma_load_2d_pair(dst0 + (uint32_t)u * sub_bytes + h_bytes, &tm_w, x, row_w, bar);
                             } else {
                                 tma_load_2d(dst0 + (uint32_t)u * sub_bytes, &tm_h, x, 0, &s_full[sc]);
-                                tma_load_2d(dst0 + (uint32_t)u * sub_bytes + kHTileBytes, &tm_w, x, row_w, &s_full[sc]);
+                                tma_load_2d(dst0 + (uint32_t)u * sub_bytes + h_bytes, &tm_w, x, row_w, &s_full[sc]);
                             }
                         }
                     }
@@ -348,7 +404,7 @@ k_head_dense(const HeadArgs a, Ctrl* ctrl, float* __restrict__ recs, const Dense
                     tc_fence_after();
                     const int subs = min(geo.sub, geo.n_kc - kc);
                     const uint64_t da0 = desc_a0 + (uint64_t)(((uint32_t)s * (uint32_t)geo.stage_bytes) >> 4);
-                    const uint64_t db0 = da0 + (uint64_t)(kHTileBytes >> 4);
+                    const uint64_t db0 = da0 + (uint64_t)(geo.h_bytes >> 4);
 #pragma unroll
                     for (int u = 0; u < kMaxSub; ++u) {
                         if (u < subs) {
@@ -381,79 +437,114 @@ k_head_dense(const HeadArgs a, Ctrl* ctrl, float* __restrict__ recs, const Dense
         const int ew = warp - 2;
         const int quad = warp & 3;                            // TMEM lanes this warp may read
         const int part = ew >> 2;                             // which share of the tile's chunks
+        const int rows = min(B - (int)rank * kBM, kBM);       // hidden rows of this CTA
         const int n_ch_tile = bn / kCh;
-        const int ch_lo = part * n_ch_tile / kParts, ch_hi = (part + 1) * n_ch_tile / kParts;
+        const int ch_lo = part * n_ch_tile / PARTS, ch_hi = (part + 1) * n_ch_tile / PARTS;
         const int b = (int)rank * kBM + quad * 32 + lane;
         const bool row_live = b < B;
-        griddep_wait();                                       // temp, uniforms and the record scratch belong to earlier work until here
-        float invT = 1.f;
-        if (row_live) {
-            const float T = a.temp[b];
-            invT = (T > 0.f && T < CUDART_INF_F) ? 1.f / T : CUDART_NAN_F;
-        }
-        RowState<KT> st;
-        st.m = -CUDART_INF_F; st.s = 0.f; st.gb_s = -CUDART_INF_F; st.gb_z = 0.f; st.gb_j = -1;
-        float thr = -CUDART_INF_F;
+        if (quad * 32 < rows) {
+            griddep_wait();                                   // temp, uniforms and the record scratch belong to earlier work until here
+            float invT = 0.f;
+            if (row_live) {
+                const float T = a.temp[b];
+                invT = (T > 0.f && T < CUDART_INF_F) ? 1.f / T : CUDART_NAN_F;
+            }
+            RowState<KT> st;
+            st.m = -CUDART_INF_F; st.s = 0.f; st.gb_s = -CUDART_INF_F; st.gb_z = 0.f; st.gb_j = -1;
 #pragma unroll
-        for (int i = 0; i < KT; ++i) { st.tv[i] = (i < KT - topk) ? CUDART_INF_F : -CUDART_INF_F; st.tj[i] = -1; }
-        const bool vec_u = a.uniforms && ((K & 3) == 0) && ((reinterpret_cast<uintptr_t>(a.uniforms) & 15) == 0);
-        const bool use_u = row_live && a.uniforms != nullptr;
-        const uint32_t acc_empty_bar = PAIR ? mapa_u32(smem_u32(&s_acc_empty[0]), 0) : 0u;
-        float u[kCh];
+            for (int i = 0; i < KT; ++i) { st.tv[i] = (i < KT - topk) ? CUDART_INF_F : -CUDART_INF_F; st.tj[i] = -1; }
+            constexpr int kEntStride = 4 * PARTS * 32;
+            float2* ent = reinterpret_cast<float2*>(ring + geo.ring_bytes) + part * kBM + quad * 32 + lane;
+            const bool vec_u = a.uniforms && ((K & 3) == 0) && ((reinterpret_cast<uintptr_t>(a.uniforms) & 15) == 0);
+            const bool use_u = row_live && a.uniforms != nullptr;
+            const uint32_t acc_empty_bar = PAIR ? mapa_u32(smem_u32(&s_acc_empty[0]), 0) : 0u;
+            const uint32_t tmem_row = tmem_base + ((uint32_t)(quad * 32) << 16);
+            // The warp's chunks one after the other, through all tiles: a chunk's uniforms are requested when the one before it has
+            // used its own.
+            float u[kCh];
 #pragma unroll
-        for (int i = 0; i < kCh; ++i) u[i] = 0.5f;
-        int t_local = 0;
-        for (int tile = group; tile < geo.n_tiles; tile += geo.n_groups, ++t_local) {
-            const int as = t_local & 1;
-            if (!mbar_wait_warp(&s_acc_full[as], (uint32_t)((t_local >> 1) & 1), abort_flag)) break;
-#ifdef VT_STAMPS
-            if (warp == 2 && lane == 0) { if (t_local == 0) VT_DSTAMP(6); VT_DSTAMP(7); }
-#endif
-            tc_fence_after();
-            const int jt = tile * bn;                         // first vocabulary row of the tile
+            for (int i = 0; i < kCh; ++i) u[i] = 0.5f;
+            auto request_u = [&](int j0) {
+                if (!use_u || j0 >= K) return;
+                const float* up = a.uniforms + (size_t)b * K + j0;
+                if (vec_u && j0 + kCh <= K) {
+#pragma unroll
+                    for (int i = 0; i < kCh / 4; ++i) {
+                        const float4 q = reinterpret_cast<const float4*>(up)[i];
+                        u[4 * i] = q.x; u[4 * i + 1] = q.y; u[4 * i + 2] = q.z; u[4 * i + 3] = q.w;
+                    }
+                } else {
+#pragma unroll
+                    for (int i = 0; i < kCh; ++i) u[i] = (j0 + i < K) ? up[i] : 0.5f;
+                }
+            };
+            // log2(-log u) of the chunk at hand: -log u from a short series in 1-u near 1 (where the fast logarithm's absolute
+            // error would dominate), fast logarithms elsewhere; u is clamped to [2^-24, 1 - 2^-24] where each of the two looks at it
+            auto noise = [&](float (&g)[kCh]) {
+#pragma unroll
+                for (int i = 0; i < kCh; ++i) {
+                    const float t = fmaxf(1.f - u[i], 0x1p-24f);
+                    const float lp = t * (1.f + t * (0.5f + t * (0.33333334f + t * (0.25f + t * 0.2f))));
+                    const float L = u[i] > 0.95f ? lp : log2_fast(fmaxf(u[i], 0x1p-24f)) * -kLn2;
+                    g[i] = log2_fast(L);
+                }
+            };
+            if (ch_lo < ch_hi) request_u(group * bn + ch_lo * kCh);
+            int t_local = 0;
+            for (int tile = group; tile < geo.n_tiles; tile += geo.n_groups, ++t_local) {
+                const int as = t_local & 1;
+                const int jt = tile * bn;                     // first vocabulary row of the tile
+                const int ch_end = min(ch_hi, (K - jt + kCh - 1) / kCh);       // (chunks that have columns)
+                const uint32_t acc = tmem_row + (uint32_t)(as * kMaxBN);
+                // The Gumbel noise of the CTA's last tile is made while its MMAs run, and parked in the accumulator stage that
+                // no further tile will use: the only epilogue that nothing hides has neither the loads nor the logarithms.
+                const bool last = tile + geo.n_groups >= geo.n_tiles;
+                const uint32_t parked = tmem_row + (uint32_t)((as ^ 1) * kMaxBN);
+                if (last && a.uniforms) {
 #pragma unroll 1
-            for (int ch = ch_lo; ch < ch_hi; ++ch) {
-                const int j0 = jt + ch * kCh;
-                // this chunk's uniforms are requested first (they are needed last), and a later
-                // chunk's line is pulled into L2 meanwhile
-                if (use_u && j0 < K) {
-                    const float* up = a.uniforms + (size_t)b * K + j0;
-                    if (vec_u && j0 + kCh <= K) {
-#pragma unroll
-                        for (int i = 0; i < kCh / 4; ++i) {
-                            const float4 q = reinterpret_cast<const float4*>(up)[i];
-                            u[4 * i] = q.x; u[4 * i + 1] = q.y; u[4 * i + 2] = q.z; u[4 * i + 3] = q.w;
-                        }
-                    } else {
-#pragma unroll
-                        for (int i = 0; i < kCh; ++i) u[i] = (j0 + i < K) ? up[i] : 0.5f;
+                    for (int ch = ch_lo; ch < ch_end; ++ch) {
+                        float g[kCh];
+                        noise(g);
+                        if (ch + 1 < ch_end) request_u(jt + (ch + 1) * kCh);
+                        __syncwarp();
+                        tc_st16(parked + (uint32_t)(ch * kCh), g);
                     }
                 }
-                const int jn = (ch + 2 < ch_hi) ? j0 + 2 * kCh : jt + geo.n_groups * bn + ch_lo * kCh;
-                if (use_u && jn < K && (ch & 1) == 0)
-                    asm volatile("prefetch.global.L2 [%0];" ::"l"(a.uniforms + (size_t)b * K + jn));
-                uint32_t r[kCh];
-                tc_ld16(tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(as * kMaxBN + ch * kCh), r);
-                // Warp-uniform from here on (j0 and K are): rows that do not exist simply carry nv = 0,
-                // i.e. columns of -inf, so the warp votes below always see all 32 lanes.
-                if (j0 < K) {
-                    // (the lane of a hidden row that does not exist goes along with whatever it has and is never looked at)
-                    const int nv = min(kCh, K - j0);
-                    float z[kCh];
-                    if (nv == kCh) {
+                if (!mbar_wait_warp(&s_acc_full[as], (uint32_t)((t_local >> 1) & 1), abort_flag)) break;
+#ifdef VT_STAMPS
+                if (warp == 2 && lane == 0) { if (t_local == 0) VT_DSTAMP(6); VT_DSTAMP(7); }
+#endif
+                tc_fence_after();
+                // z of a chunk's columns; columns that do not exist carry -inf
+                auto load_z = [&](int ch, float (&z)[kCh]) {
+                    float r[kCh];
+                    __syncwarp();
+                    tc_ld16(acc + (uint32_t)(ch * kCh), r);
+                    const int nv = K - (jt + ch * kCh);
 #pragma unroll
-                        for (int i = 0; i < kCh; ++i) z[i] = __uint_as_float(r[i]) * invT;
-                    } else {
+                    for (int i = 0; i < kCh; ++i) z[i] = r[i] * invT;
+                    if (nv < kCh) {
 #pragma unroll
-                        for (int i = 0; i < kCh; ++i) z[i] = (i < nv) ? __uint_as_float(r[i]) * invT : -CUDART_INF_F;
+                        for (int i = 0; i < kCh; ++i) z[i] = (i < nv) ? z[i] : -CUDART_INF_F;
                     }
+                };
+                // (Warp-uniform throughout: the lane of a hidden row that does not exist goes along with whatever it has and is
+                // never looked at.)
+#pragma unroll 1
+                for (int ch = ch_lo; ch < ch_end; ++ch) {
+                    const int j0 = jt + ch * kCh;
+
+                    float z[kCh];
+                    load_z(ch, z);
                     float cmax = z[0];
 #pragma unroll
                     for (int i = 1; i < kCh; ++i) cmax = fmaxf(cmax, z[i]);
-                    if (a.dbg_logits && row_live) {
+                    if (a.dbg_logits) {
+                        float r[kCh];
+                        tc_ld16(acc + (uint32_t)(ch * kCh), r);
 #pragma unroll
                         for (int i = 0; i < kCh; ++i)
-                            if (i < nv) a.dbg_logits[(size_t)b * K + j0 + i] = __uint_as_float(r[i]);
+                            if (row_live && j0 + i < K) a.dbg_logits[(size_t)b * K + j0 + i] = r[i];
                     }
                     // running max / sum-exp: one rescale per chunk, independent exponentials, two sums.  The maximum is
                     // subtracted before the scaling to base 2: z - m is exact or nearly so whatever the size of the logits,
@@ -466,113 +557,195 @@ k_head_dense(const HeadArgs a, Ctrl* ctrl, float* __restrict__ recs, const Dense
                         acc0 += exp_fast(z[i] - m_ref);
                         acc1 += exp_fast(z[i + 1] - m_ref);
                     }
-                    st.s = st.s * exp_fast(st.m - m_ref) + (acc0 + acc1);
+                    const float add = acc0 + acc1;
+                    st.s = st.s * exp_fast(st.m - m_ref) + add;
                     st.m = m_new;
+
                     if (a.uniforms) {
+                        // Gumbel maximum, score z - log(-log u)
+                        float g[kCh];
+                        if (last) {
+                            __syncwarp();
+                            tc_ld16(parked + (uint32_t)(ch * kCh), g);
+                        } else {
+                            noise(g);
+                            request_u(ch + 1 < ch_end ? j0 + kCh : jt + geo.n_groups * bn + ch_lo * kCh);
+                        }
+                        float bs[2] = {-CUDART_INF_F, -CUDART_INF_F}, bz[2] = {0.f, 0.f};       // (two halves side by side)
+                        int bj[2] = {-1, -1};
 #pragma unroll
                         for (int i = 0; i < kCh; ++i) {
-                            // g = -log(-log u): -log u from a short series in 1-u near 1 (where the fast
-                            // logarithm's absolute error would dominate), fast logarithms elsewhere; u is clamped to
-                            // [2^-24, 1 - 2^-24] where each of the two looks at it
-                            const float t = fmaxf(1.f - u[i], 0x1p-24f);
-                            const float lp = t * (1.f + t * (0.5f + t * (0.33333334f + t * (0.25f + t * 0.2f))));
-                            const float L = u[i] > 0.95f ? lp : log2_fast(fmaxf(u[i], 0x1p-24f)) * -kLn2;
-                            const float sc = fmaf(log2_fast(L), -kLn2, z[i]);
-                            const bool win = sc > st.gb_s;            // columns that do not exist carry z = -inf
-                            st.gb_s = win ? sc : st.gb_s;
-                            st.gb_j = win ? j0 + i : st.gb_j;
-                            st.gb_z = win ? z[i] : st.gb_z;
+                            const int q = i / (kCh / 2);
+                            const float sc = fmaf(g[i], -kLn2, z[i]);
+                            const bool win = sc > bs[q];              // columns that do not exist carry z = -inf
+                            bs[q] = win ? sc : bs[q];
+                            bj[q] = win ? i : bj[q];
+                            bz[q] = win ? z[i] : bz[q];
+                        }
+                        const bool second = bs[1] > bs[0];
+                        const float cs = second ? bs[1] : bs[0];
+                        if (cs > st.gb_s) {
+                            st.gb_s = cs;
+                            st.gb_j = j0 + (second ? bj[1] : bj[0]);
+                            st.gb_z = second ? bz[1] : bz[0];
                         }
                     }
-                    // top-k: pull the chunk's candidates into the list while they beat its last entry.  The loop is
-                    // warp-uniform (it runs while any row of the warp still has a candidate) and everything inside is
-                    // select-based: one row's insertions never make the other 31 rows branch.  A NaN logit poisons the
-                    // row's lse (reported through VT_FLAG_NAN_ROW) and is no candidate (it beats nothing).
-                    // candidates: the columns that beat the list's last entry as it stands; they go in by
-                    // ascending column (equal values keep the lower column ahead), one per trip of a warp-
-                    // uniform loop that runs while any row still has one.  A candidate that has fallen under
-                    // the entry that moved up meanwhile simply finds no slot.
-                    uint32_t cand = 0;
+
+                    if (t_local == 0) {
+                        // Top-k over the first tile, where nearly everything is a candidate at first: the list's values alone, by
+                        // sorting networks, whatever a chunk holds; the indices follow below.  (Inserting the candidates one by one,
+                        // a warp does as many trips as the one of its 32 rows that has most of them, 9 a chunk.)
+                        if (__any_sync(0xffffffffu, add != add)) {
+                            // a NaN logit (or an infinite one) somewhere: a NaN is no candidate, and the networks have to be without it
+                            // (min and max would drop it and keep its partner twice)
 #pragma unroll
-                    for (int i = 0; i < kCh; ++i) cand |= (z[i] > thr) ? (1u << i) : 0u;
-                    while (__any_sync(0xffffffffu, cand != 0)) {
-                        const bool take = cand != 0;
-                        const int i = take ? __ffs(cand) - 1 : 0;
-                        float q8[8], q4[4], q2[2];
+                            for (int i = 0; i < kCh; ++i) z[i] = fmaxf(z[i], -CUDART_INF_F);
+                        }
+                        sort_desc<0, KT>(z);
+                        merge_desc<0>(st.tv, z);
+                        if (KT < kCh) {
+                            sort_desc<kCh - KT, KT>(z);
+                            merge_desc<kCh - KT>(st.tv, z);
+                        }
+                    } else {
+                        // Later on a chunk has few candidates, the columns that beat the list's last entry as it stands; they go in
+                        // by ascending column (equal values keep the lower column ahead), one per trip of a warp-uniform loop that
+                        // runs while any row still has one, everything inside select-based: one row's insertions never make the
+                        // other 31 rows branch.  A candidate that has fallen under the entry that moved up meanwhile simply finds no
+                        // slot.  (A NaN logit beats nothing.)
+                        const float thr = st.tj[KT - 1] >= 0 ? st.tv[KT - 1] : -CUDART_INF_F;  // a threshold only once the list is full
+                        uint32_t cand = 0;
 #pragma unroll
-                        for (int k = 0; k < 8; ++k) q8[k] = (i & 1) ? z[2 * k + 1] : z[2 * k];
+                        for (int i = 0; i < kCh; ++i) cand |= (z[i] > thr) ? (1u << i) : 0u;
+                        while (__any_sync(0xffffffffu, cand != 0)) {
+                            const bool take = cand != 0;
+                            const int i = take ? __ffs(cand) - 1 : 0;
+                            float q8[8], q4[4], q2[2];
 #pragma unroll
-                        for (int k = 0; k < 4; ++k) q4[k] = (i & 2) ? q8[2 * k + 1] : q8[2 * k];
+                            for (int k = 0; k < 8; ++k) q8[k] = (i & 1) ? z[2 * k + 1] : z[2 * k];
 #pragma unroll
-                        for (int k = 0; k < 2; ++k) q2[k] = (i & 4) ? q4[2 * k + 1] : q4[2 * k];
-                        const float v = (i & 8) ? q2[1] : q2[0];
-                        list_insert<KT>(st.tv, st.tj, take ? v : -CUDART_INF_F, j0 + i);
-                        thr = st.tj[KT - 1] >= 0 ? st.tv[KT - 1] : -CUDART_INF_F;   // a threshold only once the list is full
-                        cand &= cand - 1;
+                            for (int k = 0; k < 4; ++k) q4[k] = (i & 2) ? q8[2 * k + 1] : q8[2 * k];
+#pragma unroll
+                            for (int k = 0; k < 2; ++k) q2[k] = (i & 4) ? q4[2 * k + 1] : q4[2 * k];
+                            const float v = (i & 8) ? q2[1] : q2[0];
+                            list_insert<KT>(st.tv, st.tj, take ? v : -CUDART_INF_F, j0 + i);
+                            cand &= cand - 1;
+                        }
                     }
                 }
-            }
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) {
-                if (PAIR) mbar_arrive_cluster(acc_empty_bar + (uint32_t)(as * sizeof(uint64_t)));
-                else mbar_arrive(&s_acc_empty[as]);
-            }
-#ifdef VT_STAMPS
-            if (warp == 2 && lane == 0) { if (t_local == 0) VT_DSTAMP(8); VT_DSTAMP(9); }
-#endif
-        }
-        // ---- the column shares of a row meet in shared memory (the ring is idle by now: the last
-        // accumulators were complete, so every MMA has read its operands and every copy has landed) ----
-        float* xch = reinterpret_cast<float*>(ring);
-        constexpr int kXchFields = 5 + 2 * KT;
-        const int slot = quad * 32 + lane;                    // row within the CTA
-        const bool ok = !*abort_flag;
-        if (part > 0 && ok) {
-            float* x = xch + (size_t)(part - 1) * kXchFields * kBM + slot;     // field-major: conflict-free
-            x[0 * kBM] = st.m; x[1 * kBM] = st.s; x[2 * kBM] = st.gb_s; x[3 * kBM] = __int_as_float(st.gb_j); x[4 * kBM] = st.gb_z;
-#pragma unroll
-            for (int p = 0; p < KT; ++p) { x[(5 + p) * kBM] = st.tv[p]; x[(5 + KT + p) * kBM] = __int_as_float(st.tj[p]); }
-        }
-        asm volatile("bar.sync 1, %0;" ::"n"(4 * kParts * 32) : "memory");
-        if (part == 0 && ok && row_live) {
+
+                if (t_local == 0) {
+                    // The threshold is known: the columns at or above it are the list, and go to shared memory with their indices in
+                    // ascending order.  More of them than fit means that columns tie at the threshold; then it is done again and of
+                    // those only the first are taken, as many as there is room for.
+                    const float thr = st.tv[KT - 1];
+                    const float least = fmaxf(thr, -FLT_MAX);          // (a list that is not full: every column but -inf)
+                    int n = 0;
 #pragma unroll 1
-            for (int o = 0; o < kParts - 1; ++o) {
-                const float* x = xch + (size_t)o * kXchFields * kBM + slot;
-                lse_merge(st.m, st.s, x[0 * kBM], x[1 * kBM]);
-                const float os = x[2 * kBM];
-                const int oj = __float_as_int(x[3 * kBM]);
-                if (better(os, oj, st.gb_s, st.gb_j) && oj >= 0) { st.gb_s = os; st.gb_j = oj; st.gb_z = x[4 * kBM]; }
+                    for (int ch = ch_lo; ch < ch_end; ++ch) {
+                        float z[kCh];
+                        load_z(ch, z);
 #pragma unroll
-                for (int p = 0; p < KT; ++p) {
-                    // entries of the other share: equal values must still order by index, so compare keys
-                    float cv = x[(5 + p) * kBM];
-                    int cj = __float_as_int(x[(5 + KT + p) * kBM]);
-                    if (p < KT - topk) continue;              // its sentinels
+                        for (int i = 0; i < kCh; ++i) {
+                            const bool in = z[i] >= least;
+                            if (in) ent[min(n, KT - 1) * kEntStride] = make_float2(z[i], __int_as_float(jt + ch * kCh + i));
+                            n += in ? 1 : 0;
+                        }
+                    }
+                    if (__any_sync(0xffffffffu, row_live && n > topk)) {
+                        int ties = KT;                        // entries equal to the threshold that there is room for
 #pragma unroll
-                    for (int q = 0; q < KT; ++q) {
-                        const bool sw = key64(cv, cj) > key64(st.tv[q], st.tj[q]) && q >= KT - topk;
-                        const float ov = st.tv[q];
-                        const int oj2 = st.tj[q];
-                        st.tv[q] = sw ? cv : ov;
-                        st.tj[q] = sw ? cj : oj2;
-                        cv = sw ? ov : cv;
-                        cj = sw ? oj2 : cj;
+                        for (int i = 0; i < KT; ++i) ties -= st.tv[i] > thr || (i < KT - topk && thr == CUDART_INF_F) ? 1 : 0;
+                        n = 0;
+#pragma unroll 1
+                        for (int ch = ch_lo; ch < ch_end; ++ch) {
+                            float z[kCh];
+                            load_z(ch, z);
+#pragma unroll
+                            for (int i = 0; i < kCh; ++i) {
+                                const bool tie = z[i] == thr;
+                                const bool in = z[i] >= least && (!tie || ties > 0);
+                                ties -= in && tie ? 1 : 0;
+                                if (in) ent[min(n, KT - 1) * kEntStride] = make_float2(z[i], __int_as_float(jt + ch * kCh + i));
+                                n += in ? 1 : 0;
+                            }
+                        }
+                    }
+
+                    unsigned long long key[KT];
+                    n = min(n, topk);
+#pragma unroll
+                    for (int i = 0; i < KT; ++i) {
+                        const float2 e = i < n ? ent[i * kEntStride] : make_float2(0.f, 0.f);
+                        // (-0 orders as 0; the sentinels in front of everything)
+                        key[i] = i < n ? key64(e.x + 0.f, __float_as_int(e.y)) : i < topk ? 0ull : ~0ull;
+                    }
+                    sort_desc<0, KT>(key);
+#pragma unroll
+                    for (int i = 0; i < KT; ++i) {
+                        st.tj[i] = i < KT - topk || key[i] == 0ull ? -1 : key_idx(key[i]);
+                        st.tv[i] = i < KT - topk ? CUDART_INF_F : key[i] == 0ull ? -CUDART_INF_F : key_val(key[i]);
+                    }
+
+                }
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) {
+                    if (PAIR) mbar_arrive_cluster(acc_empty_bar + (uint32_t)(as * sizeof(uint64_t)));
+                    else mbar_arrive(&s_acc_empty[as]);
+                }
+#ifdef VT_STAMPS
+                if (warp == 2 && lane == 0) { if (t_local == 0) VT_DSTAMP(8); VT_DSTAMP(9); }
+#endif
+            }
+
+            const bool ok = !*abort_flag;
+            unsigned long long key[KT];                       // the list as keys, behind the sentinels
+#pragma unroll
+            for (int i = 0; i < KT; ++i) key[i] = i < KT - topk ? ~0ull : st.tj[i] >= 0 ? key64(st.tv[i] + 0.f, st.tj[i]) : 0ull;
+            if (!PAIR) {
+                // the column shares of a row meet in shared memory: lists where the thread's entries were, the rest in the ring
+                // (idle by now: the last accumulators were complete, so every MMA has read its operands and every copy has landed)
+                unsigned long long* klist = reinterpret_cast<unsigned long long*>(ent);
+                float* xch = reinterpret_cast<float*>(ring) + part * kBM + quad * 32 + lane;
+#pragma unroll
+                for (int o = 1; o < PARTS; o <<= 1) {
+                    if ((part & (2 * o - 1)) == o && ok) {
+#pragma unroll
+                        for (int i = 0; i < KT; ++i) klist[((i + topk) & (KT - 1)) * kEntStride] = i < KT - topk ? 0ull : key[i];
+                        xch[0] = st.m; xch[kEntStride] = st.s; xch[2 * kEntStride] = st.gb_s;
+                        xch[3 * kEntStride] = __int_as_float(st.gb_j); xch[4 * kEntStride] = st.gb_z;
+                    }
+                    asm volatile("bar.sync 1, %0;" ::"r"(live_warps(rows) * 32) : "memory");
+                    if ((part & (2 * o - 1)) == 0 && ok) {
+                        const float* x = xch + o * kBM;
+                        unsigned long long other[KT];
+#pragma unroll
+                        for (int i = 0; i < KT; ++i) other[i] = klist[i * kEntStride + o * kBM];
+                        lse_merge(st.m, st.s, x[0], x[kEntStride]);
+                        const float os = x[2 * kEntStride];
+                        const int oj = __float_as_int(x[3 * kEntStride]);
+                        if (better(os, oj, st.gb_s, st.gb_j) && oj >= 0) { st.gb_s = os; st.gb_j = oj; st.gb_z = x[4 * kEntStride]; }
+                        merge_desc<0>(key, other);
                     }
                 }
             }
-            // ---- this CTA's record of hidden row b ---------------------------------------------------------
-            unsigned long long* kp = rec_keys(recs, b, topk);
-            float* fp = rec_f32(recs, b, topk);
-            const int c = group;
-            fp[c] = st.m;
-            fp[kMaxGrid + c] = st.s;
-            fp[2 * kMaxGrid + c] = st.gb_z;
-            kp[c] = st.gb_j >= 0 ? key64(st.gb_s, st.gb_j) : 0ull;
+
+            if ((PAIR || part == 0) && ok && row_live) {
+                // ---- the record of hidden row b: this CTA's, or this share's of the pair's columns (a pair leaves two per row, which
+                // the merge takes as well as one)
+                unsigned long long* kp = rec_keys(recs, b, topk);
+                float* fp = rec_f32(recs, b, topk);
+                const int c = PAIR ? group * PARTS + part : group;
+                fp[c] = st.m;
+                fp[kMaxGrid + c] = st.s;
+                fp[2 * kMaxGrid + c] = st.gb_z;
+                kp[c] = st.gb_j >= 0 ? key64(st.gb_s, st.gb_j) : 0ull;
 #pragma unroll
-            for (int p = 0; p < KT; ++p)
-                if (p >= KT - topk)
-                    kp[(size_t)(1 + p - (KT - topk)) * kMaxGrid + c] = st.tj[p] >= 0 ? key64(st.tv[p], st.tj[p]) : 0ull;
+                for (int p = 0; p < KT; ++p)
+                    if (p >= KT - topk) kp[(size_t)(1 + p - (KT - topk)) * kMaxGrid + c] = key[p];
+            }
+
         }
 #ifdef VT_STAMPS
         if (warp == 2 && lane == 0) VT_DSTAMP(10);
@@ -649,11 +822,13 @@ k_head_merge(const HeadArgs a, Ctrl* ctrl, float* __restrict__ recs, int G, int 
 // ---- host side ----------------------------------------------------------------------------------------
 // Tile width: the vocabulary is dealt to `groups` CTAs (pairs) in tiles of bn rows; the slowest group
 // works ceil(tiles / groups) * bn rows.  Smallest such makespan wins, the wider tile on equal terms
-// (fewer re-reads of the hidden rows).
-DenseGeo make_geo(int32_t K, int32_t d, bool pair, int max_groups) {
+// (fewer re-reads of the hidden rows).  Multiples of 16 (136 rows per CTA of 20001: 144 instead of 160); a pair takes multiples
+// of 32, with others its MMAs are several times slower (200 rows of 50001 x 3072, 240 columns: 318 us instead of 122).
+DenseGeo make_geo(int32_t K, int32_t d, bool pair, int h_rows, int max_groups, size_t ring_budget) {
     DenseGeo g{};
     long best = -1;
-    for (int bn = kMaxBN; bn >= 32; bn -= 32) {
+    const int by = pair ? 32 : 16;
+    for (int bn = kMaxBN; bn >= by; bn -= by) {
         const long tiles = (K + bn - 1) / bn;
         const long span = ((tiles + max_groups - 1) / max_groups) * bn;
         if (best < 0 || span < best) { best = span; g.bn = bn; }
@@ -661,30 +836,43 @@ DenseGeo make_geo(int32_t K, int32_t d, bool pair, int max_groups) {
     g.n_tiles = (K + g.bn - 1) / g.bn;
     g.n_kc = (d + kBK - 1) / kBK;
     g.n_groups = g.n_tiles < max_groups ? g.n_tiles : max_groups;
-    const int step_bytes = kHTileBytes + (pair ? g.bn / 2 : g.bn) * kBK * 2;
-    g.sub = (3 * kMaxSub * (size_t)step_bytes <= kRingBudget && g.n_kc >= kMaxSub) ? kMaxSub : 1;
+    g.h_rows = h_rows;
+    // (the MMA reads 128 hidden rows from here: beyond those that exist whatever follows, behind the ring's end the entries)
+    g.h_bytes = (int)align_up((size_t)h_rows * kBK * 2, 1024);
+    const int step_bytes = g.h_bytes + (pair ? g.bn / 2 : g.bn) * kBK * 2;
+    g.sub = (3 * kMaxSub * (size_t)step_bytes <= ring_budget && g.n_kc >= kMaxSub) ? kMaxSub : 1;
     g.stage_bytes = step_bytes * g.sub;
-    g.n_stages = (int)(kRingBudget / (size_t)g.stage_bytes);
+    g.n_stages = (int)(ring_budget / (size_t)g.stage_bytes);
     if (g.n_stages > kMaxStages) g.n_stages = kMaxStages;
+    g.ring_bytes = g.n_stages * g.stage_bytes;
     return g;
 }
 
-template <int KT, bool PAIR>
-cudaError_t launch_variant(const HeadArgs& a, Ctrl* ctrl, float* recs, const DenseGeo& geo, const CUtensorMap& tm_h,
-                           const CUtensorMap& tm_w, cudaStream_t s) {
+// shared memory of the candidate entries; also room for the operand rows that the last stage's MMAs read beyond it
+template <int KT, int PARTS>
+constexpr size_t entry_bytes() { return (size_t)KT * 4 * PARTS * 32 * sizeof(float2); }
+static_assert(entry_bytes<8, 2>() >= (size_t)kBM * kBK * 2, "128 operand rows from the ring's end on lie inside");
+
+template <int KT, bool PAIR, int PARTS>
+cudaError_t launch_variant(const HeadArgs& a, Ctrl* ctrl, float* recs, int max_groups, int* records, cudaStream_t s) {
+    constexpr size_t kEntries = entry_bytes<KT, PARTS>();
+    const DenseGeo geo = make_geo(a.K, a.d, PAIR, PAIR ? kBM : a.B, max_groups, kSmemBudget - kEntries);
+    CUtensorMap tm_h, tm_w;
+    if (!encode_map(&tm_h, a.h, a.B, a.d, geo.h_rows) || !encode_map(&tm_w, a.W, a.K, a.d, PAIR ? geo.bn / 2 : geo.bn))
+        return cudaErrorInvalidValue;
     static int attr_done[64] = {0};
-    const size_t smem = (size_t)geo.n_stages * geo.stage_bytes + 1024;   // + slack to align the ring to 1024 bytes
+    const size_t smem = (size_t)geo.ring_bytes + kEntries + 1024;   // + slack to align the ring to 1024 bytes
     int dev = 0;
     cudaGetDevice(&dev);
     if (dev < 0 || dev >= 64 || !attr_done[dev]) {
-        cudaError_t e = cudaFuncSetAttribute(k_head_dense<KT, PAIR>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)(kRingBudget + 1024));
+        cudaError_t e = cudaFuncSetAttribute(k_head_dense<KT, PAIR, PARTS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)(kSmemBudget + 1024));
         if (e != cudaSuccess) return e;
         if (dev >= 0 && dev < 64) attr_done[dev] = 1;
     }
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)(PAIR ? 2 * geo.n_groups : geo.n_groups));
-    cfg.blockDim = dim3(kThreads);
+    cfg.blockDim = dim3((2 + 4 * PARTS) * 32);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
     cudaLaunchAttribute at[2];
@@ -696,7 +884,8 @@ cudaError_t launch_variant(const HeadArgs& a, Ctrl* ctrl, float* recs, const Den
     at[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
     cfg.numAttrs = a.overlap ? 2 : 1;
-    return cudaLaunchKernelEx(&cfg, k_head_dense<KT, PAIR>, a, ctrl, recs, geo, tm_h, tm_w);
+    *records = PAIR ? geo.n_groups * PARTS : geo.n_groups;
+    return cudaLaunchKernelEx(&cfg, k_head_dense<KT, PAIR, PARTS>, a, ctrl, recs, geo, tm_h, tm_w);
 }
 
 }  // namespace
@@ -722,22 +911,24 @@ cudaError_t launch_head_dense(const HeadArgs& a, Ctrl* ctrl, uint8_t* scratch, c
     if (!head_dense_supported(a.B, a.K, a.d) || !head_dense_topk_ok(a.topk)) return cudaErrorInvalidValue;
     const bool pair = a.B > kBM;                       // more than one MMA's worth of hidden rows: CTA pairs
     int max_groups = pair ? num_sms() / 2 : num_sms();
-    if (max_groups > kMaxGrid) max_groups = kMaxGrid;
+    const int most = pair ? kMaxGrid / 2 : kMaxGrid;   // (a pair leaves two records per row)
+    if (max_groups > most) max_groups = most;
     if (max_groups < 1) return cudaErrorInvalidValue;
-    DenseGeo geo = make_geo(a.K, a.d, pair, max_groups);
-    geo.h_rows = pair ? kBM : a.B;
-    CUtensorMap tm_h, tm_w;
-    if (!encode_map(&tm_h, a.h, a.B, a.d, geo.h_rows) || !encode_map(&tm_w, a.W, a.K, a.d, pair ? geo.bn / 2 : geo.bn))
-        return cudaErrorInvalidValue;
     float* recs = reinterpret_cast<float*>(scratch);
     cudaError_t e;
-    if (a.topk <= 8) e = pair ? launch_variant<8, true>(a, ctrl, recs, geo, tm_h, tm_w, s)
-                              : launch_variant<8, false>(a, ctrl, recs, geo, tm_h, tm_w, s);
-    else e = pair ? launch_variant<kMaxTopk, true>(a, ctrl, recs, geo, tm_h, tm_w, s)
-                  : launch_variant<kMaxTopk, false>(a, ctrl, recs, geo, tm_h, tm_w, s);
+    int records = 0;
+    // Up to 64 rows half of the lane quadrants hold none: twice the warps on the others (above that two shares are as fast, 100 rows
+    // of 20001 x 3072 43.7 against 46.1 us).
+    const bool few = a.B <= 64;
+    if (a.topk <= 8) e = pair ? launch_variant<8, true, 2>(a, ctrl, recs, max_groups, &records, s)
+                       : few  ? launch_variant<8, false, 4>(a, ctrl, recs, max_groups, &records, s)
+                              : launch_variant<8, false, 2>(a, ctrl, recs, max_groups, &records, s);
+    else e = pair ? launch_variant<kMaxTopk, true, 2>(a, ctrl, recs, max_groups, &records, s)
+           : few  ? launch_variant<kMaxTopk, false, 4>(a, ctrl, recs, max_groups, &records, s)
+                  : launch_variant<kMaxTopk, false, 2>(a, ctrl, recs, max_groups, &records, s);
     if (e != cudaSuccess) return e;
     count_launch();
-    return launch_head_merge(a, ctrl, recs, geo.n_groups, s);
+    return launch_head_merge(a, ctrl, recs, records, s);
 }
 
 // The records of G CTAs (pairs) -> outputs; with a tree, its expansion as one more launch (it needs every row's merge).

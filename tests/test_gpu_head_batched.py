@@ -1,0 +1,101 @@
+"""The batched head's epilogue against its own logits: candidate lists, sampled ids and log-probabilities recomputed from the logits
+that the same call leaves, at the edges of tiles, column shares, lane quadrants and lists, with ties, infinities and NaN."""
+import pytest
+import torch
+
+import paper_2506_22694_b200 as vt
+import vt_inputs
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda"
+
+
+def _check(h, W, T, topk, u, flags=0):
+    B, K, d = h.shape[0], W.shape[0], W.shape[1]
+    ws = vt.Workspace(vt.workspace_bytes(vt.VT_OP_DRAFT_HEAD, 0, 0, K, d, B, topk))
+    ids, lps, logits, lse = vt.vt_draft_head(h, W, None, T, topk, u, ws=ws, debug=True)
+    z = logits * (1.0 / T)[:, None]                                    # the kernel's own two roundings
+    # candidates: by descending z, equal ones by index, NaN and -inf never.  Exact.
+    ranked = torch.where(torch.isnan(z), torch.full_like(z, -float("inf")), z)
+    order = torch.argsort(ranked, dim=1, descending=True, stable=True)[:, :topk]
+    best = ranked.gather(1, order)
+    want = torch.where(best > -float("inf"), order, torch.full_like(order, -1)).to(torch.int32)
+    assert torch.equal(ids[:, 1:], want)
+    got = lps[:, 1:]
+    expect = torch.where(want >= 0, best - lse[:, None], torch.full_like(best, float("nan")))
+    assert torch.equal(torch.isnan(got), torch.isnan(expect))
+    assert torch.equal(got[~torch.isnan(got)], expect[~torch.isnan(expect)])
+    if u is None:
+        assert torch.equal(ids[:, 0], ids[:, 1])
+    else:
+        # a score is off by the fast logarithms' 2^-21 and one rounding of its own size at most
+        uc = u.double().clamp(2.0 ** -24, 1 - 2.0 ** -24)
+        score = ranked.double() - torch.log(-torch.log(uc))
+        top = score.max(dim=1).values
+        mine = score.gather(1, ids[:, :1].long().clamp(min=0))[:, 0]
+        live = top > -float("inf")
+        slack = 2.0 ** -20 + (ranked.double().abs().amax(dim=1).clamp(max=1e30)) * 2.0 ** -23
+        assert bool(((ids[:, 0] >= 0) == live).all())
+        ok = (top - mine <= slack) | (top == mine)
+        assert bool(ok[live].all())
+    got_flags = ws.read_status()[1]
+    assert got_flags == flags, got_flags
+    again = vt.vt_draft_head(h, W, None, T, topk, u, ws=ws, overlapped=True)
+    assert torch.equal(again[0], ids) and torch.equal(again[1].view(torch.int32), lps.view(torch.int32))
+
+
+def _inputs(B, K, d, sample, seed):
+    W = vt_inputs.gaussian_bf16((K, d), 0.02, seed=seed, device=DEV)
+    h = vt_inputs.gaussian_bf16((B, d), 1.0, seed=seed + 1, device=DEV)
+    T = vt_inputs.temperatures(B, 0.5, 1.5, seed=seed + 2, device=DEV)
+    u = vt_inputs.uniforms((B, K), seed=seed + 3, device=DEV) if sample else None
+    return h, W, T, u
+
+
+@pytest.mark.parametrize("B,K,d,topk,sample", [
+    (33, 17, 64, 16, True), (64, 2369, 128, 8, True), (65, 2369, 128, 7, True),                  # tiles of 16 columns: one chunk, empty shares
+    (40, 20_001, 256, 8, True), (63, 37_888, 64, 1, False), (64, 37_889, 64, 9, True),           # one tile per CTA, the widest, two
+    (96, 20_004, 192, 8, True), (97, 19_999, 192, 16, True), (128, 80_001, 64, 3, True),         # three and four quadrants, three tiles
+    (129, 2368, 128, 8, True), (129, 2369, 72, 16, True), (160, 18_944, 64, 8, False),           # pairs: second CTA with one row and with 32
+    (161, 18_945, 64, 10, True), (255, 60_000, 64, 8, True), (256, 33_000, 136, 5, True),        # one, two and four tiles
+])
+def test_lists_and_samples_follow_from_the_logits(B, K, d, topk, sample):
+    h, W, T, u = _inputs(B, K, d, sample, seed=B + K)
+    _check(h, W, T, topk, u)
+
+
+@pytest.mark.parametrize("B,K,topk", [(40, 20_001, 8), (100, 40_001, 5), (200, 40_001, 8), (70, 20_001, 16), (130, 3000, 16)])
+def test_ties_go_to_the_lower_index(B, K, topk):
+    """Logits of a few distinct values (small whole numbers, exact in every order): tens to thousands of columns tie at the threshold."""
+    g = torch.Generator(device=DEV)
+    g.manual_seed(K + topk)
+    W = torch.randint(-1, 2, (K, 64), generator=g, device=DEV).to(torch.bfloat16)
+    W[:, 4:] = 0                                                       # nine values
+    h = torch.ones((B, 64), device=DEV).to(torch.bfloat16)
+    h[1] = 0                                                           # all columns tie
+    h[2] = -1
+    _check(h, W, torch.ones(B, device=DEV), topk, None)
+    _check(h, W, torch.ones(B, device=DEV), topk, vt_inputs.uniforms((B, K), seed=3, device=DEV))
+
+
+@pytest.mark.parametrize("B,K", [(40, 20_001), (200, 40_001)])
+def test_infinite_and_nan_logits(B, K):
+    h, W, T, u = _inputs(B, K, 64, True, seed=B)
+    W[:, 0] = 0
+    W[5, 0] = float("inf")                                             # +inf, -inf or (times 0) NaN in that column, by row
+    W[K - 3, 0] = float("nan")
+    h[:, 0] = 0
+    h[3, 0] = 1
+    h[B - 1, 0] = -1
+    _check(h, W, T, 8, u, flags=vt.VT_FLAG_NAN_ROW)
+    W[K - 3, 0] = 0
+    _check(h, W, T, 8, None, flags=vt.VT_FLAG_NAN_ROW)
+
+
+def test_uniforms_at_and_beyond_their_range_and_unaligned():
+    B, K = 70, 20_003
+    h, W, T, u = _inputs(B, K, 64, True, seed=9)
+    u[0], u[1, ::2], u[2, 7], u[3] = 0.0, 1.0, 1.0, 1.0 - 2.0 ** -24
+    flat = torch.empty(B * K + 1, device=DEV)
+    flat[1:].view(B, K).copy_(u)
+    _check(h, W, T, 8, flat[1:].view(B, K))
