@@ -12,10 +12,8 @@ constexpr int kMaxGrid = 160;                    // merge: each lane owns at mos
 constexpr int kMaxOwn = kMaxGrid / 32;
 constexpr int kMergeDepth = 4;                   // list entries per CTA staged on chip by the merge
 constexpr int kSelCap = 128;                     // entries the merge's direct selection can rank
-// staging words (32-bit) per merging warp: the staged list heads, or before it comes to that the selection buffer and the
-// output keys (all 64-bit)
+// staging words (32-bit) of a merging block: the staged list heads, or before it comes to that the selection's buffers
 constexpr int kMergeStageWords = 2 * kMergeDepth * kMaxGrid;
-static_assert(2 * (kSelCap + 4 + 64) <= kMergeStageWords, "both uses fit");
 constexpr int kStampSlots = 16;                  // phase stamps per CTA (-DVT_STAMPS builds)
 #ifdef VT_STAMPS
 constexpr size_t kStampBytes = (size_t)kMaxGrid * kStampSlots * 8;
@@ -133,239 +131,253 @@ struct MergeOut {
     int sampled;       // uniforms were given: column 0 is the Gumbel-max draw
 };
 
-// A single warp runs dependent code at a few cycles per instruction, so the merge is cut into two
-// roles that two warps can run side by side when the CTA has warps to spare:
-//   kRoleStats: log-sum-exp over all CTAs, the Gumbel-max winner (column 0 when sampling);
-//   kRoleCand : the topk best list entries over all CTAs (columns 1..topk; column 0 when not sampling).
-// The candidate log-probabilities need the row's lse: the two warps pass it through `xch` (shared memory) and
-// meet at the named barrier `bar_id` (64 threads).  All record loads of a role are issued before their first use.
-constexpr int kRoleCand = 1, kRoleStats = 2;
+// The merge of one hidden row by six warps.  A warp runs dependent code at a few cycles per instruction, and the row's result is what
+// the next step waits for, so the work is spread: five warps hold a CTA's list heads per lane (kRoleCand), the sixth the
+// statistics (log-sum-exp over all CTAs, the Gumbel-max winner).  Everything a warp needs from memory is asked for at once.
+// (Two warps, five CTAs to a lane, took 4150 cycles from the records being there to the outputs, a quarter of them one L2 round
+// trip for the abort mark in front of the records and the gathers through the index mapper behind the ranking.)
+constexpr int kMergeThreads = 32 * (kMaxOwn + 1);
 
-__device__ __noinline__ void merge_records(const MergeOut a, Ctrl* ctrl, float* recs, int b, bool row_ok, int G,
-                                           float* stage, int role, volatile float* xch, int bar_id) {
-    const int lane = threadIdx.x & 31;
-    const int topk = a.topk;
-    const unsigned long long* kp = rec_keys(recs, b, topk);
-    const float* fp = rec_f32(recs, b, topk);
-    const int row_w = 1 + topk;
-    int* oid = a.out_ids + (size_t)b * row_w;
-    float* olp = a.out_logprobs + (size_t)b * row_w;
+struct MergeLoads {                                // what a thread has asked for
+    unsigned long long ek[kMergeDepth];            // candidate warps: the best entries of a CTA's list
+    float hm[kMaxOwn], hs[kMaxOwn], hz[kMaxOwn];   // statistics warp: kMaxOwn CTAs to a lane
+    unsigned long long hk[kMaxOwn];
+};
 
-    const int depth = min(topk, kMergeDepth);
-    unsigned long long ek[kMergeDepth][kMaxOwn];
-    if (role == kRoleCand) {
+// (loads of records that do not exist go to one that does and are not looked at: no branch around any of them)
+__device__ __forceinline__ void merge_request(const MergeOut& a, float* recs, int b, int G, MergeLoads& ld) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const unsigned long long* kp = rec_keys(recs, b, a.topk);
+    if (warp < kMaxOwn) {
+        const int depth = min(a.topk, kMergeDepth), c = min(warp * 32 + lane, G - 1);
 #pragma unroll
-        for (int r = 0; r < kMergeDepth; ++r)
+        for (int r = 0; r < kMergeDepth; ++r) ld.ek[r] = ld_cg_u64(kp + (size_t)(1 + min(r, depth - 1)) * kMaxGrid + c);
+    } else {
+        const float* fp = rec_f32(recs, b, a.topk);
+#pragma unroll
+        for (int o = 0; o < kMaxOwn; ++o) {
+            const int c = min(lane + 32 * o, G - 1);
+            ld.hm[o] = ld_cg_f32(fp + c);
+            ld.hs[o] = ld_cg_f32(fp + kMaxGrid + c);
+        }
+        if (a.sampled) {
 #pragma unroll
             for (int o = 0; o < kMaxOwn; ++o) {
-                const int c = lane + 32 * o;
-                ek[r][o] = (c < G && r < depth) ? ld_cg_u64(kp + (size_t)(1 + r) * kMaxGrid + c) : 0ull;
+                const int c = min(lane + 32 * o, G - 1);
+                ld.hz[o] = ld_cg_f32(fp + 2 * kMaxGrid + c);
+                ld.hk[o] = ld_cg_u64(kp + c);
             }
+        }
     }
+}
 
-    if (role == kRoleStats) {
-        float hm[kMaxOwn], hs[kMaxOwn], hz[kMaxOwn];
-        unsigned long long hk[kMaxOwn];
+__device__ __forceinline__ void merge_stats(const MergeOut& a, Ctrl* ctrl, int b, bool row_ok, int G, MergeLoads& ld, volatile float* xch) {
+    const int lane = threadIdx.x & 31;
+    int* oid = a.out_ids + (size_t)b * (1 + a.topk);
+    float* olp = a.out_logprobs + (size_t)b * (1 + a.topk);
+    // the row's maximum over this lane's CTAs and by one warp reduction, every CTA's sum rescaled to it once, added in
+    // CTA order, a butterfly of additions (a fixed order: the result does not depend on which CTA finished when)
+    float M = -CUDART_INF_F, gz = 0.f;
+    unsigned long long gk = 0ull;
+#pragma unroll
+    for (int o = 0; o < kMaxOwn; ++o) {
+        const bool on = lane + 32 * o < G;
+        ld.hm[o] = on ? ld.hm[o] : -CUDART_INF_F;
+        ld.hs[o] = on ? ld.hs[o] : 0.f;
+        M = fmaxf(M, ld.hm[o]);
+    }
+    if (a.sampled) {
 #pragma unroll
         for (int o = 0; o < kMaxOwn; ++o) {
-            const int c = lane + 32 * o;
-            const bool on = c < G;
-            hm[o] = on ? ld_cg_f32(fp + c) : -CUDART_INF_F;
-            hs[o] = on ? ld_cg_f32(fp + kMaxGrid + c) : 0.f;
-            hz[o] = (on && a.sampled) ? ld_cg_f32(fp + 2 * kMaxGrid + c) : 0.f;
-            hk[o] = (on && a.sampled) ? ld_cg_u64(kp + c) : 0ull;
+            const bool w = lane + 32 * o < G && ld.hk[o] > gk;
+            gk = w ? ld.hk[o] : gk;
+            gz = w ? ld.hz[o] : gz;
         }
-        // the row's maximum over this lane's CTAs and by one warp reduction, every CTA's sum rescaled to it once, added in
-        // CTA order, a butterfly of additions (a fixed order: the result does not depend on which CTA finished when)
-        float M = hm[0], gz = 0.f;
-        unsigned long long gk = 0ull;
+    }
+    const float Mall = ord2f(__reduce_max_sync(0xffffffffu, f2ord(M)));
+    const float Mref = Mall == -CUDART_INF_F ? 0.f : Mall;
+    float sc = 0.f;
 #pragma unroll
-        for (int o = 1; o < kMaxOwn; ++o) M = fmaxf(M, hm[o]);
+    for (int o = 0; o < kMaxOwn; ++o) sc += ld.hs[o] * exp_fast(ld.hm[o] - Mref);     // (hm = -inf: nothing but a NaN sum counts)
 #pragma unroll
-        for (int o = 0; o < kMaxOwn; ++o) {
-            const bool w = hk[o] > gk;
-            gk = w ? hk[o] : gk;
-            gz = w ? hz[o] : gz;
-        }
-        const float Mall = ord2f(__reduce_max_sync(0xffffffffu, f2ord(M)));
-        const float Mref = Mall == -CUDART_INF_F ? 0.f : Mall;
-        float sc = 0.f;
-#pragma unroll
-        for (int o = 0; o < kMaxOwn; ++o) sc += hs[o] * exp_fast(hm[o] - Mref);   // (hm = -inf: nothing but a NaN sum counts)
-#pragma unroll
-        for (int o = 16; o; o >>= 1) sc += __shfl_xor_sync(0xffffffffu, sc, o);
-        const float lse = Mall + logf(sc);
-        if (lane == 0) *xch = lse;                          // the candidate warp of this row is waiting for it
-        asm volatile("bar.sync %0, 64;" ::"r"(bar_id) : "memory");
-        unsigned long long gwin = 0ull;
-        float gzw = 0.f;
+    for (int o = 16; o; o >>= 1) sc += __shfl_xor_sync(0xffffffffu, sc, o);
+    const float lse = Mall + logf(sc);
+    if (lane == 0) *xch = lse;                              // the ranking warp is waiting for it
+    __syncwarp();
+    asm volatile("bar.arrive 2, 64;" ::: "memory");
+    unsigned long long gwin = 0ull;
+    float gzw = 0.f;
+    if (a.sampled) {
+        const unsigned hi = (unsigned)(gk >> 32);
+        const unsigned kmax = __reduce_max_sync(0xffffffffu, hi);
+        const unsigned lomax = __reduce_max_sync(0xffffffffu, hi == kmax ? (unsigned)gk : 0u);
+        const unsigned who = __ballot_sync(0xffffffffu, hi == kmax && (unsigned)gk == lomax);
+        gzw = __shfl_sync(0xffffffffu, gz, __ffs(who) - 1);
+        gwin = ((unsigned long long)kmax << 32) | lomax;
+    }
+    if (lane == 0) {
+        bool bad = !(lse == lse);                           // a NaN logit somewhere in the row
         if (a.sampled) {
-            const unsigned hi = (unsigned)(gk >> 32);
-            const unsigned kmax = __reduce_max_sync(0xffffffffu, hi);
-            const unsigned lomax = __reduce_max_sync(0xffffffffu, hi == kmax ? (unsigned)gk : 0u);
-            const unsigned who = __ballot_sync(0xffffffffu, hi == kmax && (unsigned)gk == lomax);
-            gzw = __shfl_sync(0xffffffffu, gz, __ffs(who) - 1);
-            gwin = ((unsigned long long)kmax << 32) | lomax;
+            const bool ok = row_ok && gwin != 0ull;
+            const int gj = key_idx(gwin);
+            oid[0] = ok ? (a.map ? ld_cg_s32(a.map + gj) : gj) : -1;
+            olp[0] = ok ? gzw - lse : CUDART_NAN_F;
+            bad = bad || !ok;
         }
-        if (lane == 0) {
-            bool bad = !(lse == lse);                       // a NaN logit somewhere in the row
-            if (a.sampled) {
-                const bool ok = row_ok && gwin != 0ull;
-                const int gj = key_idx(gwin);
-                oid[0] = ok ? (a.map ? ld_cg_s32(a.map + gj) : gj) : -1;
-                olp[0] = ok ? gzw - lse : CUDART_NAN_F;
-                bad = bad || !ok;
-            }
-            if (a.dbg_lse) a.dbg_lse[b] = lse;
-            if (!row_ok) atomicOr(&ctrl->flags, (uint32_t)VT_FLAG_BAD_TEMP);
-            else if (bad) atomicOr(&ctrl->flags, (uint32_t)VT_FLAG_NAN_ROW);
-        }
-        return;
+        if (a.dbg_lse) a.dbg_lse[b] = lse;
+        if (!row_ok) atomicOr(&ctrl->flags, (uint32_t)VT_FLAG_BAD_TEMP);
+        else if (bad) atomicOr(&ctrl->flags, (uint32_t)VT_FLAG_NAN_ROW);
     }
+}
 
-    unsigned long long res_k[2] = {0ull, 0ull};
-    unsigned long long* stk = reinterpret_cast<unsigned long long*>(stage);        // [kMergeDepth][kMaxGrid] list heads
-    unsigned long long* sel = stk;                                                 // [kSelCap] (in the same place: one or the other)
-    unsigned long long* outk = sel + kSelCap + 4;                                  // [64] (behind four words of padding)
-    bool done = false;
-    if (topk <= 32) {
-        // Direct selection.  tau = the topk-th largest of the 32 lanes' best list heads is a lower
-        // bound of the topk-th best entry overall, so only staged entries >= tau can matter: a few
-        // dozen at most.  They are compacted into shared memory and every one finds its output
-        // position as its rank -- no sequential rounds.  Falls back to the rounds below when a list
-        // might hold qualifying entries beyond the staged ones, or when too many qualify.
-        unsigned lh = 0u;
+// Entry `key` of the merged list is the r-th best (r < topk): id and log-probability.  The id is asked for before the ranking.
+__device__ __forceinline__ void merge_emit(const MergeOut& a, int b, int r, int id, unsigned long long key, bool row_ok, float lse) {
+    int* oid = a.out_ids + (size_t)b * (1 + a.topk);
+    float* olp = a.out_logprobs + (size_t)b * (1 + a.topk);
+    const bool ok = row_ok && key != 0ull;
+    id = ok ? id : -1;
+    const float lp = ok ? key_val(key) - lse : CUDART_NAN_F;
+    oid[1 + r] = id;
+    olp[1 + r] = lp;
+    if (r == 0 && !a.sampled) { oid[0] = id; olp[0] = lp; }
+}
+__device__ __forceinline__ int merge_id(const MergeOut& a, unsigned long long key) {
+    const int j = key != 0ull ? key_idx(key) : 0;
+    return a.map ? ld_cg_s32(a.map + j) : j;
+}
+
+// Ranks the n keys in sel (NS to a lane) and writes the topk best of them.
+template <int NS>
+__device__ __forceinline__ void merge_rank(const MergeOut& a, const unsigned long long* sel, int n, int b, bool row_ok, volatile float* xch) {
+    const int lane = threadIdx.x & 31;
+    unsigned long long mine[NS];
+    int rk[NS], id[NS];
 #pragma unroll
-        for (int o = 0; o < kMaxOwn; ++o) {
-            const unsigned h = (unsigned)(ek[0][o] >> 32);
-            lh = h > lh ? h : lh;
-        }
-        const unsigned tau = kth_of_lanes(lh, topk, reinterpret_cast<unsigned*>(stage));
-        outk[lane] = 0ull;
-        outk[lane + 32] = 0ull;
-        // compaction: every lane counts its qualifying entries, a warp scan gives it a place to put them
-        int mine_n = 0;
+    for (int i = 0; i < NS; ++i) {
+        mine[i] = lane + 32 * i < n ? sel[lane + 32 * i] : 0ull;
+        rk[i] = 0;
+    }
+#pragma unroll
+    for (int i = 0; i < NS; ++i) id[i] = merge_id(a, mine[i]);
+    rank_among<NS>(sel, n, mine, rk);
+    asm volatile("bar.sync 2, 64;" ::: "memory");
+    const float lse = *xch;
+#pragma unroll
+    for (int i = 0; i < NS; ++i)
+        if (lane + 32 * i < n && rk[i] < a.topk) merge_emit(a, b, rk[i], id[i], mine[i], row_ok, lse);
+    for (int r = n + lane; r < a.topk; r += 32) merge_emit(a, b, r, -1, 0ull, row_ok, lse);          // fewer than topk candidates
+}
+
+__device__ __forceinline__ void merge_candidates(const MergeOut& a, Ctrl* ctrl, float* recs, int b, bool row_ok, int G, MergeLoads& ld,
+                                                 float* stage, int* s_n, int* s_deep, volatile float* xch) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int topk = a.topk, depth = min(topk, kMergeDepth), c = warp * 32 + lane;
+    unsigned long long* sel = reinterpret_cast<unsigned long long*>(stage);                    // [kSelCap] and padding
+    unsigned* heads = reinterpret_cast<unsigned*>(stage) + 2 * (kSelCap + 8);                  // [kMaxGrid]
+    unsigned* kth = heads + kMaxGrid + warp * 32;
+    static_assert(2 * (kSelCap + 8) + 2 * kMaxGrid <= kMergeStageWords, "the selection's words fit");
+#pragma unroll
+    for (int r = 0; r < kMergeDepth; ++r) ld.ek[r] = c < G && r < depth ? ld.ek[r] : 0ull;
+    bool direct = topk <= 32;
+    if (direct) {
+        // Direct selection.  tau = the topk-th largest of 32 maxima over five list heads each is a lower bound of the topk-th
+        // best entry overall, so only staged entries >= tau can matter: a few dozen at most.  They are compacted into shared
+        // memory and every one finds its output position as its rank -- no sequential rounds.  Falls back to the rounds below
+        // when a list might hold qualifying entries beyond the staged ones, or when too many qualify.
+        heads[c] = (unsigned)(ld.ek[0] >> 32);
+        asm volatile("bar.sync 1, %0;" ::"n"(32 * kMaxOwn) : "memory");
+        unsigned lh = heads[lane];
+#pragma unroll
+        for (int o = 1; o < kMaxOwn; ++o) lh = max(lh, heads[lane + 32 * o]);
+        const unsigned tau = kth_of_lanes(lh, topk, kth);
+        unsigned m[kMergeDepth];
+        int total = 0;
         bool deep = false;
 #pragma unroll
-        for (int r = 0; r < kMergeDepth; ++r)
-#pragma unroll
-            for (int o = 0; o < kMaxOwn; ++o) {
-                const bool in = ek[r][o] != 0ull && (unsigned)(ek[r][o] >> 32) >= tau;
-                mine_n += in ? 1 : 0;
-                deep = deep || (in && r == depth - 1 && depth < topk);
+        for (int r = 0; r < kMergeDepth; ++r) {
+            const bool in = ld.ek[r] != 0ull && (unsigned)(ld.ek[r] >> 32) >= tau;
+            m[r] = __ballot_sync(0xffffffffu, in);
+            total += __popc(m[r]);
+            deep = deep || (r == depth - 1 && depth < topk && m[r] != 0u);
+        }
+        if (total) {                                        // (warp-uniform; the order among the warps does not matter, ranks decide)
+            int base = 0;
+            if (lane == 0) {
+                base = atomicAdd(s_n, total);
+                if (deep) *s_deep = 1;
             }
-        int pos = mine_n;
+            base = __shfl_sync(0xffffffffu, base, 0);
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int y = __shfl_up_sync(0xffffffffu, pos, o);
-            pos += (lane >= o) ? y : 0;
+            for (int r = 0; r < kMergeDepth; ++r) {
+                const int pos = base + __popc(m[r] & lanemask_lt());
+                if (((m[r] >> lane) & 1u) && pos < kSelCap) sel[pos] = ld.ek[r];
+                base += __popc(m[r]);
+            }
         }
-        const int n = __shfl_sync(0xffffffffu, pos, 31);
-        pos -= mine_n;
-        if (n <= kSelCap) {
-#pragma unroll
-            for (int r = 0; r < kMergeDepth; ++r)
-#pragma unroll
-                for (int o = 0; o < kMaxOwn; ++o)
-                    if (ek[r][o] != 0ull && (unsigned)(ek[r][o] >> 32) >= tau) sel[pos++] = ek[r][o];
-        }
-        if (n <= kSelCap && !__any_sync(0xffffffffu, deep)) {
+        asm volatile("bar.sync 1, %0;" ::"n"(32 * kMaxOwn) : "memory");
+        const int n = *s_n;
+        direct = n <= kSelCap && !*s_deep;
+        if (direct) {
+            if (warp != 0) return;
             if (lane < 4) sel[n + lane] = 0ull;                                    // (read in groups of four)
             __syncwarp();
-            if (n <= 32) {                                                         // the usual case: one entry per lane
-                const unsigned long long mine[1] = {lane < n ? sel[lane] : 0ull};
-                int r1[1] = {0};
-                rank_among<1>(sel, n, mine, r1);
-                if (lane < n && r1[0] < topk) outk[r1[0]] = mine[0];
-            } else {
-                unsigned long long mine[kSelCap / 32];
-                int rk4[kSelCap / 32];
+            if (n <= 32) merge_rank<1>(a, sel, n, b, row_ok, xch);
+            else merge_rank<kSelCap / 32>(a, sel, n, b, row_ok, xch);
+            if (lane == 0 && row_ok && n < topk) atomicOr(&ctrl->flags, (uint32_t)VT_FLAG_NAN_ROW);
+            return;
+        }
+        asm volatile("bar.sync 1, %0;" ::"n"(32 * kMaxOwn) : "memory");            // (the words are given up)
+    }
+    // heads of the lists: entry r of CTA c at stk[r * kMaxGrid + c]
+    unsigned long long* stk = sel;
 #pragma unroll
-                for (int i = 0; i < kSelCap / 32; ++i) {
-                    mine[i] = (lane + 32 * i < n) ? sel[lane + 32 * i] : 0ull;
-                    rk4[i] = 0;
+    for (int r = 0; r < kMergeDepth; ++r) stk[r * kMaxGrid + c] = ld.ek[r];
+    asm volatile("bar.sync 1, %0;" ::"n"(32 * kMaxOwn) : "memory");
+    if (warp != 0) return;
+    // k rounds of one warp; every lane keeps the current head of each of its lists in registers, a round is two
+    // warp reductions, and the winner alone advances (from the staged entries, else from global memory)
+    const unsigned long long* kp = rec_keys(recs, b, topk);
+    unsigned long long res_k[2] = {0ull, 0ull};
+    int head[kMaxOwn];
+    unsigned long long ck[kMaxOwn];
+#pragma unroll
+    for (int o = 0; o < kMaxOwn; ++o) {
+        head[o] = 0;
+        ck[o] = stk[lane + 32 * o];
+    }
+    for (int r = 0; r < topk; ++r) {
+        unsigned long long lk = ck[0];
+#pragma unroll
+        for (int o = 1; o < kMaxOwn; ++o) lk = ck[o] > lk ? ck[o] : lk;
+        const unsigned hi = (unsigned)(lk >> 32);
+        const unsigned kmax = __reduce_max_sync(0xffffffffu, hi);
+        const unsigned lomax = __reduce_max_sync(0xffffffffu, hi == kmax ? (unsigned)lk : 0u);
+        if (kmax == 0u) break;                                // every list is exhausted
+        const unsigned long long win = ((unsigned long long)kmax << 32) | lomax;
+        if (lk == win) {                                      // one lane: advance the list it came from
+#pragma unroll
+            for (int o = 0; o < kMaxOwn; ++o)
+                if (ck[o] == win) {
+                    const int hd = ++head[o];
+                    unsigned long long nk = 0ull;
+                    if (hd < depth) nk = stk[hd * kMaxGrid + lane + 32 * o];
+                    else if (hd < topk) nk = ld_cg_u64(kp + (size_t)(1 + hd) * kMaxGrid + lane + 32 * o);
+                    ck[o] = nk;
                 }
-                rank_among<kSelCap / 32>(sel, n, mine, rk4);
-#pragma unroll
-                for (int i = 0; i < kSelCap / 32; ++i)
-                    if (lane + 32 * i < n && rk4[i] < topk) outk[rk4[i]] = mine[i];
-            }
-            __syncwarp();
-            res_k[0] = outk[lane];
-            done = true;
         }
+        if (lane == r) res_k[0] = win;
+        if (lane + 32 == r) res_k[1] = win;
     }
-    if (!done) {
-        __syncwarp();                                                              // (the selection buffer has been given up)
-        // heads of the lists: entry r of CTA c at stk[r * kMaxGrid + c]
-#pragma unroll
-        for (int o = 0; o < kMaxOwn; ++o)
-#pragma unroll
-            for (int r = 0; r < kMergeDepth; ++r) stk[r * kMaxGrid + lane + 32 * o] = ek[r][o];
-        __syncwarp();
-        // k rounds; every lane keeps the current head of each of its lists in registers, a round is two
-        // warp reductions, and the winner alone advances (from the staged entries, else from global memory)
-        int head[kMaxOwn];
-        unsigned long long ck[kMaxOwn];
-#pragma unroll
-        for (int o = 0; o < kMaxOwn; ++o) {
-            head[o] = 0;
-            ck[o] = ek[0][o];
-        }
-        for (int r = 0; r < topk; ++r) {
-            unsigned long long lk = ck[0];
-#pragma unroll
-            for (int o = 1; o < kMaxOwn; ++o) lk = ck[o] > lk ? ck[o] : lk;
-            const unsigned hi = (unsigned)(lk >> 32);
-            const unsigned kmax = __reduce_max_sync(0xffffffffu, hi);
-            const unsigned lomax = __reduce_max_sync(0xffffffffu, hi == kmax ? (unsigned)lk : 0u);
-            if (kmax == 0u) break;                                // every list is exhausted
-            const unsigned long long win = ((unsigned long long)kmax << 32) | lomax;
-            if (lk == win) {                                      // one lane: advance the list it came from
-#pragma unroll
-                for (int o = 0; o < kMaxOwn; ++o)
-                    if (ck[o] == win) {
-                        const int c = lane + 32 * o;
-                        const int hd = ++head[o];
-                        unsigned long long nk = 0ull;
-                        if (hd < depth) nk = stk[hd * kMaxGrid + c];
-                        else if (hd < topk) nk = ld_cg_u64(kp + (size_t)(1 + hd) * kMaxGrid + c);
-                        ck[o] = nk;
-                    }
-            }
-            if (lane == (r & 31)) res_k[r >> 5] = win;
-        }
-    }
-    // the gathers through the index mapper go out before the wait for the row's lse
-    int ids[2];
-    float zv[2];
-    bool okv[2];
-#pragma unroll
-    for (int sl = 0; sl < 2; ++sl) {
-        const int r = lane + 32 * sl;
-        okv[sl] = r < topk && row_ok && res_k[sl] != 0ull;
-        ids[sl] = okv[sl] ? key_idx(res_k[sl]) : 0;
-        zv[sl] = key_val(res_k[sl]);
-    }
-    if (a.map) {                                            // (both loads unconditional: no branch around either)
-        const int i0 = ld_cg_s32(a.map + ids[0]), i1 = ld_cg_s32(a.map + ids[1]);
-        ids[0] = i0;
-        ids[1] = i1;
-    }
-    ids[0] = okv[0] ? ids[0] : -1;
-    ids[1] = okv[1] ? ids[1] : -1;
-    asm volatile("bar.sync %0, 64;" ::"r"(bar_id) : "memory");
+    const int ids[2] = {merge_id(a, res_k[0]), merge_id(a, res_k[1])};
+    asm volatile("bar.sync 2, 64;" ::: "memory");
     const float lse = *xch;
     bool miss = false;
 #pragma unroll
     for (int sl = 0; sl < 2; ++sl) {
         const int r = lane + 32 * sl;
         if (r < topk) {
-            const float lp = okv[sl] ? zv[sl] - lse : CUDART_NAN_F;
-            oid[1 + r] = ids[sl];
-            olp[1 + r] = lp;
-            if (!okv[sl]) miss = true;
-            if (r == 0 && !a.sampled) { oid[0] = ids[sl]; olp[0] = lp; }
+            merge_emit(a, b, r, ids[sl], res_k[sl], row_ok, lse);
+            miss = miss || res_k[sl] == 0ull;
         }
     }
     const bool any_missing = __any_sync(0xffffffffu, miss);

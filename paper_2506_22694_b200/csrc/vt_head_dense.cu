@@ -23,7 +23,7 @@
 // columns each -- 16 columns at a time: running max / sum-exp of z = logit / T_b, Gumbel-max candidate
 // from the caller's uniforms, and a sorted top-k list kept in registers.  Logits never go to HBM.  The
 // two column halves of a row are merged through shared memory; per CTA (pair) and hidden row one
-// record goes to scratch; a second small kernel (two warps per hidden row) merges the records,
+// record goes to scratch; a second small kernel (six warps per hidden row) merges the records,
 // applies the index mapper and writes the outputs.  Every wait is bounded; on expiry the CTA raises
 // VT_FLAG_TIMEOUT and leaves after releasing its tensor memory.
 #include <cfloat>
@@ -768,36 +768,45 @@ k_head_dense(const HeadArgs a, Ctrl* ctrl, float* __restrict__ recs, const Dense
 #endif
 }
 
-// Two warps per hidden row (candidates / statistics): merge the CTA records, remap, write the outputs.  After a
-// wait that expired somewhere the records are incomplete: every row is reported as missing.  FUSE: tree drafting --
-// the block that finishes last turns the merged candidates into pool nodes and chooses the next frontier, so that
-// a tree depth needs no launch for it.  (Dynamic shared memory, sized by the need: the block has to fit beside the
-// head kernel's CTA to take its seat early.)
-constexpr int kFuseNodes = 64;                                    // new nodes that a block of 64 threads expands (see launch_head_merge)
-__global__ void __launch_bounds__(64)
+// A block of six warps per hidden row: merge the CTA records, remap, write the outputs.  After a wait that expired somewhere the records are
+// incomplete: every row is reported as missing.  FUSE: tree drafting -- the block that finishes last turns the merged
+// candidates into pool nodes and chooses the next frontier, so that a tree depth needs no launch for it.  (Dynamic shared
+// memory, sized by the need: the block has to fit beside the head kernel's CTA to take its seat early.)
+// Bound by latency: two L2 round trips (records; index mapper, behind the ranking) and about ten short dependent phases.  us per
+// chained step, two warps per row and a round trip more / this: one row of 5000 x 1024 9.7 / 8.7, of 32768 x 3072 31.6 / 30.5, 8
+// rows of 9973 x 3072 17.6 / 16.7, 100 rows of 20001 x 3072 37.3 / 35.3.
+constexpr int kFuseNodes = 64;                                    // new nodes that the last block expands (see launch_head_merge)
+__global__ void __launch_bounds__(kMergeThreads)
 k_head_merge(const HeadArgs a, Ctrl* ctrl, float* __restrict__ recs, int G, int fuse) {
     extern __shared__ __align__(16) float s_stage[];              // [kMergeStageWords], and over it the keys of the expansion
     __shared__ float s_xch;
-    __shared__ int s_last;
+    __shared__ int s_last, s_n, s_deep;
     const int b = blockIdx.x;
     griddep_launch_dependents();                                  // the next step may start fetching its weights
+    if (threadIdx.x == 0) { s_n = 0; s_deep = 0; }
+    __syncthreads();
     griddep_wait();                                               // the records are complete
 #ifdef VT_STAMPS
     unsigned long long* stamps = reinterpret_cast<unsigned long long*>(
         reinterpret_cast<uint8_t*>(recs) + align_up_dev((size_t)kMaxGrid * a.B * rec_fields(a.topk) * 4, 256));
     if (b == 0 && threadIdx.x == 0) stamps[12] = global_ns();
 #endif
-    const bool aborted = *reinterpret_cast<volatile uint32_t*>(&ctrl->head_aborted) != 0u;
+    // (everything is on its way before the mark is looked at: a round trip to L2 is a fifth of the merge)
+    const uint32_t mark = ld_cg_u32(&ctrl->head_aborted);
+    const float T = ld_cg_f32(a.temp + b);
+    const MergeOut mo{a.map, a.out_ids, a.out_logprobs, a.dbg_lse, a.topk, a.uniforms != nullptr};
+    MergeLoads ld;
+    merge_request(mo, recs, b, G, ld);
+    const bool aborted = mark != 0u;
     if (aborted) {
-        for (int i = threadIdx.x; i < 1 + a.topk; i += 64) {
+        for (int i = threadIdx.x; i < 1 + a.topk; i += kMergeThreads) {
             a.out_ids[(size_t)b * (1 + a.topk) + i] = -1;
             a.out_logprobs[(size_t)b * (1 + a.topk) + i] = CUDART_NAN_F;
         }
     } else {
-        const float T = a.temp[b];
         const bool row_ok = (T > 0.f) && (T < CUDART_INF_F);
-        const MergeOut mo{a.map, a.out_ids, a.out_logprobs, a.dbg_lse, a.topk, a.uniforms != nullptr};
-        merge_records(mo, ctrl, recs, b, row_ok, G, s_stage, threadIdx.x < 32 ? kRoleCand : kRoleStats, &s_xch, 1);
+        if (threadIdx.x < 32 * kMaxOwn) merge_candidates(mo, ctrl, recs, b, row_ok, G, ld, s_stage, &s_n, &s_deep, &s_xch);
+        else merge_stats(mo, ctrl, b, row_ok, G, ld, &s_xch);
     }
 #ifdef VT_STAMPS
     if (b == 0 && threadIdx.x == 0) stamps[13] = global_ns();
@@ -816,7 +825,7 @@ k_head_merge(const HeadArgs a, Ctrl* ctrl, float* __restrict__ recs, int G, int 
     __syncthreads();
     if (!s_last || !fuse) return;
     tree_expand_block(a.tree, a.out_ids, a.out_logprobs, a.B, a.topk, 1 + a.topk, 1, reinterpret_cast<unsigned long long*>(s_stage),
-                      (int)threadIdx.x, 64);
+                      (int)threadIdx.x, kMergeThreads);
 }
 
 // ---- host side ----------------------------------------------------------------------------------------
@@ -935,13 +944,13 @@ cudaError_t launch_head_dense(const HeadArgs& a, Ctrl* ctrl, uint8_t* scratch, c
 cudaError_t launch_head_merge(const HeadArgs& a, Ctrl* ctrl, float* recs, int G, cudaStream_t s) {
     // the merge always follows its own producer closely: it takes its seats early and waits on the device
     const int n_new = a.B * a.topk;
-    // The expansion inside the merge saves a launch; as a kernel of its own it has sixteen times the threads.  What decides is
-    // one node per thread (us per depth, fused / kernel, heads of 60, 128, 268 MB: 8 nodes 15.1 / 16.1, 23.3 / 24.0, 41.9 / 42.3; 64
-    // nodes 15.5 / 17.2, 23.8 / 24.8, 42.6 / 43.0; 100 nodes 20.7 / 20.7, 27.8 / 26.3, 46.0 / 44.7; 512 nodes 43.5 / 28.3, 49.3 / 34.8, 70.4 / 55.7).
+    // The expansion inside the merge saves a launch; as a kernel of its own it has more threads, and the blocks need not meet.  Up to
+    // 64 new nodes the one wins, from there to 170 neither, beyond the other (us per depth of a tree over 9973 x 3072, fused /
+    // kernel: 64 nodes 19.0 / 19.9, 100 nodes 22.9 / 22.7, 144 nodes 23.5 / 23.8, 169 nodes 25.1 / 24.8, 256 nodes 29.6 / 28.2).
     const bool fuse = a.tree.pool_token && n_new <= kFuseNodes;
     size_t smem = (size_t)kMergeStageWords * 4;
     if (fuse && (size_t)padded_keys(n_new) * 8 > smem) smem = (size_t)padded_keys(n_new) * 8;
-    const cudaError_t e = launch_dependent(k_head_merge, (unsigned)a.B, 64, smem, s, a, ctrl, recs, G, fuse ? 1 : 0);
+    const cudaError_t e = launch_dependent(k_head_merge, (unsigned)a.B, kMergeThreads, smem, s, a, ctrl, recs, G, fuse ? 1 : 0);
     if (e != cudaSuccess || !a.tree.pool_token || fuse) return e;
     return launch_tree_expand(a.out_ids, a.out_logprobs, a.B, a.topk, 1 + a.topk, 1, a.tree, s);
 }

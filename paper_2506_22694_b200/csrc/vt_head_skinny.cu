@@ -20,7 +20,7 @@
 // memory; then warp w owns hidden rows w, w + EW, ...: its lanes walk the tile's rows, updating running
 // max / sum-exp of z = logit / T, the Gumbel-max candidate from the caller's uniforms and the row's sorted
 // top-k list.  Logits never go to HBM.  Each CTA leaves one small record per hidden row; a second kernel, one
-// pair of warps per row, merges them in CTA order, remaps trimmed indices through `map` and writes the outputs
+// block per row, merges them in CTA order, remaps trimmed indices through `map` and writes the outputs
 // (vt_head_dense.cu).  It takes its seats while this one runs, and a CTA here is gone as soon as its record is
 // written, which lets the next step's weights in; the merge by the last CTA to finish (atomic ticket) kept them
 // out for its 4-6 us (us per chained step, one CTA / second kernel: 1 row of 5000 x 2048 14.8 / 11.7, 10 rows of
