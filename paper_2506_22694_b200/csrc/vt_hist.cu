@@ -10,7 +10,8 @@
 //     field notices, and the stream is then counted again by the kernels of the next case.
 //   * more bins than that, in two to four ranges that fit: the same kernel, every range dealt to its own share of
 //     the CTAs, each share reading the whole stream (the second and later readers find it in L2).
-//   * the recount: a short pre-pass samples the stream, picks the hottest bins that fit (about 49.8 K of
+//   * the recount, of shorter streams: ranges of 57344 32-bit bins, by the kernel that settles the packed count;
+//   * the recount of longer ones, and long streams over more bins than three counters per word hold: a short pre-pass samples the stream, picks the hottest bins that fit (about 49.8 K of
 //     them for 128256 bins), and the main pass keeps those in shared memory; the rare cold tokens go
 //     to L2 with one red.global each.  The hot set only steers traffic: counts are exact whichever
 //     bins were picked.
@@ -34,23 +35,23 @@ static_assert(kPickBins == kThreads, "one pick bin per thread");
 constexpr int kPickLoads = 16;                 // loads each thread of the one-CTA pick keeps in flight
 
 // ---- streaming loop shared by the counting kernels ---------------------------------------------
-// The CTA's share of the 16-byte-aligned body is read with four independent 128-bit loads per
-// thread per trip; the unaligned head/tail (at most 3 + 3 ids) is handled by CTA 0.
+// A share of the 16-byte-aligned body is read with four independent 128-bit loads per
+// thread per trip; the unaligned head/tail (at most 3 + 3 ids) goes to share 0.
 template <class F>
-__device__ __forceinline__ void stream_ids(const int32_t* __restrict__ ids, int64_t n, F&& tally) {
+__device__ __forceinline__ void stream_ids(const int32_t* __restrict__ ids, int64_t n, F&& tally, int share, int shares) {
     const uintptr_t addr = reinterpret_cast<uintptr_t>(ids);
     int64_t head = ((16 - (addr & 15)) & 15) >> 2;
     if (head > n) head = n;
     const int64_t nvec = (n - head) >> 2;
     const int64_t tail0 = head + nvec * 4;
-    if (blockIdx.x == 0) {
+    if (share == 0) {
         if ((int64_t)threadIdx.x < head) tally((uint32_t)ids[threadIdx.x]);
         const int64_t t = tail0 + threadIdx.x;
         if (t < n) tally((uint32_t)ids[t]);
     }
     const uint4* vec = reinterpret_cast<const uint4*>(ids + head);
-    const int64_t v0 = nvec * blockIdx.x / gridDim.x;
-    const int64_t v1 = nvec * (blockIdx.x + 1) / gridDim.x;
+    const int64_t v0 = nvec * share / shares;
+    const int64_t v1 = nvec * (share + 1) / shares;
     for (int64_t v = v0 + threadIdx.x; v < v1; v += 4 * kThreads) {
         uint4 a = ld_stream_u4(vec + v), b, c, d;
         const bool pb = v + kThreads < v1, pc = v + 2 * kThreads < v1, pd = v + 3 * kThreads < v1;
@@ -449,7 +450,22 @@ k_hist_hot(const int32_t* __restrict__ ids, int64_t n, int32_t V, uint32_t* __re
 constexpr uint32_t kFieldBits = 10, kFieldMax = (1u << kFieldBits) - 1, kSpill = 512;
 constexpr uint32_t kNoId = 0xffffffffu;        // no token id: ids are tallied only when < V <= 2^31
 constexpr int kCarefulTrips = 2;               // trips a CTA counts one add at a time, until its hot id is known
-constexpr int kGateWords = 4;                  // {recount, unused, skipped ids (64 bits)}
+constexpr int kGateWords = 4;                  // {recount, CTAs that have recounted, skipped ids (64 bits)}
+constexpr int kFlushCtas = 2;                  // CTAs (a cluster) that flush together
+constexpr int kFlushLoads = 4;                 // words of the peer a thread has in flight
+
+__device__ __forceinline__ void cluster_arrive() { __syncwarp(); asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { __syncwarp(); asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+__device__ __forceinline__ uint32_t peer_smem(uint32_t addr, uint32_t rank) {
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+    return r;
+}
+__device__ __forceinline__ uint32_t ld_peer_u32(uint32_t addr) {
+    uint32_t v;
+    asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
+    return v;
+}
 
 // Words per CTA for V bins, 0 when they do not fit: the smallest W >= ceil(V / 3) for which
 // field = (id * M) >> 32 with M = 2^32 / W + 1 is exact for every id < 3W (the quotient steps at W and 2W:
@@ -467,9 +483,15 @@ static uint32_t packed_words(int32_t V, uint32_t* magic) {
     return 0;
 }
 
-// SPLIT: the vocabulary is cut into `parts` ranges of Vp ids; CTA c counts range c % parts of share c / parts of the
-// stream, and a token outside the CTA's range costs the instructions but not the add.  (Neighbouring CTAs read the
+// SPLIT: the vocabulary is cut into `parts` ranges of Vp ids; the CTAs of cluster c count range c % parts of their shares of
+// the stream, and a token outside the CTA's range costs the instructions but not the add.  (Neighbouring clusters read the
 // same ids at about the same time: one of them from HBM, the others from L2.)
+//
+// The flush is bound by the 32-byte sectors that L2 adds to (about 110 a cycle): every CTA touches nearly all of them, 20 K
+// cycles for 128256 bins, of 32 K that a call of 3e6 ids took.  So two CTAs of a cluster flush together, each one half of
+// the words with both CTAs' counts, its peer's read through distributed shared memory.  (With that and without the two launches
+// of the recount, us per call: V = 128256 1e5 / 3e6 / 4e7 / 1e9 ids 21.8 / 28.1 / 60.9 / 759 -> 17.7 / 22.4 / 55.4 / 755; V = 256000 3e6 /
+// 4e7 34.5 / 105.5 -> 29.2 / 99.0.)
 template <bool SPLIT, bool SHORT>
 __global__ void __launch_bounds__(kThreads, 1)
 k_hist_packed(const int32_t* __restrict__ ids, int64_t n, int32_t V, int32_t Vp, int32_t parts, uint32_t W, uint32_t M,
@@ -477,12 +499,13 @@ k_hist_packed(const int32_t* __restrict__ ids, int64_t n, int32_t V, int32_t Vp,
     extern __shared__ __align__(16) uint32_t s_fields[];
     __shared__ uint32_t s_hot;
     __shared__ uint32_t s_own[32];                           // the hot id's counts, one word per lane
-    const int part = SPLIT ? (int)blockIdx.x % parts : 0;
-    const int share = SPLIT ? (int)blockIdx.x / parts : (int)blockIdx.x, shares = SPLIT ? (int)gridDim.x / parts : (int)gridDim.x;
+    const int rank = (int)blockIdx.x % kFlushCtas, cluster = (int)blockIdx.x / kFlushCtas;
+    const int part = SPLIT ? cluster % parts : 0;
+    const int share = SPLIT ? cluster / parts * kFlushCtas + rank : (int)blockIdx.x, shares = SPLIT ? (int)gridDim.x / parts : (int)gridDim.x;
     const uint32_t lo = SPLIT ? (uint32_t)part * (uint32_t)Vp : 0u;       // first id of the CTA's range
     const uint32_t mine = SPLIT ? min((uint32_t)Vp, (uint32_t)V - lo) : (uint32_t)V;
     uint32_t* __restrict__ out = all_out + lo;               // (ids are relative to lo from the range test on)
-    for (uint32_t i = threadIdx.x; i < W; i += kThreads) s_fields[i] = 0;
+    for (uint32_t i = threadIdx.x; i < (W + 3) / 4; i += kThreads) reinterpret_cast<uint4*>(s_fields)[i] = make_uint4(0, 0, 0, 0);
     if (threadIdx.x == 0) s_hot = kNoId;
     if (threadIdx.x < 32) s_own[threadIdx.x] = 0;
     __syncthreads();
@@ -629,18 +652,34 @@ k_hist_packed(const int32_t* __restrict__ ids, int64_t n, int32_t V, int32_t Vp,
         for (int64_t v = v0 + trips * (kRows * kThreads) + threadIdx.x; v < v1; v += kThreads) tally4_in_turn(ld_stream_u4(vec + v));
     }
     griddep_launch_dependents();                             // (the settling kernel waits for this one's end)
-    __syncthreads();
-    const uint32_t first = blockIdx.x * (W / gridDim.x);         // the CTAs' flushes spread over the whole array
-    for (uint32_t i = threadIdx.x; i < W; i += kThreads) {
-        const uint32_t w = i + first < W ? i + first : i + first - W;
-        const uint32_t x = s_fields[w];
-        if (x == 0) continue;
+    cluster_arrive();
+    cluster_wait();                                          // both CTAs have counted
+    {
+        // this CTA's half of the words, the CTAs starting at different places
+        const uint32_t peer = peer_smem(base, (uint32_t)rank ^ 1u);
+        const uint32_t w_lo = W * (uint32_t)rank / kFlushCtas, n_w = W * (uint32_t)(rank + 1) / kFlushCtas - w_lo;
+        const uint32_t first = n_w / gridDim.x * blockIdx.x;
+        for (uint32_t i0 = threadIdx.x; i0 < n_w; i0 += kFlushLoads * kThreads) {
+            uint32_t w[kFlushLoads], x[kFlushLoads], y[kFlushLoads];
 #pragma unroll
-        for (uint32_t f = 0; f < 3; ++f) {
-            const uint32_t c = (x >> (f * kFieldBits)) & kFieldMax, id = f * W + w;
-            if (c && id < mine) atomicAdd(&out[id], c);
+            for (int k = 0; k < kFlushLoads; ++k) {
+                const uint32_t i = min(i0 + k * kThreads, n_w - 1);
+                w[k] = w_lo + (i + first < n_w ? i + first : i + first - n_w);
+                y[k] = ld_peer_u32(peer + 4 * w[k]);
+                x[k] = s_fields[w[k]];
+            }
+#pragma unroll
+            for (int k = 0; k < kFlushLoads; ++k) {
+                if (i0 + k * kThreads >= n_w || (x[k] | y[k]) == 0) continue;
+#pragma unroll
+                for (uint32_t f = 0; f < 3; ++f) {
+                    const uint32_t c = ((x[k] >> (f * kFieldBits)) & kFieldMax) + ((y[k] >> (f * kFieldBits)) & kFieldMax), id = f * W + w[k];
+                    if (c && id < mine) atomicAdd(&out[id], c);
+                }
+            }
         }
     }
+    cluster_arrive();                                        // (its own words are the peer's until the wait at the end)
     if (threadIdx.x < 32) {                                  // (only lanes that had read s_hot added to s_own)
         uint32_t c = s_own[threadIdx.x];
         for (int o = 16; o; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
@@ -649,23 +688,30 @@ k_hist_packed(const int32_t* __restrict__ ids, int64_t n, int32_t V, int32_t Vp,
     if (wrapped) atomicOr(&gate[0], 1u);
     for (int o = 16; o; o >>= 1) bad += __shfl_xor_sync(0xffffffffu, bad, o);
     if ((threadIdx.x & 31) == 0 && bad) atomicAdd(reinterpret_cast<unsigned long long*>(gate + 2), bad);
+    cluster_wait();
 }
 
-// After the packed count: if it stood, counts (+)= packed and the skipped ids are reported; if a field
-// wrapped, counts is left as the recount needs it (zero unless accumulating) and the recount's sampling
-// pre-pass runs here.
+// After the packed count: if it stood, counts (+)= packed and the skipped ids are reported; if a field wrapped, the stream is
+// counted again.  RANGES (shorter streams, see kRangeIds): here, exactly and in one go -- 32-bit bins of a range of ids per CTA, the
+// ranges' CTAs each over their shares of the stream, the last CTA to finish adds the sums up -- so that a call whose count
+// stood has no launches behind this one.  Else counts is left as the hot / cold kernels need it (zero unless accumulating) and
+// their sampling pre-pass runs here.
+constexpr int kRangeBins = (int)(kDynSmem / 4);
+template <bool RANGES>
 __global__ void __launch_bounds__(kThreads, 1)
 k_hist_settle(const int32_t* __restrict__ ids, int64_t n, int32_t V, const uint32_t* packed,
-              uint32_t* __restrict__ counts, int accumulate, uint32_t* __restrict__ sample,
-              const uint32_t* gate, Ctrl* ctrl) {
-    __shared__ int s_tag[kSampleSlots];
-    __shared__ uint32_t s_cnt[kSampleSlots];
+              uint32_t* __restrict__ counts, int accumulate, uint32_t* sample,
+              uint32_t* gate, Ctrl* ctrl) {
+    extern __shared__ __align__(16) uint32_t s_bins[];       // RANGES: [kRangeBins]; else the sampling cache
+    __shared__ uint32_t s_last;
     griddep_launch_dependents();
     griddep_wait();
     const bool recount = ld_cg_u32(gate) != 0;
-    for (int v = blockIdx.x * kThreads + threadIdx.x; v < V; v += gridDim.x * kThreads) {
-        const uint32_t c = recount ? 0u : ld_cg_u32(packed + v);
-        counts[v] = accumulate ? counts[v] + c : c;
+    if (!recount || !RANGES) {
+        for (int v = blockIdx.x * kThreads + threadIdx.x; v < V; v += gridDim.x * kThreads) {
+            const uint32_t c = recount ? 0u : ld_cg_u32(packed + v);
+            counts[v] = accumulate ? counts[v] + c : c;
+        }
     }
     if (!recount) {
         if (blockIdx.x == 0 && threadIdx.x == 0) {
@@ -678,7 +724,41 @@ k_hist_settle(const int32_t* __restrict__ ids, int64_t n, int32_t V, const uint3
         }
         return;
     }
-    sample_stream(ids, n, V, sample, s_tag, s_cnt);
+    if (!RANGES) {
+        sample_stream(ids, n, V, sample, reinterpret_cast<int*>(s_bins), s_bins + kSampleSlots);
+        return;
+    }
+    const int ranges = (V + kRangeBins - 1) / kRangeBins;
+    const int shares = max(1, (int)gridDim.x / ranges);
+    unsigned long long bad = 0;
+    for (int job = blockIdx.x; job < ranges * shares; job += gridDim.x) {
+        const int range = job % ranges, share = job / ranges;
+        const uint32_t lo = (uint32_t)range * kRangeBins, mine = min((uint32_t)kRangeBins, (uint32_t)V - lo);
+        for (uint32_t i = threadIdx.x; i < mine; i += kThreads) s_bins[i] = 0;
+        __syncthreads();
+        const int64_t i0 = n * share / shares, i1 = n * (share + 1) / shares;
+        stream_ids(ids + i0, i1 - i0, [&](uint32_t id) {
+            if (id - lo < mine) atomicAdd(&s_bins[id - lo], 1u);
+            else if (range == 0 && id >= (uint32_t)V) ++bad;
+        }, 0, 1);
+        __syncthreads();
+        for (uint32_t i = threadIdx.x; i < mine; i += kThreads) {
+            const uint32_t c = s_bins[i];
+            if (c) atomicAdd(&sample[lo + i], c);
+        }
+        __syncthreads();
+    }
+    report_bad(bad, ctrl);
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) s_last = atomicAdd(&gate[1], 1u) == gridDim.x - 1 ? 1u : 0u;
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    for (int v = threadIdx.x; v < V; v += kThreads) {
+        const uint32_t c = ld_cg_u32(sample + v);
+        counts[v] = accumulate ? counts[v] + c : c;
+    }
 }
 
 // ---- measurement aid: directly indexed 32-bit bins, one shared-memory reduction per token, nothing else ----
@@ -698,7 +778,7 @@ k_hist_fold(const int32_t* __restrict__ ids, int64_t n, int32_t V, int32_t bins,
             else b = b % nb;
             atomicAdd(&s_bins[b], 1u);
         }
-    });
+    }, (int)blockIdx.x, (int)gridDim.x);
     __syncthreads();
     for (int i = threadIdx.x; i < bins; i += kThreads) {
         const int v = (i + blockIdx.x * 61) % bins;
@@ -773,6 +853,11 @@ static HistPlan plan_for(int32_t V, int parts) {
 // cross at 250 / 112 / 100 million ids; the ranges are taken up to 200 million / (P - 1).
 constexpr int64_t kSplitIds = 200000000;
 
+// A recount by ranges of 57344 bins reads the stream once per range and has no pre-passes, the hot / cold kernels have 50-75 us of
+// them and read it once (us per call, ranges / hot and cold, 45 % + 40 % tokens: V = 128256 3e6 ids 73 / 129, 4e7 194 / 220, 1e8 388
+// / 355; V = 256000 3e6 115 / 200, 4e7 320 / 330, 1e8 - / 535).  The lines cross at 170 million ids per further range.
+constexpr int64_t kRangeIds = 170000000;
+
 HistPlan hist_plan(int32_t V, int64_t n, size_t scratch_bytes) {
     HistPlan p{};
     p.small = (size_t)V * 4 <= kDynSmem;
@@ -796,9 +881,20 @@ static cudaError_t launch_packed(int grid, const int32_t* ids, int64_t n, int32_
     static int done[kMaxDevices] = {0};
     const cudaError_t e = set_smem_once(reinterpret_cast<const void*>(k_hist_packed<SPLIT, SHORT>), kDynSmem, done);
     if (e != cudaSuccess) return e;
-    k_hist_packed<SPLIT, SHORT><<<grid, kThreads, (size_t)W * 4, s>>>(ids, n, V, Vp, parts, W, M, packed, gate);
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = align_up((size_t)W * 4, 16);
+    cfg.stream = s;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = kFlushCtas;
+    at.val.clusterDim.y = 1;
+    at.val.clusterDim.z = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
     count_launch();
-    return cudaGetLastError();
+    return cudaLaunchKernelEx(&cfg, k_hist_packed<SPLIT, SHORT>, ids, n, V, Vp, parts, W, M, packed, gate);
 }
 
 cudaError_t launch_histogram(const int32_t* ids, int64_t n, int32_t V, uint32_t* counts,
@@ -847,17 +943,26 @@ cudaError_t launch_histogram(const int32_t* ids, int64_t n, int32_t V, uint32_t*
         const uint32_t W = packed_words(Vp, &M);
         uint32_t* packed = reinterpret_cast<uint32_t*>(scratch + p.off_packed);
         uint32_t* g = reinterpret_cast<uint32_t*>(scratch + p.off_gate);
-        int shares = parts > 1 ? sms / parts : sms;
-        if (shares < 1) shares = 1;
-        if (shares > grid) shares = grid;                  // (never more than one share per 4096 ids)
+        // (never more than one share per 4096 ids, but whole clusters)
+        const int most = sms / (parts * kFlushCtas) > 0 ? sms / (parts * kFlushCtas) * kFlushCtas : kFlushCtas;
+        int shares = (grid + kFlushCtas - 1) / kFlushCtas * kFlushCtas;
+        if (shares > most) shares = most;
         const bool brief = n <= (int64_t)shares * kShortIds;
         if (parts == 1) e = brief ? launch_packed<false, true>(shares, ids, n, V, V, 1, W, M, packed, g, s)
                                   : launch_packed<false, false>(shares, ids, n, V, V, 1, W, M, packed, g, s);
         else e = brief ? launch_packed<true, true>(shares * parts, ids, n, V, Vp, parts, W, M, packed, g, s)
                        : launch_packed<true, false>(shares * parts, ids, n, V, Vp, parts, W, M, packed, g, s);
         if (e != cudaSuccess) return e;
-        e = launch_dependent(k_hist_settle, grid, kThreads, 0, s, ids, n, V, (const uint32_t*)packed, counts, accumulate, sample,
-                             (const uint32_t*)g, ctrl);
+        const int ranges = (V + kRangeBins - 1) / kRangeBins;
+        if (n * (ranges - 1) <= kRangeIds) {
+            static int done_ranges[kMaxDevices] = {0};
+            e = set_smem_once(reinterpret_cast<const void*>(k_hist_settle<true>), kDynSmem, done_ranges);
+            if (e != cudaSuccess) return e;
+            return launch_dependent(k_hist_settle<true>, sms, kThreads, kDynSmem, s, ids, n, V, (const uint32_t*)packed, counts, accumulate,
+                                    sample, g, ctrl);
+        }
+        e = launch_dependent(k_hist_settle<false>, grid, kThreads, kSampleSlots * 8, s, ids, n, V, (const uint32_t*)packed, counts, accumulate,
+                             sample, g, ctrl);
         gate = g;
     } else {
         k_hist_sample<<<grid, kThreads, 0, s>>>(ids, n, V, sample);
