@@ -44,11 +44,14 @@ class VocabTrimError(RuntimeError):
 
 
 _lib = None
+_bind = None                                       # the calls a program makes per step or per build, marshalled in C++ (csrc/vt_bind.cpp)
+_BOUND = ("vt_draft_head", "vt_draft_head_overlapped", "vt_draft_head_host", "vt_draft_head_expand", "vt_tree_rerank", "vt_verify_greedy",
+          "vt_build_vocab", "vt_trim_head")
 
 
 def lib() -> ctypes.CDLL:
     """Loads libvocabtrim.so; raises if it has not been built (python -m paper_2506_22694_b200.build)."""
-    global _lib
+    global _lib, _bind
     if _lib is None:
         if not os.path.exists(LIB_PATH):
             raise RuntimeError("libvocabtrim.so is missing: build it with "
@@ -85,7 +88,14 @@ def lib() -> ctypes.CDLL:
         L.vt_draft_head_overlapped.argtypes = head
         L.vt_draft_head_host.argtypes = head
         L.vt_draft_head_debug.argtypes = head + [c_void_p, c_void_p]
-        _lib = L
+        try:
+            from . import _vt_bind as bind
+        except ImportError as e:
+            raise RuntimeError("_vt_bind.so is missing or was built for another Python or torch: build it with "
+                               "`python -m paper_2506_22694_b200.build` (%s)" % e) from e
+        bind.use({name: ctypes.cast(getattr(L, name), c_void_p).value for name in _BOUND}, _make_workspace,
+                 torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice)
+        _lib, _bind = L, bind
     return _lib
 
 
@@ -102,10 +112,10 @@ def _check(call: str, status: int) -> None:
         raise VocabTrimError(call, status)
 
 
-# Marshalling.  A drafting step is a few tens of microseconds on the device, so what Python does per call shows: pointers
-# go to ctypes as plain integers (None = NULL), the raw stream handle comes from torch's C layer without a Stream
-# object, outputs are allocated through an input's new_empty, and the size of a caller's workspace is checked by the
-# library, which does it anyway.
+# Marshalling.  A drafting step is a few tens of microseconds on the device, so what Python does per call shows: the calls of a
+# drafting loop and of a build go through _vt_bind.  For the others pointers go to ctypes as plain integers (None =
+# NULL), the raw stream handle comes from torch's C layer without a Stream object, outputs are allocated through an
+# input's new_empty, and the size of a caller's workspace is checked by the library, which does it anyway.
 def _ptr(t):
     return t.data_ptr() if t is not None else None
 
@@ -149,16 +159,24 @@ class Workspace:
         return int(st), int(flags.value), int(bad.value)
 
 
+def _make_workspace(op: int, n: int, V: int, K: int, d: int, B: int, topk: int, like: torch.Tensor) -> Workspace:
+    return Workspace(workspace_bytes(op, n, V, K, d, B, topk), like.device)
+
+
+def _fail(call: str, status: int, op: int, shape, ws: Workspace | None):
+    need = workspace_bytes(op, *shape) if status == 3 else 0
+    if ws is not None and ws.nbytes < need:
+        raise VocabTrimError("workspace too small (%d < %d)" % (ws.nbytes, need), 3)
+    raise VocabTrimError(call, status)
+
+
 def _run(call: str, op: int, shape, ws: Workspace | None, like: torch.Tensor, *args, tail=()) -> None:
     """One library call on the current stream: args, the workspace (the caller's, or one made for the call), the stream, tail."""
     if ws is None:
         ws = Workspace(workspace_bytes(op, *shape), like.device)
     status = getattr(lib(), call)(*args, ws.ptr, ws.nbytes, _stream(), *tail)
     if status:
-        need = workspace_bytes(op, *shape) if status == 3 else 0
-        if ws.nbytes < need:
-            raise VocabTrimError("workspace too small (%d < %d)" % (ws.nbytes, need), 3)
-        raise VocabTrimError(call, status)
+        _fail(call, status, op, shape, ws)
 
 
 def vt_histogram(ids: torch.Tensor, V: int, counts: torch.Tensor | None = None, accumulate: bool = False,
@@ -245,43 +263,20 @@ def vt_draft_head_expand(h: torch.Tensor, W_trim: torch.Tensor, map_: torch.Tens
     """One tree depth in one call: the head (as vt_draft_head(..., overlapped=True), with the same promise: W_trim is not
     written by work still pending on the stream) and the expansion of its candidates into the node pool.  Returns
     (out_ids, out_logprobs, next_frontier [n_front])."""
-    _dev(h, torch.bfloat16, "h")
-    _dev(W_trim, torch.bfloat16, "W_trim")
-    _dev(temp, torch.float32, "temp")
-    B, d = h.shape
-    K = W_trim.shape[0]
-    if W_trim.shape[1] != d or temp.numel() != B:
-        raise ValueError("shape mismatch between h, W_trim and temp")
-    if map_ is not None and _dev(map_, torch.int32, "map").numel() != K:
-        raise ValueError("map must have K entries")
-    if uniforms is not None and tuple(_dev(uniforms, torch.float32, "uniforms").shape) != (B, K):
-        raise ValueError("uniforms must be [B,K]")
-    if frontier_nodes is not None and _dev(frontier_nodes, torch.int32, "frontier_nodes").numel() != B:
-        raise ValueError("frontier_nodes must have B entries")
-    tok, par, sc = pool
-    _dev(tok, torch.int32, "pool token"), _dev(par, torch.int32, "pool parent"), _dev(sc, torch.float32, "pool score")
-    if out is None:
-        out = (torch.empty((B, 1 + topk), dtype=torch.int32, device=h.device),
-               torch.empty((B, 1 + topk), dtype=torch.float32, device=h.device))
-    ids, lps = out
-    nxt = tok.new_empty(n_front)
-    _run("vt_draft_head_expand", VT_OP_DRAFT_HEAD, (0, 0, K, d, B, topk), ws, h,
-         h.data_ptr(), W_trim.data_ptr(), _ptr(map_), B, K, d, temp.data_ptr(), topk, _ptr(uniforms), ids.data_ptr(), lps.data_ptr(),
-         _ptr(frontier_nodes), tok.data_ptr(), par.data_ptr(), sc.data_ptr(), pool_base, min(tok.numel(), par.numel(), sc.numel()),
-         n_front, nxt.data_ptr())
-    return ids, lps, nxt
+    _lib or lib()
+    r = _bind.draft_head_expand(h, W_trim, map_, temp, topk, uniforms, frontier_nodes, pool, pool_base, n_front, ws, out)
+    if r.__class__ is int:
+        _fail("vt_draft_head_expand", r, VT_OP_DRAFT_HEAD, (0, 0, W_trim.shape[0], h.shape[1], h.shape[0], topk), ws)
+    return r
 
 
 def vt_tree_rerank(pool, n: int, budget: int):
     """Final draft of the tree (Settings): returns (nodes, token, parent), each int32 [budget]."""
-    tok, par, sc = pool
-    _dev(tok, torch.int32, "pool token"), _dev(par, torch.int32, "pool parent"), _dev(sc, torch.float32, "pool score")
-    if n > min(tok.numel(), par.numel(), sc.numel()):
-        raise ValueError("n exceeds the pool")
-    outs = [tok.new_empty(budget) for _ in range(3)]
-    _check("vt_tree_rerank", lib().vt_tree_rerank(_ptr(tok), _ptr(par), _ptr(sc), n, budget, _ptr(outs[0]),
-                                                  _ptr(outs[1]), _ptr(outs[2]), _stream()))
-    return tuple(outs)
+    _lib or lib()
+    r = _bind.tree_rerank(pool, n, budget)
+    if r.__class__ is int:
+        raise VocabTrimError("vt_tree_rerank", r)
+    return r
 
 
 def vt_verify_greedy(token: torch.Tensor, parent: torch.Tensor | None, target: torch.Tensor,
@@ -290,21 +285,11 @@ def vt_verify_greedy(token: torch.Tensor, parent: torch.Tensor | None, target: t
 
     token [S,N], parent [S,N] or None (chains), target [S,N+1], all int32 on the device.  Returns
     (n_accept [S], path [S,N], emitted [S,N+1]); `tokens_total` (int64 [1], device) is added to."""
-    _dev(token, torch.int32, "token")
-    _dev(target, torch.int32, "target")
-    S, N = token.shape
-    if tuple(target.shape) != (S, N + 1):
-        raise ValueError("target must be [S, N+1]")
-    if parent is not None:
-        _dev(parent, torch.int32, "parent")
-        if tuple(parent.shape) != (S, N):
-            raise ValueError("parent must be [S, N]")
-    if tokens_total is not None:
-        _dev(tokens_total, torch.int64, "tokens_total")
-    n_accept, path, emitted = token.new_empty(S), token.new_empty((S, N)), token.new_empty((S, N + 1))
-    _check("vt_verify_greedy", lib().vt_verify_greedy(
-        _ptr(token), _ptr(parent), _ptr(target), S, N, _ptr(n_accept), _ptr(path), _ptr(emitted), _ptr(tokens_total), _stream()))
-    return n_accept, path, emitted
+    _lib or lib()
+    r = _bind.verify_greedy(token, parent, target, tokens_total)
+    if r.__class__ is int:
+        raise VocabTrimError("vt_verify_greedy", r)
+    return r
 
 
 def vt_mbsu(tau: float, draft_params: float, target_params: float, gamma: int) -> float:
@@ -331,10 +316,11 @@ def vt_build_vocab(ids: torch.Tensor, V: int, K: int, ws: Workspace | None = Non
     ids tensor goes through vt_build_vocab_host, which streams it to the device in chunks."""
     if not ids.is_cuda:
         return vt_build_vocab_host(ids, V, K, ws)
-    _dev(ids, torch.int32, "ids")
-    map_, inv, n = ids.new_empty(K), ids.new_empty(V), ids.numel()
-    _run("vt_build_vocab", VT_OP_BUILD_VOCAB, (n, V, K), ws, ids, ids.data_ptr(), n, V, K, map_.data_ptr(), inv.data_ptr())
-    return map_, inv
+    _lib or lib()
+    r = _bind.build_vocab(ids, V, K, ws)
+    if r.__class__ is int:
+        _fail("vt_build_vocab", r, VT_OP_BUILD_VOCAB, (ids.numel(), V, K), ws)
+    return r
 
 
 def vt_build_vocab_host(ids_host: torch.Tensor, V: int, K: int, ws: Workspace | None = None, device="cuda",
@@ -352,16 +338,11 @@ def vt_build_vocab_host(ids_host: torch.Tensor, V: int, K: int, ws: Workspace | 
 def vt_trim_head(W_full: torch.Tensor, map_: torch.Tensor, W_trim: torch.Tensor | None = None,
                  ws: Workspace | None = None) -> torch.Tensor:
     """Eq. 1 (head restriction).  W_full bf16 [V,d], map int32 [K] -> W_trim bf16 [K,d]."""
-    _dev(W_full, torch.bfloat16, "W_full")
-    _dev(map_, torch.int32, "map")
-    V, d = W_full.shape
-    K = map_.numel()
-    if W_trim is None:
-        W_trim = W_full.new_empty((K, d))
-    _dev(W_trim, torch.bfloat16, "W_trim")
-    _check("vt_trim_head", lib().vt_trim_head(_ptr(W_full), _ptr(map_), _ptr(W_trim), V, K, d,
-                                              ws.ptr if ws else None, _stream()))
-    return W_trim
+    _lib or lib()
+    r = _bind.trim_head(W_full, map_, W_trim, ws)
+    if r.__class__ is int:
+        raise VocabTrimError("vt_trim_head", r)
+    return r
 
 
 def vt_draft_head(h: torch.Tensor, W_trim: torch.Tensor, map_: torch.Tensor | None, temp: torch.Tensor,
@@ -372,6 +353,13 @@ def vt_draft_head(h: torch.Tensor, W_trim: torch.Tensor, map_: torch.Tensor | No
     vt_draft_head_overlapped, for drafting loops with static weights: W_trim is fetched before the work in front of the
     call has finished, so it must not be written by work still pending on the stream.  After vt_trim_head (or any other
     write to it) synchronise, or make one plain call first."""
+    _lib or lib()
+    if not debug:
+        r = _bind.draft_head(h, W_trim, map_, temp, topk, uniforms, ws, out, overlapped)
+        if r.__class__ is int:
+            _fail("vt_draft_head_overlapped" if overlapped else "vt_draft_head", r, VT_OP_DRAFT_HEAD,
+                  (0, 0, W_trim.shape[0], h.shape[1], h.shape[0], topk), ws)
+        return r
     _dev(h, torch.bfloat16, "h")
     _dev(W_trim, torch.bfloat16, "W_trim")
     _dev(temp, torch.float32, "temp")
@@ -387,15 +375,12 @@ def vt_draft_head(h: torch.Tensor, W_trim: torch.Tensor, map_: torch.Tensor | No
         out = (torch.empty((B, 1 + topk), dtype=torch.int32, device=h.device),
                torch.empty((B, 1 + topk), dtype=torch.float32, device=h.device))
     ids, lps = out
-    args = (h.data_ptr(), W_trim.data_ptr(), _ptr(map_), B, K, d, temp.data_ptr(), topk, _ptr(uniforms), ids.data_ptr(), lps.data_ptr())
-    shape = (0, 0, K, d, B, topk)
-    if debug:
-        logits = torch.empty((B, K), dtype=torch.float32, device=h.device)
-        lse = torch.empty(B, dtype=torch.float32, device=h.device)
-        _run("vt_draft_head_debug", VT_OP_DRAFT_HEAD, shape, ws, h, *args, tail=(logits.data_ptr(), lse.data_ptr()))
-        return ids, lps, logits, lse
-    _run("vt_draft_head_overlapped" if overlapped else "vt_draft_head", VT_OP_DRAFT_HEAD, shape, ws, h, *args)
-    return ids, lps
+    logits = torch.empty((B, K), dtype=torch.float32, device=h.device)
+    lse = torch.empty(B, dtype=torch.float32, device=h.device)
+    _run("vt_draft_head_debug", VT_OP_DRAFT_HEAD, (0, 0, K, d, B, topk), ws, h,
+         h.data_ptr(), W_trim.data_ptr(), _ptr(map_), B, K, d, temp.data_ptr(), topk, _ptr(uniforms), ids.data_ptr(), lps.data_ptr(),
+         tail=(logits.data_ptr(), lse.data_ptr()))
+    return ids, lps, logits, lse
 
 
 def vt_draft_head_host(h_host: torch.Tensor, W_trim: torch.Tensor, map_: torch.Tensor | None,
@@ -407,7 +392,6 @@ def vt_draft_head_host(h_host: torch.Tensor, W_trim: torch.Tensor, map_: torch.T
     B, d = h_host.shape
     K = W_trim.shape[0]
     ids, lps = out_host
-    _check("vt_draft_head_host", lib().vt_draft_head_host(
-        h_host.data_ptr(), _ptr(W_trim), _ptr(map_), B, K, d, temp_host.data_ptr(), topk, _ptr(uniforms_host),
-        ids.data_ptr(), lps.data_ptr(), ws.ptr, ws.nbytes, _stream()))
+    _lib or lib()
+    _check("vt_draft_head_host", _bind.draft_head_host(h_host, W_trim, map_, B, K, d, temp_host, topk, uniforms_host, ids, lps, ws))
     return ids, lps

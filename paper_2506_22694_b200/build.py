@@ -1,4 +1,5 @@
-"""Builds libvocabtrim.so (the C-ABI CUDA library) in-tree with nvcc for sm_100a.
+"""Builds libvocabtrim.so (the C-ABI CUDA library) in-tree with nvcc for sm_100a, and _vt_bind.so (the argument marshalling of the
+Python binding) with the C++ compiler against torch's headers.
 
 Usage: python -m paper_2506_22694_b200.build [--force] [--verbose]
 """
@@ -8,12 +9,15 @@ import glob
 import os
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libvocabtrim.so")
 OBJ_DIR = os.path.join(HERE, "_build")
+BIND_SRC = os.path.join(CSRC, "vt_bind.cpp")
+BIND = os.path.join(HERE, "_vt_bind.so")
 LIB_STAMPS = os.path.join(HERE, "libvocabtrim_stamps.so")     # -DVT_STAMPS: phase stamps in the head kernel
 OBJ_DIR_STAMPS = os.path.join(HERE, "_build_stamps")
 
@@ -40,10 +44,28 @@ def needs_build(lib: str = LIB) -> bool:
     return any(os.path.getmtime(p) > t for p in _deps())
 
 
+def build_bind(force: bool = False) -> str:
+    """Compile the binding's extension module; its objects come from torch, already loaded when it is imported."""
+    header = os.path.join(ROOT, "include", "vocabtrim.h")
+    if not force and os.path.exists(BIND) and os.path.getmtime(BIND) > max(os.path.getmtime(BIND_SRC), os.path.getmtime(header)):
+        return BIND
+    import torch
+
+    top = os.path.dirname(torch.__file__)
+    tmp = BIND + ".%d.tmp" % os.getpid()
+    subprocess.check_call([os.environ.get("CXX", "g++"), "-std=c++17", "-O2", "-fPIC", "-shared",
+                           "-D_GLIBCXX_USE_CXX11_ABI=%d" % torch._C._GLIBCXX_USE_CXX11_ABI, "-I", os.path.join(ROOT, "include"),
+                           "-isystem", sysconfig.get_paths()["include"], "-isystem", os.path.join(top, "include"),
+                           BIND_SRC, "-o", tmp, "-L", os.path.join(top, "lib"), "-lc10", "-ltorch_cpu", "-ltorch_python"])
+    os.replace(tmp, BIND)
+    return BIND
+
+
 def build(force: bool = False, verbose: bool = False, stamps: bool = False) -> str:
     """Compile every .cu under csrc/ (one object each, in parallel) and link the shared library.
     stamps=True builds the instrumented twin (libvocabtrim_stamps.so, -DVT_STAMPS) instead."""
     LIB, OBJ_DIR = (LIB_STAMPS, OBJ_DIR_STAMPS) if stamps else (globals()["LIB"], globals()["OBJ_DIR"])
+    build_bind(force)
     if not force and not needs_build(LIB):
         return LIB
     nvcc = os.environ.get("NVCC", "nvcc")
