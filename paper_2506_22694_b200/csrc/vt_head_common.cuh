@@ -127,9 +127,17 @@ struct MergeOut {
     int32_t* out_ids;
     float* out_logprobs;
     float* dbg_lse;
+    const float* temp;
     int topk;
     int sampled;       // uniforms were given: column 0 is the Gumbel-max draw
 };
+
+// What a row without a full result is reported as.  (A row of unusable temperature has NaN for every z and so no candidates: nothing
+// else looks at the temperature, which may lie in host memory.)
+__device__ __forceinline__ uint32_t merge_flag(const MergeOut& a, int b) {
+    const float T = ld_cg_f32(a.temp + b);
+    return T > 0.f && T < CUDART_INF_F ? (uint32_t)VT_FLAG_NAN_ROW : (uint32_t)VT_FLAG_BAD_TEMP;
+}
 
 // The merge of one hidden row by six warps.  A warp runs dependent code at a few cycles per instruction, and the row's result is what
 // the next step waits for, so the work is spread: five warps hold a CTA's list heads per lane (kRoleCand), the sixth the
@@ -171,7 +179,7 @@ __device__ __forceinline__ void merge_request(const MergeOut& a, float* recs, in
     }
 }
 
-__device__ __forceinline__ void merge_stats(const MergeOut& a, Ctrl* ctrl, int b, bool row_ok, int G, MergeLoads& ld, volatile float* xch) {
+__device__ __forceinline__ void merge_stats(const MergeOut& a, Ctrl* ctrl, int b, int G, MergeLoads& ld, volatile float* xch) {
     const int lane = threadIdx.x & 31;
     int* oid = a.out_ids + (size_t)b * (1 + a.topk);
     float* olp = a.out_logprobs + (size_t)b * (1 + a.topk);
@@ -216,25 +224,24 @@ __device__ __forceinline__ void merge_stats(const MergeOut& a, Ctrl* ctrl, int b
         gwin = ((unsigned long long)kmax << 32) | lomax;
     }
     if (lane == 0) {
-        bool bad = !(lse == lse);                           // a NaN logit somewhere in the row
+        bool bad = !(lse == lse);                           // a NaN logit somewhere in the row, or an unusable temperature
         if (a.sampled) {
-            const bool ok = row_ok && gwin != 0ull;
+            const bool ok = gwin != 0ull;
             const int gj = key_idx(gwin);
             oid[0] = ok ? (a.map ? ld_cg_s32(a.map + gj) : gj) : -1;
             olp[0] = ok ? gzw - lse : CUDART_NAN_F;
             bad = bad || !ok;
         }
         if (a.dbg_lse) a.dbg_lse[b] = lse;
-        if (!row_ok) atomicOr(&ctrl->flags, (uint32_t)VT_FLAG_BAD_TEMP);
-        else if (bad) atomicOr(&ctrl->flags, (uint32_t)VT_FLAG_NAN_ROW);
+        if (bad) atomicOr(&ctrl->flags, merge_flag(a, b));
     }
 }
 
 // Entry `key` of the merged list is the r-th best (r < topk): id and log-probability.  The id is asked for before the ranking.
-__device__ __forceinline__ void merge_emit(const MergeOut& a, int b, int r, int id, unsigned long long key, bool row_ok, float lse) {
+__device__ __forceinline__ void merge_emit(const MergeOut& a, int b, int r, int id, unsigned long long key, float lse) {
     int* oid = a.out_ids + (size_t)b * (1 + a.topk);
     float* olp = a.out_logprobs + (size_t)b * (1 + a.topk);
-    const bool ok = row_ok && key != 0ull;
+    const bool ok = key != 0ull;
     id = ok ? id : -1;
     const float lp = ok ? key_val(key) - lse : CUDART_NAN_F;
     oid[1 + r] = id;
@@ -248,7 +255,7 @@ __device__ __forceinline__ int merge_id(const MergeOut& a, unsigned long long ke
 
 // Ranks the n keys in sel (NS to a lane) and writes the topk best of them.
 template <int NS>
-__device__ __forceinline__ void merge_rank(const MergeOut& a, const unsigned long long* sel, int n, int b, bool row_ok, volatile float* xch) {
+__device__ __forceinline__ void merge_rank(const MergeOut& a, const unsigned long long* sel, int n, int b, volatile float* xch) {
     const int lane = threadIdx.x & 31;
     unsigned long long mine[NS];
     int rk[NS], id[NS];
@@ -264,11 +271,11 @@ __device__ __forceinline__ void merge_rank(const MergeOut& a, const unsigned lon
     const float lse = *xch;
 #pragma unroll
     for (int i = 0; i < NS; ++i)
-        if (lane + 32 * i < n && rk[i] < a.topk) merge_emit(a, b, rk[i], id[i], mine[i], row_ok, lse);
-    for (int r = n + lane; r < a.topk; r += 32) merge_emit(a, b, r, -1, 0ull, row_ok, lse);          // fewer than topk candidates
+        if (lane + 32 * i < n && rk[i] < a.topk) merge_emit(a, b, rk[i], id[i], mine[i], lse);
+    for (int r = n + lane; r < a.topk; r += 32) merge_emit(a, b, r, -1, 0ull, lse);          // fewer than topk candidates
 }
 
-__device__ __forceinline__ void merge_candidates(const MergeOut& a, Ctrl* ctrl, float* recs, int b, bool row_ok, int G, MergeLoads& ld,
+__device__ __forceinline__ void merge_candidates(const MergeOut& a, Ctrl* ctrl, float* recs, int b, int G, MergeLoads& ld,
                                                  float* stage, int* s_n, int* s_deep, volatile float* xch) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int topk = a.topk, depth = min(topk, kMergeDepth), c = warp * 32 + lane;
@@ -321,9 +328,9 @@ __device__ __forceinline__ void merge_candidates(const MergeOut& a, Ctrl* ctrl, 
             if (warp != 0) return;
             if (lane < 4) sel[n + lane] = 0ull;                                    // (read in groups of four)
             __syncwarp();
-            if (n <= 32) merge_rank<1>(a, sel, n, b, row_ok, xch);
-            else merge_rank<kSelCap / 32>(a, sel, n, b, row_ok, xch);
-            if (lane == 0 && row_ok && n < topk) atomicOr(&ctrl->flags, (uint32_t)VT_FLAG_NAN_ROW);
+            if (n <= 32) merge_rank<1>(a, sel, n, b, xch);
+            else merge_rank<kSelCap / 32>(a, sel, n, b, xch);
+            if (lane == 0 && n < topk) atomicOr(&ctrl->flags, merge_flag(a, b));
             return;
         }
         asm volatile("bar.sync 1, %0;" ::"n"(32 * kMaxOwn) : "memory");            // (the words are given up)
@@ -376,12 +383,12 @@ __device__ __forceinline__ void merge_candidates(const MergeOut& a, Ctrl* ctrl, 
     for (int sl = 0; sl < 2; ++sl) {
         const int r = lane + 32 * sl;
         if (r < topk) {
-            merge_emit(a, b, r, ids[sl], res_k[sl], row_ok, lse);
+            merge_emit(a, b, r, ids[sl], res_k[sl], lse);
             miss = miss || res_k[sl] == 0ull;
         }
     }
     const bool any_missing = __any_sync(0xffffffffu, miss);
-    if (lane == 0 && row_ok && any_missing) atomicOr(&ctrl->flags, (uint32_t)VT_FLAG_NAN_ROW);
+    if (lane == 0 && any_missing) atomicOr(&ctrl->flags, merge_flag(a, b));
 }
 
 }  // namespace

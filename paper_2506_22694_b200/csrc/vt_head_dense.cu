@@ -793,8 +793,7 @@ k_head_merge(const HeadArgs a, Ctrl* ctrl, float* __restrict__ recs, int G, int 
 #endif
     // (everything is on its way before the mark is looked at: a round trip to L2 is a fifth of the merge)
     const uint32_t mark = ld_cg_u32(&ctrl->head_aborted);
-    const float T = ld_cg_f32(a.temp + b);
-    const MergeOut mo{a.map, a.out_ids, a.out_logprobs, a.dbg_lse, a.topk, a.uniforms != nullptr};
+    const MergeOut mo{a.map, a.out_ids, a.out_logprobs, a.dbg_lse, a.temp, a.topk, a.uniforms != nullptr};
     MergeLoads ld;
     merge_request(mo, recs, b, G, ld);
     const bool aborted = mark != 0u;
@@ -804,9 +803,8 @@ k_head_merge(const HeadArgs a, Ctrl* ctrl, float* __restrict__ recs, int G, int 
             a.out_logprobs[(size_t)b * (1 + a.topk) + i] = CUDART_NAN_F;
         }
     } else {
-        const bool row_ok = (T > 0.f) && (T < CUDART_INF_F);
-        if (threadIdx.x < 32 * kMaxOwn) merge_candidates(mo, ctrl, recs, b, row_ok, G, ld, s_stage, &s_n, &s_deep, &s_xch);
-        else merge_stats(mo, ctrl, b, row_ok, G, ld, &s_xch);
+        if (threadIdx.x < 32 * kMaxOwn) merge_candidates(mo, ctrl, recs, b, G, ld, s_stage, &s_n, &s_deep, &s_xch);
+        else merge_stats(mo, ctrl, b, G, ld, &s_xch);
     }
 #ifdef VT_STAMPS
     if (b == 0 && threadIdx.x == 0) stamps[13] = global_ns();
