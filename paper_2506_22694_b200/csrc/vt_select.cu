@@ -751,6 +751,94 @@ k_select_sort(const uint32_t* counts, int32_t V, int32_t K, int32_t* map, int32_
     }
 }
 
+// ---- small vocabularies: every rank by comparison with all counts ------------------------------------------
+// The cluster kernel above is a chain of some twenty short phases, 11 us however few the ids.  Of a small vocabulary an id's
+// rank is simply counted -- the ids of greater count, and of equal count those before it -- by 32 warps per 32 * NK
+// ids, each over its part of the counts: no exchange between CTAs, one round trip to memory.  The counts are compared as fp32
+// (exact below 2^24; whole numbers, so that the saturated difference is the outcome of the comparison), which takes two
+// instructions of the FMA pipe; integer comparisons run at half their rate.  Bound by those: V * V / 64 cycles over all SMs.
+constexpr int kRankThreads = 1024;
+constexpr int32_t kRankMaxIds = 12000;            // 4 bytes each: what shared memory holds without being asked for more
+
+template <int NK>
+__global__ void __launch_bounds__(kRankThreads, 1)
+k_select_rank(const uint32_t* counts, int32_t V, int32_t K, int32_t* __restrict__ map, int32_t* __restrict__ inv_map) {
+    extern __shared__ __align__(16) uint32_t s_count[];          // [V, rounded up to 128]: as fp32, or as they are where one is too large
+    __shared__ int s_rank[32 * NK];
+    griddep_launch_dependents();
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int first = blockIdx.x * (32 * NK), n = (V + 127) & ~127;
+    if (threadIdx.x < 32 * NK) s_rank[threadIdx.x] = 0;
+    griddep_wait();                                              // (the counts come from the kernel before)
+    int large = 0;
+    for (int j = threadIdx.x; j < n; j += kRankThreads) {
+        const uint32_t c = j < V ? ld_cg_u32(counts + j) : 0u;
+        large |= c >> 24 ? 1 : 0;
+        s_count[j] = j < V ? c : 0u;
+    }
+    const bool exact = !__syncthreads_or(large);
+    if (exact) {                                                 // (every thread its own ones)
+        for (int j = threadIdx.x; j < n; j += kRankThreads) s_count[j] = __float_as_uint((float)s_count[j]);
+        __syncthreads();
+    }
+    auto count_of = [&](uint32_t x) { return exact ? (uint32_t)__uint_as_float(x) : x; };
+    // this lane's ids: i[k] = first + 32 k + lane
+    uint32_t ci[NK];
+    int r[NK];
+#pragma unroll
+    for (int k = 0; k < NK; ++k) {
+        ci[k] = count_of(s_count[min(first + 32 * k + lane, n - 1)]);
+        r[k] = 0;
+    }
+    // the warp's part of the others, in groups of four: those of ids below the CTA's and those above
+    const int j_lo = n / 4 * warp / 32 * 4, j_hi = n / 4 * (warp + 1) / 32 * 4;
+    const int a_hi = min(max(first, j_lo), j_hi), b_lo = min(max(first + 32 * NK, j_lo), j_hi);
+    const uint4* c4 = reinterpret_cast<const uint4*>(s_count);
+    auto one = [&](int j) {
+        const uint32_t cj = count_of(s_count[j]);
+#pragma unroll
+        for (int k = 0; k < NK; ++k) r[k] += cj > ci[k] || (cj == ci[k] && j < first + 32 * k + lane) ? 1 : 0;
+    };
+    // of the CTA's own ids (as of a count that fp32 does not hold) every warp takes as many
+    for (int j = first + warp; j < min(first + 32 * NK, V); j += 32) one(j);
+    if (exact) {
+        float f[NK][2], fc[NK];
+#pragma unroll
+        for (int k = 0; k < NK; ++k) { f[k][0] = f[k][1] = 0.f; fc[k] = (float)ci[k]; }
+        auto walk = [&](int lo, int hi, float less) {            // counts greater than ci - less
+            float t[NK];
+#pragma unroll
+            for (int k = 0; k < NK; ++k) t[k] = fc[k] - less;
+#pragma unroll 4
+            for (int j = lo; j < hi; j += 4) {
+                const uint4 q = c4[j >> 2];
+                const float x[4] = {__uint_as_float(q.x), __uint_as_float(q.y), __uint_as_float(q.z), __uint_as_float(q.w)};
+#pragma unroll
+                for (int k = 0; k < NK; ++k)
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) f[k][e & 1] += __saturatef(x[e] - t[k]);
+            }
+        };
+        walk(j_lo, a_hi, 1.f);                                   // equal counts of lower ids go first
+        walk(b_lo, j_hi, 0.f);                                   // (ids that do not exist count nothing and are above)
+#pragma unroll
+        for (int k = 0; k < NK; ++k) r[k] += (int)(f[k][0] + f[k][1]);
+    } else {
+        for (int j = j_lo; j < a_hi; ++j) one(j);
+        for (int j = b_lo; j < min(j_hi, V); ++j) one(j);
+    }
+#pragma unroll
+    for (int k = 0; k < NK; ++k)
+        if (r[k]) atomicAdd(&s_rank[32 * k + lane], r[k]);
+    __syncthreads();
+    const int i = first + threadIdx.x;
+    if (threadIdx.x < 32 * NK && i < V) {
+        const int rk = s_rank[threadIdx.x];
+        if (rk < K) map[rk] = i;
+        inv_map[i] = rk < K ? rk : -1;
+    }
+}
+
 }  // namespace
 
 // Attributes of one instance on the current device, and whether it can run there at all.
@@ -839,6 +927,16 @@ cudaError_t launch_select_topk(const uint32_t* counts, int32_t V, int32_t K, int
                                int32_t* inv_map, uint8_t* scratch, cudaStream_t s) {
     // (whatever K: even K = V is the selection's work when most ids were seen fewer than 1024 times -- 31 against
     // 56 us on the counts of 3 M tokens -- and costs it one bucket pass, 13 us, before the full ranking when not)
+    // Ranks by comparison while one CTA to an SM does, with one or two ids to a lane (us per call, cluster kernel / this: V = 1000 11.1 /
+    // 2.8, 4096 11.8 / 4.5, 5000 13.3 / 7.3, 8192 14.3 / 10.0, 9472 13.5 / 11.7; two CTAs to an SM: 12000 14.0 / 24.7).
+    const int sms = num_sms();
+    if (V <= 64 * sms && V <= kRankMaxIds) {
+        const size_t smem = align_up((size_t)V, 128) * 4;
+        const int per = V <= 32 * sms ? 1 : 2;
+        const unsigned grid = (unsigned)((V + 32 * per - 1) / (32 * per));
+        return per == 1 ? launch_dependent(k_select_rank<1>, grid, kRankThreads, smem, s, counts, V, K, map, inv_map)
+                        : launch_dependent(k_select_rank<2>, grid, kRankThreads, smem, s, counts, V, K, map, inv_map);
+    }
     return launch_select<0>(counts, V, K, map, inv_map, scratch, 1.0, 0u, nullptr, s);
 }
 
