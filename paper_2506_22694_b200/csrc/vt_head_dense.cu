@@ -20,12 +20,19 @@
 // the epilogue of tile t overlaps the MMAs of tile t+1.  tcgen05.commit releases ring stages and
 // publishes accumulators (to both CTAs of a pair).  Eight epilogue warps read the accumulators back
 // with tcgen05.ld -- TMEM lane = hidden row; the two warps of a lane quadrant take one half of a tile's
-// columns each -- 16 columns at a time: running max / sum-exp of z = logit / T_b, Gumbel-max candidate
-// from the caller's uniforms, and a sorted top-k list kept in registers.  Logits never go to HBM.  The
-// two column halves of a row are merged through shared memory; per CTA (pair) and hidden row one
-// record goes to scratch; a second small kernel (six warps per hidden row) merges the records,
-// applies the index mapper and writes the outputs.  Every wait is bounded; on expiry the CTA raises
+// columns each (up to 64 rows a tile is computed in two halves, on lanes of their own) -- 16 columns at a time: running max /
+// sum-exp of z = logit / T_b, Gumbel-max candidate from the caller's uniforms, and a sorted top-k list kept in registers.
+// Logits never go to HBM.  The column shares of a row are merged through shared memory (a pair's two shares leave a record
+// each); per CTA and hidden row one record goes to scratch; a second small kernel (six warps per hidden row) merges the
+// records, applies the index mapper and writes the outputs.  Every wait is bounded; on expiry the CTA raises
 // VT_FLAG_TIMEOUT and leaves after releasing its tensor memory.
+//
+// What bounds it: W_trim and the uniforms stream in at 6 TB/s while MMAs and all but the last tile's epilogue run; then the last
+// epilogue and the merge are exposed, while HBM idles.  So that epilogue is kept short: the Gumbel noise of the last
+// tile is made while its MMAs run, and over a CTA's only tile the top-k list is found by sorting networks.  The epilogue issues
+// at half the schedulers' rate at most (two warps on each, selects and minima at half rate).  us per chained step before
+// any of this / now (the merge's share included): 40 rows of 20001 x 3072 41.3 / 31.9, 64 rows 42.7 / 33.5, 100 rows 46.2 / 34.8,
+// 90 rows of 10000 x 4096 with top-10 43.7 / 27.2, 256 rows of 32768 x 4096 74.5 / 72.2.
 #include <cfloat>
 
 #include "vt_common.cuh"
@@ -42,6 +49,7 @@ constexpr int kMaxBN = 256;               // vocabulary rows per tile at most (T
 constexpr int kMaxSub = 2;                // d-steps of kBK columns one ring stage holds at most
 constexpr int kMaxStages = 8;
 constexpr int kCh = 16;                   // accumulator columns per epilogue step (keeps the row state in registers)
+constexpr int kParts = 2;                  // epilogue warps per TMEM lane quadrant
 constexpr int kTmemCols = 512;            // 2 accumulator stages x kMaxBN columns
 constexpr int kMaxTopk = 16;              // the list's values live in registers
 constexpr unsigned long long kWaitLimitNs = 2000000000ull;
@@ -161,6 +169,8 @@ struct DenseGeo {
     int h_rows;       // hidden rows a copy brings (the rest of the MMA's 128 is whatever lies there: lanes nobody looks at)
     int h_bytes;      // shared memory of a step's hidden rows (a multiple of 1024); its vocabulary rows lie behind them
     int ring_bytes;
+    int bn0;          // SPLIT: columns of a tile's first half (a multiple of 16, <= kHalfCols; the second has no more)
+    int tail_bytes;   // behind the ring, for operand rows that the last stage's MMAs read beyond it
     int sub;          // d-steps per ring stage (1 or 2): one wait and one release per stage, so two steps per stage halve
                       // what the two single threads that drive the ring spend per MMA; taken when three such stages fit
 };
@@ -237,10 +247,16 @@ __device__ __forceinline__ void merge_desc(T (&list)[N], const T (&v)[A]) {
             if ((i & k) == 0) order2(list[i], list[i + k]);
 }
 
-// KT: capacity of the list (8 or kMaxTopk).  PAIR: two CTAs of a cluster form one MMA.  PARTS: epilogue warps per TMEM lane
-// quadrant, each with a contiguous share of a tile's 16-column chunks.  Warps whose lanes hold no hidden row leave at once.
-template <int KT, bool PAIR, int PARTS>
-__global__ void __launch_bounds__((2 + 4 * PARTS) * 32, 1)
+// KT: capacity of the list (8 or kMaxTopk).  PAIR: two CTAs of a cluster form one MMA.  Two epilogue warps per TMEM lane
+// quadrant, each with a contiguous share of the quadrant's 16-column chunks.  Warps whose lanes hold no hidden row leave at once.
+// SPLIT (up to 64 hidden rows): an MMA's first 64 rows are the hidden rows and its second 64 nobody's, and a quadrant's warps sit on
+// one scheduler, so half of them would do the whole epilogue.  So a tile's columns are computed in two halves: one with the
+// hidden rows as rows 0-63, the other with the operand's start 64 rows earlier, which makes them rows 64-127; each half
+// of the lanes then has half of the columns (in TMEM kHalfCols apart) and all eight warps work.  (40 rows of 20001 x 3072, four
+// warps on each of two quadrants / this: 34.2 / 31.9 us.)
+constexpr int kHalfCols = kMaxBN / 2;
+template <int KT, bool PAIR, bool SPLIT>
+__global__ void __launch_bounds__((2 + 4 * kParts) * 32, 1)
 k_head_dense(const HeadArgs a, Ctrl* ctrl, float* __restrict__ recs, const DenseGeo geo,
              const __grid_constant__ CUtensorMap tm_h, const __grid_constant__ CUtensorMap tm_w) {
     extern __shared__ uint8_t s_dyn[];
@@ -254,7 +270,11 @@ k_head_dense(const HeadArgs a, Ctrl* ctrl, float* __restrict__ recs, const Dense
     if (threadIdx.x == 0) VT_DSTAMP(0);
 #endif
     // identical in both CTAs of a pair: the MMA addresses the peer's operands by the leader's offsets
-    uint8_t* ring = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(s_dyn) + 1023) & ~(uintptr_t)1023);
+    // (the candidate entries lie in front of the ring)
+    constexpr int kShares = SPLIT ? 2 * kParts : kParts;           // column shares of a hidden row
+    constexpr int kRows = SPLIT ? kBM / 2 : kBM, kEntStride = kShares * kRows;
+    uint8_t* entries = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(s_dyn) + 1023) & ~(uintptr_t)1023);
+    uint8_t* ring = entries + KT * kEntStride * sizeof(float2);
     const uint32_t ring_u32 = smem_u32(ring);
     const int B = a.B, K = a.K, topk = a.topk;
     const uint32_t rank = PAIR ? cluster_ctarank() : 0u;          // 0 = leader: issues the MMAs, owns the full barriers
@@ -262,7 +282,7 @@ k_head_dense(const HeadArgs a, Ctrl* ctrl, float* __restrict__ recs, const Dense
     const int bn = geo.bn, n_stages = geo.n_stages;
     const int w_rows = PAIR ? bn / 2 : bn;                         // vocabulary rows this CTA stages per step
     // epilogue warps of a CTA with this many of the hidden rows that have any of them to look after
-    auto live_warps = [&](int rows) { return (min(max(rows, 0), kBM) + 31) / 32 * PARTS; };
+    auto live_warps = [&](int rows) { return (min(max(rows, 0), kBM) + 31) / 32 * kShares; };
 
     if (threadIdx.x == 0) {
         // the two tensor maps are fetched now, not by the first copy that needs them
@@ -382,7 +402,8 @@ k_head_dense(const HeadArgs a, Ctrl* ctrl, float* __restrict__ recs, const Dense
     } else if (warp == 1) {
         // ================= MMA issuer (leader CTA only) ================================================
         if (rank == 0 && elect_one()) {
-            const uint32_t idesc = make_idesc(PAIR ? 2 * kBM : kBM, bn);
+            const int bn0 = SPLIT ? geo.bn0 : bn;                               // columns of the (first) MMA
+            const uint32_t idesc = make_idesc(PAIR ? 2 * kBM : kBM, bn0), idesc1 = make_idesc(kBM, max(bn - bn0, 16));
             const uint64_t desc_a0 = make_desc(ring_u32);                       // (the ring is 1024-byte aligned and under 256 KB:
             const uint64_t sub16 = (uint64_t)(((uint32_t)geo.stage_bytes / (uint32_t)geo.sub) >> 4);   //  adding byte offsets >> 4 stays inside the address field)
             int s = 0, t_local = 0;
@@ -413,6 +434,9 @@ k_head_dense(const HeadArgs a, Ctrl* ctrl, float* __restrict__ recs, const Dense
                                 const uint64_t step = (uint64_t)u * sub16 + (uint64_t)(k * 2);
                                 if (PAIR) tc_mma_pair(d_tmem, da0 + step, db0 + step, idesc, (kc | u | k) != 0 ? 1u : 0u);
                                 else tc_mma(d_tmem, da0 + step, db0 + step, idesc, (kc | u | k) != 0 ? 1u : 0u);
+                                if (SPLIT && bn > bn0)
+                                    tc_mma(d_tmem + kHalfCols, da0 + step - (uint64_t)(kRows * kBK * 2 >> 4),
+                                           db0 + step + (uint64_t)(bn0 * kBK * 2 >> 4), idesc1, (kc | u | k) != 0 ? 1u : 0u);
                             }
                         }
                     }
@@ -436,13 +460,17 @@ k_head_dense(const HeadArgs a, Ctrl* ctrl, float* __restrict__ recs, const Dense
         // ================= epilogue warps: one hidden row and one share of the tile's columns per thread =
         const int ew = warp - 2;
         const int quad = warp & 3;                            // TMEM lanes this warp may read
-        const int part = ew >> 2;                             // which share of the tile's chunks
+        const int half = SPLIT ? quad >> 1 : 0;               // which columns the quadrant has
+        const int row0 = SPLIT ? (quad & 1) * 32 : quad * 32; // first of its hidden rows
+        const int share = half * kParts + (ew >> 2);          // which of the row's columns this warp takes
         const int rows = min(B - (int)rank * kBM, kBM);       // hidden rows of this CTA
-        const int n_ch_tile = bn / kCh;
-        const int ch_lo = part * n_ch_tile / PARTS, ch_hi = (part + 1) * n_ch_tile / PARTS;
-        const int b = (int)rank * kBM + quad * 32 + lane;
+        const int n_ch = bn / kCh, n_ch0 = SPLIT ? geo.bn0 / kCh : n_ch;
+        const int ch0 = half ? n_ch0 : 0, n_mine = half ? n_ch - n_ch0 : n_ch0;
+        const int ch_lo = ch0 + (ew >> 2) * n_mine / kParts, ch_hi = ch0 + ((ew >> 2) + 1) * n_mine / kParts;
+        const int col_off = half ? kHalfCols - geo.bn0 : 0;   // from a column of the tile to its place in the accumulator stage
+        const int b = (int)rank * kBM + row0 + lane;
         const bool row_live = b < B;
-        if (quad * 32 < rows) {
+        if (row0 < rows) {
             griddep_wait();                                   // temp, uniforms and the record scratch belong to earlier work until here
             float invT = 0.f;
             if (row_live) {
@@ -453,12 +481,11 @@ k_head_dense(const HeadArgs a, Ctrl* ctrl, float* __restrict__ recs, const Dense
             st.m = -CUDART_INF_F; st.s = 0.f; st.gb_s = -CUDART_INF_F; st.gb_z = 0.f; st.gb_j = -1;
 #pragma unroll
             for (int i = 0; i < KT; ++i) { st.tv[i] = (i < KT - topk) ? CUDART_INF_F : -CUDART_INF_F; st.tj[i] = -1; }
-            constexpr int kEntStride = 4 * PARTS * 32;
-            float2* ent = reinterpret_cast<float2*>(ring + geo.ring_bytes) + part * kBM + quad * 32 + lane;
+            float2* ent = reinterpret_cast<float2*>(entries) + share * kRows + row0 + lane;
             const bool vec_u = a.uniforms && ((K & 3) == 0) && ((reinterpret_cast<uintptr_t>(a.uniforms) & 15) == 0);
             const bool use_u = row_live && a.uniforms != nullptr;
             const uint32_t acc_empty_bar = PAIR ? mapa_u32(smem_u32(&s_acc_empty[0]), 0) : 0u;
-            const uint32_t tmem_row = tmem_base + ((uint32_t)(quad * 32) << 16);
+            const uint32_t tmem_row = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)col_off;
             // The warp's chunks one after the other, through all tiles: a chunk's uniforms are requested when the one before it has
             // used its own.
             float u[kCh];
@@ -707,21 +734,21 @@ k_head_dense(const HeadArgs a, Ctrl* ctrl, float* __restrict__ recs, const Dense
                 // the column shares of a row meet in shared memory: lists where the thread's entries were, the rest in the ring
                 // (idle by now: the last accumulators were complete, so every MMA has read its operands and every copy has landed)
                 unsigned long long* klist = reinterpret_cast<unsigned long long*>(ent);
-                float* xch = reinterpret_cast<float*>(ring) + part * kBM + quad * 32 + lane;
+                float* xch = reinterpret_cast<float*>(ring) + share * kRows + row0 + lane;
 #pragma unroll
-                for (int o = 1; o < PARTS; o <<= 1) {
-                    if ((part & (2 * o - 1)) == o && ok) {
+                for (int o = 1; o < kShares; o <<= 1) {
+                    if ((share & (2 * o - 1)) == o && ok) {
 #pragma unroll
                         for (int i = 0; i < KT; ++i) klist[((i + topk) & (KT - 1)) * kEntStride] = i < KT - topk ? 0ull : key[i];
                         xch[0] = st.m; xch[kEntStride] = st.s; xch[2 * kEntStride] = st.gb_s;
                         xch[3 * kEntStride] = __int_as_float(st.gb_j); xch[4 * kEntStride] = st.gb_z;
                     }
                     asm volatile("bar.sync 1, %0;" ::"r"(live_warps(rows) * 32) : "memory");
-                    if ((part & (2 * o - 1)) == 0 && ok) {
-                        const float* x = xch + o * kBM;
+                    if ((share & (2 * o - 1)) == 0 && ok) {
+                        const float* x = xch + o * kRows;
                         unsigned long long other[KT];
 #pragma unroll
-                        for (int i = 0; i < KT; ++i) other[i] = klist[i * kEntStride + o * kBM];
+                        for (int i = 0; i < KT; ++i) other[i] = klist[i * kEntStride + o * kRows];
                         lse_merge(st.m, st.s, x[0], x[kEntStride]);
                         const float os = x[2 * kEntStride];
                         const int oj = __float_as_int(x[3 * kEntStride]);
@@ -731,12 +758,12 @@ k_head_dense(const HeadArgs a, Ctrl* ctrl, float* __restrict__ recs, const Dense
                 }
             }
 
-            if ((PAIR || part == 0) && ok && row_live) {
+            if ((PAIR || share == 0) && ok && row_live) {
                 // ---- the record of hidden row b: this CTA's, or this share's of the pair's columns (a pair leaves two per row, which
                 // the merge takes as well as one)
                 unsigned long long* kp = rec_keys(recs, b, topk);
                 float* fp = rec_f32(recs, b, topk);
-                const int c = PAIR ? group * PARTS + part : group;
+                const int c = PAIR ? group * kParts + share : group;
                 fp[c] = st.m;
                 fp[kMaxGrid + c] = st.s;
                 fp[2 * kMaxGrid + c] = st.gb_z;
@@ -844,9 +871,12 @@ DenseGeo make_geo(int32_t K, int32_t d, bool pair, int h_rows, int max_groups, s
     g.n_kc = (d + kBK - 1) / kBK;
     g.n_groups = g.n_tiles < max_groups ? g.n_tiles : max_groups;
     g.h_rows = h_rows;
-    // (the MMA reads 128 hidden rows from here: beyond those that exist whatever follows, behind the ring's end the entries)
+    // (the MMA reads 128 hidden rows from here: beyond those that exist whatever follows)
     g.h_bytes = (int)align_up((size_t)h_rows * kBK * 2, 1024);
     const int step_bytes = g.h_bytes + (pair ? g.bn / 2 : g.bn) * kBK * 2;
+    g.bn0 = (g.bn / 2 + 15) / 16 * 16;
+    g.tail_bytes = kBM * kBK * 2 > step_bytes ? kBM * kBK * 2 - step_bytes : 0;
+    ring_budget -= (size_t)g.tail_bytes;
     g.sub = (3 * kMaxSub * (size_t)step_bytes <= ring_budget && g.n_kc >= kMaxSub) ? kMaxSub : 1;
     g.stage_bytes = step_bytes * g.sub;
     g.n_stages = (int)(ring_budget / (size_t)g.stage_bytes);
@@ -855,31 +885,31 @@ DenseGeo make_geo(int32_t K, int32_t d, bool pair, int h_rows, int max_groups, s
     return g;
 }
 
-// shared memory of the candidate entries; also room for the operand rows that the last stage's MMAs read beyond it
-template <int KT, int PARTS>
-constexpr size_t entry_bytes() { return (size_t)KT * 4 * PARTS * 32 * sizeof(float2); }
-static_assert(entry_bytes<8, 2>() >= (size_t)kBM * kBK * 2, "128 operand rows from the ring's end on lie inside");
+// shared memory of the candidate entries (in front of the ring: also what a split tile's second operand reads before it)
+template <int KT>
+constexpr size_t entry_bytes() { return (size_t)KT * kParts * kBM * sizeof(float2); }
+static_assert(entry_bytes<8>() >= (size_t)kBM / 2 * kBK * 2 && entry_bytes<8>() % 1024 == 0, "64 operand rows before the ring lie inside");
 
-template <int KT, bool PAIR, int PARTS>
+template <int KT, bool PAIR, bool SPLIT>
 cudaError_t launch_variant(const HeadArgs& a, Ctrl* ctrl, float* recs, int max_groups, int* records, cudaStream_t s) {
-    constexpr size_t kEntries = entry_bytes<KT, PARTS>();
+    constexpr size_t kEntries = entry_bytes<KT>();
     const DenseGeo geo = make_geo(a.K, a.d, PAIR, PAIR ? kBM : a.B, max_groups, kSmemBudget - kEntries);
     CUtensorMap tm_h, tm_w;
     if (!encode_map(&tm_h, a.h, a.B, a.d, geo.h_rows) || !encode_map(&tm_w, a.W, a.K, a.d, PAIR ? geo.bn / 2 : geo.bn))
         return cudaErrorInvalidValue;
     static int attr_done[64] = {0};
-    const size_t smem = (size_t)geo.ring_bytes + kEntries + 1024;   // + slack to align the ring to 1024 bytes
+    const size_t smem = (size_t)geo.ring_bytes + kEntries + geo.tail_bytes + 1024;   // + slack to align the ring to 1024 bytes
     int dev = 0;
     cudaGetDevice(&dev);
     if (dev < 0 || dev >= 64 || !attr_done[dev]) {
-        cudaError_t e = cudaFuncSetAttribute(k_head_dense<KT, PAIR, PARTS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        cudaError_t e = cudaFuncSetAttribute(k_head_dense<KT, PAIR, SPLIT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              (int)(kSmemBudget + 1024));
         if (e != cudaSuccess) return e;
         if (dev >= 0 && dev < 64) attr_done[dev] = 1;
     }
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)(PAIR ? 2 * geo.n_groups : geo.n_groups));
-    cfg.blockDim = dim3((2 + 4 * PARTS) * 32);
+    cfg.blockDim = dim3((2 + 4 * kParts) * 32);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
     cudaLaunchAttribute at[2];
@@ -891,8 +921,8 @@ cudaError_t launch_variant(const HeadArgs& a, Ctrl* ctrl, float* recs, int max_g
     at[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
     cfg.numAttrs = a.overlap ? 2 : 1;
-    *records = PAIR ? geo.n_groups * PARTS : geo.n_groups;
-    return cudaLaunchKernelEx(&cfg, k_head_dense<KT, PAIR, PARTS>, a, ctrl, recs, geo, tm_h, tm_w);
+    *records = PAIR ? geo.n_groups * kParts : geo.n_groups;
+    return cudaLaunchKernelEx(&cfg, k_head_dense<KT, PAIR, SPLIT>, a, ctrl, recs, geo, tm_h, tm_w);
 }
 
 }  // namespace
@@ -924,15 +954,13 @@ cudaError_t launch_head_dense(const HeadArgs& a, Ctrl* ctrl, uint8_t* scratch, c
     float* recs = reinterpret_cast<float*>(scratch);
     cudaError_t e;
     int records = 0;
-    // Up to 64 rows half of the lane quadrants hold none: twice the warps on the others (above that two shares are as fast, 100 rows
-    // of 20001 x 3072 43.7 against 46.1 us).
-    const bool few = a.B <= 64;
-    if (a.topk <= 8) e = pair ? launch_variant<8, true, 2>(a, ctrl, recs, max_groups, &records, s)
-                       : few  ? launch_variant<8, false, 4>(a, ctrl, recs, max_groups, &records, s)
-                              : launch_variant<8, false, 2>(a, ctrl, recs, max_groups, &records, s);
-    else e = pair ? launch_variant<kMaxTopk, true, 2>(a, ctrl, recs, max_groups, &records, s)
-           : few  ? launch_variant<kMaxTopk, false, 4>(a, ctrl, recs, max_groups, &records, s)
-                  : launch_variant<kMaxTopk, false, 2>(a, ctrl, recs, max_groups, &records, s);
+    const bool split = a.B <= kBM / 2;
+    if (a.topk <= 8) e = pair  ? launch_variant<8, true, false>(a, ctrl, recs, max_groups, &records, s)
+                       : split ? launch_variant<8, false, true>(a, ctrl, recs, max_groups, &records, s)
+                               : launch_variant<8, false, false>(a, ctrl, recs, max_groups, &records, s);
+    else e = pair  ? launch_variant<kMaxTopk, true, false>(a, ctrl, recs, max_groups, &records, s)
+           : split ? launch_variant<kMaxTopk, false, true>(a, ctrl, recs, max_groups, &records, s)
+                   : launch_variant<kMaxTopk, false, false>(a, ctrl, recs, max_groups, &records, s);
     if (e != cudaSuccess) return e;
     count_launch();
     return launch_head_merge(a, ctrl, recs, records, s);
