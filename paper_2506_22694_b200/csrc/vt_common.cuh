@@ -124,7 +124,7 @@ cudaError_t launch_head_skinny(const HeadArgs& a, Ctrl* ctrl, uint8_t* scratch, 
 size_t head_stamps_offset(int32_t B, int32_t topk);   // offset of the phase stamps in the scratch of either head
 #endif
 
-cudaError_t launch_head_merge(const HeadArgs& a, Ctrl* ctrl, float* recs, int G, cudaStream_t s);
+cudaError_t launch_head_merge(const HeadArgs& a, Ctrl* ctrl, float* recs, int G, bool lean, cudaStream_t s);
 
 bool head_dense_supported(int32_t B, int32_t K, int32_t d);
 bool head_dense_topk_ok(int32_t topk);

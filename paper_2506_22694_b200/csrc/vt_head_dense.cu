@@ -803,7 +803,12 @@ k_head_dense(const HeadArgs a, Ctrl* ctrl, float* __restrict__ recs, const Dense
 // chained step, two warps per row and a round trip more / this: one row of 5000 x 1024 9.7 / 8.7, of 32768 x 3072 31.6 / 30.5, 8
 // rows of 9973 x 3072 17.6 / 16.7, 100 rows of 20001 x 3072 37.3 / 35.3.
 constexpr int kFuseNodes = 64;                                    // new nodes that the last block expands (see launch_head_merge)
-__global__ void __launch_bounds__(kMergeThreads)
+// LEAN: 32 registers, with spills, where the head's CTAs have eighteen warps of 96 (9 to 64 rows of the streaming kernel): beside five
+// of those in a quarter of the register file there is room for one warp of 32 and none of 48, and a merge that does not find
+// its seat early starts 1.5-2 us late (48 / 32 registers, us per step: 12 rows of 4757 x 2048 15.4 / 13.2, 10 rows of 9973 x 3072 19.2 /
+// 17.7, 24 rows of 5000 x 2048 17.1 / 15.6; beside the other heads the spills show: 8 rows of 9973 x 3072 16.2 / 16.8).
+template <bool LEAN>
+__global__ void __launch_bounds__(kMergeThreads, LEAN ? 10 : 1)
 k_head_merge(const HeadArgs a, Ctrl* ctrl, float* __restrict__ recs, int G, int fuse) {
     extern __shared__ __align__(16) float s_stage[];              // [kMergeStageWords], and over it the keys of the expansion
     __shared__ float s_xch;
@@ -963,11 +968,11 @@ cudaError_t launch_head_dense(const HeadArgs& a, Ctrl* ctrl, uint8_t* scratch, c
                    : launch_variant<kMaxTopk, false, false>(a, ctrl, recs, max_groups, &records, s);
     if (e != cudaSuccess) return e;
     count_launch();
-    return launch_head_merge(a, ctrl, recs, records, s);
+    return launch_head_merge(a, ctrl, recs, records, false, s);
 }
 
 // The records of G CTAs (pairs) -> outputs; with a tree, its expansion as one more launch (it needs every row's merge).
-cudaError_t launch_head_merge(const HeadArgs& a, Ctrl* ctrl, float* recs, int G, cudaStream_t s) {
+cudaError_t launch_head_merge(const HeadArgs& a, Ctrl* ctrl, float* recs, int G, bool lean, cudaStream_t s) {
     // the merge always follows its own producer closely: it takes its seats early and waits on the device
     const int n_new = a.B * a.topk;
     // The expansion inside the merge saves a launch; as a kernel of its own it has more threads, and the blocks need not meet.  Up to
@@ -976,7 +981,10 @@ cudaError_t launch_head_merge(const HeadArgs& a, Ctrl* ctrl, float* recs, int G,
     const bool fuse = a.tree.pool_token && n_new <= kFuseNodes;
     size_t smem = (size_t)kMergeStageWords * 4;
     if (fuse && (size_t)padded_keys(n_new) * 8 > smem) smem = (size_t)padded_keys(n_new) * 8;
-    const cudaError_t e = launch_dependent(k_head_merge, (unsigned)a.B, kMergeThreads, smem, s, a, ctrl, recs, G, fuse ? 1 : 0);
+    // (in front of an expansion kernel the early seat does not pay: 10 rows of 32768 x 4096 six depths deep 305 us without, 312 with it)
+    lean = lean && (!a.tree.pool_token || fuse);
+    const cudaError_t e = lean ? launch_dependent(k_head_merge<true>, (unsigned)a.B, kMergeThreads, smem, s, a, ctrl, recs, G, fuse ? 1 : 0)
+                               : launch_dependent(k_head_merge<false>, (unsigned)a.B, kMergeThreads, smem, s, a, ctrl, recs, G, fuse ? 1 : 0);
     if (e != cudaSuccess || !a.tree.pool_token || fuse) return e;
     return launch_tree_expand(a.out_ids, a.out_logprobs, a.B, a.topk, 1 + a.topk, 1, a.tree, s);
 }

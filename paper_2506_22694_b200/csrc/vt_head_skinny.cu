@@ -876,7 +876,7 @@ cudaError_t launch_head_skinny(const HeadArgs& a, Ctrl* ctrl, uint8_t* scratch, 
                         : a.B <= 32 ? launch_variant<16, 2, false>(a, ctrl, recs, geo, tm_h, tm_w, smem, s)
                                     : launch_variant<16, 4, false>(a, ctrl, recs, geo, tm_h, tm_w, smem, s);
     if (e != cudaSuccess) return e;
-    return launch_head_merge(a, ctrl, recs, geo.grid, s);
+    return launch_head_merge(a, ctrl, recs, geo.grid, a.B > 8, s);
 }
 
 }  // namespace vt
