@@ -25,10 +25,11 @@ __device__ __forceinline__ bool better(float v, int j, float bv, int bj) {
     return v > bv || (v == bv && j < bj);
 }
 
-// (m, s) <- (m, s) (+) (m2, s2) for running max / sum of exponentials
+// (m, s) <- (m, s) (+) (m2, s2) for running max / sum of exponentials.  (A NaN is left out of the maximum and lives in the sum, also
+// where neither side has a maximum: 0 + 0 stays 0, NaN stays NaN.)
 __device__ __forceinline__ void lse_merge(float& m, float& s, float m2, float s2) {
     const float M = fmaxf(m, m2);
-    if (M == -CUDART_INF_F) { m = M; s = 0.f; return; }
+    if (M == -CUDART_INF_F) { m = M; s = s + s2; return; }
     s = s * __expf(m - M) + s2 * __expf(m2 - M);
     m = M;
 }

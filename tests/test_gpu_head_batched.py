@@ -34,10 +34,13 @@ def _check(h, W, T, topk, u, flags=0):
         top = score.max(dim=1).values
         mine = score.gather(1, ids[:, :1].long().clamp(min=0))[:, 0]
         live = top > -float("inf")
-        slack = 2.0 ** -20 + (ranked.double().abs().amax(dim=1).clamp(max=1e30)) * 2.0 ** -23
+        size = torch.where(torch.isfinite(ranked), ranked.abs(), torch.zeros_like(ranked)).double().amax(dim=1)
+        slack = 2.0 ** -20 + size * 2.0 ** -23
         assert bool(((ids[:, 0] >= 0) == live).all())
-        ok = (top - mine <= slack) | (top == mine)
+        ok = torch.where(torch.isinf(top), top == mine, top - mine <= slack)       # (a winner of +inf: one of +inf)
         assert bool(ok[live].all())
+    # a NaN logit leaves no log-sum-exp, and neither does +inf (inf - inf)
+    assert torch.equal(torch.isnan(lse), (torch.isnan(z) | (z == float("inf"))).any(dim=1))
     got_flags = ws.read_status()[1]
     assert got_flags == flags, got_flags
     again = vt.vt_draft_head(h, W, None, T, topk, u, ws=ws, overlapped=True)
@@ -90,6 +93,23 @@ def test_infinite_and_nan_logits(B, K):
     _check(h, W, T, 8, u, flags=vt.VT_FLAG_NAN_ROW)
     W[K - 3, 0] = 0
     _check(h, W, T, 8, None, flags=vt.VT_FLAG_NAN_ROW)
+
+
+@pytest.mark.parametrize("B,K", [
+    (8, 19_953), (10, 129),                                            # streaming
+    (33, 17), (40, 19_953), (64, 33),                                  # the last column alone in a half of its tile, the other share empty
+    (65, 17), (100, 2369), (128, 145),                                 # alone in the last tile
+    (129, 33), (200, 2369), (256, 4737),                               # pairs
+])
+def test_a_nan_or_minus_infinity_alone_in_the_last_column(B, K):
+    """Beside shares of a tile that have no column at all, or none but -inf."""
+    h, W, T, u = _inputs(B, K, 64, True, seed=B + 1)
+    W[K - 1] = float("nan")
+    _check(h, W, T, 8, None, flags=vt.VT_FLAG_NAN_ROW)
+    _check(h, W, T, 8, u, flags=vt.VT_FLAG_NAN_ROW)
+    W[:, 0], W[K - 1], h[:, 0] = 0, 0, 1
+    W[K - 1, 0] = float("-inf")                                        # (no candidate, and nothing of the sum)
+    _check(h, W, T, 8, u)
 
 
 def test_uniforms_at_and_beyond_their_range_and_unaligned():
