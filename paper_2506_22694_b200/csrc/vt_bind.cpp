@@ -83,6 +83,23 @@ void expect_args(Py_ssize_t n, Py_ssize_t want) {
     if (n != want) raise(PyExc_TypeError, "expected %zd arguments, got %zd", want, n);
 }
 
+// The interpreter's lock given up for a scope (an exception that leaves it has the lock again).
+struct Unlocked {
+    PyThreadState* state = PyEval_SaveThread();
+    Unlocked() = default;
+    Unlocked(const Unlocked&) = delete;
+    Unlocked& operator=(const Unlocked&) = delete;
+    ~Unlocked() { PyEval_RestoreThread(state); }
+};
+
+// A call into the library without the lock.  Its arguments are plain pointers and numbers, all of them made before the lock is given
+// up: a tensor may refuse its data pointer, which raises.
+template <class F, class... A>
+int call(F* function, A... arguments) {
+    const Unlocked u;
+    return function(arguments...);
+}
+
 // the parts of a tuple or list, checked for their number as Python's unpacking does
 struct Parts {
     Ref seq;
@@ -117,8 +134,11 @@ struct Space {
     }
 };
 
+// (without the lock, as torch.empty: an allocation may wait for the device)
 at::Tensor make(const at::Tensor& like, at::ScalarType dtype, at::IntArrayRef shape) {
-    return at::empty(shape, like.options().dtype(dtype).requires_grad(false));
+    const at::TensorOptions options = like.options().dtype(dtype).requires_grad(false);
+    const Unlocked u;
+    return at::empty(shape, options);
 }
 
 // what a head call takes, checked
@@ -176,11 +196,6 @@ struct Pool {
     }
 };
 
-#define VT_CALL(status, ...)      \
-    Py_BEGIN_ALLOW_THREADS        \
-    status = __VA_ARGS__;         \
-    Py_END_ALLOW_THREADS
-
 // (h, W_trim, map, temp, topk, uniforms, ws, out, overlapped)
 PyObject* draft_head(PyObject*, PyObject* const* a, Py_ssize_t n) {
     HANDLE_TH_ERRORS
@@ -193,10 +208,9 @@ PyObject* draft_head(PyObject*, PyObject* const* a, Py_ssize_t n) {
     const int overlapped = PyObject_IsTrue(a[8]);
     if (overlapped < 0) raise();
     void* s = stream();
-    int status;
-    VT_CALL(status, (overlapped ? g_head_overlapped : g_head)(data<uint16_t>(in.h), data<uint16_t>(in.W), in.map, (int32_t)in.B, (int32_t)in.K,
+    const int status = call(overlapped ? g_head_overlapped : g_head, data<uint16_t>(in.h), data<uint16_t>(in.W), in.map, (int32_t)in.B, (int32_t)in.K,
                                                               (int32_t)in.d, data<float>(in.temp), (int32_t)in.topk, in.u, ids, lps,
-                                                              ws.ptr, ws.bytes, s));
+                                                              ws.ptr, ws.bytes, s);
     if (status != VT_OK) return PyLong_FromLong(status);
     return PyTuple_Pack(2, out.ids.p, out.lps.p);
     END_HANDLE_TH_ERRORS
@@ -218,11 +232,10 @@ PyObject* draft_head_expand(PyObject*, PyObject* const* a, Py_ssize_t n) {
     const Space ws(a[10], VT_OP_DRAFT_HEAD, a[0], 0, 0, in.K, in.d, in.B, in.topk);
     const int32_t* frontier = data_of<int32_t>(a[6]);
     void* s = stream();
-    int status;
-    VT_CALL(status, g_expand(data<uint16_t>(in.h), data<uint16_t>(in.W), in.map, (int32_t)in.B, (int32_t)in.K, (int32_t)in.d,
+    const int status = call(g_expand, data<uint16_t>(in.h), data<uint16_t>(in.W), in.map, (int32_t)in.B, (int32_t)in.K, (int32_t)in.d,
                              data<float>(in.temp), (int32_t)in.topk, in.u, ids, lps, frontier, data<int32_t>(pool.token),
                              data<int32_t>(pool.parent), data<float>(pool.score), (int32_t)base, (int32_t)pool.capacity, (int32_t)n_front,
-                             data<int32_t>(next), ws.ptr, ws.bytes, s));
+                             data<int32_t>(next), ws.ptr, ws.bytes, s);
     if (status != VT_OK) return PyLong_FromLong(status);
     Ref nx(THPVariable_Wrap(next));
     if (!nx.p) raise();
@@ -242,8 +255,7 @@ PyObject* draft_head_host(PyObject*, PyObject* const* a, Py_ssize_t n) {
     int32_t* ids = data_of<int32_t>(a[9]);
     float* lps = data_of<float>(a[10]);
     void* s = stream();
-    int status;
-    VT_CALL(status, g_head_host(h, W, map, B, K, d, temp, topk, u, ids, lps, ws.ptr, ws.bytes, s));
+    const int status = call(g_head_host, h, W, map, B, K, d, temp, topk, u, ids, lps, ws.ptr, ws.bytes, s);
     return PyLong_FromLong(status);
     END_HANDLE_TH_ERRORS
 }
@@ -258,9 +270,8 @@ PyObject* tree_rerank(PyObject*, PyObject* const* a, Py_ssize_t n) {
     at::Tensor t[3];
     for (at::Tensor& x : t) x = make(pool.token, at::kInt, {budget});
     void* s = stream();
-    int status;
-    VT_CALL(status, g_rerank(data<int32_t>(pool.token), data<int32_t>(pool.parent), data<float>(pool.score), (int32_t)nodes, (int32_t)budget,
-                             data<int32_t>(t[0]), data<int32_t>(t[1]), data<int32_t>(t[2]), s));
+    const int status = call(g_rerank, data<int32_t>(pool.token), data<int32_t>(pool.parent), data<float>(pool.score), (int32_t)nodes, (int32_t)budget,
+                             data<int32_t>(t[0]), data<int32_t>(t[1]), data<int32_t>(t[2]), s);
     if (status != VT_OK) return PyLong_FromLong(status);
     Ref r0(THPVariable_Wrap(t[0])), r1(THPVariable_Wrap(t[1])), r2(THPVariable_Wrap(t[2]));
     if (!r0.p || !r1.p || !r2.p) raise();
@@ -285,9 +296,8 @@ PyObject* verify_greedy(PyObject*, PyObject* const* a, Py_ssize_t n) {
     const int32_t* parent = data_of<int32_t>(a[1]);
     uint64_t* total = data_of<uint64_t>(a[3]);
     void* s = stream();
-    int status;
-    VT_CALL(status, g_verify(data<int32_t>(token), parent, data<int32_t>(target), (int32_t)S, (int32_t)N, data<int32_t>(n_accept),
-                             data<int32_t>(path), data<int32_t>(emitted), total, s));
+    const int status = call(g_verify, data<int32_t>(token), parent, data<int32_t>(target), (int32_t)S, (int32_t)N, data<int32_t>(n_accept),
+                             data<int32_t>(path), data<int32_t>(emitted), total, s);
     if (status != VT_OK) return PyLong_FromLong(status);
     Ref r0(THPVariable_Wrap(n_accept)), r1(THPVariable_Wrap(path)), r2(THPVariable_Wrap(emitted));
     if (!r0.p || !r1.p || !r2.p) raise();
@@ -304,8 +314,7 @@ PyObject* build_vocab(PyObject*, PyObject* const* a, Py_ssize_t n) {
     const at::Tensor map = make(ids, at::kInt, {K}), inv = make(ids, at::kInt, {V});
     const Space ws(a[3], VT_OP_BUILD_VOCAB, a[0], count, V, K, 0, 0, 0);
     void* s = stream();
-    int status;
-    VT_CALL(status, g_build(data<int32_t>(ids), count, (int32_t)V, (int32_t)K, data<int32_t>(map), data<int32_t>(inv), ws.ptr, ws.bytes, s));
+    const int status = call(g_build, data<int32_t>(ids), count, (int32_t)V, (int32_t)K, data<int32_t>(map), data<int32_t>(inv), ws.ptr, ws.bytes, s);
     if (status != VT_OK) return PyLong_FromLong(status);
     Ref r0(THPVariable_Wrap(map)), r1(THPVariable_Wrap(inv));
     if (!r0.p || !r1.p) raise();
@@ -334,8 +343,7 @@ PyObject* trim_head(PyObject*, PyObject* const* a, Py_ssize_t n) {
         ws = pointer(p.p);
     }
     void* s = stream();
-    int status;
-    VT_CALL(status, g_trim(data<uint16_t>(W), data<int32_t>(map), data<uint16_t>(trim), (int32_t)V, (int32_t)K, (int32_t)d, ws, s));
+    const int status = call(g_trim, data<uint16_t>(W), data<int32_t>(map), data<uint16_t>(trim), (int32_t)V, (int32_t)K, (int32_t)d, ws, s);
     if (status != VT_OK) return PyLong_FromLong(status);
     Py_INCREF(out.p);
     return out.p;
