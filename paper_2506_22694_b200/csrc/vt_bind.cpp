@@ -100,16 +100,17 @@ int call(F* function, A... arguments) {
     return function(arguments...);
 }
 
-// the parts of a tuple or list, checked for their number as Python's unpacking does
+// the parts of a tuple or list, checked for their number as Python's unpacking does, and kept (a list may lose them meanwhile)
 struct Parts {
-    Ref seq;
+    Ref own[3];
     PyObject* at[3];
-    Parts(PyObject* o, Py_ssize_t want) : seq(PySequence_Fast(o, "cannot unpack non-iterable object")) {
+    Parts(PyObject* o, Py_ssize_t want) {
+        const Ref seq(PySequence_Fast(o, "cannot unpack non-iterable object"));
         if (!seq.p) raise();
         const Py_ssize_t n = PySequence_Fast_GET_SIZE(seq.p);
         if (n < want) raise(PyExc_ValueError, "not enough values to unpack (expected %zd, got %zd)", want, n);
         if (n > want) raise(PyExc_ValueError, "too many values to unpack (expected %zd)", want);
-        for (Py_ssize_t i = 0; i < want; ++i) at[i] = PySequence_Fast_GET_ITEM(seq.p, i);
+        for (Py_ssize_t i = 0; i < want; ++i) Py_INCREF(own[i].p = at[i] = PySequence_Fast_GET_ITEM(seq.p, i));
     }
 };
 

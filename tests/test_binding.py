@@ -1,5 +1,6 @@
 """The C++ marshalling of the Python calls, without a GPU: fake tensors on a CUDA device and recorded calls in the library's place."""
 import ctypes
+import weakref
 
 import pytest
 import torch
@@ -125,3 +126,19 @@ def test_a_pool_or_outputs_of_another_number_of_parts_are_refused(calls, parts):
         with pytest.raises(ValueError):
             vt.vt_draft_head(a["h"], a["W"], None, a["temp"], 8, ws=Space(), out=[a["ids"]] * parts)
     assert not calls
+
+
+def test_a_pool_given_as_a_list_is_kept_while_the_call_runs(calls):
+    a = _cases()["expand"][1]()
+    pool = [a.pop("token"), a.pop("parent"), a.pop("score")]
+    refs, alive = [weakref.ref(t) for t in pool], []
+
+    class Emptying(Space):
+        @property
+        def ptr(self):                                      # runs in the middle of the call, as another thread may
+            pool.clear()
+            alive.append([r() is not None for r in refs])
+            return 4096
+
+    vt.vt_draft_head_expand(a["h"], a["W"], a["map"], a["temp"], 8, a["u"], None, pool, 0, 8, ws=Emptying(), out=(a["ids"], a["lps"]))
+    assert alive == [[True] * 3] and len(calls) == 1
