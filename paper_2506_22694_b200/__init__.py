@@ -95,7 +95,8 @@ def lib() -> ctypes.CDLL:
                                "`python -m paper_2506_22694_b200.build` (%s)" % e) from e
         bind.use({name: ctypes.cast(getattr(L, name), c_void_p).value for name in _BOUND}, _make_workspace,
                  torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice)
-        _lib, _bind = L, bind
+        _bind = bind
+        _lib = L                                   # (last: where it is set, another thread takes both for loaded)
     return _lib
 
 

@@ -44,16 +44,31 @@ def needs_build(lib: str = LIB) -> bool:
     return any(os.path.getmtime(p) > t for p in _deps())
 
 
+def bind_for() -> str:
+    """The Python and torch that an extension module built now is for."""
+    import torch
+
+    return "%s, torch %s, C++ ABI %d" % (sys.implementation.cache_tag, torch.__version__, torch._C._GLIBCXX_USE_CXX11_ABI)
+
+
+def bind_fresh() -> bool:
+    """Whether the module is younger than its sources and says that it was built for this Python and torch."""
+    newest = max(os.path.getmtime(p) for p in (BIND_SRC, os.path.join(ROOT, "include", "vocabtrim.h")))
+    if not os.path.exists(BIND) or os.path.getmtime(BIND) <= newest:
+        return False
+    with open(BIND, "rb") as f:
+        return b"_vt_bind for " + bind_for().encode() + b"\0" in f.read()
+
+
 def build_bind(force: bool = False) -> str:
     """Compile the binding's extension module; its objects come from torch, already loaded when it is imported."""
-    header = os.path.join(ROOT, "include", "vocabtrim.h")
-    if not force and os.path.exists(BIND) and os.path.getmtime(BIND) > max(os.path.getmtime(BIND_SRC), os.path.getmtime(header)):
+    if not force and bind_fresh():
         return BIND
     import torch
 
     top = os.path.dirname(torch.__file__)
     tmp = BIND + ".%d.tmp" % os.getpid()
-    subprocess.check_call([os.environ.get("CXX", "g++"), "-std=c++17", "-O2", "-fPIC", "-shared",
+    subprocess.check_call([os.environ.get("CXX", "g++"), "-std=c++17", "-O2", "-fPIC", "-shared", '-DVT_BIND_FOR="%s"' % bind_for(),
                            "-D_GLIBCXX_USE_CXX11_ABI=%d" % torch._C._GLIBCXX_USE_CXX11_ABI, "-I", os.path.join(ROOT, "include"),
                            "-isystem", sysconfig.get_paths()["include"], "-isystem", os.path.join(top, "include"),
                            BIND_SRC, "-o", tmp, "-L", os.path.join(top, "lib"), "-lc10", "-ltorch_cpu", "-ltorch_python"])

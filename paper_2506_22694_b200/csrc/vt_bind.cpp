@@ -385,7 +385,26 @@ PyModuleDef g_module = {PyModuleDef_HEAD_INIT, "_vt_bind", "Argument marshalling
 
 }  // namespace
 
+// What the module was compiled for: its view of torch's and Python's objects is theirs only.  (VT_BIND_FOR comes from build.py, which also
+// looks for this text in the file to know whether it is up to date.)
+static const char kFor[] = "_vt_bind for " VT_BIND_FOR;
+
+static bool fits() {
+    Ref torch(PyImport_ImportModule("torch")), sys(PyImport_ImportModule("sys"));
+    Ref core(torch.p ? PyObject_GetAttrString(torch.p, "_C") : nullptr), impl(sys.p ? PyObject_GetAttrString(sys.p, "implementation") : nullptr);
+    if (!core.p || !impl.p) return false;
+    Ref tag(PyObject_GetAttrString(impl.p, "cache_tag")), version(PyObject_GetAttrString(torch.p, "__version__"));
+    Ref abi(PyObject_GetAttrString(core.p, "_GLIBCXX_USE_CXX11_ABI"));
+    if (!tag.p || !version.p || !abi.p) return false;
+    Ref now(PyUnicode_FromFormat("_vt_bind for %S, torch %S, C++ ABI %d", tag.p, version.p, PyObject_IsTrue(abi.p)));
+    if (!now.p) return false;
+    if (PyUnicode_CompareWithASCIIString(now.p, kFor) == 0) return true;
+    PyErr_Format(PyExc_ImportError, "built as %s, this is %U", kFor, now.p);
+    return false;
+}
+
 PyMODINIT_FUNC PyInit__vt_bind() {
+    if (!fits()) return nullptr;
     s_ptr = PyUnicode_InternFromString("ptr");
     s_nbytes = PyUnicode_InternFromString("nbytes");
     return s_ptr && s_nbytes ? PyModule_Create(&g_module) : nullptr;

@@ -1,5 +1,9 @@
 """The C++ marshalling of the Python calls, without a GPU: fake tensors on a CUDA device and recorded calls in the library's place."""
 import ctypes
+import os
+import shutil
+import subprocess
+import sys
 import weakref
 
 import pytest
@@ -7,6 +11,7 @@ import torch
 from torch._subclasses.fake_tensor import FakeTensorMode
 
 import paper_2506_22694_b200 as vt
+from paper_2506_22694_b200 import build as vt_build
 
 pytestmark = pytest.mark.filterwarnings("ignore:Accessing the data pointer of FakeTensor")
 I32, F32, BF16 = torch.int32, torch.float32, torch.bfloat16
@@ -142,3 +147,22 @@ def test_a_pool_given_as_a_list_is_kept_while_the_call_runs(calls):
 
     vt.vt_draft_head_expand(a["h"], a["W"], a["map"], a["temp"], 8, a["u"], None, pool, 0, 8, ws=Emptying(), out=(a["ids"], a["lps"]))
     assert alive == [[True] * 3] and len(calls) == 1
+
+
+def test_a_module_for_another_torch_is_built_anew(monkeypatch, tmp_path):
+    copy = str(tmp_path / "_vt_bind.so")
+    shutil.copyfile(vt_build.BIND, copy)
+    monkeypatch.setattr(vt_build, "BIND", copy)
+    asked = []
+    monkeypatch.setattr(vt_build.subprocess, "check_call", lambda cmd: asked.append(cmd) or shutil.copyfile(copy, cmd[cmd.index("-o") + 1]))
+    vt_build.build_bind()
+    assert not asked
+    monkeypatch.setattr(torch, "__version__", "0.0.1")
+    vt_build.build_bind()
+    assert len(asked) == 1 and any("torch 0.0.1" in a for a in asked[0])
+
+
+def test_a_module_for_another_torch_is_not_loaded():
+    code = "import torch; torch.__version__ = '0.0.1'; import paper_2506_22694_b200 as vt; vt.lib()"
+    r = subprocess.run([sys.executable, "-c", code], cwd=os.path.dirname(os.path.dirname(os.path.abspath(__file__))), capture_output=True, text=True)
+    assert r.returncode != 0 and "built for another Python or torch" in r.stderr and "this is" in r.stderr
