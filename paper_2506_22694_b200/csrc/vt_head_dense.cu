@@ -20,7 +20,7 @@
 // the epilogue of tile t overlaps the MMAs of tile t+1.  tcgen05.commit releases ring stages and
 // publishes accumulators (to both CTAs of a pair).  Eight epilogue warps read the accumulators back
 // with tcgen05.ld -- TMEM lane = hidden row; the two warps of a lane quadrant take one half of a tile's
-// columns each (up to 64 rows a tile is computed in two halves, on lanes of their own) -- 16 columns at a time: running max /
+// columns each (up to 64 rows a wide tile is computed in two halves, on lanes of their own) -- 16 columns at a time: running max /
 // sum-exp of z = logit / T_b, Gumbel-max candidate from the caller's uniforms, and a sorted top-k list kept in registers.
 // Logits never go to HBM.  The column shares of a row are merged through shared memory (a pair's two shares leave a record
 // each); per CTA and hidden row one record goes to scratch; a second small kernel (six warps per hidden row) merges the
@@ -34,6 +34,7 @@
 // any of this / now (the merge's share included): 40 rows of 20001 x 3072 41.3 / 31.9, 64 rows 42.7 / 33.5, 100 rows 46.2 / 34.8,
 // 90 rows of 10000 x 4096 with top-10 43.7 / 27.2, 256 rows of 32768 x 4096 74.5 / 72.2.
 #include <cfloat>
+#include <cmath>
 
 #include "vt_common.cuh"
 #include "vt_head_common.cuh"
@@ -249,7 +250,7 @@ __device__ __forceinline__ void merge_desc(T (&list)[N], const T (&v)[A]) {
 
 // KT: capacity of the list (8 or kMaxTopk).  PAIR: two CTAs of a cluster form one MMA.  Two epilogue warps per TMEM lane
 // quadrant, each with a contiguous share of the quadrant's 16-column chunks.  Warps whose lanes hold no hidden row leave at once.
-// SPLIT (up to 64 hidden rows): an MMA's first 64 rows are the hidden rows and its second 64 nobody's, and a quadrant's warps sit on
+// SPLIT (up to 64 hidden rows, tiles of kSplitCols columns and more): an MMA's first 64 rows are the hidden rows and its second 64 nobody's, and a quadrant's warps sit on
 // one scheduler, so half of them would do the whole epilogue.  So a tile's columns are computed in two halves: one with the
 // hidden rows as rows 0-63, the other with the operand's start 64 rows earlier, which makes them rows 64-127; each half
 // of the lanes then has half of the columns (in TMEM kHalfCols apart) and all eight warps work.  (40 rows of 20001 x 3072, four
@@ -403,7 +404,7 @@ k_head_dense(const HeadArgs a, Ctrl* ctrl, float* __restrict__ recs, const Dense
         // ================= MMA issuer (leader CTA only) ================================================
         if (rank == 0 && elect_one()) {
             const int bn0 = SPLIT ? geo.bn0 : bn;                               // columns of the (first) MMA
-            const uint32_t idesc = make_idesc(PAIR ? 2 * kBM : kBM, bn0), idesc1 = make_idesc(kBM, max(bn - bn0, 16));
+            const uint32_t idesc = make_idesc(PAIR ? 2 * kBM : kBM, bn0), idesc1 = make_idesc(kBM, SPLIT ? bn - bn0 : 16);
             const uint64_t desc_a0 = make_desc(ring_u32);                       // (the ring is 1024-byte aligned and under 256 KB:
             const uint64_t sub16 = (uint64_t)(((uint32_t)geo.stage_bytes / (uint32_t)geo.sub) >> 4);   //  adding byte offsets >> 4 stays inside the address field)
             int s = 0, t_local = 0;
@@ -434,7 +435,7 @@ k_head_dense(const HeadArgs a, Ctrl* ctrl, float* __restrict__ recs, const Dense
                                 const uint64_t step = (uint64_t)u * sub16 + (uint64_t)(k * 2);
                                 if (PAIR) tc_mma_pair(d_tmem, da0 + step, db0 + step, idesc, (kc | u | k) != 0 ? 1u : 0u);
                                 else tc_mma(d_tmem, da0 + step, db0 + step, idesc, (kc | u | k) != 0 ? 1u : 0u);
-                                if (SPLIT && bn > bn0)
+                                if (SPLIT)
                                     tc_mma(d_tmem + kHalfCols, da0 + step - (uint64_t)(kRows * kBK * 2 >> 4),
                                            db0 + step + (uint64_t)(bn0 * kBK * 2 >> 4), idesc1, (kc | u | k) != 0 ? 1u : 0u);
                             }
@@ -859,19 +860,45 @@ k_head_merge(const HeadArgs a, Ctrl* ctrl, float* __restrict__ recs, int G, int 
 }
 
 // ---- host side ----------------------------------------------------------------------------------------
-// Tile width: the vocabulary is dealt to `groups` CTAs (pairs) in tiles of bn rows; the slowest group
-// works ceil(tiles / groups) * bn rows.  Smallest such makespan wins, the wider tile on equal terms
-// (fewer re-reads of the hidden rows).  Multiples of 16 (136 rows per CTA of 20001: 144 instead of 160); a pair takes multiples
-// of 32, with others its MMAs are several times slower (200 rows of 50001 x 3072, 240 columns: 318 us instead of 122).
-DenseGeo make_geo(int32_t K, int32_t d, bool pair, int h_rows, int max_groups, size_t ring_budget) {
-    DenseGeo g{};
-    long best = -1;
-    const int by = pair ? 32 : 16;
+// Tile width: the vocabulary is dealt to `groups` CTAs (pairs) in tiles of bn rows.  A CTA's time is that of its tiles -- what it takes
+// from HBM (its rows of W, and the uniforms of its columns) or, where that is longer, what it stages through L2 (those and all hidden
+// rows again, per tile), and the turn-around of a tile and of its steps -- and of the last tile's epilogue, which nothing hides.  The
+// rates are a CTA's share with all SMs at work, fitted to 2500 timed pairs of shape and width (3000 to 111000 rows, d = 512 to 4096, 33 to
+// 256 hidden rows): the width they choose was within 2 % of the best of them in the median.  Evening out the rows per CTA alone, as
+// this did before, takes 16 columns for one K in five, and each such tile brings the hidden rows again (us per call, even rows / this,
+// with uniforms: 100 hidden rows of 40000 x 3072 152 / 53, of 95000 x 3072 386 / 108, 40 of 40000 x 2048 137 / 37; pairs: 200 of
+// 95000 x 3072 395 / 150, 256 of 40000 x 1024 72 / 47).  On equal terms the wider tile.  Multiples of 16, for a pair of 32: the columns
+// of an MMA over two CTAs come in those.
+struct TileCost {
+    double hbm, staged;                   // bytes / ns
+    double tile, step, column;            // ns per tile, per 64-column step, per column of the last epilogue
+};
+constexpr TileCost kCostSplit{41., 90., 200., 10., 10.}, kCostNarrow{41., 90., 800., 10., 20.}, kCostSingle{44., 90., 400., 10., 20.},
+    kCostPair{41., 120., 1800., 5., 60.};
+// Columns from which a tile of up to 64 hidden rows is computed in two halves.  Its MMAs are twice as many, and one takes some 40 cycles
+// however few its columns; what the second set of lanes saves is epilogue, by the column (us per call, one / two halves: 40 rows of
+// 3000 x 3072 in tiles of 32 16.7 / 21.9, of 9973 x 4096 in 80 24.3 / 28.8, of 14000 x 1024 in 96 16.5 / 17.6, in 112 16.3 / 16.2, of
+// 16668 x 3072 in 128 29.1 / 28.2, of 20001 x 2048 in 160 25.4 / 24.3, of 60000 x 1024 in 208 41.7 / 34.4).
+constexpr int kSplitCols = 112;
+
+int tile_width(int32_t B, int32_t K, int32_t d, bool sampled, int max_groups) {
+    const bool pair = B > kBM;
+    const int by = pair ? 32 : 16, h_rows = pair ? kBM : B, n_kc = (d + kBK - 1) / kBK;
+    int best_bn = kMaxBN;
+    double best = -1.;
     for (int bn = kMaxBN; bn >= by; bn -= by) {
-        const long tiles = (K + bn - 1) / bn;
-        const long span = ((tiles + max_groups - 1) / max_groups) * bn;
-        if (best < 0 || span < best) { best = span; g.bn = bn; }
+        const TileCost& c = pair ? kCostPair : B > kBM / 2 ? kCostSingle : bn >= kSplitCols ? kCostSplit : kCostNarrow;
+        const int tiles = (K + bn - 1) / bn, own = (tiles + max_groups - 1) / max_groups, w_rows = pair ? bn / 2 : bn;
+        const double hbm = 2. * w_rows * d + (sampled ? 4. * bn * h_rows : 0.), staged = 2. * (h_rows + w_rows) * d;
+        const double ns = own * (fmax(hbm / c.hbm, staged / c.staged) + c.tile + c.step * n_kc) + c.column * bn;
+        if (best < 0. || ns < best) { best = ns; best_bn = bn; }
     }
+    return best_bn;
+}
+
+DenseGeo make_geo(int32_t K, int32_t d, bool pair, int h_rows, int bn, int max_groups, size_t ring_budget) {
+    DenseGeo g{};
+    g.bn = bn;
     g.n_tiles = (K + g.bn - 1) / g.bn;
     g.n_kc = (d + kBK - 1) / kBK;
     g.n_groups = g.n_tiles < max_groups ? g.n_tiles : max_groups;
@@ -896,9 +923,9 @@ constexpr size_t entry_bytes() { return (size_t)KT * kParts * kBM * sizeof(float
 static_assert(entry_bytes<8>() >= (size_t)kBM / 2 * kBK * 2 && entry_bytes<8>() % 1024 == 0, "64 operand rows before the ring lie inside");
 
 template <int KT, bool PAIR, bool SPLIT>
-cudaError_t launch_variant(const HeadArgs& a, Ctrl* ctrl, float* recs, int max_groups, int* records, cudaStream_t s) {
+cudaError_t launch_variant(const HeadArgs& a, Ctrl* ctrl, float* recs, int bn, int max_groups, int* records, cudaStream_t s) {
     constexpr size_t kEntries = entry_bytes<KT>();
-    const DenseGeo geo = make_geo(a.K, a.d, PAIR, PAIR ? kBM : a.B, max_groups, kSmemBudget - kEntries);
+    const DenseGeo geo = make_geo(a.K, a.d, PAIR, PAIR ? kBM : a.B, bn, max_groups, kSmemBudget - kEntries);
     CUtensorMap tm_h, tm_w;
     if (!encode_map(&tm_h, a.h, a.B, a.d, geo.h_rows) || !encode_map(&tm_w, a.W, a.K, a.d, PAIR ? geo.bn / 2 : geo.bn))
         return cudaErrorInvalidValue;
@@ -959,13 +986,14 @@ cudaError_t launch_head_dense(const HeadArgs& a, Ctrl* ctrl, uint8_t* scratch, c
     float* recs = reinterpret_cast<float*>(scratch);
     cudaError_t e;
     int records = 0;
-    const bool split = a.B <= kBM / 2;
-    if (a.topk <= 8) e = pair  ? launch_variant<8, true, false>(a, ctrl, recs, max_groups, &records, s)
-                       : split ? launch_variant<8, false, true>(a, ctrl, recs, max_groups, &records, s)
-                               : launch_variant<8, false, false>(a, ctrl, recs, max_groups, &records, s);
-    else e = pair  ? launch_variant<kMaxTopk, true, false>(a, ctrl, recs, max_groups, &records, s)
-           : split ? launch_variant<kMaxTopk, false, true>(a, ctrl, recs, max_groups, &records, s)
-                   : launch_variant<kMaxTopk, false, false>(a, ctrl, recs, max_groups, &records, s);
+    const int bn = tile_width(a.B, a.K, a.d, a.uniforms != nullptr, max_groups);
+    const bool split = a.B <= kBM / 2 && bn >= kSplitCols;
+    if (a.topk <= 8) e = pair  ? launch_variant<8, true, false>(a, ctrl, recs, bn, max_groups, &records, s)
+                       : split ? launch_variant<8, false, true>(a, ctrl, recs, bn, max_groups, &records, s)
+                               : launch_variant<8, false, false>(a, ctrl, recs, bn, max_groups, &records, s);
+    else e = pair  ? launch_variant<kMaxTopk, true, false>(a, ctrl, recs, bn, max_groups, &records, s)
+           : split ? launch_variant<kMaxTopk, false, true>(a, ctrl, recs, bn, max_groups, &records, s)
+                   : launch_variant<kMaxTopk, false, false>(a, ctrl, recs, bn, max_groups, &records, s);
     if (e != cudaSuccess) return e;
     count_launch();
     return launch_head_merge(a, ctrl, recs, records, false, s);

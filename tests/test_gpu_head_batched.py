@@ -56,11 +56,14 @@ def _inputs(B, K, d, sample, seed):
 
 
 @pytest.mark.parametrize("B,K,d,topk,sample", [
-    (33, 17, 64, 16, True), (64, 2369, 128, 8, True), (65, 2369, 128, 7, True),                  # tiles of 16 columns: one chunk, empty shares
-    (40, 20_001, 256, 8, True), (63, 37_888, 64, 1, False), (64, 37_889, 64, 9, True),           # one tile per CTA, the widest, two
-    (96, 20_004, 192, 8, True), (97, 19_999, 192, 16, True), (128, 80_001, 64, 3, True),         # three and four quadrants, three tiles
+    (33, 17, 64, 16, True), (64, 2369, 128, 8, True), (65, 2369, 128, 7, True),                  # tiles of 16 and 32 columns: one chunk, empty shares
+    (40, 20_001, 256, 8, True), (63, 37_888, 64, 1, False), (64, 37_889, 64, 9, True),           # halved tiles: one per CTA, two, a last one of 17
+    (48, 14_200, 512, 8, True), (40, 16_576, 64, 16, False), (50, 14_208, 1024, 7, True),        # the narrowest that are halved
+    (64, 11_840, 64, 8, True), (33, 9973, 512, 16, True), (45, 3476, 512, 1, False),             # up to 64 rows in one piece
+    (96, 20_004, 192, 8, True), (97, 19_999, 192, 16, True), (128, 80_001, 64, 3, True),         # three and four quadrants, three tiles and more
     (129, 2368, 128, 8, True), (129, 2369, 72, 16, True), (160, 18_944, 64, 8, False),           # pairs: second CTA with one row and with 32
-    (161, 18_945, 64, 10, True), (255, 60_000, 64, 8, True), (256, 33_000, 136, 5, True),        # one, two and four tiles
+    (161, 18_945, 64, 10, True), (255, 60_000, 64, 8, True), (256, 33_000, 136, 5, True),        # three to seven tiles
+    (100, 37_000, 1024, 8, True), (64, 60_000, 512, 8, True), (256, 33_000, 2048, 8, True),      # two and three wide ones
 ])
 def test_lists_and_samples_follow_from_the_logits(B, K, d, topk, sample):
     h, W, T, u = _inputs(B, K, d, sample, seed=B + K)
