@@ -55,6 +55,11 @@ constexpr int kTmemCols = 512;            // 2 accumulator stages x kMaxBN colum
 constexpr int kMaxTopk = 16;              // the list's values live in registers
 constexpr unsigned long long kWaitLimitNs = 2000000000ull;
 constexpr size_t kSmemBudget = 225 * 1024;   // ring and candidate entries at most (227 KB per CTA less alignment slack and statics)
+// What of it a pair leaves to L1 where the uniforms come one by one (K no multiple of four, or an unaligned pointer).  Sixteen loads then
+// share the 256 lines of the eight epilogue warps, 32 KB; beside more than 196 KB of shared memory L1 has 28 KB, and 60 beside this
+// (us per call, 28 / 60 KB: 256 rows of 33001 x 2048 69.3 / 49.5, of 15073 x 1024 38.4 / 28.3, of 7142 x 512 24.2 / 19.1, of 32769 x 4096
+// 75.8 / 70.9; up to 128 rows no difference).
+constexpr size_t kL1Room = 32 * 1024;
 
 // Phase stamps (-DVT_STAMPS builds only): one thread per role writes %globaltimer into a region behind the
 // records; bench.py --case stamps reads them back.  Slots per CTA: 0 entry, 1 set up (barriers, tensor
@@ -175,6 +180,11 @@ struct DenseGeo {
     int sub;          // d-steps per ring stage (1 or 2): one wait and one release per stage, so two steps per stage halve
                       // what the two single threads that drive the ring spend per MMA; taken when three such stages fit
 };
+
+// Rows of uniforms that 16-byte loads can read.
+__host__ __device__ __forceinline__ bool uniforms_aligned(const float* u, int K) {
+    return (K & 3) == 0 && (reinterpret_cast<uintptr_t>(u) & 15) == 0;
+}
 
 // Per-thread state of one hidden row over the columns the thread has seen.
 template <int KT>
@@ -483,7 +493,7 @@ k_head_dense(const HeadArgs a, Ctrl* ctrl, float* __restrict__ recs, const Dense
 #pragma unroll
             for (int i = 0; i < KT; ++i) { st.tv[i] = (i < KT - topk) ? CUDART_INF_F : -CUDART_INF_F; st.tj[i] = -1; }
             float2* ent = reinterpret_cast<float2*>(entries) + share * kRows + row0 + lane;
-            const bool vec_u = a.uniforms && ((K & 3) == 0) && ((reinterpret_cast<uintptr_t>(a.uniforms) & 15) == 0);
+            const bool vec_u = a.uniforms && uniforms_aligned(a.uniforms, K);
             const bool use_u = row_live && a.uniforms != nullptr;
             const uint32_t acc_empty_bar = PAIR ? mapa_u32(smem_u32(&s_acc_empty[0]), 0) : 0u;
             const uint32_t tmem_row = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)col_off;
@@ -925,7 +935,8 @@ static_assert(entry_bytes<8>() >= (size_t)kBM / 2 * kBK * 2 && entry_bytes<8>() 
 template <int KT, bool PAIR, bool SPLIT>
 cudaError_t launch_variant(const HeadArgs& a, Ctrl* ctrl, float* recs, int bn, int max_groups, int* records, cudaStream_t s) {
     constexpr size_t kEntries = entry_bytes<KT>();
-    const DenseGeo geo = make_geo(a.K, a.d, PAIR, PAIR ? kBM : a.B, bn, max_groups, kSmemBudget - kEntries);
+    const bool one_by_one = a.uniforms && !uniforms_aligned(a.uniforms, a.K);
+    const DenseGeo geo = make_geo(a.K, a.d, PAIR, PAIR ? kBM : a.B, bn, max_groups, kSmemBudget - kEntries - (PAIR && one_by_one ? kL1Room : 0));
     CUtensorMap tm_h, tm_w;
     if (!encode_map(&tm_h, a.h, a.B, a.d, geo.h_rows) || !encode_map(&tm_w, a.W, a.K, a.d, PAIR ? geo.bn / 2 : geo.bn))
         return cudaErrorInvalidValue;
