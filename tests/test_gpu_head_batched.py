@@ -115,6 +115,16 @@ def test_a_nan_or_minus_infinity_alone_in_the_last_column(B, K):
     _check(h, W, T, 8, u)
 
 
+@pytest.mark.parametrize("B,K", [(33, 14_209), (64, 4738), (70, 20_003), (130, 9474), (256, 7143)])
+@pytest.mark.parametrize("shift", [0, 1, 2, 3])
+def test_uniforms_at_every_offset_from_a_16_byte_boundary(B, K, shift):
+    """Rows of every remainder, in a buffer that begins at any of the four places and ends with the last row."""
+    h, W, T, u = _inputs(B, K, 128, True, seed=K + shift)
+    flat = torch.empty(B * K + shift, device=DEV)
+    flat[shift:].view(B, K).copy_(u)
+    _check(h, W, T, 8, flat[shift:].view(B, K))
+
+
 def test_uniforms_at_and_beyond_their_range_and_unaligned():
     B, K = 70, 20_003
     h, W, T, u = _inputs(B, K, 64, True, seed=9)
