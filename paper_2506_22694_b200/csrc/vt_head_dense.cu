@@ -885,7 +885,7 @@ struct TileCost {
     double tile, step, column;            // ns per tile, per 64-column step, per column of the last epilogue
 };
 constexpr TileCost kCostSplit{41., 90., 200., 10., 10.}, kCostNarrow{41., 90., 800., 10., 20.}, kCostSingle{44., 90., 400., 10., 20.},
-    kCostPair{41., 120., 1800., 5., 60.};
+    kCostPair{44., 160., 1800., 5., 20.};
 // Columns from which a tile of up to 64 hidden rows is computed in two halves.  Its MMAs are twice as many, and one takes some 40 cycles
 // however few its columns; what the second set of lanes saves is epilogue, by the column (us per call, one / two halves: 40 rows of
 // 3000 x 3072 in tiles of 32 16.7 / 21.9, of 9973 x 4096 in 80 24.3 / 28.8, of 14000 x 1024 in 96 16.5 / 17.6, in 112 16.3 / 16.2, of
