@@ -57,9 +57,9 @@ constexpr unsigned long long kWaitLimitNs = 2000000000ull;
 constexpr size_t kSmemBudget = 225 * 1024;   // ring and candidate entries at most (227 KB per CTA less alignment slack and statics)
 // What of it a pair leaves to L1 where the uniforms come one by one (K no multiple of four, or an unaligned pointer).  Sixteen loads then
 // share the 256 lines of the eight epilogue warps, 32 KB; beside more than 196 KB of shared memory L1 has 28 KB, and 60 beside this.
-// Over a long d the shorter ring costs more than that, but for the widest tiles (us per call, 28 / 60 KB: 256 rows of 33001 x 2048
-// 69.3 / 49.5, of 16573 x 1536 41.6 / 28.8, of 9109 x 3072 30.9 / 28.8, of 18941 x 4096 54.9 / 50.4; of 4735 x 4096 24.9 / 27.5, of 11801 x 4096
-// 36.4 / 37.6; up to 128 rows no difference).
+// Over a long d a single narrow tile has its noise made behind its MMAs, and the shorter ring costs more than that (us per call, 28 / 60
+// KB: 256 rows of 33001 x 2048 69.3 / 49.5, of 16573 x 1536 41.6 / 28.8, of 9109 x 3072 30.9 / 28.8, of 18941 x 4096 54.9 / 50.4; of 4735 x
+// 4096 24.9 / 27.5, of 11801 x 4096 36.4 / 37.6; up to 128 rows no difference).
 constexpr size_t kL1Room = 32 * 1024;
 
 // Phase stamps (-DVT_STAMPS builds only): one thread per role writes %globaltimer into a region behind the
@@ -936,7 +936,7 @@ static_assert(entry_bytes<8>() >= (size_t)kBM / 2 * kBK * 2 && entry_bytes<8>() 
 template <int KT, bool PAIR, bool SPLIT>
 cudaError_t launch_variant(const HeadArgs& a, Ctrl* ctrl, float* recs, int bn, int max_groups, int* records, cudaStream_t s) {
     constexpr size_t kEntries = entry_bytes<KT>();
-    const bool one_by_one = a.uniforms && !uniforms_aligned(a.uniforms, a.K) && (a.d <= 3072 || bn >= 224);
+    const bool one_by_one = a.uniforms && !uniforms_aligned(a.uniforms, a.K) && (a.d <= 3072 || bn >= 224 || a.K > bn * max_groups);
     const DenseGeo geo = make_geo(a.K, a.d, PAIR, PAIR ? kBM : a.B, bn, max_groups, kSmemBudget - kEntries - (PAIR && one_by_one ? kL1Room : 0));
     CUtensorMap tm_h, tm_w;
     if (!encode_map(&tm_h, a.h, a.B, a.d, geo.h_rows) || !encode_map(&tm_w, a.W, a.K, a.d, PAIR ? geo.bn / 2 : geo.bn))
