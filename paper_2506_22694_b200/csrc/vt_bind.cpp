@@ -1,6 +1,6 @@
 // Argument marshalling of the calls that a drafting loop or a vocabulary build makes, as a CPython extension: the checks, the outputs'
-// allocation and the call into libvocabtrim.so, without Python in between.  A drafting step is 9 to 40 us on the device and
-// its call cost 7 us of Python (us per call on the host, Python / here: a head 12.9 / 8.5, a rerank 9.9 / 5.8); nothing of the method
+// allocation and the call into libvocabtrim.so, without Python in between.  A drafting step is 9 to 40 us on the device, and
+// Python marshalling added 4 us to a call on the host (us, Python / here: a head 12.9 / 8.5, a rerank 9.9 / 5.8); nothing of the method
 // happens here.  The functions of the library are registered by address (`use`), so that the library can be another build.
 //
 // Every function returns its outputs, or the library's status as an int when that is not VT_OK.

@@ -54,7 +54,7 @@ struct HistPlan {
     int parts;             // id ranges the packed kernel deals to different CTAs (0: not packed)
     size_t off_sample;     // uint32 [V]   sampled counts
     size_t off_packed;     // uint32 [V]   what the packed kernel counted (only when three bins per word fit)
-    size_t off_gate;       // uint32 [4]   {recount, -, skipped ids (64 bits)} of the packed kernel
+    size_t off_gate;       // uint32 [4]   {recount, CTAs that have recounted, skipped ids (64 bits)}
     size_t clear_bytes;    // the scratch prefix every call zeroes
     size_t off_table;      // uint2  [ceil(V/32)] hot-bin table {bitmap word, slot base}
     size_t bytes;          // scratch after the control block

@@ -141,7 +141,7 @@ __device__ __forceinline__ uint32_t merge_flag(const MergeOut& a, int b) {
 }
 
 // The merge of one hidden row by six warps.  A warp runs dependent code at a few cycles per instruction, and the row's result is what
-// the next step waits for, so the work is spread: five warps hold a CTA's list heads per lane (kRoleCand), the sixth the
+// the next step waits for, so the work is spread: five warps hold a CTA's list heads per lane, the sixth the
 // statistics (log-sum-exp over all CTAs, the Gumbel-max winner).  Everything a warp needs from memory is asked for at once.
 // (Two warps, five CTAs to a lane, took 4150 cycles from the records being there to the outputs, a quarter of them one L2 round
 // trip for the abort mark in front of the records and the gathers through the index mapper behind the ranking.)

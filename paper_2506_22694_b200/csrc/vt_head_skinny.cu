@@ -844,10 +844,12 @@ cudaError_t launch_variant(const HeadArgs& a, Ctrl* ctrl, float* recs, const Geo
 
 bool head_skinny_supported(int32_t B, int32_t d) { return shape_ok(B, d); }
 
-// Up to 32 rows this kernel is the faster one at every size (us per call, this / batched kernel: 24 rows of 5000 x 2048
-// 15.8 / 18.5, of 20001 x 3072 30.7 / 39.2, of 80000 x 3072 83 / 146).  From 33 to 64 its second pass over h for slabs of
-// more than 128 rows and four hidden rows per epilogue warp cost as much as the batched kernel's idle lanes: 40 rows of
-// 123 MB 40.4 / 39.6, of 268 MB 58.5 / 64.0, of 491 MB 99.5 / 146.5; the line is drawn between the first two.
+// Up to 32 rows the two kernels are within 11 % of one another (us per call, this / batched kernel, greedy: 24 rows of 5000 x 2048
+// 15.9 / 14.9, of 20001 x 3072 32.7 / 30.8, of 80000 x 3072 85.2 / 87.0; 32 rows of 32768 x 3072 41.6 / 43.4), and the smaller sums are this
+// one's advantage: it adds up phases of eight steps, and its logits' rms error is a tenth of the batched kernel's (2.6e-7 against
+// 3.6e-6 at 40 rows).  From 33 to 64 rows its second pass over h for slabs of more than 128 rows and four hidden rows per
+// epilogue warp make it the slower one throughout: 40 rows of 123 MB 39.9 / 33.1, of 201 MB 47.1 / 44.1, of 268 MB 58.8 / 53.9, of 491
+// MB 95.1 / 88.5.  It keeps the heads of 192 MB and more there for the sake of those logits.
 bool head_stream_takes(int32_t B, int32_t K, int32_t d) {
     return B >= 1 && (B <= 32 || (B <= kMaxB && (size_t)K * d * 2 >= ((size_t)192 << 20)));
 }

@@ -7,14 +7,14 @@
 //   * ceil(V / 3) * 4 bytes fit (Llama-3: 128256 bins = 171 KB)  -> every CTA still keeps all bins,
 //     three 10-bit fields to a word (k_hist_packed): one shared-memory add per token and nothing else.
 //     A field hands 512 counts on to global memory whenever it gets there; the add that would wrap a
-//     field notices, and the stream is then counted again by the kernels of the next case.
+//     field notices, and the stream is then counted again (the last two cases).
 //   * more bins than that, in two to four ranges that fit: the same kernel, every range dealt to its own share of
 //     the CTAs, each share reading the whole stream (the second and later readers find it in L2).
-//   * the recount, of shorter streams: ranges of 57344 32-bit bins, by the kernel that settles the packed count;
-//   * the recount of longer ones, and long streams over more bins than three counters per word hold: a short pre-pass samples the stream, picks the hottest bins that fit (about 49.8 K of
-//     them for 128256 bins), and the main pass keeps those in shared memory; the rare cold tokens go
-//     to L2 with one red.global each.  The hot set only steers traffic: counts are exact whichever
-//     bins were picked.
+//   * the recount of a shorter stream (kRangeIds): ranges of 57344 32-bit bins, by the kernel that settles the packed count;
+//   * the recount of a longer one, and the first count of a long stream over several ranges or of a vocabulary that no ranges hold
+//     (kSplitIds): a short pre-pass samples the stream, picks the hottest bins that fit (about 49.8 K of them for 128256
+//     bins), and the main pass keeps those in shared memory; the rare cold tokens go to L2 with one red.global each.
+//     The hot set only steers traffic: counts are exact whichever bins were picked.
 //       hot lookup: entry[id >> 4] = {16 membership bits, 16-bit slot of the group's first member};
 //       slot = base + popc(bits & below(id)), one 4-byte shared load per token.
 #include "vt_common.cuh"
@@ -457,8 +457,8 @@ k_hist_hot(const int32_t* __restrict__ ids, int64_t n, int32_t V, uint32_t* __re
 // token gets to kSpill first), and from then on a lane that meets it adds 1 to a 32-bit word of its own
 // instead (one per lane, so those adds never collide).  Until the hot id is known (kCarefulTrips trips)
 // every add is tested before the thread's next one is issued.  An add that finds kFieldMax in its field has
-// carried into the neighbour: it raises the gate, and the launcher's next kernels throw this count away
-// and count the stream again with the hot / cold kernels.
+// carried into the neighbour: it raises the gate, and the next kernel throws this count away and has the
+// stream counted again, by itself or, of a long one, by the hot / cold kernels.
 constexpr uint32_t kFieldBits = 10, kFieldMax = (1u << kFieldBits) - 1, kSpill = 512;
 constexpr uint32_t kNoId = 0xffffffffu;        // no token id: ids are tallied only when < V <= 2^31
 constexpr int kCarefulTrips = 2;               // trips a CTA counts one add at a time, until its hot id is known
@@ -955,7 +955,8 @@ cudaError_t launch_histogram(const int32_t* ids, int64_t n, int32_t V, uint32_t*
     // a refused launch must stop the chain: the main pass would count through an unwritten table
     const uint32_t* gate = nullptr;
     if (packed_path) {
-        // all bins in shared memory, packed; of the three kernels after it two return at once unless a field wrapped
+        // all bins in shared memory, packed; behind it one kernel that settles the count or recounts by ranges, or for a long stream
+        // three, of which the last two return at once unless a field wrapped
         uint32_t M = 0;
         int32_t Vp = V;
         const int parts = packed_parts(V, &Vp);

@@ -64,6 +64,7 @@ def _inputs(B, K, d, sample, seed):
     (129, 2368, 128, 8, True), (129, 2369, 72, 16, True), (160, 18_944, 64, 8, False),           # pairs: second CTA with one row and with 32
     (161, 18_945, 64, 10, True), (255, 60_000, 64, 8, True), (256, 33_000, 136, 5, True),        # three to seven tiles
     (100, 37_000, 1024, 8, True), (64, 60_000, 512, 8, True), (256, 33_000, 2048, 8, True),      # two and three wide ones
+    (140, 9475, 3080, 8, True), (140, 18_941, 3080, 16, True), (256, 16_573, 3080, 9, True),     # uneven uniforms over a long d: long and short ring
 ])
 def test_lists_and_samples_follow_from_the_logits(B, K, d, topk, sample):
     h, W, T, u = _inputs(B, K, d, sample, seed=B + K)
