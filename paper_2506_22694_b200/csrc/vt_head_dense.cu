@@ -874,12 +874,12 @@ k_head_merge(const HeadArgs a, Ctrl* ctrl, float* __restrict__ recs, int G, int 
 // Tile width: the vocabulary is dealt to `groups` CTAs (pairs) in tiles of bn rows.  A CTA's time is that of its tiles -- what it takes
 // from HBM (its rows of W, and the uniforms of its columns) or, where that is longer, what it stages through L2 (those and all hidden
 // rows again, per tile), and the turn-around of a tile and of its steps -- and of the last tile's epilogue, which nothing hides.  The
-// rates are a CTA's share with all SMs at work, fitted to 2500 timed pairs of shape and width (3000 to 111000 rows, d = 512 to 4096, 33 to
-// 256 hidden rows): the width they choose was within 2 % of the best of them in the median.  Evening out the rows per CTA alone, as
-// this did before, takes 16 columns for one K in five, and each such tile brings the hidden rows again (us per call, even rows / this,
-// with uniforms: 100 hidden rows of 40000 x 3072 152 / 53, of 95000 x 3072 386 / 108, 40 of 40000 x 2048 137 / 37; pairs: 200 of
-// 95000 x 3072 395 / 150, 256 of 40000 x 1024 72 / 47).  On equal terms the wider tile.  Multiples of 16, for a pair of 32: the columns
-// of an MMA over two CTAs come in those.
+// rates are a CTA's share with all SMs at work, fitted to 2500 timed widths of 183 shapes (3000 to 111000 rows, d = 512 to 4096, 33 to 256
+// hidden rows): the width they choose is the fastest one for half of the shapes and within 6 % of it for nine in ten.  Evening out the
+// rows per CTA alone, as this did before, takes 16 columns for one K in five, and each such tile brings the hidden rows again (us per
+// call, even rows / this, with uniforms: 100 hidden rows of 40000 x 3072 150 / 52, of 95000 x 3072 346 / 105, 40 of 40000 x 2048 137 / 37;
+// pairs: 200 of 95000 x 3072 306 / 141, 256 of 40000 x 1024 72 / 47).  On equal terms the wider tile.  Multiples of 16, for a pair of 32:
+// the columns of an MMA over two CTAs come in those.
 struct TileCost {
     double hbm, staged;                   // bytes / ns
     double tile, step, column;            // ns per tile, per 64-column step, per column of the last epilogue
